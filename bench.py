@@ -195,8 +195,8 @@ def run_reference(args):
     print(json.dumps(line), flush=True)
 
 
-OZ_DIGITS = 7  # base-2^7 digits of the fp64e step
-OZ_PRODUCTS = OZ_DIGITS * (OZ_DIGITS + 1) // 2  # BF16 digit products per tile (28)
+OZ_DIGITS = 5  # digits of the fp64e step (11, 8, 11, 9 and 11 bits)
+OZ_PRODUCTS = OZ_DIGITS * (OZ_DIGITS + 1) // 2  # FP16 digit products per tile (15)
 
 
 def tc_exec_flops(sizes, kstage, products, trim=False):
@@ -216,15 +216,15 @@ def tc_exec_flops(sizes, kstage, products, trim=False):
 def alg_flops(sizes, products=1):
     """Algorithmic flops of one symmetric squaring of every part: the upper triangle with the
     diagonal, s (s + 1) / 2 dot products of length s, 2 s flops each: s^2 (s + 1); the
-    tensor-core forms multiply it by their products per element (28 digit products, 3 for a
+    tensor-core forms multiply it by their products per element (15 digit products, 3 for a
     hi + lo split)."""
     import numpy as np
     return float(np.sum(sizes * sizes * (sizes + 1.0))) * products
 
 
 def fp64_roofline(precision, sizes, avg_launch_ms, peaks, src, workload):
-    """Roofline of one FP64-result step: native (FP64 pipe) or rebuilt from BF16 digits
-    (tensor pipe); `achieved` from the algorithmic flops s^2 (s+1) per part (times the 28
+    """Roofline of one FP64-result step: native (FP64 pipe) or rebuilt from FP16 digits
+    (tensor pipe); `achieved` from the algorithmic flops s^2 (s+1) per part (times the 15
     digit products for the emulated step), the emulated step's executed flops (128-tile
     padding, whole diagonal tiles) beside it."""
     import numpy as np
@@ -236,10 +236,10 @@ def fp64_roofline(precision, sizes, avg_launch_ms, peaks, src, workload):
         peak = peaks["bf16_tflops"]
         return {"bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
                 "traffic": TRAFFIC.get((workload, precision)),
-                "kernel": "oz_step_kernel (one FP64-accurate step: 28 BF16 digit products per upper tile, fused)",
+                "kernel": "oz_step_kernel (one FP64-accurate step: 15 FP16 digit products per upper tile, fused)",
                 "peak_source": f"{src}: bf16 burst (of measured)", "avg_launch_ms": avg_launch_ms,
                 "flops_per_launch": flops,
-                "flops": f"algorithmic: {OZ_PRODUCTS} BF16 digit products x s^2 (s+1) per part (upper triangle "
+                "flops": f"algorithmic: {OZ_PRODUCTS} FP16 digit products x s^2 (s+1) per part (upper triangle "
                          f"of X^2)",
                 "executed_flops_per_launch": exe, "executed_tflops": exe / t / 1e12,
                 "executed_frac": exe / t / 1e12 / peak}
@@ -382,7 +382,7 @@ def adjoint_block(dev, peaks, src, workload="tb4k", reps=3, precisions=("fp64", 
             flops = (2.0 * n + rebuilt) * alg_flops(sz, OZ_PRODUCTS)
             peak, psrc = peaks["bf16_tflops"], f"{src}: bf16 burst (of measured)"
             kern, fdesc = ("oz_step_kernel<adjoint> + oz_step_kernel recompute",
-                           f"algorithmic BF16 flops of the {OZ_PRODUCTS} digit products: reverse steps 2 s^2 (s+1), "
+                           f"algorithmic FP16 flops of the {OZ_PRODUCTS} digit products: reverse steps 2 s^2 (s+1), "
                            "rebuilt iterates s^2 (s+1), per part and product")
             bound = "tensor"
         elif prec == "fp32":
@@ -509,7 +509,7 @@ def run_ours(args):
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
         "warmup": warm, "ms_per_step": ms_per_step, "higher_is_better": True,
         "scaling": "weak", "vs_baseline": None,
-        "dtype": {"fp64": "f64", "fp64e": "f64 (bf16 digit products, int64 sums)"}.get(args.precision, args.precision),
+        "dtype": {"fp64": "f64", "fp64e": "f64 (fp16 digit products, int64 sums)"}.get(args.precision, args.precision),
         "data": "synthetic",
         "config": workload_config(args, s, sizes, world),
         "arith": args.precision, "sp2_steps": int(steps_applied),

@@ -66,8 +66,8 @@ typedef enum {
   GSP2_PREC_BF16 = 3,
   GSP2_PREC_BF16X3 = 4, /* split operands hi+lo in BF16, three products, FP32 accumulate */
   GSP2_PREC_TF32X3 = 5, /* split operands hi+lo in TF32, three products, FP32 accumulate */
-  GSP2_PREC_FP64_EMU = 6, /* FP64 results; every product X X rebuilt from 7 base-2^7 digits of X
-                             held in BF16 (28 exact BF16 tensor-core products per tile, groups
+  GSP2_PREC_FP64_EMU = 6, /* FP64 results; every product X X rebuilt from 5 digits of X (11, 8,
+                             11, 9 and 11 bits) held in FP16 (15 tensor-core products per tile, groups
                              summed as 64-bit fixed point), master copy in that fixed point */
   GSP2_PREC_FP16X3 = 7  /* split operands hi+lo in FP16 of X 2^14 (22 bits like TF32X3, entries
                            down to 2^-28 in FP16's normal range), three products at the
@@ -108,7 +108,7 @@ typedef struct {
   int32_t report_idem;     /* 1: after each density call, one extra FP64 pass over the final
                               iterates computes the idempotency report idem_fro (default 0) */
   int32_t fp64_tail_emulated; /* low-precision modes: 1 (default) runs the FP64 tail steps with
-                                 the products rebuilt from BF16 digits (as GSP2_PREC_FP64_EMU),
+                                 the products rebuilt from FP16 digits (as GSP2_PREC_FP64_EMU),
                                  0 on the FP64 units */
   int32_t tile_order;      /* order of the 128x128 tiles walked by the persistent kernels
                               (tensor-core steps with tc_schedule = 0, FP64_EMU steps): 0 = parts
@@ -131,9 +131,10 @@ typedef struct {
                               small problems); 0 = one item per tile; -1 (default) = 1 when the
                               plan has at most 512 upper 128-tiles.  Needs every part above 128
                               orbitals (else 0) and 2 x 128 KB of workspace per tile; gsp2_autotune
-                              may turn it off.  The 64-bit sums are exact; the group sums of each
-                              half are rounded in FP32 like the whole K's, so results agree to the
-                              last bits only */
+                              may turn it off.  The 64-bit sums are exact and, in plans of at most
+                              512 upper tiles, items of either kind round their FP32 sums at the
+                              same K, so both give the same bits (larger plans agree to the last
+                              few) */
   int32_t tile_claim;      /* persistent 128 x 128 steps (tensor-core steps and reverse steps, FP64_EMU
                               forward and reverse steps): 1 (default) = each CTA takes its first
                               tile by its index and claims every next one from a counter in the
@@ -322,7 +323,7 @@ gsp2_status gsp2_autotune(gsp2_handle h, const double* d_hvals, double* d_pvals,
  * held fixed).  X^2 steps map Xbar -> Xbar X + X Xbar, 2X - X^2 steps map
  * Xbar -> 2 Xbar - Xbar X - X Xbar; dX0/dH = -1/(eps_max - eps_min) (Eq. 1).
  * Iterates are recomputed from checkpoints kept every `ckpt_every` steps.  FP64 plans
- * run it on the FP64 pipe, FP64_EMU plans from BF16 digit products (Xbar's digits scaled
+ * run it on the FP64 pipe, FP64_EMU plans from FP16 digit products (Xbar's digits scaled
  * by a power of two per part taken from its row norms), the low-precision plans in FP32
  * with FP16 hi + lo products (Xbar's operands scaled by a power of two per part).
  *  d_pbar  device double[nnz_p]

@@ -35,8 +35,8 @@ struct WsLayout {
   size_t maps_mn;      // 16-bit kinds: the same with MN-major boxes (upper tiles only kept)
   size_t master_of_step;
   size_t d[2];         // FP64 arenas of the tail steps
-  // FP64 products from BF16 digits
-  size_t oz_slice[2][OZ_SLICES];  // BF16 digit arenas, two buffers (read / written by a step)
+  // FP64 products from FP16 digits
+  size_t oz_slice[2][OZ_SLICES];  // FP16 digit arenas, two buffers (read / written by a step)
   size_t oz_maps;                 // CUtensorMap[2][OZ_SLICES][nparts], K-major boxes
   size_t oz_maps_mn;              // the same, MN-major boxes
   size_t oz_acc;                  // int64[OZ_MAX_GRID][128 * 128] partial sums of the emulated step
@@ -107,9 +107,10 @@ struct gsp2_plan {
   std::vector<ColBlock> gblocks_ld;        // low-precision gather: every column up to ld
   int32_t nslots_tc = 0;
   int32_t total_steps = 0;  // FP64 path: max_steps + tail steps (static launches of a call)
-  bool use_oz = false;      // FP64 products from BF16 digits (fp64e steps or emulated tail steps)
+  bool use_oz = false;      // FP64 products from FP16 digits (fp64e steps or emulated tail steps)
   bool split_ok = false;    // emulated steps: buffers for split-K work items are in the workspace
   bool split_on = false;    // emulated steps split each tile's K into two work items
+  bool halves = false;      // unsplit items drain at the halves too: bitwise the sums of split ones
   std::vector<int64_t> pcolptr;
   std::vector<int32_t> prowind;
   int32_t nslots = 0, max_s = 0, min_s = 0;
@@ -185,7 +186,7 @@ static size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 constexpr int HIST_EXTRA = 16;
 constexpr int MAX_TAIL = 8;
 
-// FP64 results: native FP64 steps or FP64 products rebuilt from BF16 digits
+// FP64 results: native FP64 steps or FP64 products rebuilt from FP16 digits
 static bool fp64_like(int prec) { return prec == GSP2_PREC_FP64 || prec == GSP2_PREC_FP64_EMU; }
 
 // tensor-core operand kind (-1: FP32 CUDA cores, 0: BF16, 1: TF32, 2: FP16 of x 2^14) and
@@ -408,6 +409,8 @@ static void build_layout(gsp2_plan* h) {
   h->split_ok = h->opt.precision == GSP2_PREC_FP64_EMU && h->min_s > 128 &&
                 (h->opt.split_k == 1 || (h->opt.split_k < 0 && h->tc_tiles.size() <= 512));
   h->split_on = h->split_ok;
+  h->halves = h->split_ok ||
+              (h->opt.precision == GSP2_PREC_FP64_EMU && h->min_s > 128 && h->tc_tiles.size() <= 512);
   if (h->split_ok) {
     L.split_acc = take(2 * h->tc_tiles.size() * 128 * 128 * sizeof(long long));
     L.split_cnt = take(h->tc_tiles.size() * sizeof(uint32_t));
@@ -890,7 +893,7 @@ extern "C" gsp2_status gsp2_bind_workspace(gsp2_handle h, void* d_ws, size_t byt
       return fail(h, GSP2_E_CUDA, "cuTensorMapEncodeTiled not available from the driver");
     const size_t np = h->parts.size();
     // per digit set, K-major and MN-major maps whose boxes take all OZ_SLICES digits (the
-    // high pass) or the first OZ_SPLIT (the low pass) of a tile slice in one request; a set's
+    // high pass) or the first OZ_LOW (the low pass) of a tile slice in one request; a set's
     // digit arenas lie one arena apart (consecutive equal allocations)
     const size_t dstride = (size_t)h->arena_elems * 2;
     auto encode_set = [&](unsigned char* mk, unsigned char* mm, const size_t* dig) -> int {
@@ -900,7 +903,7 @@ extern "C" gsp2_status gsp2_bind_workspace(gsp2_handle h, void* d_ws, size_t byt
                                       OZ_SLICES, OZ_BK);
       if (r == 0)
         r = encode_part_maps_digits(enc, mk + np * 128, mm + np * 128, h->parts.data(), (int)np, h->ws + dig[0],
-                                    dstride, OZ_SLICES, OZ_SPLIT, OZ_BK);
+                                    dstride, OZ_SLICES, OZ_LOW, OZ_BK);
       return r;
     };
     std::vector<unsigned char> maps((size_t)2 * OZ_SLICES * np * 128, 0), maps_mn(maps.size(), 0);
@@ -1046,6 +1049,7 @@ static OzStepArgs oz_args(gsp2_plan* h, const StepCtl& ctl) {
   a.acc = (long long*)(w + L.oz_acc);
   a.ctl = ctl;
   a.tile_ctr = h->opt.tile_claim ? (uint32_t*)(w + L.tile_ctr) : nullptr;
+  a.halves = h->halves ? 1 : 0;
   if (h->split_on) {
     a.split = 1;
     a.split_acc = (long long*)(w + L.split_acc);
@@ -1204,7 +1208,7 @@ static gsp2_status enqueue_forward(gsp2_plan* h, const double* hv, double* pv, i
       CU(h, launch_square_tc(kind, nprod, a, a.ntiles, pgrid, s));
     }
     // FP64 tail: convert the last FP32 iterate, then purification steps in FP64 (native, or
-    // with the products rebuilt from BF16 digits); the conversions open the segment of the
+    // with the products rebuilt from FP16 digits); the conversions open the segment of the
     // first tail step (or the last segment when there is no tail)
     double* d[2] = {(double*)(w + L.d[0]), (double*)(w + L.d[1])};
     const int T = h->opt.fp64_tail_steps;

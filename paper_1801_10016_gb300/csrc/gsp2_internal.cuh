@@ -140,14 +140,14 @@ struct TcStepArgs {
 };
 constexpr int TC_SIG_MIN = -98, TC_SIG_MAX = 126;  // range of the FP16 adjoint's scale exponents
 
-// FP64 products rebuilt from BF16 digits (k_oz.cu)
-constexpr int OZ_SLICES = 7;  // base-2^7 digits per entry
-constexpr int OZ_SPLIT = 3;   // digit groups d < OZ_SPLIT form the second pass of a tile
+// FP64 products rebuilt from FP16 digits (k_oz.cu)
+constexpr int OZ_SLICES = 5;  // digits per entry (11, 8, 11, 11 and 11 bits)
+constexpr int OZ_LOW = 2;     // digits the second pass of a tile multiplies
 constexpr int OZ_MAX_GRID = 256;  // CTAs of the emulated step (one 128x128 int64 scratch each)
 constexpr int OZ_BK = 32;         // K per pipeline stage of the emulated step (64-byte rows)
 
 struct OzSlices {
-  uint16_t* s[OZ_SLICES];  // BF16 digit arenas (same element indexing as the arenas)
+  uint16_t* s[OZ_SLICES];  // FP16 digit arenas (same element indexing as the arenas)
 };
 
 // One emulated step: digits of X_{step-1} are read from buffer (step-1)&1 and the digits
@@ -161,7 +161,7 @@ struct OzStepArgs {
   const Tile* tiles;   // 128x128 upper tiles
   int ntiles;
   const void* maps;    // per digit buffer (OZ_SLICES x nparts maps apart): CUtensorMap[2][nparts], K-major
-                       // boxes of all OZ_SLICES digits ([0]) or the first OZ_SPLIT ([1]) of a tile slice
+                       // boxes of all OZ_SLICES digits ([0]) or the first OZ_LOW ([1]) of a tile slice
   const void* maps_mn; // the same with MN-major boxes (each tile 128 rows x OZ_BK columns as two 64-row atoms,
                        // 128-byte swizzle)
   const void* maps_b;    // adjoint: the same two K-major map arrays over the digits of Xbar / 2^sig
@@ -184,6 +184,7 @@ struct OzStepArgs {
   // its 64-bit partial tile to split_acc[2 t + h] and the second of the two to finish
   // (split_cnt[t], left at zero) adds both and forms the tile (X_new, digits, traces)
   int split;
+  int halves;            // the plan's items may be split: unsplit ones drain at the same boundary
   long long* split_acc;  // [2 ntiles][128 x 128], indexed by item code 2 t + h
   uint32_t* split_cnt;   // [ntiles]
   const int32_t* split_items;  // [2 ntiles]: item codes in the order the CTAs take them

@@ -56,7 +56,7 @@ cudaError_t launch_copy_iterate(const float* const* master_of_step, float* out, 
                                 int back, cudaStream_t s);
 cudaError_t launch_convert(const float* const* master_of_step, double* out, int64_t n, const DevState* st,
                            cudaStream_t s);
-// FP64 products from BF16 digits (k_oz.cu)
+// FP64 products from FP16 digits (k_oz.cu)
 cudaError_t launch_oz_step(const OzStepArgs& a, int grid, cudaStream_t s, bool adjoint = false);
 // the last FP32 iterate of a low-precision run as fixed-point master and digits (upper rows only)
 cudaError_t launch_oz_convert_slice(const PartDesc* parts, const ColBlock* blocks, int nblocks,

@@ -1,32 +1,34 @@
-// FP64-accurate purification steps on the BF16 tensor cores (sm_103a).
+// FP64-accurate purification steps on the FP16 tensor cores (sm_103a).
 //
-// GB300 runs FP64 at 1/1800 of its BF16 rate, so the FP64 product X X is rebuilt from
-// exact BF16 products, in the spirit of the Ozaki splitting (Ozaki, Ogita, Oishi and
-// Rump, 2012).  With T = OZ_SLICES digits:
+// GB300 runs FP64 at 1/1800 of its 16-bit rate, so the FP64 product X X is rebuilt from
+// FP16 products, in the spirit of the Ozaki splitting (Ozaki, Ogita, Oishi and Rump, 2012):
 //
-//   every entry of X (|x| <= 1: the spectrum of X stays in [0, 1]) is written in base 2^7
-//   with rounded signed digits, x = sum_{t<T} S_t 2^{-7(t+1)} + r, |S_0| <= 2^7 |x| + 1,
-//   |S_t| <= 2^6 (t >= 1), |r| <= 2^{-7T-1} (+ 2^-57 from the fixed point); every S_t is an
-//   integer of at most 8 bits, stored in BF16 as S_t 2^{-7t} (still exact) so that the
-//   product of digits a and b carries the factor 2^{-7(a+b)} of its group;
+//   every entry of X (|x| <= 1: the spectrum of X stays in [0, 1]) is written with T = 5
+//   balanced digits of 11, 8, 11, 9 and 11 bits, x = sum_t S_t 2^{-e_t} + r with
+//   e = 11, 19, 30, 39, 50, |S_0| <= 2^11 |x| + 1, |S_t| at most half of digit t's range
+//   (t >= 1), |r| <= 2^-51 (+ 2^-57 from the fixed point); every S_t is an integer that FP16
+//   holds exactly (11 significant bits);
 //
-//   X X = sum_{d<T} 2^{-7(d+2)} G_d + (terms below 2^{-7(T+2)}), G_d = sum_{a+b=d} S_a S_b.
+//   X X = sum_{a+b<T} 2^{-(e_a+e_b)} S_a S_b + (terms of order 2^-47): 15 products.
 //
-// Each 2^{-7d} G_d is a sum of such products accumulated in FP32 in TMEM.  Because
-// ||X||_2 <= 1, sum_k |x_ik x_kj| <= 1 bounds G_0; the groups up to d = 4 add products of
-// lower digits, which behave like independent values except on the diagonal (sums of
-// squares, about K 2^10.4), and stay below 2^24 (in units of their own scale) for K up to
-// 4096, so they are exact; later groups carry a rounding of 2^-24 relative on a value
-// scaled by 2^{-49} or less.  G_0 and G_1 share one
-// accumulator, G_0 + 2^-7 G_1: its terms are multiples of 2^-7 whose magnitudes sum to at
-// most 2^14 + 3 2^7 (sum_k |x_ik| + |x_kj|) / 2 + 2 K (with sum_k |x_ik| <= sqrt(K)), below
-// 2^16 for K <= 4096, so it is exact as well.  The groups are added as integers into a
-// 64-bit fixed-point accumulator (resolution 2^-56), and a final elementwise pass forms
-// X_new = Y or 2X - Y on that grid (the master copy of the iterate stays in this fixed
-// point), the core traces in FP64, and the digits of X_new for the next step by integer
-// arithmetic.  With T = 7 (28 BF16 products per tile) the digits hold x to 2^-49 and the
-// dropped products are of order 2^-63 K 2^12; the error of Y is about 1e-13, far below the
-// 1e-10 parity of the FP64 path.
+// The products are summed in FP32 in TMEM, in six accumulators.  Five of them hold integers
+// (in units of their own scale) that stay below 2^24 and so are exact: (0,0), because
+// ||X||_2 <= 1 bounds sum_k |x_ik x_kj| by 1; (0,1) + (1,0) and (0,2) + (2,0), at most 2^19
+// and 2^22 times the row 1-norm sum_k |x_ik| (1 to 2 for the localised iterates of a gapped
+// system; for rows spread over all K columns the digits behave like independent values,
+// about 2^18 and 2^21); (1,1), whose diagonal is a sum of squares, K 2^12.4 for digits
+// spread over their range; and 2 [(1,2) + (2,1)] + (0,3) + (3,0), about sqrt(K) 2^17.  The
+// width of digit 1 follows from (1,1) staying below 2^24 up to K = 2048 (longer K is drained
+// every 2048), that of digit 3 from its accumulator; digits 0 and 2 are as wide as FP16
+// allows, which leaves so little behind them that (1,3), (0,4), (2,2) and their mirrors, of
+// order 2^-36 (2^-31 on the diagonal), share the sixth accumulator, whose FP32 rounding lies
+// below the dropped products.  Digits of 7 bits in BF16, whose 8-bit significand caps the
+// width, took 7 digits and 28 products for an error per entry of 1.3e-14 at K = 1,184 on
+// dense rows; these give 0.8e-14.
+// The accumulators are added as integers into a 64-bit fixed point (resolution 2^-56; the
+// sixth rounded to it), and a final elementwise pass forms X_new = Y or 2X - Y on that
+// grid (the master copy of the iterate stays in this fixed point), the core traces in FP64,
+// and the digits of X_new for the next step by integer arithmetic.
 //
 // The adjoint step Xbar <- Xbar X + X Xbar (or 2 Xbar minus that) runs on the same
 // machinery: an upper tile (I, J) of Xbar X + X Xbar is one product over K = 2s, rows I of
@@ -35,8 +37,8 @@
 // part, chosen from the largest row 2-norm of Xbar so that every row of Xbar / 2^sig has
 // 2-norm <= 1/2.  With ||X||_2 <= 1, Cauchy-Schwarz gives
 // sum_k |xbar_ik x_kj| + |x_ik xbar_kj| <= 1/2 + 1/2, the bound the forward step rests on,
-// so the digit groups stay exact in the same way and the result carries an error of
-// order 2^-49 2^sig.
+// so the accumulators behave in the same way and the result carries an error of
+// order 2^-47 2^sig.
 #include <cuda.h>
 
 #include "gsp2_internal.cuh"
@@ -45,44 +47,64 @@
 
 namespace gsp2 {
 
-// Digits of a value held in 64-bit fixed point v = x 2^56 (|x| < 1.5): rounded to
-// w = x 2^{7T}, then written as balanced base-2^7 digits, S_t in [-64, 63] for t >= 1 and
-// the rest in S_0 (|S_0| <= 2^7 + 1 for |x| <= 1), w = sum_t S_t 2^{7(T-1-t)} exactly.
-// The balanced digits of w are the plain base-2^7 digits of w + 64 (1 + 2^7 + ... +
-// 2^{7(T-2)}) less 64, so each is one shift-and-mask; the small integer becomes exact BF16
-// bits through the FP32 magic-number form.  Digit t is stored as S_t 2^{-7t} (exact: a
-// power-of-two scale of an integer of at most 8 bits): the float 2^{23-7t} + u 2^{-7t}
-// less (2^23 + 64) 2^{-7t}, one OR and one exact subtraction, so that the product of digits
-// a and b lands at 2^{-7(a+b)} and groups can share an accumulator at their own scale.
-// Returned are the FP32 bit patterns whose upper halves are the BF16 digits (S_t weighs
-// 2^{-7(t+1)} in x, so every stored digit S_t 2^{-7t} weighs 2^-7).
-__device__ __forceinline__ void digit_words(long long v, uint32_t (&fw)[OZ_SLICES]) {
-  constexpr int drop = 56 - 7 * OZ_SLICES;
-  constexpr long long bias = 64ll * (((1ll << (7 * (OZ_SLICES - 1))) - 1) / 127);
-  const long long w = (drop > 0 ? ((v + (1ll << (drop - 1))) >> drop) : v) + bias;
+// Digits of a value held in 64-bit fixed point v = x 2^56 (|x| < 2): rounded to
+// w = x 2^50, then written as balanced digits of 8, 11, 9 and 11 bits below S_0, so that
+// w = S_0 2^39 + S_1 2^31 + S_2 2^20 + S_3 2^11 + S_4 exactly.  The balanced digits of w are
+// the plain bit fields of w + bias less half of each field's range, so each is one
+// shift-and-mask.  Digit t is stored as S_t 2^-rho_t with rho = -3, -4, -2, -2, 0: exact in
+// FP16, and the products that share an accumulator land at one scale (rho_a + rho_b - e_a -
+// e_b is the same for (1,2) and (0,3), and for (1,3), (0,4) and (2,2)).  S_0 beyond 2^11
+// (|x| > 1, after low-precision steps) is kept even, which FP16 holds up to 2^12, and S_1
+// takes the rest.  Each value is the float 2^{23-rho} + u 2^-rho less (2^23 + half) 2^-rho, one
+// OR and one exact subtraction.
+__host__ __device__ constexpr int oz_e(int t) {  // x = sum_t S_t 2^-e_t
+  return t == 0 ? 11 : (t == 1 ? 19 : (t == 2 ? 30 : (t == 3 ? 39 : 50)));
+}
+__host__ __device__ constexpr int oz_rho(int t) {  // stored: S_t 2^-rho_t
+  return t == 0 ? -3 : (t == 1 ? -4 : (t == 4 ? 0 : -2));
+}
+__device__ __forceinline__ float digit_float(uint32_t u, int t, int half) {
+  const uint32_t e = (uint32_t)(150 - oz_rho(t)) << 23;  // exponent field of 2^{23-rho}
+  return __fsub_rn(__uint_as_float(e | u), __uint_as_float(e | (uint32_t)half));
+}
+__device__ __forceinline__ void digit_floats(long long v, float (&f)[OZ_SLICES]) {
+  constexpr int drop = 56 - oz_e(4);
+  constexpr long long bias = 1024ll + (256ll << 11) + (1024ll << 20) + (128ll << 31);
+  const long long w = ((v + (1ll << (drop - 1))) >> drop) + bias;
+  const uint32_t lo = (uint32_t)w, hi = (uint32_t)(w >> 31);
+  f[4] = digit_float(lo & 2047u, 4, 1024);
+  f[3] = digit_float((lo >> 11) & 511u, 3, 256);
+  f[2] = digit_float((lo >> 20) & 2047u, 2, 1024);
+  int s0 = (int)hi >> 8;
+  const int odd = (s0 > 2048 || s0 < -2048) ? (s0 & 1) : 0;
+  f[1] = digit_float((hi & 255u) + 256u * (uint32_t)odd, 1, 128);
+  f[0] = digit_float((uint32_t)(s0 - odd + 8192), 0, 8192);
+}
+// two digits as packed FP16 (lo in the lower half)
+__device__ __forceinline__ uint32_t pack_f16(float lo, float hi) {
+  uint32_t d;
+  asm("cvt.rn.f16x2.f32 %0, %1, %2;\n" : "=r"(d) : "f"(hi), "f"(lo));
+  return d;
+}
+// the digits of four values, packed: d[t][0] values 0 and 1, d[t][1] values 2 and 3
+__device__ __forceinline__ void digits4(const long long (&v)[4], uint32_t (&d)[OZ_SLICES][2]) {
 #pragma unroll
-  for (int t = OZ_SLICES - 1; t >= 1; --t) {
-    const uint32_t u = (uint32_t)(w >> (7 * (OZ_SLICES - 1 - t))) & 127u;
-    const uint32_t e = (uint32_t)(150 - 7 * t) << 23;  // exponent field of 2^{23-7t}
-    fw[t] = __float_as_uint(__fsub_rn(__uint_as_float(e | u), __uint_as_float(e | 64u)));  // (2^23 + 64) 2^{-7t}
+  for (int h = 0; h < 2; ++h) {
+    float a[OZ_SLICES], b[OZ_SLICES];
+    digit_floats(v[2 * h], a);
+    digit_floats(v[2 * h + 1], b);
+#pragma unroll
+    for (int t = 0; t < OZ_SLICES; ++t) d[t][h] = pack_f16(a[t], b[t]);
   }
-  const int s0 = (int)(w >> (7 * (OZ_SLICES - 1)));  // |s0| < 256
-  fw[0] = __float_as_uint(__fsub_rn(__uint_as_float(0x4B000000u | (uint32_t)(s0 + 256)), 8388864.0f));
 }
 
 // The digits of four consecutive elements e .. e + 3 (e a multiple of 4), one 8-byte store
 // per digit array (a warp's lanes on consecutive groups of four write 256 B per store).
 __device__ __forceinline__ void store_digits4(uint16_t* const* slices, int64_t e, const long long (&v)[4]) {
-  uint32_t fw[4][OZ_SLICES];
+  uint32_t d[OZ_SLICES][2];
+  digits4(v, d);
 #pragma unroll
-  for (int i = 0; i < 4; ++i) digit_words(v[i], fw[i]);
-#pragma unroll
-  for (int t = 0; t < OZ_SLICES; ++t) {
-    uint2 pk;  // upper halves of two words per 32 bits
-    pk.x = __byte_perm(fw[0][t], fw[1][t], 0x7632);
-    pk.y = __byte_perm(fw[2][t], fw[3][t], 0x7632);
-    *reinterpret_cast<uint2*>(slices[t] + e) = pk;
-  }
+  for (int t = 0; t < OZ_SLICES; ++t) *reinterpret_cast<uint2*>(slices[t] + e) = make_uint2(d[t][0], d[t][1]);
 }
 
 // Start of the emulated FP64 tail of a low-precision run: the last FP32 iterate (found on the
@@ -299,47 +321,41 @@ __global__ void __launch_bounds__(256) oz_digits_kernel(const PartDesc* __restri
 // per SM walks the upper 128x128 tiles: blockIdx.x, then the ones it claims from a counter,
 // or blockIdx.x + gridDim.x, ... in the static deal).
 //
-// The T(T+1)/2 digit products of a tile need an FP32 accumulator per group d = a + b
-// (128 TMEM columns each; G_0 and G_1 share one), more than the 512 columns of an SM, so a
-// tile takes two passes over K: first the high groups d >= OZ_SPLIT (all seven digits; 22
-// of the 28 products, columns 0-511), then the low groups d < OZ_SPLIT (digits below
-// OZ_SPLIT, columns 0-255).  A stage of the TMA ring holds one K = OZ_BK slice of every
-// digit the pass needs, for rows I (A) and rows J (B; diagonal tiles reuse A), so each
-// distinct digit tile is loaded once per slice and feeds all its products (one K = 16 BF16
-// MMA each).  The epilogue warps turn the high groups' sums into 64-bit fixed point (2^-56)
-// and park them in TMEM columns 256-511, which the low pass leaves alone; after the low
-// pass they add the low groups, hand all 512 columns back and keep the tile's sums in a
+// The 15 digit products of a tile need six FP32 accumulators of 128 TMEM columns, more than
+// the 512 columns of an SM, so a tile takes two passes over K: first the 12 products other
+// than (0,0), (0,1) and (1,0) (all five digits, columns 0-511), then those three (digits 0
+// and 1, columns 0-255).  A unit of the TMA ring holds one operand (rows I or rows J) of the
+// pass: one K = OZ_BK slice of all five digits, or in the second pass two slices of two
+// digits; diagonal tiles load rows I only.  Each distinct digit tile is loaded once per slice
+// and feeds all its products (one K = 16 FP16 MMA each).  Five units of 40 KB keep two and a
+// half slices in flight.  The epilogue warps turn the first pass's sums into 64-bit fixed
+// point (2^-56) and park them in TMEM columns 256-511, which the second pass leaves alone;
+// after it they add its sums, hand all 512 columns back and keep the tile's sums in a
 // per-CTA scratch tile (L2-resident) for the final pass, which forms X_new = Y or 2X - Y,
 // writes the master copy (64-bit fixed point) and the digits of X_new (into the other
 // digit buffer) at (I, J) and mirrored at (J, I) (diagonal tiles from their upper
-// triangle), and adds the core traces, while the MMAs of the next tile's high pass run.  The new
+// triangle), and adds the core traces, while the MMAs of the next tile's first pass run.  The new
 // iterate is written with evict-first stores: the next step reads it after this launch,
 // and keeping it out of L2 leaves room for the digit panels the running tiles share.  The last block
-// runs the step bookkeeping.
+// runs the step bookkeeping.  K beyond OZ_CHUNK slices is taken in rounds of both passes, the
+// later ones adding to the scratch tile, so that the sums stay exact (see the top).
 //
 // 20 warps: warp 0 lane 0 TMA, warp 1 TMEM owner and MMA issuer, warps 4..19 epilogue
 // (warp w: TMEM lanes 32 (w % 4) .. + 31, columns 32 ((w - 4) / 4) .. + 31 of each group,
 // in two chunks of 16), sized so that four epilogue warps per scheduler hide latency.
-constexpr int OZ_STAGES = 2;
+constexpr int OZ_UNITS = 5;                                      // operand units of the TMA ring
 constexpr uint32_t OZ_DTILE = 128u * OZ_BK * 2u;                 // one digit tile: 128 rows x 64 B
-constexpr uint32_t OZ_STAGE_B = 2u * OZ_SLICES * OZ_DTILE;       // all A and B digit tiles
+constexpr uint32_t OZ_UNIT_B = OZ_SLICES * OZ_DTILE;             // one operand's digit tiles
+constexpr int OZ_LOW_SUB = 2;                                    // K slices per unit of the second pass
+constexpr int OZ_CHUNK = 2048 / OZ_BK;                           // K slices per round of both passes
 constexpr int OZ_EPI_WARPS = 16;                                 // 4 per TMEM lane quarter
 constexpr int OZ_THREADS = 32 * (4 + OZ_EPI_WARPS);
 constexpr int OZ_RING = 4;  // dynamic schedule: tiles claimed ahead of the MMA and epilogue warps
-constexpr int OZ_SMEM = OZ_STAGES * (int)OZ_STAGE_B + 1024 + 8 * (2 * OZ_STAGES + 4) + 16 + 16 * OZ_EPI_WARPS +
+constexpr int OZ_SMEM = OZ_UNITS * (int)OZ_UNIT_B + 1024 + 8 * (2 * OZ_UNITS + 4) + 16 + 16 * OZ_EPI_WARPS +
                         8 * 2 * OZ_RING + 4 * OZ_RING;
-static_assert(OZ_SLICES - OZ_SPLIT <= 4 && OZ_SPLIT <= 4, "groups of one pass must fit in 512 TMEM columns");
+static_assert(OZ_LOW_SUB * OZ_LOW <= OZ_SLICES, "a unit holds the second pass's slices");
+static_assert((2 * OZ_UNITS + 4) % 2 == 0, "alignment of the reduction slots");
 static_assert(OZ_SMEM <= 232448, "shared memory of the emulated step");
-
-// K slices per stage: as many as the stage's 2 T tile slots hold (a slice needs nd digit tiles
-// of A, and as many of B unless the tile is diagonal), at most one 128-block of K, a power of 2
-// so that the slices of a stage never cross a 128-block.
-__host__ __device__ constexpr int oz_slices_per_stage(int nd, bool diag) {
-  const int fit = (2 * OZ_SLICES) / ((diag ? 1 : 2) * nd), cap = 128 / OZ_BK;
-  const int m = fit < cap ? fit : cap;
-  return m >= 4 ? 4 : (m >= 2 ? 2 : 1);
-}
-static_assert(oz_slices_per_stage(OZ_SLICES, false) >= 1, "a high-pass slice fits a stage");
 
 // Columns of tile column block tj that an MMA must cover: those inside the part, rounded up
 // to 16 (N of an M = 128 MMA is a multiple of 16); the rest of the block is zero padding.
@@ -347,41 +363,44 @@ __host__ __device__ constexpr int oz_tile_cols(int s, int tj) {
   return s - tj * 128 >= 128 ? 128 : ((s - tj * 128 + 15) & ~15);
 }
 
-// Accumulator of group d: the high pass's groups 5, 6, 3, 4 in columns 0-127, 128-255,
-// 256-383, 384-511; the low pass's G_0 + 2^-7 G_1 in columns 0-127 and G_2 in 128-255, so the
-// low pass can start once groups 5 and 6 are read, and columns 256-511 hold the high pass's
-// 64-bit sums (low and high words) until the low pass is drained.
-static_assert(OZ_SPLIT == 3 && OZ_SLICES - OZ_SPLIT == 4, "the TMEM plan of the emulated step");
+// Accumulators (first TMEM column): of the first pass, (1,3), (0,4) and (2,2) in columns
+// 0-127, (1,2) and (0,3) in 128-255, (0,2) in 256-383 and (1,1) in 384-511; of the second,
+// (0,0) in 0-127 and (0,1) in 128-255.  The second pass can start once the columns 0-255 are
+// read, and columns 256-511 then hold the first pass's 64-bit sums (low and high words).
 constexpr uint32_t OZ_PARK_LO = 256, OZ_PARK_HI = 384;
-__host__ __device__ constexpr uint32_t oz_group_col(int d) {
-  return (uint32_t)(d >= OZ_SPLIT ? (d >= 5 ? 128 * (d - 5) : 256 + 128 * (d - 3)) : (d <= 1 ? 0 : 128));
+__host__ __device__ constexpr bool oz_low_pass(int a, int b) { return a + b <= 1; }
+__host__ __device__ constexpr uint32_t oz_col(int a, int b) {
+  return a + b == 0 || a + b == 4 ? 0u : (a + b == 2 ? (a == 1 ? 384u : 256u) : 128u);
 }
+// products of A digit q in a pass: (q, b) for lo <= b < hi
+template <bool LOW>
+__host__ __device__ constexpr int oz_b_lo(int q) { return LOW ? 0 : (q < 2 ? 2 - q : 0); }
+template <bool LOW>
+__host__ __device__ constexpr int oz_b_hi(int q) { return (LOW ? OZ_LOW : OZ_SLICES) - q; }
 
-// The MMAs of one stage for the groups d0 <= d < d1, fully unrolled: every pair (q, d - q)
-// of a group into the group's accumulator, descriptors formed by adding compile-time
-// offsets to the stage's base descriptors (the 14-bit address field cannot carry: shared
-// addresses stay below 2^18).  The products are issued A digit by A digit: the products of
-// A digit q (one per group d >= q) follow one another and share their A operand through the
+// The MMAs of one K slice of a pass, fully unrolled, descriptors formed by adding
+// compile-time offsets to the slice's base descriptors (the 14-bit address field cannot
+// carry: shared addresses stay below 2^18).  The products are issued A digit by A digit: the products of
+// A digit q follow one another and share their A operand through the
 // collector buffer, so each A digit tile is read from shared memory once per K = 16 slice
 // instead of once per product (the MMAs' shared-memory reads, A and B, set the pace of the
-// tensor pipe otherwise).  Every accumulator's first product is the one with q = 0 (for the
-// shared G_0 + 2^-7 G_1, the product (0, 0)).
-template <int D0, int D1>
-__device__ __forceinline__ void oz_issue_stage(uint32_t tmem, uint64_t da, uint64_t db, uint32_t adv_a,
+// tensor pipe otherwise).
+template <bool LOW>
+__device__ __forceinline__ void oz_issue_slice(uint32_t tmem, uint64_t da, uint64_t db, uint32_t adv_a,
                                                uint32_t adv_b, uint32_t idesc, bool first_k) {
   constexpr uint64_t step = OZ_DTILE >> 4;
 #pragma unroll
-  for (int kk = 0; kk < OZ_BK / 16; ++kk) {  // K = 16 slices of the stage
+  for (int kk = 0; kk < OZ_BK / 16; ++kk) {  // K = 16 steps of the slice
 #pragma unroll
-    for (int q = 0; q < D1; ++q) {
-      const int dlo = q > D0 ? q : D0;  // groups holding a product of A digit q
+    for (int q = 0; q < (LOW ? OZ_LOW : OZ_SLICES); ++q) {
+      const int b0 = oz_b_lo<LOW>(q), b1 = oz_b_hi<LOW>(q);
 #pragma unroll
-      for (int d = dlo; d < D1; ++d) {
-        const int op = (D1 - dlo == 1) ? 0 : (d == dlo ? 1 : (d == D1 - 1 ? 3 : 2));
-        // the first product into each accumulator is (0, d) of its lowest group
-        const bool opens = q == 0 && !(D0 == 0 && d == 1);
-        mma_f16_col(op, tmem + oz_group_col(d), da + (uint64_t)q * step + (uint64_t)(adv_a * kk),
-                    db + (uint64_t)(d - q) * step + (uint64_t)(adv_b * kk), idesc,
+      for (int b = b0; b < b1; ++b) {
+        const int op = (b1 - b0 == 1) ? 0 : (b == b0 ? 1 : (b == b1 - 1 ? 3 : 2));
+        // the first product into each accumulator: (0,0), (0,1); (0,2), (0,3), (0,4), (1,1)
+        const bool opens = q == 0 || (q == 1 && b == 1);
+        mma_f16_col(op, tmem + oz_col(q, b), da + (uint64_t)q * step + (uint64_t)(adv_a * kk),
+                    db + (uint64_t)b * step + (uint64_t)(adv_b * kk), idesc,
                     (!opens || kk > 0 || !first_k) ? 1u : 0u);
       }
     }
@@ -389,9 +408,8 @@ __device__ __forceinline__ void oz_issue_stage(uint32_t tmem, uint64_t da, uint6
 }
 
 // z[j] += u[j] 2^SHIFT for one accumulator of one 16-column chunk, where u = v 2^M is the
-// integer its FP32 sums v hold at the scale 2^-M: the groups d >= 3 alone (M = 7 d, SHIFT =
-// 56 - 7 (d + 2)), G_2 (M = 14, SHIFT = 28), G_0 + 2^-7 G_1 (M = 7, SHIFT = 35: u = 2^7 G_0 +
-// G_1).  A chunk whose integers all lie below 2^22 in magnitude is converted without the
+// integer its FP32 sums v hold at the scale 2^-M (the sixth accumulator: v 2^M rounded).
+// A chunk whose integers all lie below 2^22 in magnitude is converted without the
 // conversion unit: v + 1.5 2^(23 - M) is a float in [2^(23 - M), 2^(24 - M)) with spacing 2^-M,
 // whose bit pattern less that of 1.5 2^(23 - M) is u, and a 32 x 32 -> 64-bit multiply-add
 // (by the power of two, or on the upper word for shifts of 32 and more) accumulates it; any
@@ -425,21 +443,30 @@ __device__ __forceinline__ void oz_drain_slot(uint32_t taddr, long long (&z)[16]
   }
 }
 
-// The high pass of one chunk, in two halves: groups 5 and 6 (the columns the low pass
-// reuses), then groups 3 and 4 (the columns that then hold the sums), into z.
-__device__ __forceinline__ void oz_drain_high56(uint32_t taddr, long long (&z)[16]) {
-  oz_drain_slot<35, 7>(taddr + oz_group_col(5), z);
-  oz_drain_slot<42, 0>(taddr + oz_group_col(6), z);
-}
-__device__ __forceinline__ void oz_drain_high34(uint32_t taddr, long long (&z)[16]) {
-  oz_drain_slot<21, 21>(taddr + oz_group_col(3), z);
-  oz_drain_slot<28, 14>(taddr + oz_group_col(4), z);
+// The drain of the accumulator of product (a, b): stored products carry 2^-(rho_a+rho_b),
+// their integers weigh 2^(56-e_a-e_b) on the fixed point's grid.  GRID: the sums are taken as
+// multiples of 2^-GRID (the sixth accumulator, not an integer, rounded to 2^-56).
+template <int A, int B, int GRID = oz_e(A) + oz_e(B)>
+__device__ __forceinline__ void oz_drain(uint32_t taddr, long long (&z)[16]) {
+  constexpr int M = oz_rho(A) + oz_rho(B) - (oz_e(A) + oz_e(B) - GRID);
+  oz_drain_slot<M, 56 - GRID>(taddr + oz_col(A, B), z);
 }
 
-// The low pass of one chunk: G_0 + 2^-7 G_1 and G_2 into z.
+// The first pass of one chunk, in two halves: the columns the second pass reuses, then the
+// columns that hold the sums from then on, into z.
+__device__ __forceinline__ void oz_drain_high_a(uint32_t taddr, long long (&z)[16]) {
+  oz_drain<0, 4, 56>(taddr, z);
+  oz_drain<0, 3>(taddr, z);
+}
+__device__ __forceinline__ void oz_drain_high_b(uint32_t taddr, long long (&z)[16]) {
+  oz_drain<0, 2>(taddr, z);
+  oz_drain<1, 1>(taddr, z);
+}
+
+// The second pass of one chunk into z.
 __device__ __forceinline__ void oz_drain_low(uint32_t taddr, long long (&z)[16]) {
-  oz_drain_slot<7, 35>(taddr + oz_group_col(0), z);
-  oz_drain_slot<14, 28>(taddr + oz_group_col(2), z);
+  oz_drain<0, 0>(taddr, z);
+  oz_drain<0, 1>(taddr, z);
 }
 
 // |v| 2^-56 as FP32 (integer instructions, truncated: at most 2^-23 below), for the row
@@ -480,8 +507,8 @@ __device__ __forceinline__ float warp_colsum16(const float (&v)[16], int lane, i
 template <bool ADJ>
 __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
   constexpr int T = OZ_SLICES;
-  // instruction descriptor without N (bits 17..22, N / 8): FP32 accumulate, BF16 A and B, M = 128
-  constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((128u >> 4) << 24);
+  // instruction descriptor without N (bits 17..22, N / 8): FP32 accumulate, FP16 A and B, M = 128
+  constexpr uint32_t IDESC = (1u << 4) | ((128u >> 4) << 24);
 
   int step = a.step;
   const bool rec = !ADJ && a.mode == SQ_RECOMPUTE;
@@ -504,11 +531,11 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
   uint8_t* sb = smem_raw + (base - raw);
-  const uint32_t bars = base + OZ_STAGES * OZ_STAGE_B;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(sb + OZ_STAGES * OZ_STAGE_B + 8 * (2 * OZ_STAGES + 4));
+  const uint32_t bars = base + OZ_UNITS * OZ_UNIT_B;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(sb + OZ_UNITS * OZ_UNIT_B + 8 * (2 * OZ_UNITS + 4));
   int* s_err = reinterpret_cast<int*>(tmem_slot + 1);
-  int* s_half = reinterpret_cast<int*>(tmem_slot + 2);  // split adjoint: halves of the tile done before
-  double2* red = reinterpret_cast<double2*>(sb + OZ_STAGES * OZ_STAGE_B + 8 * (2 * OZ_STAGES + 4) + 16);
+  int* s_half = reinterpret_cast<int*>(tmem_slot + 2);  // split K: halves of the tile done before
+  double2* red = reinterpret_cast<double2*>(sb + OZ_UNITS * OZ_UNIT_B + 8 * (2 * OZ_UNITS + 4) + 16);
   // dynamic schedule: the producer claims each next tile from a counter in global memory and
   // passes it on through a ring (full: claimed; empty: read by the MMA thread and every
   // epilogue warp); -1 ends the walk
@@ -517,12 +544,11 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
   auto item_full = [&](int q) { return ring_bars + 8u * q; };
   auto item_empty = [&](int q) { return ring_bars + 8u * (OZ_RING + q); };
   auto full = [&](int s) { return bars + 8u * s; };
-  auto empty = [&](int s) { return bars + 8u * (OZ_STAGES + s); };
-  // accumulator barriers: [0] high groups, [1] low groups
-  auto afull = [&](int pass) { return bars + 8u * (2 * OZ_STAGES + pass); };
-  auto aempty = [&](int pass) { return bars + 8u * (2 * OZ_STAGES + 2 + pass); };
-  auto tileA = [&](int s, int q) { return base + (uint32_t)s * OZ_STAGE_B + (uint32_t)q * OZ_DTILE; };
-  auto tileB = [&](int s, int q) { return base + (uint32_t)s * OZ_STAGE_B + (uint32_t)(OZ_SLICES + q) * OZ_DTILE; };
+  auto empty = [&](int s) { return bars + 8u * (OZ_UNITS + s); };
+  // accumulator barriers: [0] first pass, [1] second
+  auto afull = [&](int pass) { return bars + 8u * (2 * OZ_UNITS + pass); };
+  auto aempty = [&](int pass) { return bars + 8u * (2 * OZ_UNITS + 2 + pass); };
+  auto unit = [&](int s) { return base + (uint32_t)s * OZ_UNIT_B; };
   int32_t* abort_flag = &a.ctl.st->timeout;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const CUtensorMap* maps = reinterpret_cast<const CUtensorMap*>(a.maps) + (size_t)dbi * T * a.nparts;
@@ -532,12 +558,25 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
   // work items: the upper tiles, or (split K) each tile's two K halves
   const bool split = a.split != 0;
   const int nitems = split ? 2 * a.ntiles : a.ntiles;
+  // K slices [x, y) of an item of a part of size sz: all of them (the adjoint's first ns slices
+  // multiply Xbar by X, the rest X by Xbar) or one half, up to or from slice z
+  auto slices = [&](int sz, int half) {
+    const int ns = (sz + OZ_BK - 1) / OZ_BK, all = ADJ ? 2 * ns : ns, mid = ADJ ? ns : (ns + 1) / 2;
+    return make_int3(half == 1 ? mid : 0, half == 0 ? mid : all, mid);
+  };
+  // end of the round of both passes that starts at slice c0: OZ_CHUNK slices, and (plans whose
+  // items may be split) never across the halves, so that a tile's sums are rounded alike
+  // whether one item forms it or two
+  auto round_end = [&](int c0, int3 kr) {
+    const int c1 = min(c0 + OZ_CHUNK, kr.y);
+    return a.halves && c0 < kr.z ? min(c1, kr.z) : c1;
+  };
   // items claimed at run time (forward, tail and reverse steps; the list order) or dealt in turn
   // (the rebuilt iterates, which may run beside reverse steps and have no last block)
   const bool dyn = a.tile_ctr != nullptr && !rec;
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < OZ_STAGES; ++s) {
+    for (int s = 0; s < OZ_UNITS; ++s) {
       mbar_init(full(s), 1);
       mbar_init(empty(s), 1);
     }
@@ -587,48 +626,38 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
       const Tile t = a.tiles[ti];
       const int sz = a.parts[t.part].s;
       const bool dg = !ADJ && t.ti == t.tj;  // X X on a diagonal tile: B is A
-      for (int pass = 0; pass < 2 && !bad; ++pass) {
-        const int nd = pass == 0 ? T : OZ_SPLIT;  // digits the pass multiplies
-        const int sub = oz_slices_per_stage(nd, dg);
-        const int nk = (sz + sub * OZ_BK - 1) / (sub * OZ_BK);
-        // K stages of the item: the adjoint's halves are Xbar X and X Xbar, the forward's the
-        // two halves of the stages of the pass
-        const int kb0 = half < 1 ? 0 : (ADJ ? nk : (nk + 1) / 2);
-        const int kb1 = ADJ ? (half == 0 ? nk : 2 * nk) : (half == 0 ? (nk + 1) / 2 : nk);
-        for (int kb = kb0; kb < kb1; ++kb, ++g) {
-          // the adjoint's first nk stages multiply Xbar (rows I) by X (rows J), the rest X by Xbar
-          const bool h2 = ADJ && kb >= nk;
-          const int kq = h2 ? kb - nk : kb;
-          const CUtensorMap* const mA = (ADJ && !h2) ? maps_b : maps;
-          const CUtensorMap* const mmA = (ADJ && !h2) ? maps_mn_b : maps_mn;
-          const CUtensorMap* const mB = h2 ? maps_b : maps;
-          const CUtensorMap* const mmB = h2 ? maps_mn_b : maps_mn;
-          const int s = g % OZ_STAGES;
-          if (g >= OZ_STAGES && !mbar_wait(empty(s), ((g / OZ_STAGES) - 1) & 1, abort_flag)) {
-            bad = true;
-            break;
-          }
-          mbar_expect_tx(full(s), (uint32_t)(sub * (dg ? nd : 2 * nd)) * OZ_DTILE);
-          // rows I over the K slice: K-major from columns I of the tiles on or above the
-          // diagonal (slice block <= I's block), else MN-major from rows I of tile (I, slice);
-          // the slices of one stage lie in one 128-block of K.  One request per slice and
-          // operand brings all nd digit tiles (slots u nd .. u nd + nd - 1): the maps of the
-          // high pass take OZ_SLICES digits per box, those of the low pass OZ_SPLIT
-          const size_t at = (size_t)(nd == T ? 0 : 1) * a.nparts + t.part;
-          for (int u = 0; u < sub; ++u) {
-            const int k0 = (kq * sub + u) * OZ_BK;
-            const int kt = k0 / 128;
-            const int slot = u * nd;
-            if (kt <= t.ti) {
-              tma_load_3d(tileA(s, slot), mA + at, k0, t.ti * 128, 0, full(s));
-            } else {
-              tma_load_4d(tileA(s, slot), mmA + at, 0, k0, 2 * t.ti, 0, full(s));  // 64-row atoms x digits
-            }
-            if (dg) continue;
-            if (kt <= t.tj) {
-              tma_load_3d(tileB(s, slot), mB + at, k0, t.tj * 128, 0, full(s));
-            } else {
-              tma_load_4d(tileB(s, slot), mmB + at, 0, k0, 2 * t.tj, 0, full(s));
+      const int ns = (sz + OZ_BK - 1) / OZ_BK;
+      const int3 kr = slices(sz, half);
+      for (int c0 = kr.x, c1; c0 < kr.y && !bad; c0 = c1) {
+        c1 = round_end(c0, kr);
+        for (int pass = 0; pass < 2 && !bad; ++pass) {
+          const int nd = pass == 0 ? T : OZ_LOW, sub = pass == 0 ? 1 : OZ_LOW_SUB;
+          const size_t at = (size_t)pass * a.nparts + t.part;  // maps whose boxes take nd digits
+          for (int kb = c0; kb < c1 && !bad; kb += sub) {
+            const int m = min(sub, c1 - kb);
+            for (int op = 0; op < (dg ? 1 : 2); ++op, ++g) {  // rows I, then rows J
+              const int s = g % OZ_UNITS;
+              if (g >= OZ_UNITS && !mbar_wait(empty(s), ((g / OZ_UNITS) - 1) & 1, abort_flag)) {
+                bad = true;
+                break;
+              }
+              mbar_expect_tx(full(s), (uint32_t)(m * nd) * OZ_DTILE);
+              const int blk = op == 0 ? t.ti : t.tj;
+              for (int u = 0; u < m; ++u) {
+                // the adjoint's first ns slices take Xbar for rows I and X for rows J, the rest
+                // X for rows I and Xbar for rows J
+                const bool h2 = ADJ && kb + u >= ns;
+                const bool xb = ADJ && (op == 0) != h2;
+                const int k0 = (h2 ? kb + u - ns : kb + u) * OZ_BK;
+                const uint32_t dst = unit(s) + (uint32_t)(u * nd) * OZ_DTILE;
+                // K-major from columns `blk` of the tiles on or above the diagonal (slice block
+                // <= blk), else MN-major from rows `blk` of the tile (blk, slice); one request
+                // brings the slice's nd digit tiles
+                if (k0 / 128 <= blk)
+                  tma_load_3d(dst, (xb ? maps_b : maps) + at, k0, blk * 128, 0, full(s));
+                else
+                  tma_load_4d(dst, (xb ? maps_mn_b : maps_mn) + at, 0, k0, 2 * blk, 0, full(s));  // 64-row atoms x digits
+              }
             }
           }
         }
@@ -636,17 +665,17 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
     }
     if (bad) {
       *s_err = 1;
-      const uint32_t first = g > OZ_STAGES ? g - OZ_STAGES : 0;
-      for (uint32_t q = first; q < g; ++q) (void)mbar_wait_own(full(q % OZ_STAGES), (q / OZ_STAGES) & 1);
+      const uint32_t first = g > OZ_UNITS ? g - OZ_UNITS : 0;
+      for (uint32_t q = first; q < g; ++q) (void)mbar_wait_own(full(q % OZ_UNITS), (q / OZ_UNITS) & 1);
     }
   } else if (warp == 1 && lane == 0) {
     uint32_t g = 0;
-    int u = 0;  // items done by this CTA
+    int v = 0, r = 0;  // items taken, rounds of both passes done by this CTA
     bool bad = false;
-    for (int it = blockIdx.x; !bad; it += gridDim.x, ++u) {
+    for (int it = blockIdx.x; !bad; it += gridDim.x, ++v) {
       if (dyn) {
-        const int q = u % OZ_RING;
-        if (!mbar_wait(item_full(q), (u / OZ_RING) & 1, abort_flag)) {
+        const int q = v % OZ_RING;
+        if (!mbar_wait(item_full(q), (v / OZ_RING) & 1, abort_flag)) {
           bad = true;
           break;
         }
@@ -660,58 +689,61 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
       const Tile t = a.tiles[ti];
       const int sz = a.parts[t.part].s;
       const bool dg = !ADJ && t.ti == t.tj;
-      for (int pass = 0; pass < 2 && !bad; ++pass) {
-        const int nd = pass == 0 ? T : OZ_SPLIT;
-        const int sub = oz_slices_per_stage(nd, dg);
-        const int nk = (sz + sub * OZ_BK - 1) / (sub * OZ_BK);
-        // K stages of the item: the adjoint's halves are Xbar X and X Xbar, the forward's the
-        // two halves of the stages of the pass
-        const int kb0 = half < 1 ? 0 : (ADJ ? nk : (nk + 1) / 2);
-        const int kb1 = ADJ ? (half == 0 ? nk : 2 * nk) : (half == 0 ? (nk + 1) / 2 : nk);
-        // the high pass reuses the columns of the previous tile's low groups, the low pass
-        // those of this tile's high groups: wait until the epilogue has read them
-        const bool ready = pass == 0 ? (u == 0 || mbar_wait(aempty(1), (u - 1) & 1, abort_flag))
-                                     : mbar_wait(aempty(0), u & 1, abort_flag);
-        if (!ready) {
-          bad = true;
-          break;
-        }
-        tc_fence_after();
-        for (int kb = kb0; kb < kb1; ++kb, ++g) {
-          const int kq = (ADJ && kb >= nk) ? kb - nk : kb;
-          const int s = g % OZ_STAGES;
-          if (!mbar_wait(full(s), (g / OZ_STAGES) & 1, abort_flag)) {
+      const int ns = (sz + OZ_BK - 1) / OZ_BK;
+      const int3 kr = slices(sz, half);
+      const uint32_t idesc0 = IDESC | ((uint32_t)(oz_tile_cols(sz, t.tj) >> 3) << 17);
+      for (int c0 = kr.x, c1; c0 < kr.y && !bad; c0 = c1, ++r) {
+        c1 = round_end(c0, kr);
+        for (int pass = 0; pass < 2 && !bad; ++pass) {
+          const int nd = pass == 0 ? T : OZ_LOW, sub = pass == 0 ? 1 : OZ_LOW_SUB;
+          // the first pass reuses the columns of the previous round's second, the second pass
+          // those of this round's first: wait until the epilogue has read them
+          const bool ready = pass == 0 ? (r == 0 || mbar_wait(aempty(1), (r - 1) & 1, abort_flag))
+                                       : mbar_wait(aempty(0), r & 1, abort_flag);
+          if (!ready) {
             bad = true;
             break;
           }
           tc_fence_after();
-          // pairs (q, d - q) of every group of the pass; both digits are < d1 <= T.  Operands
-          // right of the tile's own block came in MN-major (transpose bits 15 / 16); a K = 16
-          // step advances 32 B in a K-major row, 2 KB (16 K values) in an MN-major tile
-          const int kt = kq * sub * OZ_BK / 128;
-          const bool amn = kt > t.ti, bmn = kt > t.tj;
-          const uint64_t da = amn ? smem_desc_mn128(tileA(s, 0), OZ_DTILE / 2) : smem_desc_sw<2 * OZ_BK>(tileA(s, 0));
-          const uint64_t db = dg ? da
-                                 : (bmn ? smem_desc_mn128(tileB(s, 0), OZ_DTILE / 2)
-                                        : smem_desc_sw<2 * OZ_BK>(tileB(s, 0)));
-          const uint32_t adv_a = amn ? (2048u >> 4) : (32u >> 4), adv_b = bmn ? (2048u >> 4) : (32u >> 4);
-          const uint32_t idesc =
-              IDESC | ((uint32_t)(oz_tile_cols(sz, t.tj) >> 3) << 17) | ((amn ? 1u : 0u) << 15) | ((bmn ? 1u : 0u) << 16);
-          for (int u = 0; u < sub; ++u) {  // the stage's K slices, nd tiles apart
-            const uint64_t off = (uint64_t)(u * nd) * (OZ_DTILE >> 4);
-            if (pass == 0) oz_issue_stage<OZ_SPLIT, T>(tmem, da + off, db + off, adv_a, adv_b, idesc, kb == kb0 && u == 0);
-            else oz_issue_stage<0, OZ_SPLIT>(tmem, da + off, db + off, adv_a, adv_b, idesc, kb == kb0 && u == 0);
+          for (int kb = c0; kb < c1; kb += sub) {
+            const int m = min(sub, c1 - kb);
+            const int sa = g % OZ_UNITS, sB = dg ? sa : (g + 1) % OZ_UNITS;
+            if (!mbar_wait(full(sa), (g / OZ_UNITS) & 1, abort_flag) ||
+                (!dg && !mbar_wait(full(sB), ((g + 1) / OZ_UNITS) & 1, abort_flag))) {
+              bad = true;
+              break;
+            }
+            tc_fence_after();
+            for (int u = 0; u < m; ++u) {
+              // operands right of the tile's own block came in MN-major (transpose bits 15 / 16);
+              // a K = 16 step advances 32 B in a K-major row, 2 KB (16 K values) in an MN-major tile
+              const int ks = kb + u;
+              const int kt = (ADJ && ks >= ns ? ks - ns : ks) * OZ_BK / 128;
+              const bool amn = kt > t.ti, bmn = kt > t.tj;
+              const uint32_t off = (uint32_t)(u * nd) * OZ_DTILE;
+              const uint64_t da = amn ? smem_desc_mn128(unit(sa) + off, OZ_DTILE / 2)
+                                      : smem_desc_sw<2 * OZ_BK>(unit(sa) + off);
+              const uint64_t db = dg ? da
+                                     : (bmn ? smem_desc_mn128(unit(sB) + off, OZ_DTILE / 2)
+                                            : smem_desc_sw<2 * OZ_BK>(unit(sB) + off));
+              const uint32_t adv_a = amn ? (2048u >> 4) : (32u >> 4), adv_b = bmn ? (2048u >> 4) : (32u >> 4);
+              const uint32_t idesc = idesc0 | ((amn ? 1u : 0u) << 15) | ((bmn ? 1u : 0u) << 16);
+              if (pass == 0) oz_issue_slice<false>(tmem, da, db, adv_a, adv_b, idesc, ks == c0);
+              else oz_issue_slice<true>(tmem, da, db, adv_a, adv_b, idesc, ks == c0);
+            }
+            mma_commit(empty(sa));
+            if (!dg) mma_commit(empty(sB));
+            g += dg ? 1 : 2;
           }
-          mma_commit(empty(s));
+          if (!bad) mma_commit(afull(pass));
         }
-        if (!bad) mma_commit(afull(pass));
       }
     }
     if (bad) {
       *s_err = 1;
       // MMAs already issued keep reading shared memory and writing TMEM: wait (on this
       // thread's own limit) for the last commit, which covers all of them
-      if (g > 0) (void)mbar_wait_own(empty((g - 1) % OZ_STAGES), ((g - 1) / OZ_STAGES) & 1);
+      if (g > 0) (void)mbar_wait_own(empty((g - 1) % OZ_UNITS), ((g - 1) / OZ_UNITS) & 1);
     }
   } else if (warp >= 4) {
     const int quarter = warp & 3, colq = (warp - 4) >> 2;
@@ -731,11 +763,11 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
       xout = const_cast<double*>(a.xin);
     }
     long long* const xq = reinterpret_cast<long long*>(xout);
-    int u = 0;
-    for (int it = blockIdx.x;; it += gridDim.x, ++u) {
+    int v = 0, rd = 0;  // items taken, rounds of both passes drained
+    for (int it = blockIdx.x;; it += gridDim.x, ++v) {
       if (dyn) {
-        const int q = u % OZ_RING;
-        const bool got = __all_sync(0xffffffffu, mbar_wait(item_full(q), (u / OZ_RING) & 1, abort_flag));
+        const int q = v % OZ_RING;
+        const bool got = __all_sync(0xffffffffu, mbar_wait(item_full(q), (v / OZ_RING) & 1, abort_flag));
         if (!got) {
           *s_err = 1;
           break;
@@ -747,14 +779,14 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
       }
       if (it >= nitems) break;
       const int code = split ? a.split_items[it] : it;
-      const int ti = split ? code >> 1 : it;
+      const int ti = split ? code >> 1 : it, half = split ? code & 1 : -1;
       // a split item's 64-bit partial goes to its own tile of split_acc, which the item that
       // finishes the tile reads; otherwise the sums wait in this CTA's scratch tile
       long long* const acc = split ? a.split_acc + (size_t)code * (128 * 128) : cta_acc;
       const Tile t = a.tiles[ti];
       const PartDesc p = a.parts[t.part];
       const int64_t ld = p.ld;
-      const int r = t.ti * 128 + m, c0 = t.tj * 128;
+      const int r = t.ti * 128 + m;
       const bool diag = t.slot >= 0;
       const int sg = ADJ ? a.sig[t.part] : 0;  // the adjoint's sums hold (Xbar X + X Xbar) / 2^sg
       // columns the MMAs covered; the 16-column chunks beyond them lie in the part's zero
@@ -765,15 +797,16 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
       const int cskip = (t.ti == t.tj) ? quarter * 32 : 0;
       double tY = 0.0, tN = 0.0;
       bool ok = true;
-      // the two passes: read the groups' sums (integers at their groups' scales, held
-      // exactly in FP32) and add them as 64-bit integers, parked in TMEM between the passes
-      // and then in the scratch tile (thread-private entries: column cl, row m); each pass
-      // hands its columns back
-      for (int pass = 0; pass < 2; ++pass) {
-        ok = __all_sync(0xffffffffu, mbar_wait(afull(pass), u & 1, abort_flag)) && ok;
+      // the two passes of every round: read the accumulators' sums (integers at their scales,
+      // held exactly in FP32, but for the sixth) and add them as 64-bit integers, parked in
+      // TMEM between the passes and then in the scratch tile (thread-private entries: column
+      // cl, row m); each pass hands its columns back
+      const int3 kr = slices(p.s, half);
+      for (int c0 = kr.x, pass = 0; c0 < kr.y; pass ^= 1) {
+        ok = __all_sync(0xffffffffu, mbar_wait(afull(pass), rd & 1, abort_flag)) && ok;
         tc_fence_after();
-        // the high pass hands its columns back as soon as the warp's last chunk has read
-        // groups 5 and 6, which the low pass reuses (-1: no chunk, hand back at the end)
+        // the first pass hands its columns back as soon as the warp's last chunk has read
+        // columns 0-255, which the second reuses (-1: no chunk, hand back at the end)
         const int clast = (colq * 32 + 16 < ncols && colq * 32 + 32 > cskip) ? 1
                           : (colq * 32 < ncols && colq * 32 + 16 > cskip)   ? 0
                                                                             : -1;
@@ -786,18 +819,18 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
           long long z[16];
           uint32_t w[16];
           if (pass == 0) {
-            // the high groups' sum waits in the columns this warp has just drained (its own
-            // columns of groups 3 and 4), which the low pass leaves alone
+            // the first pass's sum waits in the columns this warp has just drained (its own
+            // columns among 256-511), which the second pass leaves alone
 #pragma unroll
             for (int j = 0; j < 16; ++j) z[j] = 0ll;
-            oz_drain_high56(tc, z);
+            oz_drain_high_a(tc, z);
             if (cc == clast) {
               tc_fence_before();
               __syncwarp();
               if (lane == 0) mbar_arrive(aempty(0));
               released = true;
             }
-            oz_drain_high34(tc, z);
+            oz_drain_high_b(tc, z);
 #pragma unroll
             for (int j = 0; j < 16; ++j) w[j] = (uint32_t)(unsigned long long)z[j];
             tmem_st16(tc + OZ_PARK_LO, w);
@@ -813,6 +846,10 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
             for (int j = 0; j < 16; ++j) z[j] += (long long)((unsigned long long)w[j] << 32);
             oz_drain_low(tc, z);
             long long* zp = acc + (size_t)cl * 128 + m;
+            if (c0 > kr.x) {  // the rounds before
+#pragma unroll
+              for (int j = 0; j < 16; ++j) z[j] += zp[(size_t)j * 128];
+            }
 #pragma unroll
             for (int j = 0; j < 16; ++j) zp[(size_t)j * 128] = z[j];
           }
@@ -822,6 +859,10 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
           tc_fence_before();
           __syncwarp();
           if (lane == 0) mbar_arrive(aempty(pass));
+        }
+        if (pass == 1) {
+          c0 = round_end(c0, kr);
+          ++rd;
         }
       }
       if (!ok) *s_err = 1;
@@ -852,7 +893,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
       for (int cc = 0; cc < 2 && ok; ++cc) {
         const int cl = colq * 32 + cc * 16;
         if (cl >= ncols || cl + 16 <= cskip) continue;
-        const int cbase = c0 + cl;
+        const int cbase = t.tj * 128 + cl;
         const long long* zp = acc + (size_t)cl * 128 + m;
         const long long* zo = other ? other + (size_t)cl * 128 + m : nullptr;
         float coln[16];  // adjoint: squares of the entries (r, c) for the norms of rows c
@@ -872,7 +913,6 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
                             : 0ll;
           }
           long long xn4[4];  // the words stored: fixed point (forward) or FP64 bits (adjoint)
-          uint32_t dw4[4][OZ_SLICES];
 #pragma unroll
           for (int w = 0; w < 4; ++w) {
             const int c = cbase + sub * 4 + w;
@@ -885,7 +925,6 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
               xn4[w] = sg == OZ_SIG_NONFINITE ? 0x7FF8000000000000ll : __double_as_longlong(from_fixed(xf, sg));
             else
               xn4[w] = xf;
-            if (!ADJ) digit_words(xf, dw4[w]);
             if (ADJ && upper && r < p.s && c < p.s) {
               // every stored entry (r, c) adds to the norm of row r, and of row c unless c = r
               const float f = fixed_to_f32_abs(xf);
@@ -894,15 +933,23 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
             }
             if (upper) {
               __stcs(xq + p.off + e, xn4[w]);
-              if (!ADJ) {
-#pragma unroll
-                for (int q = 0; q < OZ_SLICES; ++q)
-                  __stcs(a.digits[dbo].s[q] + p.off + e, (unsigned short)(dw4[w][q] >> 16));
-              }
               if (!ADJ && !rec && c == r && diag && r < p.c) {
                 tY += from_fixed(yf);
                 tN += from_fixed(xf);
               }
+            }
+          }
+          uint32_t dw[OZ_SLICES][2];  // the four columns' digits, two packed per word
+          if (!ADJ) {
+            digits4(xn4, dw);
+#pragma unroll
+            for (int w = 0; w < 4; ++w) {
+              const int c = cbase + sub * 4 + w;
+              if (!offd && c < r) continue;
+              const int64_t e = p.off + (int64_t)c * ld + r;
+#pragma unroll
+              for (int q = 0; q < OZ_SLICES; ++q)
+                __stcs(a.digits[dbo].s[q] + e, (unsigned short)(w & 1 ? dw[q][w >> 1] >> 16 : dw[q][w >> 1]));
             }
           }
           const int64_t em = p.off + (int64_t)r * ld + cbase + sub * 4;
@@ -914,12 +961,8 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
             __stcs(xm + 1, make_longlong2(xn4[2], xn4[3]));
             if (!ADJ) {
 #pragma unroll
-              for (int q = 0; q < OZ_SLICES; ++q) {
-                uint2 pk;  // upper halves of two words per 32 bits
-                pk.x = __byte_perm(dw4[0][q], dw4[1][q], 0x7632);
-                pk.y = __byte_perm(dw4[2][q], dw4[3][q], 0x7632);
-                __stcs(reinterpret_cast<uint2*>(a.digits[dbo].s[q] + em), pk);
-              }
+              for (int q = 0; q < OZ_SLICES; ++q)
+                __stcs(reinterpret_cast<uint2*>(a.digits[dbo].s[q] + em), make_uint2(dw[q][0], dw[q][1]));
             }
           } else if (!offd) {
 #pragma unroll
@@ -929,7 +972,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
               if (!ADJ) {
 #pragma unroll
                 for (int q = 0; q < OZ_SLICES; ++q)
-                  __stcs(a.digits[dbo].s[q] + em + w, (unsigned short)(dw4[w][q] >> 16));
+                  __stcs(a.digits[dbo].s[q] + em + w, (unsigned short)(w & 1 ? dw[q][w >> 1] >> 16 : dw[q][w >> 1]));
               }
             }
           }

@@ -1366,7 +1366,7 @@ int encode_part_maps(void* enc_fn, void* out_maps, const PartDesc* parts, int np
   return 0;
 }
 
-// Maps over the ndig consecutive BF16 digit arenas of the emulated step (digit t at
+// Maps over the ndig consecutive FP16 digit arenas of the emulated step (digit t at
 // arena0 + t dstride bytes) whose boxes take `nbox` digits at once, so that one request
 // fills nbox consecutive 128 x box_k digit tiles of a stage.  K-major: (column, row, digit),
 // strides 2 ld B and dstride B, box box_k x 128 x nbox, 64-byte rows and swizzle.  MN-major:
@@ -1390,7 +1390,7 @@ int encode_part_maps_digits(void* enc_fn, void* out_k, void* out_mn, const PartD
       cuuint64_t strides[2] = {ld * 2, (cuuint64_t)dstride};
       cuuint32_t box[3] = {(cuuint32_t)box_k, 128, (cuuint32_t)nbox};
       cuuint32_t estr[3] = {1u, 1u, 1u};
-      CUresult r = enc(&ok[k], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, addr, dims, strides, box, estr,
+      CUresult r = enc(&ok[k], CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 3, addr, dims, strides, box, estr,
                        CU_TENSOR_MAP_INTERLEAVE_NONE, box_k * 2 == 64 ? CU_TENSOR_MAP_SWIZZLE_64B
                                                                        : CU_TENSOR_MAP_SWIZZLE_128B,
                        CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
@@ -1401,7 +1401,7 @@ int encode_part_maps_digits(void* enc_fn, void* out_k, void* out_mn, const PartD
       cuuint64_t strides[3] = {ld * 2, 128, (cuuint64_t)dstride};
       cuuint32_t box[4] = {64, (cuuint32_t)box_k, 2, (cuuint32_t)nbox};
       cuuint32_t estr[4] = {1u, 1u, 1u, 1u};
-      CUresult r = enc(&om[k], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, addr, dims, strides, box, estr,
+      CUresult r = enc(&om[k], CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 4, addr, dims, strides, box, estr,
                        CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                        CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
       if (r != CUDA_SUCCESS) return (int)r;
