@@ -11,20 +11,21 @@
 //
 //   X X = sum_{a+b<T} 2^{-(e_a+e_b)} S_a S_b + (terms of order 2^-47): 15 products.
 //
-// The products are summed in FP32 in TMEM, in six accumulators.  Five of them hold integers
+// The products are summed in FP32 in TMEM, in six accumulators.  Four of them hold integers
 // (in units of their own scale) that stay below 2^24 and so are exact: (0,0), because
 // ||X||_2 <= 1 bounds sum_k |x_ik x_kj| by 1; (0,1) + (1,0) and (0,2) + (2,0), at most 2^19
 // and 2^22 times the row 1-norm sum_k |x_ik| (1 to 2 for the localised iterates of a gapped
 // system; for rows spread over all K columns the digits behave like independent values,
-// about 2^18 and 2^21); (1,1), whose diagonal is a sum of squares, K 2^12.4 for digits
-// spread over their range; and 2 [(1,2) + (2,1)] + (0,3) + (3,0), about sqrt(K) 2^17.  The
-// width of digit 1 follows from (1,1) staying below 2^24 up to K = 2048 (longer K is drained
-// every 2048), that of digit 3 from its accumulator; digits 0 and 2 are as wide as FP16
-// allows, which leaves so little behind them that (1,3), (0,4), (2,2) and their mirrors, of
-// order 2^-36 (2^-31 on the diagonal), share the sixth accumulator, whose FP32 rounding lies
-// below the dropped products.  Digits of 7 bits in BF16, whose 8-bit significand caps the
-// width, took 7 digits and 28 products for an error per entry of 1.3e-14 at K = 1,184 on
-// dense rows; these give 0.8e-14.
+// about 2^18 and 2^21); and (1,1), whose diagonal is a sum of squares, K 2^12.4 for digits
+// spread over their range.  The fifth, 2 [(1,2) + (2,1)] + (0,3) + (3,0) in units of 2^-50,
+// is exact too on localised iterates; on dense rows it is about sqrt(K) 2^17, and its
+// largest sums at K = 2048 round at 2^-49.  The width of digit 1 follows from (1,1) staying
+// below 2^24 up to K = 2048 (longer K is drained every 2048), that of digit 3 from the fifth
+// accumulator; digits 0 and 2 are as wide as FP16 allows, which leaves so little behind them
+// that (1,3), (0,4), (2,2) and their mirrors, of order 2^-36 (2^-31 on the diagonal), share
+// the sixth accumulator, whose FP32 rounding lies below the dropped products.  Digits of 7
+// bits in BF16, whose 8-bit significand caps the width, took 7 digits and 28 products for an
+// error per entry of 1.3e-14 at K = 1,184 on dense rows; these give 0.8e-14.
 // The accumulators are added as integers into a 64-bit fixed point (resolution 2^-56; the
 // sixth rounded to it), and a final elementwise pass forms X_new = Y or 2X - Y on that
 // grid (the master copy of the iterate stays in this fixed point), the core traces in FP64,
