@@ -56,30 +56,42 @@ namespace gsp2 {
 // FP16, and the products that share an accumulator land at one scale (rho_a + rho_b - e_a -
 // e_b is the same for (1,2) and (0,3), and for (1,3), (0,4) and (2,2)).  S_0 beyond 2^11
 // (|x| > 1, after low-precision steps) is kept even, which FP16 holds up to 2^12, and S_1
-// takes the rest.  Each value is the float 2^{23-rho} + u 2^-rho less (2^23 + half) 2^-rho, one
-// OR and one exact subtraction.
+// takes the rest.  Each value is a float whose significand
+// holds the field, less the same float of half its range: one AND/OR and one exact subtraction.
 __host__ __device__ constexpr int oz_e(int t) {  // x = sum_t S_t 2^-e_t
   return t == 0 ? 11 : (t == 1 ? 19 : (t == 2 ? 30 : (t == 3 ? 39 : 50)));
 }
 __host__ __device__ constexpr int oz_rho(int t) {  // stored: S_t 2^-rho_t
   return t == 0 ? -3 : (t == 1 ? -4 : (t == 4 ? 0 : -2));
 }
-__device__ __forceinline__ float digit_float(uint32_t u, int t, int half) {
-  const uint32_t e = (uint32_t)(150 - oz_rho(t)) << 23;  // exponent field of 2^{23-rho}
-  return __fsub_rn(__uint_as_float(e | u), __uint_as_float(e | (uint32_t)half));
+// Digit t, found biased by `half` at bit P of m (its field only): no shift is needed where the
+// field lies in the float's significand
+template <int T, int P>
+__device__ __forceinline__ float digit_float(uint32_t m, uint32_t half) {
+  constexpr uint32_t e = (uint32_t)(150 - oz_rho(T) - P) << 23;  // bit P weighs 2^-rho
+  return __fsub_rn(__uint_as_float(e | m), __uint_as_float(e | (half << P)));
 }
-__device__ __forceinline__ void digit_floats(long long v, float (&f)[OZ_SLICES]) {
-  constexpr int drop = 56 - oz_e(4);
-  constexpr long long bias = 1024ll + (256ll << 11) + (1024ll << 20) + (128ll << 31);
-  const long long w = ((v + (1ll << (drop - 1))) >> drop) + bias;
-  const uint32_t lo = (uint32_t)w, hi = (uint32_t)(w >> 31);
-  f[4] = digit_float(lo & 2047u, 4, 1024);
-  f[3] = digit_float((lo >> 11) & 511u, 3, 256);
-  f[2] = digit_float((lo >> 20) & 2047u, 2, 1024);
-  int s0 = (int)hi >> 8;
-  const int odd = (s0 > 2048 || s0 < -2048) ? (s0 & 1) : 0;
-  f[1] = digit_float((hi & 255u) + 256u * (uint32_t)odd, 1, 128);
-  f[0] = digit_float((uint32_t)(s0 - odd + 8192), 0, 8192);
+// Returns whether |S_0| > 2^11, where FP16 holds even integers only (digits_even).
+__device__ __forceinline__ bool digit_floats(long long v, float (&f)[OZ_SLICES]) {
+  // the rounding at 2^-50 and every field's bias in one addition; fields: S_4 bits 6-16, S_3
+  // 17-25, S_2 26-36, S_1 37-44, S_0 45-58
+  constexpr unsigned long long bias =
+      (1ull << 5) + (1024ull << 6) + (256ull << 17) + (1024ull << 26) + (128ull << 37) + (8192ull << 45);
+  const unsigned long long w = (unsigned long long)v + bias;
+  const uint32_t lo = (uint32_t)w, hi = (uint32_t)(w >> 32);
+  f[4] = digit_float<4, 6>(lo & (2047u << 6), 1024u);
+  f[3] = digit_float<3, 14>((lo >> 3) & (511u << 14), 256u);
+  f[2] = digit_float<2, 0>(__funnelshift_r(lo, hi, 26) & 2047u, 1024u);
+  f[1] = digit_float<1, 5>(hi & (255u << 5), 128u);
+  f[0] = digit_float<0, 9>((hi >> 4) & (16383u << 9), 8192u);
+  return hi - ((8192u - 2048u) << 13) >= (4097u << 13);
+}
+__device__ __forceinline__ void digits_even(float (&f)[OZ_SLICES]) {
+  const int s0 = (int)(f[0] * (1.0f / (float)(1 << -oz_rho(0))));
+  if ((s0 > 2048 || s0 < -2048) && (s0 & 1)) {
+    f[0] -= (float)(1 << -oz_rho(0));
+    f[1] += (float)(256 << -oz_rho(1));
+  }
 }
 // two digits as packed FP16 (lo in the lower half)
 __device__ __forceinline__ uint32_t pack_f16(float lo, float hi) {
@@ -92,8 +104,11 @@ __device__ __forceinline__ void digits4(const long long (&v)[4], uint32_t (&d)[O
 #pragma unroll
   for (int h = 0; h < 2; ++h) {
     float a[OZ_SLICES], b[OZ_SLICES];
-    digit_floats(v[2 * h], a);
-    digit_floats(v[2 * h + 1], b);
+    const bool big_a = digit_floats(v[2 * h], a), big_b = digit_floats(v[2 * h + 1], b);
+    if (big_a || big_b) {
+      digits_even(a);
+      digits_even(b);
+    }
 #pragma unroll
     for (int t = 0; t < OZ_SLICES; ++t) d[t][h] = pack_f16(a[t], b[t]);
   }
@@ -341,7 +356,8 @@ __global__ void __launch_bounds__(256) oz_digits_kernel(const PartDesc* __restri
 // runs the step bookkeeping.  K beyond OZ_CHUNK slices is taken in rounds of both passes, the
 // later ones adding to the scratch tile, so that the sums stay exact (see the top).
 //
-// 20 warps: warp 0 lane 0 TMA, warp 1 TMEM owner and MMA issuer, warps 4..19 epilogue
+// 20 warps: warps 0 and 2 lane 0 TMA (rows I and rows J: one thread's work per unit would hold
+// the ring back), warp 1 TMEM owner and MMA issuer, warps 4..19 epilogue
 // (warp w: TMEM lanes 32 (w % 4) .. + 31, columns 32 ((w - 4) / 4) .. + 31 of each group,
 // in two chunks of 16), sized so that four epilogue warps per scheduler hide latency.
 constexpr int OZ_UNITS = 5;                                      // operand units of the TMA ring
@@ -352,10 +368,16 @@ constexpr int OZ_CHUNK = 2048 / OZ_BK;                           // K slices per
 constexpr int OZ_EPI_WARPS = 16;                                 // 4 per TMEM lane quarter
 constexpr int OZ_THREADS = 32 * (4 + OZ_EPI_WARPS);
 constexpr int OZ_RING = 4;  // dynamic schedule: tiles claimed ahead of the MMA and epilogue warps
+// a claimed item as the producer passes it on: code < 0 ends the walk
+struct alignas(16) OzItem {
+  int64_t off, soff;
+  int32_t code, ti, tj, slot;
+  int32_t part, s, c, ld;
+};
 constexpr int OZ_SMEM = OZ_UNITS * (int)OZ_UNIT_B + 1024 + 8 * (2 * OZ_UNITS + 4) + 16 + 16 * OZ_EPI_WARPS +
-                        8 * 2 * OZ_RING + 4 * OZ_RING;
+                        8 * 2 * OZ_RING + (int)sizeof(OzItem) * OZ_RING;
 static_assert(OZ_LOW_SUB * OZ_LOW <= OZ_SLICES, "a unit holds the second pass's slices");
-static_assert((2 * OZ_UNITS + 4) % 2 == 0, "alignment of the reduction slots");
+static_assert((2 * OZ_UNITS + 4) % 2 == 0, "alignment of the reduction slots and items");
 static_assert(OZ_SMEM <= 232448, "shared memory of the emulated step");
 
 // Columns of tile column block tj that an MMA must cover: those inside the part, rounded up
@@ -379,67 +401,74 @@ __host__ __device__ constexpr int oz_b_lo(int q) { return LOW ? 0 : (q < 2 ? 2 -
 template <bool LOW>
 __host__ __device__ constexpr int oz_b_hi(int q) { return (LOW ? OZ_LOW : OZ_SLICES) - q; }
 
-// The MMAs of one K slice of a pass, fully unrolled, descriptors formed by adding
-// compile-time offsets to the slice's base descriptors (the 14-bit address field cannot
+// Descriptors of one K slice: lower words at the slice's first digit tile, upper words,
+// advance of a K = 16 step (16-byte units) and instruction descriptor.
+struct OzOperands {
+  uint32_t alo, ahi, blo, bhi, adv_a, adv_b, idesc;
+};
+
+// The MMAs of the K = 16 step KK of one slice of a pass, fully unrolled, descriptors formed by adding
+// compile-time offsets to the slice's lower words (the 14-bit address field cannot
 // carry: shared addresses stay below 2^18).  The products are issued A digit by A digit: the products of
 // A digit q follow one another and share their A operand through the
 // collector buffer, so each A digit tile is read from shared memory once per K = 16 slice
 // instead of once per product (the MMAs' shared-memory reads, A and B, set the pace of the
 // tensor pipe otherwise).
-template <bool LOW>
-__device__ __forceinline__ void oz_issue_slice(uint32_t tmem, uint64_t da, uint64_t db, uint32_t adv_a,
-                                               uint32_t adv_b, uint32_t idesc, bool first_k) {
-  constexpr uint64_t step = OZ_DTILE >> 4;
+template <bool LOW, int KK>
+__device__ __forceinline__ void oz_issue(uint32_t tmem, const OzOperands& o, bool first_k) {
+  constexpr uint32_t step = OZ_DTILE >> 4;
+  const uint32_t alo = o.alo + (KK ? KK * o.adv_a : 0u), blo = o.blo + (KK ? KK * o.adv_b : 0u);
 #pragma unroll
-  for (int kk = 0; kk < OZ_BK / 16; ++kk) {  // K = 16 steps of the slice
+  for (int q = 0; q < (LOW ? OZ_LOW : OZ_SLICES); ++q) {
+    const int b0 = oz_b_lo<LOW>(q), b1 = oz_b_hi<LOW>(q);
 #pragma unroll
-    for (int q = 0; q < (LOW ? OZ_LOW : OZ_SLICES); ++q) {
-      const int b0 = oz_b_lo<LOW>(q), b1 = oz_b_hi<LOW>(q);
-#pragma unroll
-      for (int b = b0; b < b1; ++b) {
-        const int op = (b1 - b0 == 1) ? 0 : (b == b0 ? 1 : (b == b1 - 1 ? 3 : 2));
-        // the first product into each accumulator: (0,0), (0,1); (0,2), (0,3), (0,4), (1,1)
-        const bool opens = q == 0 || (q == 1 && b == 1);
-        mma_f16_col(op, tmem + oz_col(q, b), da + (uint64_t)q * step + (uint64_t)(adv_a * kk),
-                    db + (uint64_t)b * step + (uint64_t)(adv_b * kk), idesc,
-                    (!opens || kk > 0 || !first_k) ? 1u : 0u);
-      }
+    for (int b = b0; b < b1; ++b) {
+      const int op = (b1 - b0 == 1) ? 0 : (b == b0 ? 1 : (b == b1 - 1 ? 3 : 2));
+      // the first product into each accumulator: (0,0), (0,1); (0,2), (0,3), (0,4), (1,1)
+      const bool opens = q == 0 || (q == 1 && b == 1);
+      mma_f16_lo(op, tmem + oz_col(q, b), alo + (uint32_t)q * step, o.ahi, blo + (uint32_t)b * step, o.bhi, o.idesc,
+                 (KK == 0 && opens && first_k) ? 0u : 1u);
     }
   }
 }
 
-// z[j] += u[j] 2^SHIFT for one accumulator of one 16-column chunk, where u = v 2^M is the
-// integer its FP32 sums v hold at the scale 2^-M (the sixth accumulator: v 2^M rounded).
-// A chunk whose integers all lie below 2^22 in magnitude is converted without the
-// conversion unit: v + 1.5 2^(23 - M) is a float in [2^(23 - M), 2^(24 - M)) with spacing 2^-M,
-// whose bit pattern less that of 1.5 2^(23 - M) is u, and a 32 x 32 -> 64-bit multiply-add
-// (by the power of two, or on the upper word for shifts of 32 and more) accumulates it; any
-// other chunk goes through the exact rounding conversion of v 2^M (|u| < 2^31).
+// The float bits of 1.5 2^(23 - M): a sum v of magnitude below 2^(22 - M) plus this float lies in
+// [2^(23 - M), 2^(24 - M)) with spacing 2^-M, so the bits of the sum are these plus v 2^M (rounded).
+__host__ __device__ constexpr uint32_t oz_magic(int M) { return ((uint32_t)(150 - M) << 23) | 0x400000u; }
+
+// z[j] += sgn (u[j] + oz_magic(M)) 2^SHIFT for one accumulator of one 16-column chunk, where
+// u = v 2^M is the integer its FP32 sums v hold at the scale 2^-M (the sixth accumulator: v 2^M
+// rounded); the constants oz_magic(M) 2^SHIFT of all accumulators are taken off once, where z
+// starts (oz_offset; 64-bit arithmetic modulo 2^64).  A chunk whose integers all lie below
+// 2^22 in magnitude is converted without the conversion unit, through the float bits, and a 32 x 32 ->
+// 64-bit multiply-add (by the power of two, or on the upper word for shifts of 32 and more)
+// accumulates it; any other chunk goes through the exact rounding conversion of v 2^M (|u| < 2^31).
 template <int M, int SHIFT>
-__device__ __forceinline__ void oz_drain_slot(uint32_t taddr, long long (&z)[16]) {
+__device__ __forceinline__ void oz_drain_slot(uint32_t taddr, int sgn, long long (&z)[16]) {
   uint32_t v[16];
   tmem_ld16(taddr, v);
-  const float magic = __uint_as_float(((uint32_t)(150 - M) << 23) | 0x400000u);  // 1.5 2^(23 - M)
-  const float lim = __uint_as_float((uint32_t)(149 - M) << 23);                   // 2^(22 - M)
+  const float magic = __uint_as_float(oz_magic(M));
+  const float lim = __uint_as_float((uint32_t)(149 - M) << 23);  // 2^(22 - M)
   float mx = 0.0f;
 #pragma unroll
   for (int j = 0; j < 16; ++j) mx = fmaxf(mx, fabsf(__uint_as_float(v[j])));
   if (__all_sync(0xffffffffu, mx < lim)) {
+    const int32_t mult = sgn * (1 << (SHIFT & 31));
 #pragma unroll
     for (int j = 0; j < 16; ++j) {
-      const int32_t g = (int32_t)(__float_as_uint(__fadd_rn(__uint_as_float(v[j]), magic)) - __float_as_uint(magic));
+      const int32_t g = (int32_t)__float_as_uint(__fadd_rn(__uint_as_float(v[j]), magic));
       if constexpr (SHIFT < 32) {
-        asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(z[j]) : "r"(g), "r"(1 << SHIFT));
+        asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(z[j]) : "r"(g), "r"(mult));
       } else {
-        z[j] += (long long)((unsigned long long)((uint32_t)g << (SHIFT - 32)) << 32);
+        z[j] += (long long)((unsigned long long)((uint32_t)g * (uint32_t)mult) << 32);
       }
     }
   } else {
     const float scale = __uint_as_float((uint32_t)(127 + M) << 23);  // 2^M
 #pragma unroll
     for (int j = 0; j < 16; ++j) {
-      const long long g = (long long)__float2int_rn(__fmul_rn(__uint_as_float(v[j]), scale));
-      z[j] += (long long)((unsigned long long)g << SHIFT);
+      const long long g = (long long)__float2int_rn(__fmul_rn(__uint_as_float(v[j]), scale)) + (long long)oz_magic(M);
+      z[j] += (long long)((unsigned long long)(sgn < 0 ? -g : g) << SHIFT);
     }
   }
 }
@@ -448,26 +477,51 @@ __device__ __forceinline__ void oz_drain_slot(uint32_t taddr, long long (&z)[16]
 // their integers weigh 2^(56-e_a-e_b) on the fixed point's grid.  GRID: the sums are taken as
 // multiples of 2^-GRID (the sixth accumulator, not an integer, rounded to 2^-56).
 template <int A, int B, int GRID = oz_e(A) + oz_e(B)>
-__device__ __forceinline__ void oz_drain(uint32_t taddr, long long (&z)[16]) {
-  constexpr int M = oz_rho(A) + oz_rho(B) - (oz_e(A) + oz_e(B) - GRID);
-  oz_drain_slot<M, 56 - GRID>(taddr + oz_col(A, B), z);
-}
+struct OzSlot {
+  static constexpr int M = oz_rho(A) + oz_rho(B) - (oz_e(A) + oz_e(B) - GRID);
+  static constexpr int SHIFT = 56 - GRID;
+  static constexpr unsigned long long offset = (unsigned long long)oz_magic(M) << SHIFT;
+  static __device__ __forceinline__ void drain(uint32_t taddr, int sgn, long long (&z)[16]) {
+    oz_drain_slot<M, SHIFT>(taddr + oz_col(A, B), sgn, z);
+  }
+};
+using OzSixth = OzSlot<0, 4, 56>;
 
 // The first pass of one chunk, in two halves: the columns the second pass reuses, then the
-// columns that hold the sums from then on, into z.
-__device__ __forceinline__ void oz_drain_high_a(uint32_t taddr, long long (&z)[16]) {
-  oz_drain<0, 4, 56>(taddr, z);
-  oz_drain<0, 3>(taddr, z);
+// columns that hold the sums from then on, into z (negated for sgn < 0).
+__device__ __forceinline__ void oz_drain_high_a(uint32_t taddr, int sgn, long long (&z)[16]) {
+  OzSixth::drain(taddr, sgn, z);
+  OzSlot<0, 3>::drain(taddr, sgn, z);
 }
-__device__ __forceinline__ void oz_drain_high_b(uint32_t taddr, long long (&z)[16]) {
-  oz_drain<0, 2>(taddr, z);
-  oz_drain<1, 1>(taddr, z);
+__device__ __forceinline__ void oz_drain_high_b(uint32_t taddr, int sgn, long long (&z)[16]) {
+  OzSlot<0, 2>::drain(taddr, sgn, z);
+  OzSlot<1, 1>::drain(taddr, sgn, z);
 }
 
 // The second pass of one chunk into z.
-__device__ __forceinline__ void oz_drain_low(uint32_t taddr, long long (&z)[16]) {
-  oz_drain<0, 0>(taddr, z);
-  oz_drain<0, 1>(taddr, z);
+__device__ __forceinline__ void oz_drain_low(uint32_t taddr, int sgn, long long (&z)[16]) {
+  OzSlot<0, 0>::drain(taddr, sgn, z);
+  OzSlot<0, 1>::drain(taddr, sgn, z);
+}
+
+// Where z starts: less the constants that the six drains of a round add.
+constexpr unsigned long long kOzOffset = OzSixth::offset + OzSlot<0, 3>::offset + OzSlot<0, 2>::offset +
+                                         OzSlot<1, 1>::offset + OzSlot<0, 0>::offset + OzSlot<0, 1>::offset;
+
+// z of a warp's 32 rows x 16 columns (lane l, z[j]: row l, column j) transposed within each half
+// warp: lane l, z[j] becomes row 16 (l / 16) + j, column l % 16.
+__device__ __forceinline__ void transpose16(long long (&z)[16], int lane) {
+#pragma unroll
+  for (int d = 8; d > 0; d >>= 1) {
+    const bool up = lane & d;
+#pragma unroll
+    for (int j = 0; j < 16; ++j) {
+      if (j & d) continue;
+      const long long got = __shfl_xor_sync(0xffffffffu, up ? z[j] : z[j + d], d);
+      if (up) z[j] = got;
+      else z[j + d] = got;
+    }
+  }
 }
 
 // |v| 2^-56 as FP32 (integer instructions, truncated: at most 2^-23 below), for the row
@@ -505,6 +559,29 @@ __device__ __forceinline__ float warp_colsum16(const float (&v)[16], int lane, i
 // diagonal tiles load both operands, the epilogue forms Xbar_new in FP64 without digits
 // or traces and adds its squared row norms (FP32, on the grid of the input scale); the last
 // block turns them into each part's new scale.
+// Predicated evict-first stores: the columns of a diagonal tile differ in the lanes that store,
+// and a branch per column costs more than the stores.
+__device__ __forceinline__ void store_word_if(bool on, long long* q, long long v) {
+  asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %0, 0;\n @p st.global.cs.b64 [%1], %2;\n}\n" ::"r"((int)on),
+               "l"(q), "l"(v)
+               : "memory");
+}
+// the digits of one element: word w (0..3) of the packed digits of four, dstr elements apart
+__device__ __forceinline__ void store_digits_if(bool on, uint16_t* d, size_t dstr, const uint32_t (&dw)[OZ_SLICES][2],
+                                                int w) {
+  static_assert(OZ_SLICES == 5, "five digit arenas");
+  unsigned short h[OZ_SLICES];
+#pragma unroll
+  for (int q = 0; q < OZ_SLICES; ++q) h[q] = (unsigned short)(w & 1 ? dw[q][w >> 1] >> 16 : dw[q][w >> 1]);
+  asm volatile(
+      "{\n .reg .pred p;\n setp.ne.b32 p, %0, 0;\n @p st.global.cs.u16 [%1], %6;\n @p st.global.cs.u16 [%2], %7;\n"
+      " @p st.global.cs.u16 [%3], %8;\n @p st.global.cs.u16 [%4], %9;\n @p st.global.cs.u16 [%5], %10;\n}\n" ::"r"(
+          (int)on),
+      "l"(d), "l"(d + dstr), "l"(d + 2 * dstr), "l"(d + 3 * dstr), "l"(d + 4 * dstr), "h"(h[0]), "h"(h[1]), "h"(h[2]),
+      "h"(h[3]), "h"(h[4])
+      : "memory");
+}
+
 template <bool ADJ>
 __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
   constexpr int T = OZ_SLICES;
@@ -537,11 +614,11 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
   int* s_err = reinterpret_cast<int*>(tmem_slot + 1);
   int* s_half = reinterpret_cast<int*>(tmem_slot + 2);  // split K: halves of the tile done before
   double2* red = reinterpret_cast<double2*>(sb + OZ_UNITS * OZ_UNIT_B + 8 * (2 * OZ_UNITS + 4) + 16);
-  // dynamic schedule: the producer claims each next tile from a counter in global memory and
-  // passes it on through a ring (full: claimed; empty: read by the MMA thread and every
-  // epilogue warp); -1 ends the walk
+  // warp 0's producer takes each next tile (claimed from a counter in global memory, or dealt)
+  // and passes it on with its part through a ring (full: taken; empty: read by the other
+  // producer, the MMA thread and every epilogue warp)
   const uint32_t ring_bars = smem_u32(red + OZ_EPI_WARPS);
-  int* s_items = reinterpret_cast<int*>(reinterpret_cast<uint8_t*>(red + OZ_EPI_WARPS) + 8 * 2 * OZ_RING);
+  OzItem* s_items = reinterpret_cast<OzItem*>(reinterpret_cast<uint8_t*>(red + OZ_EPI_WARPS) + 8 * 2 * OZ_RING);
   auto item_full = [&](int q) { return ring_bars + 8u * q; };
   auto item_empty = [&](int q) { return ring_bars + 8u * (OZ_RING + q); };
   auto full = [&](int s) { return bars + 8u * s; };
@@ -551,7 +628,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
   auto aempty = [&](int pass) { return bars + 8u * (2 * OZ_UNITS + 2 + pass); };
   auto unit = [&](int s) { return base + (uint32_t)s * OZ_UNIT_B; };
   int32_t* abort_flag = &a.ctl.st->timeout;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   const CUtensorMap* maps = reinterpret_cast<const CUtensorMap*>(a.maps) + (size_t)dbi * T * a.nparts;
   const CUtensorMap* maps_mn = reinterpret_cast<const CUtensorMap*>(a.maps_mn) + (size_t)dbi * T * a.nparts;
   const CUtensorMap* maps_b = reinterpret_cast<const CUtensorMap*>(a.maps_b);
@@ -587,7 +664,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
     }
     for (int q = 0; q < OZ_RING; ++q) {
       mbar_init(item_full(q), 1);
-      mbar_init(item_empty(q), 1 + OZ_EPI_WARPS);
+      mbar_init(item_empty(q), 2 + OZ_EPI_WARPS);
     }
     *s_err = 0;
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
@@ -599,152 +676,281 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = *tmem_slot;
+  const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
 
-  if (warp == 0 && lane == 0) {
-    uint32_t g = 0;
+  // warp-collective bounded wait (the same outcome in every lane)
+  auto wait = [&](uint32_t bar, uint32_t parity) {
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag)) != 0;
+  };
+  if (warp == 0 || warp == 2) {
+    // Like the issuing warp below, the whole warp walks the units with warp-uniform values and
+    // one elected lane issues the loads.
+    const int op = warp >> 1;      // 0: rows I, 1: rows J
+    uint32_t su = 0, ph = 0;       // next unit of the ring and its phase
+    uint32_t used = 0, phase = 0;  // units this warp has filled, and the phases of the last fills
     bool bad = false;
     // dynamic: the first item is blockIdx.x, the next ones gridDim.x + the counter's count,
     // each claimed one item ahead so that the atomic's latency hides behind an item's loads
-    int nxt = dyn && (int)blockIdx.x < nitems ? (int)gridDim.x + (int)atomicAdd(a.tile_ctr, 1u) : nitems;
+    int nxt = nitems;
+    if (op == 0 && lane == 0 && dyn && (int)blockIdx.x < nitems)
+      nxt = (int)gridDim.x + (int)atomicAdd(a.tile_ctr, 1u);
     for (int v = 0, it = blockIdx.x; !bad; ++v, it += gridDim.x) {
-      if (dyn) {
-        if (v > 0) {
-          it = nxt;
-          if (it < nitems) nxt = (int)gridDim.x + (int)atomicAdd(a.tile_ctr, 1u);
-        }
-        const int q = v % OZ_RING;
-        if (v >= OZ_RING && !mbar_wait(item_empty(q), ((v / OZ_RING) - 1) & 1, abort_flag)) {
+      const int q = v % OZ_RING;
+      if (op == 0) {
+        if (v >= OZ_RING && !wait(item_empty(q), ((v / OZ_RING) - 1) & 1)) {
           bad = true;
           break;
         }
-        s_items[q] = it < nitems ? it : -1;
-        mbar_arrive(item_full(q));
+        if (lane == 0) {
+          if (dyn && v > 0) {
+            it = nxt;
+            if (it < nitems) nxt = (int)gridDim.x + (int)atomicAdd(a.tile_ctr, 1u);
+          }
+          OzItem w;
+          w.code = -1;
+          if (it < nitems) {
+            w.code = split ? a.split_items[it] : it;
+            const Tile t = a.tiles[split ? w.code >> 1 : it];
+            const PartDesc p = a.parts[t.part];
+            w.ti = t.ti;
+            w.tj = t.tj;
+            w.slot = t.slot;
+            w.part = t.part;
+            w.off = p.off;
+            w.soff = p.soff;
+            w.s = p.s;
+            w.c = p.c;
+            w.ld = p.ld;
+          }
+          s_items[q] = w;
+          mbar_arrive(item_full(q));
+        }
+        __syncwarp();
+      } else if (!wait(item_full(q), (v / OZ_RING) & 1)) {
+        bad = true;
+        break;
       }
-      if (it >= nitems) break;
-      const int code = split ? a.split_items[it] : it;
-      const int ti = split ? code >> 1 : it, half = split ? code & 1 : -1;
-      const Tile t = a.tiles[ti];
-      const int sz = a.parts[t.part].s;
-      const bool dg = !ADJ && t.ti == t.tj;  // X X on a diagonal tile: B is A
-      const int ns = (sz + OZ_BK - 1) / OZ_BK;
-      const int3 kr = slices(sz, half);
+      OzItem w;
+      w.code = __shfl_sync(0xffffffffu, s_items[q].code, 0);
+      w.ti = __shfl_sync(0xffffffffu, s_items[q].ti, 0);
+      w.tj = __shfl_sync(0xffffffffu, s_items[q].tj, 0);
+      w.part = __shfl_sync(0xffffffffu, s_items[q].part, 0);
+      w.s = __shfl_sync(0xffffffffu, s_items[q].s, 0);
+      if (op == 1 && lane == 0) mbar_arrive(item_empty(q));
+      if (w.code < 0) break;
+      const int half = split ? w.code & 1 : -1;
+      const bool dg = !ADJ && w.ti == w.tj;  // X X on a diagonal tile: B is A
+      const int blk = op == 0 ? w.ti : w.tj;
+      const int ns = (w.s + OZ_BK - 1) / OZ_BK;
+      const int3 kr = slices(w.s, half);
+      // the next unit of this thread; false if the wait gave up
+      auto acquire = [&](uint32_t bytes, uint32_t& u) {
+        if (op == 1 && ++su == OZ_UNITS) {
+          su = 0;
+          ph ^= 1;
+        }
+        u = su;
+        if (!wait(empty(u), ph ^ 1u)) return false;
+        if (elect_one()) mbar_expect_tx(full(u), bytes);
+        used |= 1u << u;
+        phase = (phase & ~(1u << u)) | (ph << u);
+        if (++su == OZ_UNITS) {
+          su = 0;
+          ph ^= 1;
+        }
+        if (op == 0 && !dg && ++su == OZ_UNITS) {
+          su = 0;
+          ph ^= 1;
+        }
+        return true;
+      };
+      // one request brings a slice's digit tiles: K-major from columns `blk` of the tiles on or
+      // above the diagonal (slice block <= blk), else MN-major from rows `blk` of the tile (blk,
+      // slice).  The adjoint's first ns slices take Xbar for rows I and X for rows J, the rest
+      // X for rows I and Xbar for rows J
+      auto load = [&](uint32_t dst, uint32_t bar, int ks, size_t at) {
+        const bool h2 = ADJ && ks >= ns;
+        const bool xb = ADJ && (op == 0) != h2;
+        const int k0 = (h2 ? ks - ns : ks) * OZ_BK;
+        if (elect_one()) {
+          if (k0 / 128 <= blk) tma_load_3d(dst, (xb ? maps_b : maps) + at, k0, blk * 128, 0, bar);
+          else tma_load_4d(dst, (xb ? maps_mn_b : maps_mn) + at, 0, k0, 2 * blk, 0, bar);  // 64-row atoms x digits
+        }
+      };
+      if (op == 1 && dg) {  // rows I only: this thread's place in the ring moves past them
+        for (int c0 = kr.x, c1; c0 < kr.y; c0 = c1) {
+          c1 = round_end(c0, kr);
+          su += (uint32_t)(c1 - c0 + (c1 - c0 + OZ_LOW_SUB - 1) / OZ_LOW_SUB);
+        }
+        ph ^= (su / OZ_UNITS) & 1u;
+        su %= OZ_UNITS;
+        continue;
+      }
       for (int c0 = kr.x, c1; c0 < kr.y && !bad; c0 = c1) {
         c1 = round_end(c0, kr);
-        for (int pass = 0; pass < 2 && !bad; ++pass) {
-          const int nd = pass == 0 ? T : OZ_LOW, sub = pass == 0 ? 1 : OZ_LOW_SUB;
-          const size_t at = (size_t)pass * a.nparts + t.part;  // maps whose boxes take nd digits
-          for (int kb = c0; kb < c1 && !bad; kb += sub) {
-            const int m = min(sub, c1 - kb);
-            for (int op = 0; op < (dg ? 1 : 2); ++op, ++g) {  // rows I, then rows J
-              const int s = g % OZ_UNITS;
-              if (g >= OZ_UNITS && !mbar_wait(empty(s), ((g / OZ_UNITS) - 1) & 1, abort_flag)) {
-                bad = true;
-                break;
-              }
-              mbar_expect_tx(full(s), (uint32_t)(m * nd) * OZ_DTILE);
-              const int blk = op == 0 ? t.ti : t.tj;
-              for (int u = 0; u < m; ++u) {
-                // the adjoint's first ns slices take Xbar for rows I and X for rows J, the rest
-                // X for rows I and Xbar for rows J
-                const bool h2 = ADJ && kb + u >= ns;
-                const bool xb = ADJ && (op == 0) != h2;
-                const int k0 = (h2 ? kb + u - ns : kb + u) * OZ_BK;
-                const uint32_t dst = unit(s) + (uint32_t)(u * nd) * OZ_DTILE;
-                // K-major from columns `blk` of the tiles on or above the diagonal (slice block
-                // <= blk), else MN-major from rows `blk` of the tile (blk, slice); one request
-                // brings the slice's nd digit tiles
-                if (k0 / 128 <= blk)
-                  tma_load_3d(dst, (xb ? maps_b : maps) + at, k0, blk * 128, 0, full(s));
-                else
-                  tma_load_4d(dst, (xb ? maps_mn_b : maps_mn) + at, 0, k0, 2 * blk, 0, full(s));  // 64-row atoms x digits
-              }
-            }
+        uint32_t u;
+        for (int kb = c0; kb < c1; ++kb) {
+          if (!acquire(T * OZ_DTILE, u)) {
+            bad = true;
+            break;
           }
+          load(unit(u), full(u), kb, (size_t)w.part);
+        }
+        for (int kb = c0; kb < c1 && !bad; kb += OZ_LOW_SUB) {
+          const int m = min(OZ_LOW_SUB, c1 - kb);
+          if (!acquire((uint32_t)(m * OZ_LOW) * OZ_DTILE, u)) {
+            bad = true;
+            break;
+          }
+          for (int x = 0; x < m; ++x)
+            load(unit(u) + (uint32_t)(x * OZ_LOW) * OZ_DTILE, full(u), kb + x, (size_t)a.nparts + w.part);
         }
       }
     }
     if (bad) {
       *s_err = 1;
-      const uint32_t first = g > OZ_UNITS ? g - OZ_UNITS : 0;
-      for (uint32_t q = first; q < g; ++q) (void)mbar_wait_own(full(q % OZ_UNITS), (q / OZ_UNITS) & 1);
+      for (uint32_t u = 0; u < (uint32_t)OZ_UNITS; ++u)
+        if (used >> u & 1u) (void)mbar_wait_own(full(u), phase >> u & 1u);
     }
-  } else if (warp == 1 && lane == 0) {
-    uint32_t g = 0;
+  } else if (warp == 1) {
+    // The whole warp walks the slices with warp-uniform values (the item's fields through a
+    // shuffle), so that descriptors are formed in uniform registers, and one elected lane
+    // issues.  The issuing warp's own work between two slices (barrier tests, descriptors, commits) would
+    // leave the tensor pipe idle: the descriptors of the next unit are formed between the two K = 16
+    // steps of a slice, while the first step's MMAs run.
+    uint32_t su = 0, ph = 0;  // next unit of the ring and its phase
+    int last = -1;            // last unit released by a commit
+    uint32_t lastph = 0;
     int v = 0, r = 0;  // items taken, rounds of both passes done by this CTA
     bool bad = false;
-    for (int it = blockIdx.x; !bad; it += gridDim.x, ++v) {
-      if (dyn) {
-        const int q = v % OZ_RING;
-        if (!mbar_wait(item_full(q), (v / OZ_RING) & 1, abort_flag)) {
+    for (; !bad; ++v) {
+      const int q = v % OZ_RING;
+      if (!wait(item_full(q), (v / OZ_RING) & 1)) {
+        bad = true;
+        break;
+      }
+      const int code = __shfl_sync(0xffffffffu, s_items[q].code, 0);
+      const int ti = __shfl_sync(0xffffffffu, s_items[q].ti, 0), tj = __shfl_sync(0xffffffffu, s_items[q].tj, 0);
+      const int sz = __shfl_sync(0xffffffffu, s_items[q].s, 0);
+      if (lane == 0) mbar_arrive(item_empty(q));
+      if (code < 0) break;
+      const int half = split ? code & 1 : -1;
+      const bool dg = !ADJ && ti == tj;
+      const int ns = (sz + OZ_BK - 1) / OZ_BK;
+      const int3 kr = slices(sz, half);
+      const uint32_t idesc0 = IDESC | ((uint32_t)(oz_tile_cols(sz, tj) >> 3) << 17);
+      // operands of slice ks, tile `off` of the units sa (rows I) and sb (rows J): those right of
+      // the tile's own block came in MN-major (transpose bits 15 / 16); a K = 16 step advances
+      // 32 B in a K-major row, 2 KB (16 K values) in an MN-major tile
+      const uint64_t dk = smem_desc_sw<2 * OZ_BK>(0), dm = smem_desc_mn128(0, OZ_DTILE / 2);
+      auto operands = [&](int ks, uint32_t sa, uint32_t sb, int off) {
+        const int kt = (ADJ && ks >= ns ? ks - ns : ks) / (128 / OZ_BK);
+        const bool amn = kt > ti, bmn = kt > tj;
+        OzOperands o;
+        o.ahi = (uint32_t)((amn ? dm : dk) >> 32);
+        o.alo = (uint32_t)(amn ? dm : dk) + ((unit(sa) + (uint32_t)off * OZ_DTILE) >> 4);
+        o.adv_a = amn ? (2048u >> 4) : (32u >> 4);
+        o.bhi = (uint32_t)((bmn ? dm : dk) >> 32);
+        o.blo = (uint32_t)(bmn ? dm : dk) + ((unit(sb) + (uint32_t)off * OZ_DTILE) >> 4);
+        o.adv_b = bmn ? (2048u >> 4) : (32u >> 4);
+        o.idesc = idesc0 | ((amn ? 1u : 0u) << 15) | ((bmn ? 1u : 0u) << 16);
+        return o;
+      };
+      // the units of the next K step of the ring: rows I, rows J (the same on a diagonal tile)
+      uint32_t sa, pa, sb, pb;
+      auto take = [&]() {
+        sa = su;
+        pa = ph;
+        if (++su == OZ_UNITS) {
+          su = 0;
+          ph ^= 1;
+        }
+        sb = sa;
+        pb = pa;
+        if (!dg) {
+          sb = su;
+          pb = ph;
+          if (++su == OZ_UNITS) {
+            su = 0;
+            ph ^= 1;
+          }
+        }
+      };
+      auto loaded = [&]() {
+        if (!wait(full(sa), pa) || (!dg && !wait(full(sb), pb))) return false;
+        tc_fence_after();
+        return true;
+      };
+      auto release = [&](uint32_t ua, uint32_t ub, uint32_t pub) {
+        if (elect_one()) {
+          mma_commit(empty(ua));
+          if (!dg) mma_commit(empty(ub));
+        }
+        last = (int)ub;
+        lastph = pub;
+      };
+      for (int c0 = kr.x, c1; c0 < kr.y && !bad; c0 = c1, ++r) {
+        c1 = round_end(c0, kr);
+        // first pass: it reuses the columns of the previous round's second
+        take();
+        OzOperands o = operands(c0, sa, sb, 0);
+        if (r > 0 && !wait(aempty(1), (r - 1) & 1)) {
           bad = true;
           break;
         }
-        it = s_items[q];
-        mbar_arrive(item_empty(q));
-        if (it < 0) break;
-      }
-      if (it >= nitems) break;
-      const int code = split ? a.split_items[it] : it;
-      const int ti = split ? code >> 1 : it, half = split ? code & 1 : -1;
-      const Tile t = a.tiles[ti];
-      const int sz = a.parts[t.part].s;
-      const bool dg = !ADJ && t.ti == t.tj;
-      const int ns = (sz + OZ_BK - 1) / OZ_BK;
-      const int3 kr = slices(sz, half);
-      const uint32_t idesc0 = IDESC | ((uint32_t)(oz_tile_cols(sz, t.tj) >> 3) << 17);
-      for (int c0 = kr.x, c1; c0 < kr.y && !bad; c0 = c1, ++r) {
-        c1 = round_end(c0, kr);
-        for (int pass = 0; pass < 2 && !bad; ++pass) {
-          const int nd = pass == 0 ? T : OZ_LOW, sub = pass == 0 ? 1 : OZ_LOW_SUB;
-          // the first pass reuses the columns of the previous round's second, the second pass
-          // those of this round's first: wait until the epilogue has read them
-          const bool ready = pass == 0 ? (r == 0 || mbar_wait(aempty(1), (r - 1) & 1, abort_flag))
-                                       : mbar_wait(aempty(0), r & 1, abort_flag);
-          if (!ready) {
+        tc_fence_after();
+        for (int kb = c0; kb < c1; ++kb) {
+          if (!loaded()) {
             bad = true;
             break;
           }
-          tc_fence_after();
-          for (int kb = c0; kb < c1; kb += sub) {
-            const int m = min(sub, c1 - kb);
-            const int sa = g % OZ_UNITS, sB = dg ? sa : (g + 1) % OZ_UNITS;
-            if (!mbar_wait(full(sa), (g / OZ_UNITS) & 1, abort_flag) ||
-                (!dg && !mbar_wait(full(sB), ((g + 1) / OZ_UNITS) & 1, abort_flag))) {
-              bad = true;
-              break;
-            }
-            tc_fence_after();
-            for (int u = 0; u < m; ++u) {
-              // operands right of the tile's own block came in MN-major (transpose bits 15 / 16);
-              // a K = 16 step advances 32 B in a K-major row, 2 KB (16 K values) in an MN-major tile
-              const int ks = kb + u;
-              const int kt = (ADJ && ks >= ns ? ks - ns : ks) * OZ_BK / 128;
-              const bool amn = kt > t.ti, bmn = kt > t.tj;
-              const uint32_t off = (uint32_t)(u * nd) * OZ_DTILE;
-              const uint64_t da = amn ? smem_desc_mn128(unit(sa) + off, OZ_DTILE / 2)
-                                      : smem_desc_sw<2 * OZ_BK>(unit(sa) + off);
-              const uint64_t db = dg ? da
-                                     : (bmn ? smem_desc_mn128(unit(sB) + off, OZ_DTILE / 2)
-                                            : smem_desc_sw<2 * OZ_BK>(unit(sB) + off));
-              const uint32_t adv_a = amn ? (2048u >> 4) : (32u >> 4), adv_b = bmn ? (2048u >> 4) : (32u >> 4);
-              const uint32_t idesc = idesc0 | ((amn ? 1u : 0u) << 15) | ((bmn ? 1u : 0u) << 16);
-              if (pass == 0) oz_issue_slice<false>(tmem, da, db, adv_a, adv_b, idesc, ks == c0);
-              else oz_issue_slice<true>(tmem, da, db, adv_a, adv_b, idesc, ks == c0);
-            }
-            mma_commit(empty(sa));
-            if (!dg) mma_commit(empty(sB));
-            g += dg ? 1 : 2;
-          }
-          if (!bad) mma_commit(afull(pass));
+          if (elect_one()) oz_issue<false, 0>(tmem, o, kb == c0);
+          const OzOperands cur = o;
+          const uint32_t ua = sa, ub = sb, pub = pb;
+          take();  // after the last slice: the first unit of the second pass
+          if (kb + 1 < c1) o = operands(kb + 1, sa, sb, 0);
+          if (elect_one()) oz_issue<false, 1>(tmem, cur, false);
+          release(ua, ub, pub);
         }
+        if (bad) break;
+        if (elect_one()) mma_commit(afull(0));
+        // second pass: it reuses columns of this round's first
+        o = operands(c0, sa, sb, 0);
+        if (!wait(aempty(0), r & 1)) {
+          bad = true;
+          break;
+        }
+        tc_fence_after();
+        for (int kb = c0; kb < c1; kb += OZ_LOW_SUB) {
+          const bool two = kb + 1 < c1;
+          if (!loaded()) {
+            bad = true;
+            break;
+          }
+          if (elect_one()) {
+            oz_issue<true, 0>(tmem, o, kb == c0);
+            oz_issue<true, 1>(tmem, o, false);
+          }
+          const uint32_t ua = sa, ub = sb, pub = pb;
+          if (two) o = operands(kb + 1, sa, sb, OZ_LOW);
+          const bool more = kb + OZ_LOW_SUB < c1;
+          if (two && elect_one()) oz_issue<true, 0>(tmem, o, false);
+          const OzOperands cur = o;
+          if (more) {
+            take();
+            o = operands(kb + OZ_LOW_SUB, sa, sb, 0);
+          }
+          if (two && elect_one()) oz_issue<true, 1>(tmem, cur, false);
+          release(ua, ub, pub);
+        }
+        if (!bad && elect_one()) mma_commit(afull(1));
       }
     }
     if (bad) {
       *s_err = 1;
       // MMAs already issued keep reading shared memory and writing TMEM: wait (on this
-      // thread's own limit) for the last commit, which covers all of them
-      if (g > 0) (void)mbar_wait_own(empty((g - 1) % OZ_UNITS), ((g - 1) / OZ_UNITS) & 1);
+      // warp's own limit) for the last commit, which covers all of them
+      if (last >= 0) (void)mbar_wait_own(empty(last), lastph);
     }
   } else if (warp >= 4) {
     const int quarter = warp & 3, colq = (warp - 4) >> 2;
@@ -764,28 +970,37 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
       xout = const_cast<double*>(a.xin);
     }
     long long* const xq = reinterpret_cast<long long*>(xout);
+    // the sums are formed with the sign the step needs: X_new = 2X + z, z = -Y, or z = Y alone
+    const int sgn = alf > 0 ? -1 : 1;
+    // the digit arenas of a set lie one arena apart
+    const size_t dstr = ADJ ? 0 : (size_t)(a.digits[dbo].s[1] - a.digits[dbo].s[0]);
     int v = 0, rd = 0;  // items taken, rounds of both passes drained
-    for (int it = blockIdx.x;; it += gridDim.x, ++v) {
-      if (dyn) {
-        const int q = v % OZ_RING;
-        const bool got = __all_sync(0xffffffffu, mbar_wait(item_full(q), (v / OZ_RING) & 1, abort_flag));
-        if (!got) {
-          *s_err = 1;
-          break;
-        }
-        it = s_items[q];
-        __syncwarp();
-        if (lane == 0) mbar_arrive(item_empty(q));
-        if (it < 0) break;
+    for (;; ++v) {
+      const int iq = v % OZ_RING;
+      const bool got = __all_sync(0xffffffffu, mbar_wait(item_full(iq), (v / OZ_RING) & 1, abort_flag));
+      if (!got) {
+        *s_err = 1;
+        break;
       }
-      if (it >= nitems) break;
-      const int code = split ? a.split_items[it] : it;
-      const int ti = split ? code >> 1 : it, half = split ? code & 1 : -1;
+      OzItem t;  // warp-uniform
+      t.code = __shfl_sync(0xffffffffu, s_items[iq].code, 0);
+      t.ti = __shfl_sync(0xffffffffu, s_items[iq].ti, 0);
+      t.tj = __shfl_sync(0xffffffffu, s_items[iq].tj, 0);
+      t.slot = __shfl_sync(0xffffffffu, s_items[iq].slot, 0);
+      t.part = __shfl_sync(0xffffffffu, s_items[iq].part, 0);
+      t.s = __shfl_sync(0xffffffffu, s_items[iq].s, 0);
+      t.c = __shfl_sync(0xffffffffu, s_items[iq].c, 0);
+      t.ld = __shfl_sync(0xffffffffu, s_items[iq].ld, 0);
+      t.off = __shfl_sync(0xffffffffu, s_items[iq].off, 0);
+      t.soff = __shfl_sync(0xffffffffu, s_items[iq].soff, 0);
+      if (lane == 0) mbar_arrive(item_empty(iq));
+      if (t.code < 0) break;
+      const int code = t.code;
+      const int ti = split ? code >> 1 : code, half = split ? code & 1 : -1;
       // a split item's 64-bit partial goes to its own tile of split_acc, which the item that
       // finishes the tile reads; otherwise the sums wait in this CTA's scratch tile
       long long* const acc = split ? a.split_acc + (size_t)code * (128 * 128) : cta_acc;
-      const Tile t = a.tiles[ti];
-      const PartDesc p = a.parts[t.part];
+      const OzItem& p = t;
       const int64_t ld = p.ld;
       const int r = t.ti * 128 + m;
       const bool diag = t.slot >= 0;
@@ -796,42 +1011,53 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
       // a diagonal tile keeps its upper triangle and mirrors it: a chunk wholly left of the
       // warp's first row (all its entries below the diagonal) is neither drained nor formed
       const int cskip = (t.ti == t.tj) ? quarter * 32 : 0;
-      double tY = 0.0, tN = 0.0;
       bool ok = true;
+      // the warp's chunks of 16 columns: the last one's sums stay in registers for the final
+      // pass, the other one's wait in the scratch tile (-1: no chunk)
+      const int clast = (colq * 32 + 16 < ncols && colq * 32 + 32 > cskip) ? 1
+                        : (colq * 32 < ncols && colq * 32 + 16 > cskip)   ? 0
+                                                                          : -1;
+      const int cfirst = clast == 1 && colq * 32 + 16 > cskip ? 0 : -1;
+      // the previous iterate's lines of this warp (not written by this launch; read from HBM) come
+      // to L2 while the MMAs run: lane l, column l of the warp's 32, two lines of 128 B
+      if (alf > 0 && clast >= 0) {
+        const int c = t.tj * 128 + colq * 32 + lane;
+        if (c < p.s) {
+          const double* x = xin + p.off + (int64_t)c * ld + t.ti * 128 + quarter * 32;
+          asm volatile("prefetch.global.L2 [%0];\n prefetch.global.L2 [%0 + 128];\n" ::"l"(x));
+        }
+      }
+      long long z[16];
       // the two passes of every round: read the accumulators' sums (integers at their scales,
       // held exactly in FP32, but for the sixth) and add them as 64-bit integers, parked in
       // TMEM between the passes and then in the scratch tile (thread-private entries: column
-      // cl, row m); each pass hands its columns back
+      // cl, row m) or in registers; each pass hands its columns back
       const int3 kr = slices(p.s, half);
       for (int c0 = kr.x, pass = 0; c0 < kr.y; pass ^= 1) {
         ok = __all_sync(0xffffffffu, mbar_wait(afull(pass), rd & 1, abort_flag)) && ok;
         tc_fence_after();
         // the first pass hands its columns back as soon as the warp's last chunk has read
-        // columns 0-255, which the second reuses (-1: no chunk, hand back at the end)
-        const int clast = (colq * 32 + 16 < ncols && colq * 32 + 32 > cskip) ? 1
-                          : (colq * 32 < ncols && colq * 32 + 16 > cskip)   ? 0
-                                                                            : -1;
+        // columns 0-255, which the second reuses
         bool released = false;
 #pragma unroll 1
         for (int cc = 0; cc < 2 && ok; ++cc) {
+          if (cc != clast && cc != cfirst) continue;
           const int cl = colq * 32 + cc * 16;
-          if (cl >= ncols || cl + 16 <= cskip) continue;
           const uint32_t tc = tmem + lane_off + (uint32_t)cl;
-          long long z[16];
           uint32_t w[16];
           if (pass == 0) {
             // the first pass's sum waits in the columns this warp has just drained (its own
             // columns among 256-511), which the second pass leaves alone
 #pragma unroll
-            for (int j = 0; j < 16; ++j) z[j] = 0ll;
-            oz_drain_high_a(tc, z);
+            for (int j = 0; j < 16; ++j) z[j] = (long long)(sgn < 0 ? kOzOffset : 0ull - kOzOffset);
+            oz_drain_high_a(tc, sgn, z);
             if (cc == clast) {
               tc_fence_before();
               __syncwarp();
               if (lane == 0) mbar_arrive(aempty(0));
               released = true;
             }
-            oz_drain_high_b(tc, z);
+            oz_drain_high_b(tc, sgn, z);
 #pragma unroll
             for (int j = 0; j < 16; ++j) w[j] = (uint32_t)(unsigned long long)z[j];
             tmem_st16(tc + OZ_PARK_LO, w);
@@ -845,14 +1071,22 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
             tmem_ld16(tc + OZ_PARK_HI, w);
 #pragma unroll
             for (int j = 0; j < 16; ++j) z[j] += (long long)((unsigned long long)w[j] << 32);
-            oz_drain_low(tc, z);
+            oz_drain_low(tc, sgn, z);
+            if (cc == clast) {
+              tc_fence_before();
+              __syncwarp();
+              if (lane == 0) mbar_arrive(aempty(1));
+              released = true;
+            }
             long long* zp = acc + (size_t)cl * 128 + m;
             if (c0 > kr.x) {  // the rounds before
 #pragma unroll
               for (int j = 0; j < 16; ++j) z[j] += zp[(size_t)j * 128];
             }
+            if (split || cc != clast || round_end(c0, kr) < kr.y) {
 #pragma unroll
-            for (int j = 0; j < 16; ++j) zp[(size_t)j * 128] = z[j];
+              for (int j = 0; j < 16; ++j) zp[(size_t)j * 128] = z[j];
+            }
           }
         }
         if (pass == 0) tmem_wait_st();
@@ -886,108 +1120,121 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
       // final pass of the tile: X_new on the 2^-56 grid, fixed-point master, digits, traces (the
       // adjoint: Xbar_new, FP64 only); column writes are coalesced across the warp.  Only
       // tiles on or above the diagonal are kept (the next step reads the rest MN-major from
-      // them); a diagonal tile mirrors its upper triangle, each thread's row segment in
-      // groups of 4 as 32-byte (FP64) and 8-byte (digit) vectors
-      const bool offd = t.ti != t.tj;
-      float rown = 0.0f;  // adjoint: squared norm of row r over this thread's upper entries
-#pragma unroll 1
-      for (int cc = 0; cc < 2 && ok; ++cc) {
-        const int cl = colq * 32 + cc * 16;
-        if (cl >= ncols || cl + 16 <= cskip) continue;
+      // them); a diagonal tile mirrors its upper triangle, transposed among the lanes so that the
+      // mirrored columns are written 128 B (master) and 32 B (each digit) at a time
+      long long yd = 0ll, xd = 0ll;  // diagonal entry (r, r) of sgn Y and X_new
+      float rown = 0.0f;             // adjoint: squared norm of row r over this thread's upper entries
+      auto stored = [&](long long xf) {  // the word stored: fixed point (forward) or FP64 bits (adjoint)
+        if (!ADJ) return xf;
+        return sg == OZ_SIG_NONFINITE ? 0x7FF8000000000000ll : __double_as_longlong(from_fixed(xf, sg));
+      };
+      const bool dgt = t.ti == t.tj;
+      // A tile is formed once, so straight-line code for all 16 columns of a chunk would be fetched
+      // from L2 as often as it runs (a diagonal tile took 42,000 cycles, most of them waiting
+      // for instructions): the columns are taken eight at a time in loops, z turning in registers.
+      auto chunk = [&](int cl) {
         const int cbase = t.tj * 128 + cl;
-        const long long* zp = acc + (size_t)cl * 128 + m;
-        const long long* zo = other ? other + (size_t)cl * 128 + m : nullptr;
+        // element (first row of the warp, column cbase), uniform; the lane's row is added to it
+        int64_t e = p.off + (int64_t)cbase * ld + (t.ti * 128 + quarter * 32);
         float coln[16];  // adjoint: squares of the entries (r, c) for the norms of rows c
+#pragma unroll 1
+        for (int b = 0; b < 2; ++b, e += 8 * ld) {
+          const int cb = cbase + 8 * b;
+          long long xn[8];  // the forward iterates are kept in the fixed point itself; the adjoint's Xbar in FP64
 #pragma unroll
-        for (int j = 0; j < 16; ++j) coln[j] = 0.0f;
+          for (int j = 0; j < 8; ++j)
+            xn[j] = alf > 0 ? __ldg(reinterpret_cast<const long long*>(xin) + (e + (int64_t)j * ld) + lane) : 0ll;
 #pragma unroll
-        for (int sub = 0; sub < 4; ++sub) {
-          // loads of the group first (xin is not written by this launch), so that they are
-          // in flight together rather than each behind the previous group's stores
-          // the forward iterates are kept in the fixed point itself; the adjoint's Xbar in FP64
-          long long yv[4], xv[4];
-#pragma unroll
-          for (int w = 0; w < 4; ++w) {
-            const int j = sub * 4 + w;
-            yv[w] = zp[(size_t)j * 128] + (zo ? __ldcg(zo + (size_t)j * 128) : 0ll);
-            xv[w] = alf > 0 ? __ldg(reinterpret_cast<const long long*>(xin) + p.off + (int64_t)(cbase + j) * ld + r)
-                            : 0ll;
-          }
-          long long xn4[4];  // the words stored: fixed point (forward) or FP64 bits (adjoint)
-#pragma unroll
-          for (int w = 0; w < 4; ++w) {
-            const int c = cbase + sub * 4 + w;
-            const long long yf = yv[w];
-            const int64_t e = (int64_t)c * ld + r;
-            const bool upper = offd || c >= r;  // diagonal tiles: upper triangle only
-            const long long xi = ADJ ? to_fixed(__longlong_as_double(xv[w]), sg) : xv[w];
-            const long long xf = (alf > 0 && upper) ? 2 * xi - yf : yf;
-            if (ADJ)
-              xn4[w] = sg == OZ_SIG_NONFINITE ? 0x7FF8000000000000ll : __double_as_longlong(from_fixed(xf, sg));
-            else
-              xn4[w] = xf;
-            if (ADJ && upper && r < p.s && c < p.s) {
+          for (int j = 0; j < 8; ++j) {
+            const int c = cb + j;
+            const bool upper = !dgt || c >= r;
+            const long long xf = 2 * (ADJ ? to_fixed(__longlong_as_double(xn[j]), sg) : xn[j]) + z[j];
+            if (!ADJ && dgt && c == r) {  // the thread's one diagonal entry, if it has it
+              yd = z[j];
+              xd = xf;
+            }
+            if (ADJ) {
+              float f = 0.0f;
+              if (upper && r < p.s && c < p.s) f = fixed_to_f32_abs(xf);
               // every stored entry (r, c) adds to the norm of row r, and of row c unless c = r
-              const float f = fixed_to_f32_abs(xf);
               rown = fmaf(f, f, rown);
-              if (c != r) coln[sub * 4 + w] = f * f;
+              coln[j] = coln[8 + j];
+              coln[8 + j] = c != r ? f * f : 0.0f;
             }
-            if (upper) {
-              __stcs(xq + p.off + e, xn4[w]);
-              if (!ADJ && !rec && c == r && diag && r < p.c) {
-                tY += from_fixed(yf);
-                tN += from_fixed(xf);
-              }
-            }
+            xn[j] = stored(xf);
+            store_word_if(upper, xq + (e + (int64_t)j * ld) + lane, xn[j]);
           }
-          uint32_t dw[OZ_SLICES][2];  // the four columns' digits, two packed per word
           if (!ADJ) {
-            digits4(xn4, dw);
 #pragma unroll
-            for (int w = 0; w < 4; ++w) {
-              const int c = cbase + sub * 4 + w;
-              if (!offd && c < r) continue;
-              const int64_t e = p.off + (int64_t)c * ld + r;
+            for (int h = 0; h < 2; ++h) {
+              uint32_t dw[OZ_SLICES][2];  // four columns' digits, two packed per word
+              digits4({xn[4 * h], xn[4 * h + 1], xn[4 * h + 2], xn[4 * h + 3]}, dw);
 #pragma unroll
-              for (int q = 0; q < OZ_SLICES; ++q)
-                __stcs(a.digits[dbo].s[q] + e, (unsigned short)(w & 1 ? dw[q][w >> 1] >> 16 : dw[q][w >> 1]));
-            }
-          }
-          const int64_t em = p.off + (int64_t)r * ld + cbase + sub * 4;
-          if (!offd && cbase + sub * 4 > r) {
-            // the four mirrored elements are contiguous in column r: vector stores whenever
-            // all four lie right of the diagonal
-            longlong2* xm = reinterpret_cast<longlong2*>(xq + em);
-            __stcs(xm, make_longlong2(xn4[0], xn4[1]));
-            __stcs(xm + 1, make_longlong2(xn4[2], xn4[3]));
-            if (!ADJ) {
-#pragma unroll
-              for (int q = 0; q < OZ_SLICES; ++q)
-                __stcs(reinterpret_cast<uint2*>(a.digits[dbo].s[q] + em), make_uint2(dw[q][0], dw[q][1]));
-            }
-          } else if (!offd) {
-#pragma unroll
-            for (int w = 0; w < 4; ++w) {
-              if (cbase + sub * 4 + w <= r) continue;
-              __stcs(xq + em + w, xn4[w]);
-              if (!ADJ) {
-#pragma unroll
-                for (int q = 0; q < OZ_SLICES; ++q)
-                  __stcs(a.digits[dbo].s[q] + em + w, (unsigned short)(w & 1 ? dw[q][w >> 1] >> 16 : dw[q][w >> 1]));
+              for (int w = 0; w < 4; ++w) {
+                uint16_t* d = a.digits[dbo].s[0] + (e + (int64_t)(4 * h + w) * ld) + lane;
+                store_digits_if(!dgt || cb + 4 * h + w >= r, d, dstr, dw, w);
               }
             }
+          }
+#pragma unroll
+          for (int j = 0; j < 8; ++j) {
+            z[j] = z[8 + j];
+            z[8 + j] = xn[j];
           }
         }
-        if (ADJ) {
+        if (dgt) {
+          // the mirrored entries: lane l has column cbase + l % 16 of rows rb + j, which go to row
+          // cbase + l % 16 of columns rb + j
+          transpose16(z, lane);
+          int rb = t.ti * 128 + quarter * 32 + (lane & 16);
+          const int c = cbase + (lane & 15);
+          int64_t em = p.off + (int64_t)rb * ld + c;
+#pragma unroll 1
+          for (int b = 0; b < 4; ++b, rb += 4, em += 4 * ld) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+              store_word_if(c > rb + j, xq + em + (int64_t)j * ld, z[j]);
+            if (!ADJ) {
+              uint32_t dw[OZ_SLICES][2];
+              digits4({z[0], z[1], z[2], z[3]}, dw);
+#pragma unroll
+              for (int w = 0; w < 4; ++w) {
+                store_digits_if(c > rb + w, a.digits[dbo].s[0] + em + (int64_t)w * ld, dstr, dw, w);
+              }
+            }
+#pragma unroll
+            for (int j = 0; j < 12; ++j) z[j] = z[j + 4];
+          }
+        }
+        if constexpr (ADJ) {
           int col;
           const float cs = warp_colsum16(coln, lane, col);
           if (!(lane & 1) && cbase + col < p.s && cs != 0.0f) atomicAdd(&a.normf[p.soff + cbase + col], cs);
         }
+      };
+#pragma unroll 1
+      for (int pc = 0; pc < 2 && ok; ++pc) {
+        const int cc = pc == 0 ? clast : cfirst;
+        if (cc < 0) continue;
+        const int cl = colq * 32 + cc * 16;
+        if (pc == 1) {
+          const long long* zp = acc + (size_t)cl * 128 + m;
+#pragma unroll
+          for (int j = 0; j < 16; ++j) z[j] = zp[(size_t)j * 128];
+        }
+        if (other) {
+          const long long* zo = other + (size_t)cl * 128 + m;
+#pragma unroll
+          for (int j = 0; j < 16; ++j) z[j] += __ldcg(zo + (size_t)j * 128);
+        }
+        chunk(cl);
       }
       if (ADJ && ok && r < p.s && rown != 0.0f) atomicAdd(&a.normf[p.soff + r], rown);
       if (!ADJ && !rec && diag) {
-        tY = warp_sum(tY);
-        tN = warp_sum(tN);
+        // one conversion and FP64 sum per thread (zero where another warp has the entry)
+        const bool core = ok && r < p.c;
+        const double tY = warp_sum(core ? from_fixed(sgn < 0 ? -yd : yd) : 0.0);
+        const double tN = warp_sum(core ? from_fixed(xd) : 0.0);
         if (lane == 0) red[warp - 4] = make_double2(tY, tN);
         asm volatile("bar.sync 1, %0;\n" ::"n"(32 * OZ_EPI_WARPS) : "memory");
         if (warp == 4 && lane == 0) {
