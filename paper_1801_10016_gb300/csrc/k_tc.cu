@@ -301,8 +301,8 @@ __global__ void __launch_bounds__(256, 2) square_tc_kernel(TcStepArgs a) {
 // Persistent variant: one CTA per SM walks the tiles (largest parts first): blockIdx.x,
 // then the ones its producer claims from a counter (steps and reverse steps), or
 // blockIdx.x + gridDim.x, ... in the static deal.  Two TMEM accumulators let the epilogue of one tile run
-// while the tensor cores work on the next.  20 warps: warp 0 lane 0 issues TMA loads,
-// warp 1 owns TMEM and its lane 0 issues tcgen05.mma, warps 4..19 drain TMEM (four per
+// while the tensor cores work on the next.  20 warps: warps 0 and 2 issue TMA loads (rows I and
+// rows J), warp 1 owns TMEM and issues tcgen05.mma, warps 4..19 drain TMEM (four per
 // lane quarter, so that the epilogue, which writes the master and operand copies of the
 // tile and its mirror, keeps up with the tensor cores).  Same arithmetic and the same
 // bookkeeping as square_tc_kernel, bitwise; the MMAs of a part's last column block cover
@@ -327,6 +327,12 @@ __host__ __device__ constexpr int tc_tile_cols(int s, int tj) {
 constexpr int TC_EPI_WARPS = 16;  // 4 per TMEM lane quarter, 32 columns each
 constexpr int TC_RING = 4;        // dynamic schedule: tiles claimed ahead of the MMA and epilogue warps
 constexpr int TC_THREADS = 32 * (4 + TC_EPI_WARPS);
+// a taken tile as the producer passes it on with its part: part < 0 ends the walk
+struct alignas(16) TcItem {
+  int64_t off;
+  int32_t part, ti, tj, slot;
+  int32_t s, c, ld;
+};
 enum : int { TC_STEP = 0, TC_REBUILD = 1, TC_ADJOINT = 2 };
 
 template <int KIND, int NPROD, int MODE = TC_STEP>
@@ -388,21 +394,21 @@ __global__ void __launch_bounds__(TC_THREADS, 1) square_tc_persistent_kernel(TcS
   auto tempty = [&](int b) { return bars + 8u * (2 * STAGES + 2 + b); };
   auto tile_addr = [&](int s, int op) { return base + (uint32_t)s * STAGE_B + (uint32_t)op * kTileBytes; };
   int32_t* abort_flag = &a.ctl.st->timeout;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   // dynamic schedule (steps and reverse steps; the rebuilt iterates, which may run beside
-  // reverse steps and have no last block, keep the static deal): the producer claims each
-  // next tile from a counter in global memory and passes it to the MMA thread and the
-  // epilogue warps through a ring in shared memory (full: claimed; empty: read by all of
-  // them); -1 ends the walk
+  // reverse steps and have no last block, keep the static deal): tiles are claimed from a
+  // counter in global memory.  Warp 0 takes each next tile and passes it with its part to the other
+  // producer, the MMA warp and the epilogue warps through a ring in shared memory (full:
+  // taken; empty: read by all of them)
   const bool dyn = a.tile_ctr != nullptr && MODE != TC_REBUILD;
   const uint32_t ring_bars = smem_u32(red + TC_EPI_WARPS);
-  int* s_items = reinterpret_cast<int*>(reinterpret_cast<uint8_t*>(red + TC_EPI_WARPS) + 8 * 2 * TC_RING);
+  TcItem* s_items = reinterpret_cast<TcItem*>(reinterpret_cast<uint8_t*>(red + TC_EPI_WARPS) + 8 * 2 * TC_RING);
   auto item_full = [&](int q) { return ring_bars + 8u * q; };
   auto item_empty = [&](int q) { return ring_bars + 8u * (TC_RING + q); };
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) {
-      mbar_init(full(s), 1);
+      mbar_init(full(s), 2);  // both producers
       mbar_init(empty(s), 1);
     }
     for (int b = 0; b < 2; ++b) {
@@ -411,7 +417,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) square_tc_persistent_kernel(TcS
     }
     for (int q = 0; q < TC_RING; ++q) {
       mbar_init(item_full(q), 1);
-      mbar_init(item_empty(q), 1 + TC_EPI_WARPS);
+      mbar_init(item_empty(q), 2 + TC_EPI_WARPS);
     }
     *s_err = 0;
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
@@ -423,208 +429,247 @@ __global__ void __launch_bounds__(TC_THREADS, 1) square_tc_persistent_kernel(TcS
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = *tmem_slot;
+  const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
 
-  if (warp == 0 && lane == 0) {
-    // producer: one ring of stages across all tiles of this CTA
-    uint32_t g = 0;
+  // warp-collective bounded wait (the same outcome in every lane)
+  auto wait = [&](uint32_t bar, uint32_t parity) {
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag)) != 0;
+  };
+  // The producers and the MMA warp walk the stages as whole warps with warp-uniform values (the
+  // item's fields through a shuffle), so that addresses and descriptors are formed in uniform
+  // registers, and one elected lane issues: a single thread's own work per stage left the
+  // tensor pipe waiting for it.
+  if (warp == 0 || warp == 2) {
+    // producers, one ring of stages across all tiles of this CTA: warp 0 loads rows I, warp 2
+    // rows J (a diagonal tile of X X needs rows I only, B = A: each loads one of the two K
+    // blocks that a stage then holds)
+    const int op = warp >> 1;
+    uint32_t s = 0, ph = 0;        // next stage and its phase
+    uint32_t used = 0, phase = 0;  // stages this warp has loaded into, and the phases of the last loads
     bool bad = false;
     // dynamic: the first item is blockIdx.x, the next ones gridDim.x + the counter's count,
     // each claimed one item ahead so that the atomic's latency hides behind an item's loads
-    int nxt = dyn && (int)blockIdx.x < a.ntiles ? (int)gridDim.x + (int)atomicAdd(a.tile_ctr, 1u) : a.ntiles;
+    int nxt = a.ntiles;
+    if (op == 0 && lane == 0 && dyn && (int)blockIdx.x < a.ntiles)
+      nxt = (int)gridDim.x + (int)atomicAdd(a.tile_ctr, 1u);
+    // operand maps: the step's input iterate (MODE 0: by parity; 1 and 2: the rebuilt X), Xbar
+    // (adjoint), and the same arenas through MN-major boxes (16-bit kinds)
+    const CUtensorMap* const xhi = reinterpret_cast<const CUtensorMap*>(MODE == TC_STEP ? a.map_hi[bi] : a.xmap_hi);
+    const CUtensorMap* const xlo = reinterpret_cast<const CUtensorMap*>(MODE == TC_STEP ? a.map_lo[bi] : a.xmap_lo);
+    const CUtensorMap* const xhi_mn =
+        reinterpret_cast<const CUtensorMap*>(MODE == TC_STEP ? a.map_mn_hi[bi] : a.xmap_mn_hi);
+    const CUtensorMap* const xlo_mn =
+        reinterpret_cast<const CUtensorMap*>(MODE == TC_STEP ? a.map_mn_lo[bi] : a.xmap_mn_lo);
+    const CUtensorMap* const bhi = reinterpret_cast<const CUtensorMap*>(a.map_hi[bi]);
+    const CUtensorMap* const blo = reinterpret_cast<const CUtensorMap*>(a.map_lo[bi]);
+    const CUtensorMap* const bhi_mn = reinterpret_cast<const CUtensorMap*>(a.map_mn_hi[bi]);
+    const CUtensorMap* const blo_mn = reinterpret_cast<const CUtensorMap*>(a.map_mn_lo[bi]);
     for (int v = 0, ti = blockIdx.x; !bad; ++v, ti += gridDim.x) {
-      if (dyn) {
-        if (v > 0) {
-          ti = nxt;
-          if (ti < a.ntiles) nxt = (int)gridDim.x + (int)atomicAdd(a.tile_ctr, 1u);
-        }
-        const int q = v % TC_RING;
-        if (v >= TC_RING && !mbar_wait(item_empty(q), ((v / TC_RING) - 1) & 1, abort_flag)) {
+      const int q = v % TC_RING;
+      if (op == 0) {
+        if (v >= TC_RING && !wait(item_empty(q), ((v / TC_RING) - 1) & 1)) {
           bad = true;
           break;
         }
-        s_items[q] = ti < a.ntiles ? ti : -1;
-        mbar_arrive(item_full(q));
+        if (lane == 0) {
+          if (dyn && v > 0) {
+            ti = nxt;
+            if (ti < a.ntiles) nxt = (int)gridDim.x + (int)atomicAdd(a.tile_ctr, 1u);
+          }
+          TcItem w;
+          w.part = -1;
+          if (ti < a.ntiles) {
+            const Tile t = a.tiles[ti];
+            const PartDesc p = a.parts[t.part];
+            w.off = p.off;
+            w.part = t.part;
+            w.ti = t.ti;
+            w.tj = t.tj;
+            w.slot = t.slot;
+            w.s = p.s;
+            w.c = p.c;
+            w.ld = p.ld;
+          }
+          s_items[q] = w;
+          mbar_arrive(item_full(q));
+        }
+        __syncwarp();
+      } else if (!wait(item_full(q), (v / TC_RING) & 1)) {
+        bad = true;
+        break;
       }
-      if (ti >= a.ntiles) break;
-      const Tile t = a.tiles[ti];
-      const PartDesc p = a.parts[t.part];
-      // operand maps: the step's input iterate (MODE 0: by parity; 1 and 2: the rebuilt X)
-      const CUtensorMap* mhi =
-          reinterpret_cast<const CUtensorMap*>(MODE == TC_STEP ? a.map_hi[bi] : a.xmap_hi) + t.part;
-      const CUtensorMap* mlo =
-          reinterpret_cast<const CUtensorMap*>(MODE == TC_STEP ? a.map_lo[bi] : a.xmap_lo) + t.part;
-      const CUtensorMap* bhi =  // Xbar (adjoint)
-          MODE == TC_ADJOINT ? reinterpret_cast<const CUtensorMap*>(a.map_hi[bi]) + t.part : nullptr;
-      const CUtensorMap* blo = MODE == TC_ADJOINT ? reinterpret_cast<const CUtensorMap*>(a.map_lo[bi]) + t.part : nullptr;
-      // the same arenas through MN-major boxes (16-bit kinds)
-      const CUtensorMap* mhi_mn =
-          UPPER ? reinterpret_cast<const CUtensorMap*>(MODE == TC_STEP ? a.map_mn_hi[bi] : a.xmap_mn_hi) + t.part
-                : nullptr;
-      const CUtensorMap* mlo_mn =
-          UPPER ? reinterpret_cast<const CUtensorMap*>(MODE == TC_STEP ? a.map_mn_lo[bi] : a.xmap_mn_lo) + t.part
-                : nullptr;
-      const CUtensorMap* bhi_mn =
-          (UPPER && MODE == TC_ADJOINT) ? reinterpret_cast<const CUtensorMap*>(a.map_mn_hi[bi]) + t.part : nullptr;
-      const CUtensorMap* blo_mn =
-          (UPPER && MODE == TC_ADJOINT) ? reinterpret_cast<const CUtensorMap*>(a.map_mn_lo[bi]) + t.part : nullptr;
-      // a diagonal tile of X X needs rows I only (B = A): two K blocks per stage
-      const bool dg = MODE != TC_ADJOINT && t.ti == t.tj;
-      const int sub = dg ? 2 : 1;
-      const int nk = (p.s + sub * BKE - 1) / (sub * BKE);
-      for (int kb = 0; kb < (MODE == TC_ADJOINT ? 2 * nk : nk); ++kb, ++g) {
-        const int s = g % STAGES;
-        if (g >= STAGES && !mbar_wait(empty(s), ((g / STAGES) - 1) & 1, abort_flag)) {
+      const int part = __shfl_sync(0xffffffffu, s_items[q].part, 0), sz = __shfl_sync(0xffffffffu, s_items[q].s, 0);
+      const int bI = __shfl_sync(0xffffffffu, s_items[q].ti, 0), bJ = __shfl_sync(0xffffffffu, s_items[q].tj, 0);
+      if (op == 1 && lane == 0) mbar_arrive(item_empty(q));
+      if (part < 0) break;
+      const bool dg = MODE != TC_ADJOINT && bI == bJ;
+      const int nk = (sz + (dg ? 2 : 1) * BKE - 1) / ((dg ? 2 : 1) * BKE);
+      const int blk = op == 0 ? bI : bJ;
+      for (int kb = 0; kb < (MODE == TC_ADJOINT ? 2 * nk : nk); ++kb) {
+        if (!wait(empty(s), ph ^ 1u)) {
           bad = true;
           break;
         }
-        mbar_expect_tx(full(s), STAGE_B);
-        // rows `blk` of the K block at k0: K-major from the tile (k block, blk) where it is on
-        // or above the diagonal, else (16-bit kinds) MN-major from the upper tile (blk, k block)
-        auto load = [&](uint32_t dst, const CUtensorMap* mk, const CUtensorMap* mm, int k0, int blk) {
-          if (UPPER && k0 / 128 > blk) {
-            tma_load_2d(dst, mm, blk * 128, k0, full(s));
-            tma_load_2d(dst + kTileBytes / 2, mm, blk * 128 + 64, k0, full(s));
-          } else {
-            tma_load_2d(dst, mk, k0, blk * 128, full(s));
-          }
-        };
-        if (MODE == TC_ADJOINT) {
-          // first nk blocks: Xbar (rows I) times X (rows J); then X (rows I) times Xbar (rows J)
-          const bool h2 = kb >= nk;
-          const int k0 = (h2 ? kb - nk : kb) * BKE;
-          load(tile_addr(s, 0), h2 ? mhi : bhi, h2 ? mhi_mn : bhi_mn, k0, t.ti);
-          load(tile_addr(s, 1), h2 ? bhi : mhi, h2 ? bhi_mn : mhi_mn, k0, t.tj);
-          load(tile_addr(s, 2), h2 ? mlo : blo, h2 ? mlo_mn : blo_mn, k0, t.ti);
-          load(tile_addr(s, 3), h2 ? blo : mlo, h2 ? blo_mn : mlo_mn, k0, t.tj);
-        } else if (dg) {
-          for (int u = 0; u < 2; ++u) {
-            const int k0 = (2 * kb + u) * BKE;
-            load(tile_addr(s, u * (NOPS / 2)), mhi, mhi_mn, k0, t.ti);
-            if (NPROD == 3) load(tile_addr(s, u * 2 + 1), mlo, mlo_mn, k0, t.ti);
-          }
-        } else {
-          const int k0 = kb * BKE;
-          load(tile_addr(s, 0), mhi, mhi_mn, k0, t.ti);
-          load(tile_addr(s, 1), mhi, mhi_mn, k0, t.tj);
-          if (NPROD == 3) {
-            load(tile_addr(s, 2), mlo, mlo_mn, k0, t.ti);
-            load(tile_addr(s, 3), mlo, mlo_mn, k0, t.tj);
-          }
+        // the adjoint's first nk blocks: Xbar (rows I) times X (rows J); then X (rows I) times Xbar (rows J)
+        const bool h2 = MODE == TC_ADJOINT && kb >= nk;
+        const bool xb = MODE == TC_ADJOINT && (op == 0) != h2;
+        const int k0 = (dg ? 2 * kb + op : (h2 ? kb - nk : kb)) * BKE;
+        // slots of this warp's operand: hi, lo at 0, 2 (rows I) or 1, 3 (rows J); on a diagonal tile
+        // K block u at slots u NOPS / 2 (hi) and u 2 + 1 (lo)
+        const int sh = dg ? op * (NOPS / 2) : op, sl = dg ? op * 2 + 1 : 2 + op;
+        if (elect_one()) {
+          mbar_expect_tx(full(s), STAGE_B / 2);
+          // rows `blk` of the K block at k0: K-major from the tile (k block, blk) where it is on
+          // or above the diagonal, else (16-bit kinds) MN-major from the upper tile (blk, k block)
+          auto load = [&](uint32_t dst, const CUtensorMap* mk, const CUtensorMap* mm) {
+            if (UPPER && k0 / 128 > blk) {
+              tma_load_2d(dst, mm + part, blk * 128, k0, full(s));
+              tma_load_2d(dst + kTileBytes / 2, mm + part, blk * 128 + 64, k0, full(s));
+            } else {
+              tma_load_2d(dst, mk + part, k0, blk * 128, full(s));
+            }
+          };
+          load(tile_addr(s, sh), xb ? bhi : xhi, xb ? bhi_mn : xhi_mn);
+          if (NPROD == 3) load(tile_addr(s, sl), xb ? blo : xlo, xb ? blo_mn : xlo_mn);
+        }
+        used |= 1u << s;
+        phase = (phase & ~(1u << s)) | (ph << s);
+        if (++s == (uint32_t)STAGES) {
+          s = 0;
+          ph ^= 1;
         }
       }
     }
     if (bad) {
       *s_err = 1;
-      // do not leave while copies are in flight: bounded wait for the last stages issued
-      const uint32_t first = g > STAGES ? g - STAGES : 0;
-      for (uint32_t q = first; q < g; ++q) (void)mbar_wait_own(full(q % STAGES), (q / STAGES) & 1);
+      // do not leave while copies are in flight: bounded wait for the last stages loaded into
+      for (uint32_t u = 0; u < (uint32_t)STAGES; ++u)
+        if (used >> u & 1u) (void)mbar_wait_own(full(u), phase >> u & 1u);
     }
-  } else if (warp == 1 && lane == 0) {
-    // MMA issuer: tile i accumulates in TMEM columns [128 (i & 1), + 128)
-    uint32_t g = 0;
-    int i = 0;
+  } else if (warp == 1) {
+    // MMA warp: tile i accumulates in TMEM columns [128 (i & 1), + 128).  A stage's descriptors are
+    // formed before the last K step of the stage before it is issued, while the MMAs run.
+    uint32_t s = 0, ph = 0;  // next stage and its phase
+    int last = -1;           // last stage released by a commit
+    uint32_t lastph = 0;
     bool bad = false;
-    for (int ti = blockIdx.x; !bad; ti += gridDim.x, ++i) {
-      if (dyn) {
-        const int q = i % TC_RING;
-        if (!mbar_wait(item_full(q), (i / TC_RING) & 1, abort_flag)) {
-          bad = true;
-          break;
-        }
-        ti = s_items[q];
-        mbar_arrive(item_empty(q));
-        if (ti < 0) break;
+    for (int i = 0; !bad; ++i) {
+      const int q = i % TC_RING;
+      if (!wait(item_full(q), (i / TC_RING) & 1)) {
+        bad = true;
+        break;
       }
-      if (ti >= a.ntiles) break;
-      const Tile t = a.tiles[ti];
-      const PartDesc p = a.parts[t.part];
-      const bool dg = MODE != TC_ADJOINT && t.ti == t.tj;
-      const int nk = (MODE == TC_ADJOINT ? 2 : 1) * ((p.s + (dg ? 2 : 1) * BKE - 1) / ((dg ? 2 : 1) * BKE));
+      const int part = __shfl_sync(0xffffffffu, s_items[q].part, 0), sz = __shfl_sync(0xffffffffu, s_items[q].s, 0);
+      const int bI = __shfl_sync(0xffffffffu, s_items[q].ti, 0), bJ = __shfl_sync(0xffffffffu, s_items[q].tj, 0);
+      if (lane == 0) mbar_arrive(item_empty(q));
+      if (part < 0) break;
+      const bool dg = MODE != TC_ADJOINT && bI == bJ;
+      const int nb = dg ? 2 : 1;  // K blocks per stage
+      const int nk = (MODE == TC_ADJOINT ? 2 : 1) * ((sz + nb * BKE - 1) / (nb * BKE));
       const int b = i & 1, u = i >> 1;
-      if (u >= 1 && !mbar_wait(tempty(b), (u - 1) & 1, abort_flag)) {
+      const uint32_t d = tmem + (uint32_t)(b * 128);
+      const uint32_t IDESC = IDESC0 | ((uint32_t)(tc_tile_cols(sz, bJ) >> 3) << 17);
+      // operands of K block `v` of stage kb in slot group `st`: lower descriptor words of A hi, A lo,
+      // B hi, B lo, the upper words, the advance of a K step and the instruction descriptor
+      struct Ops {
+        uint32_t ah, al, bh, bl, ahi, bhi, adv_a, adv_b, idesc;
+      };
+      const uint64_t dk = smem_desc(0), dm = smem_desc_mn128(0, kTileBytes / 2);
+      auto operands = [&](int kb, int v, uint32_t st) {
+        // the K block and how each operand came in (MN-major right of the tile's block)
+        const int kq = dg ? 2 * kb + v : (MODE == TC_ADJOINT && kb >= nk / 2 ? kb - nk / 2 : kb);
+        const int kt = kq * BKE / 128;
+        const bool amn = UPPER && kt > bI, bmn = dg ? amn : UPPER && kt > bJ;
+        const uint32_t da = (uint32_t)(amn ? dm : dk), db = (uint32_t)(bmn ? dm : dk);
+        Ops o;
+        o.ah = da + (tile_addr(st, dg ? v * (NOPS / 2) : 0) >> 4);
+        o.al = da + (tile_addr(st, dg ? v * 2 + 1 : 2) >> 4);
+        o.bh = dg ? o.ah : db + (tile_addr(st, 1) >> 4);
+        o.bl = dg ? o.al : db + (tile_addr(st, 3) >> 4);
+        o.ahi = (uint32_t)((amn ? dm : dk) >> 32);
+        o.bhi = (uint32_t)((bmn ? dm : dk) >> 32);
+        // a K = KMMA step advances KMMA elements along a K-major row, KMMA rows of 128 B
+        // (64 MN elements) in an MN-major box
+        o.adv_a = amn ? (uint32_t)(KMMA * 128) >> 4 : (uint32_t)(KMMA * ES) >> 4;
+        o.adv_b = bmn ? (uint32_t)(KMMA * 128) >> 4 : (uint32_t)(KMMA * ES) >> 4;
+        o.idesc = IDESC | ((amn ? 1u : 0u) << 15) | ((bmn ? 1u : 0u) << 16);
+        return o;
+      };
+      auto issue = [&](const Ops& o, int kk, bool first) {
+        const uint32_t aa = o.adv_a * kk, ab = o.adv_b * kk;
+        // hi x hi and hi x lo share their A operand (collector buffer)
+        mma_lo<KIND>(NPROD == 3 ? 1 : 0, d, o.ah + aa, o.ahi, o.bh + ab, o.bhi, o.idesc, first ? 0u : 1u);
+        if (NPROD == 3) {
+          mma_lo<KIND>(3, d, o.ah + aa, o.ahi, o.bl + ab, o.bhi, o.idesc, 1u);
+          mma_lo<KIND>(0, d, o.al + aa, o.ahi, o.bh + ab, o.bhi, o.idesc, 1u);
+        }
+      };
+      Ops o = operands(0, 0, s);
+      if (u >= 1 && !wait(tempty(b), (u - 1) & 1)) {
         bad = true;
         break;
       }
       tc_fence_after();
-      const uint32_t d = tmem + (uint32_t)(b * 128);
-      const uint32_t IDESC = IDESC0 | ((uint32_t)(tc_tile_cols(p.s, t.tj) >> 3) << 17);
-      for (int kb = 0; kb < nk; ++kb, ++g) {
-        const int s = g % STAGES;
-        if (!mbar_wait(full(s), (g / STAGES) & 1, abort_flag)) {
+      for (int kb = 0; kb < nk; ++kb) {
+        if (!wait(full(s), ph)) {
           bad = true;
           break;
         }
         tc_fence_after();
-        for (int v = 0; v < (dg ? 2 : 1); ++v) {  // K blocks of the stage, in K order
-          // the K block and how each operand came in (MN-major right of the tile's block)
-          const int kq = dg ? 2 * kb + v : (MODE == TC_ADJOINT && kb >= nk / 2 ? kb - nk / 2 : kb);
-          const int kt = kq * BKE / 128;
-          const bool amn = UPPER && kt > t.ti, bmn = UPPER && kt > t.tj;
-          auto desc = [&](uint32_t addr, bool mn) {
-            return mn ? smem_desc_mn128(addr, kTileBytes / 2) : smem_desc(addr);
-          };
-          uint64_t ah, bh, al, bl;
-          if (dg) {
-            ah = bh = desc(tile_addr(s, v * (NOPS / 2)), amn);
-            al = bl = desc(tile_addr(s, v * 2 + 1), amn);
-          } else {
-            ah = desc(tile_addr(s, 0), amn);
-            bh = desc(tile_addr(s, 1), bmn);
-            al = desc(tile_addr(s, 2), amn);
-            bl = desc(tile_addr(s, 3), bmn);
-          }
-          // a K = KMMA step advances KMMA elements along a K-major row, KMMA rows of 128 B
-          // (64 MN elements) in an MN-major box
-          const uint32_t adv_a = amn ? (uint32_t)(KMMA * 128) >> 4 : (uint32_t)(KMMA * ES) >> 4;
-          const uint32_t adv_b = (dg ? amn : bmn) ? (uint32_t)(KMMA * 128) >> 4 : (uint32_t)(KMMA * ES) >> 4;
-          const uint32_t idesc = IDESC | ((amn ? 1u : 0u) << 15) | (((dg ? amn : bmn) ? 1u : 0u) << 16);
-#pragma unroll
-          for (int kk = 0; kk < NMMA; ++kk) {
-            const uint64_t aa = (uint64_t)(adv_a * kk), ab = (uint64_t)(adv_b * kk);
-            // hi x hi and hi x lo share their A operand (collector buffer)
-            mma_col<KIND>(NPROD == 3 ? 1 : 0, d, ah + aa, bh + ab, idesc, (kb > 0 || v > 0 || kk > 0) ? 1u : 0u);
-            if (NPROD == 3) {
-              mma_col<KIND>(3, d, ah + aa, bl + ab, idesc, 1u);
-              mma<KIND>(d, al + aa, bh + ab, idesc, 1u);
-            }
-          }
+        const uint32_t st = s, sp = ph;
+        if (++s == (uint32_t)STAGES) {
+          s = 0;
+          ph ^= 1;
         }
-        mma_commit(empty(s));
+        for (int v = 0; v < nb; ++v) {  // K blocks of the stage, in K order
+          if (elect_one()) {
+#pragma unroll
+            for (int kk = 0; kk < NMMA - 1; ++kk) issue(o, kk, kb == 0 && v == 0 && kk == 0);
+          }
+          const Ops cur = o;
+          if (v + 1 < nb) o = operands(kb, v + 1, st);
+          else if (kb + 1 < nk) o = operands(kb + 1, 0, s);
+          if (elect_one()) issue(cur, NMMA - 1, false);
+        }
+        if (elect_one()) mma_commit(empty(st));
+        last = (int)st;
+        lastph = sp;
       }
-      mma_commit(tfull(b));
+      if (!bad && elect_one()) mma_commit(tfull(b));
     }
     if (bad) {
       *s_err = 1;
       // MMAs already issued keep reading shared memory and writing TMEM: wait (on this
-      // thread's own limit) for the last commit, which covers all of them
-      if (g > 0) (void)mbar_wait_own(empty((g - 1) % STAGES), ((g - 1) / STAGES) & 1);
+      // warp's own limit) for the last commit, which covers all of them
+      if (last >= 0) (void)mbar_wait_own(empty(last), lastph);
     }
   } else if (warp >= 4) {
     // epilogue: warp w drains TMEM lanes 32 (w % 4) .. + 31, columns 32 ((w - 4) / 4) .. + 31,
     // in two halves of 16
     const int quarter = warp & 3, colq = (warp - 4) >> 2;
     const int m = quarter * 32 + lane;
-    int i = 0;
-    for (int ti = blockIdx.x;; ti += gridDim.x, ++i) {
-      if (dyn) {
-        const int q = i % TC_RING;
-        const bool got = __all_sync(0xffffffffu, mbar_wait(item_full(q), (i / TC_RING) & 1, abort_flag));
-        if (!got) {
-          *s_err = 1;
-          break;
-        }
-        ti = s_items[q];
-        __syncwarp();
-        if (lane == 0) mbar_arrive(item_empty(q));
-        if (ti < 0) break;
+    for (int i = 0;; ++i) {
+      const int q = i % TC_RING;
+      const bool got = __all_sync(0xffffffffu, mbar_wait(item_full(q), (i / TC_RING) & 1, abort_flag));
+      if (!got) {
+        *s_err = 1;
+        break;
       }
-      if (ti >= a.ntiles) break;
+      TcItem t;  // warp-uniform
+      t.off = __shfl_sync(0xffffffffu, s_items[q].off, 0);
+      t.part = __shfl_sync(0xffffffffu, s_items[q].part, 0);
+      t.ti = __shfl_sync(0xffffffffu, s_items[q].ti, 0);
+      t.tj = __shfl_sync(0xffffffffu, s_items[q].tj, 0);
+      t.slot = __shfl_sync(0xffffffffu, s_items[q].slot, 0);
+      t.s = __shfl_sync(0xffffffffu, s_items[q].s, 0);
+      t.c = __shfl_sync(0xffffffffu, s_items[q].c, 0);
+      t.ld = __shfl_sync(0xffffffffu, s_items[q].ld, 0);
+      if (lane == 0) mbar_arrive(item_empty(q));
+      if (t.part < 0) break;
+      const TcItem& p = t;
       const int b = i & 1, u = i >> 1;
       const bool ok = __all_sync(0xffffffffu, mbar_wait(tfull(b), u & 1, abort_flag));
       tc_fence_after();
-      const Tile t = a.tiles[ti];
-      const PartDesc p = a.parts[t.part];
       int8_t alf;
       if (MODE != TC_STEP) alf = a.ctl.alpha[step];  // the recorded branch
       else if (a.tail == 1) alf = (a.ctl.traces[step - 1] <= (double)a.ctl.nocc) ? (int8_t)1 : (int8_t)-1;
@@ -1092,7 +1137,7 @@ static cudaError_t launch_tc_persistent(const TcStepArgs& a, int grid, cudaStrea
   constexpr int NOPS = NPROD == 3 ? 4 : 2;
   constexpr int STAGES = NPROD == 3 ? 3 : 4;
   const int smem =
-      STAGES * NOPS * (int)kTileBytes + 1024 + 8 * (2 * STAGES + 4) + 16 + 16 * TC_EPI_WARPS + 8 * 2 * TC_RING + 4 * TC_RING;
+      STAGES * NOPS * (int)kTileBytes + 1024 + 8 * (2 * STAGES + 4) + 16 + 16 * TC_EPI_WARPS + 8 * 2 * TC_RING + (int)sizeof(TcItem) * TC_RING;
   cudaError_t e = cudaFuncSetAttribute(square_tc_persistent_kernel<KIND, NPROD, MODE>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;

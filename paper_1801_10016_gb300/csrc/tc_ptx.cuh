@@ -184,20 +184,33 @@ __device__ __forceinline__ bool elect_one() {
   return p != 0;
 }
 
-// The same for 16-bit operands from descriptor halves: the lower words carry the addresses,
-// which is all that changes from one MMA of a slice to the next (32-bit adds).
-#define GSP2_MMA_LO(OPSTR)                                                                                   \
+// The same from descriptor halves: the lower words carry the addresses, which is all that
+// changes from one MMA of a slice to the next (32-bit adds).
+#define GSP2_MMA_LO(KINDSTR, OPSTR)                                                                          \
   asm volatile("{\n .reg .pred p;\n .reg .b64 a, b;\n setp.ne.b32 p, %6, 0;\n mov.b64 a, {%1, %2};\n"       \
-               " mov.b64 b, {%3, %4};\n tcgen05.mma.cta_group::1.kind::f16" OPSTR " [%0], a, b, %5, p;\n}\n" \
+               " mov.b64 b, {%3, %4};\n tcgen05.mma.cta_group::1.kind::" KINDSTR OPSTR " [%0], a, b, %5, p;\n}\n" \
                ::"r"(tmem), "r"(alo), "r"(ahi), "r"(blo), "r"(bhi), "r"(idesc), "r"(acc))
-__device__ __forceinline__ void mma_f16_lo(int op, uint32_t tmem, uint32_t alo, uint32_t ahi, uint32_t blo,
-                                           uint32_t bhi, uint32_t idesc, uint32_t acc) {
-  if (op == 0) GSP2_MMA_LO("");
-  else if (op == 1) GSP2_MMA_LO(".collector::a::fill");
-  else if (op == 2) GSP2_MMA_LO(".collector::a::use");
-  else GSP2_MMA_LO(".collector::a::lastuse");
+template <int KIND>
+__device__ __forceinline__ void mma_lo(int op, uint32_t tmem, uint32_t alo, uint32_t ahi, uint32_t blo, uint32_t bhi,
+                                       uint32_t idesc, uint32_t acc) {
+  if (KIND != 1) {
+    if (op == 0) GSP2_MMA_LO("f16", "");
+    else if (op == 1) GSP2_MMA_LO("f16", ".collector::a::fill");
+    else if (op == 2) GSP2_MMA_LO("f16", ".collector::a::use");
+    else GSP2_MMA_LO("f16", ".collector::a::lastuse");
+  } else {
+    if (op == 0) GSP2_MMA_LO("tf32", "");
+    else if (op == 1) GSP2_MMA_LO("tf32", ".collector::a::fill");
+    else if (op == 2) GSP2_MMA_LO("tf32", ".collector::a::use");
+    else GSP2_MMA_LO("tf32", ".collector::a::lastuse");
+  }
 }
 #undef GSP2_MMA_LO
+// operands of 16-bit kinds (the emulated FP64 step)
+__device__ __forceinline__ void mma_f16_lo(int op, uint32_t tmem, uint32_t alo, uint32_t ahi, uint32_t blo,
+                                           uint32_t bhi, uint32_t idesc, uint32_t acc) {
+  mma_lo<0>(op, tmem, alo, ahi, blo, bhi, idesc, acc);
+}
 
 __device__ __forceinline__ void mma_commit(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(bar)
