@@ -335,6 +335,65 @@ struct alignas(16) TcItem {
 };
 enum : int { TC_STEP = 0, TC_REBUILD = 1, TC_ADJOINT = 2 };
 
+// Predicated stores of one element (master and operands): the columns of a diagonal tile differ
+// in the lanes that store, and a branch per column costs more than the stores.
+template <int KIND, int NPROD>
+__device__ __forceinline__ void store_element_if(bool on, float* master, void* hi, void* lo, int64_t e, float x, float xs) {
+  if (KIND != 1) {
+    const uint16_t h = Operand<KIND>::bits(xs);
+    uint16_t* ph = reinterpret_cast<uint16_t*>(hi) + e;
+    if (NPROD == 3) {
+      const uint16_t l = Operand<KIND>::bits(xs - Operand<KIND>::value(h));
+      uint16_t* pl = reinterpret_cast<uint16_t*>(lo) + e;
+      asm volatile(
+          "{\n .reg .pred p;\n setp.ne.b32 p, %0, 0;\n @p st.global.f32 [%1], %2;\n @p st.global.u16 [%3], %4;\n"
+          " @p st.global.u16 [%5], %6;\n}\n" ::"r"((int)on),
+          "l"(master + e), "f"(x), "l"(ph), "h"(h), "l"(pl), "h"(l)
+          : "memory");
+    } else {
+      asm volatile(
+          "{\n .reg .pred p;\n setp.ne.b32 p, %0, 0;\n @p st.global.f32 [%1], %2;\n @p st.global.u16 [%3], %4;\n}\n" ::"r"(
+              (int)on),
+          "l"(master + e), "f"(x), "l"(ph), "h"(h)
+          : "memory");
+    }
+  } else {
+    const uint32_t h = Operand<1>::bits(xs);
+    uint32_t* ph = reinterpret_cast<uint32_t*>(hi) + e;
+    if (NPROD == 3) {
+      const uint32_t l = Operand<1>::bits(xs - Operand<1>::value(h));
+      uint32_t* pl = reinterpret_cast<uint32_t*>(lo) + e;
+      asm volatile(
+          "{\n .reg .pred p;\n setp.ne.b32 p, %0, 0;\n @p st.global.f32 [%1], %2;\n @p st.global.b32 [%3], %4;\n"
+          " @p st.global.b32 [%5], %6;\n}\n" ::"r"((int)on),
+          "l"(master + e), "f"(x), "l"(ph), "r"(h), "l"(pl), "r"(l)
+          : "memory");
+    } else {
+      asm volatile(
+          "{\n .reg .pred p;\n setp.ne.b32 p, %0, 0;\n @p st.global.f32 [%1], %2;\n @p st.global.b32 [%3], %4;\n}\n" ::"r"(
+              (int)on),
+          "l"(master + e), "f"(x), "l"(ph), "r"(h)
+          : "memory");
+    }
+  }
+}
+
+// x of a warp's 32 rows x 16 columns (lane l, x[j]: row l, column j) transposed within each half
+// warp: lane l, x[j] becomes row 16 (l / 16) + j, column l % 16.
+__device__ __forceinline__ void transpose16(float (&x)[16], int lane) {
+#pragma unroll
+  for (int d = 8; d > 0; d >>= 1) {
+    const bool up = lane & d;
+#pragma unroll
+    for (int j = 0; j < 16; ++j) {
+      if (j & d) continue;
+      const float got = __shfl_xor_sync(0xffffffffu, up ? x[j] : x[j + d], d);
+      if (up) x[j] = got;
+      else x[j + d] = got;
+    }
+  }
+}
+
 template <int KIND, int NPROD, int MODE = TC_STEP>
 __global__ void __launch_bounds__(TC_THREADS, 1) square_tc_persistent_kernel(TcStepArgs a) {
   constexpr int NOPS = NPROD == 3 ? 4 : 2;
@@ -668,42 +727,59 @@ __global__ void __launch_bounds__(TC_THREADS, 1) square_tc_persistent_kernel(TcS
       if (t.part < 0) break;
       const TcItem& p = t;
       const int b = i & 1, u = i >> 1;
-      const bool ok = __all_sync(0xffffffffu, mbar_wait(tfull(b), u & 1, abort_flag));
-      tc_fence_after();
       int8_t alf;
       if (MODE != TC_STEP) alf = a.ctl.alpha[step];  // the recorded branch
       else if (a.tail == 1) alf = (a.ctl.traces[step - 1] <= (double)a.ctl.nocc) ? (int8_t)1 : (int8_t)-1;
       else if (a.tail == 2) alf = (int8_t)(-a.ctl.alpha[step - 1]);
       else alf = a.ctl.alpha[step];
       const float* Xi = (MODE == TC_REBUILD ? a.xin : a.master[bi]) + p.off;
-      float* Xo = (MODE == TC_REBUILD ? a.xout : a.master[bo]) + p.off;
+      float* Xo = MODE == TC_REBUILD ? a.xout : a.master[bo];
       void* ohi = MODE == TC_REBUILD ? a.xo_hi : a.op_hi[bo];
       void* olo = MODE == TC_REBUILD ? a.xo_lo : a.op_lo[bo];
       const int64_t ld = p.ld;
       const int r0 = t.ti * 128, c0 = t.tj * 128;
       const int r = r0 + m;
-      const bool diag = t.slot >= 0;
+      const bool diag = t.slot >= 0, dgt = t.ti == t.tj;
+      // the previous iterate's lines of this warp come to L2 while the MMAs run (lane l: column l
+      // of the warp's 32, one line of 128 B)
+      if (alf > 0 && c0 + colq * 32 + lane < p.s)
+        asm volatile("prefetch.global.L2 [%0];\n" ::"l"(Xi + (int64_t)(c0 + colq * 32 + lane) * ld + r0 + quarter * 32));
+      const bool ok = __all_sync(0xffffffffu, mbar_wait(tfull(b), u & 1, abort_flag));
+      tc_fence_after();
+      if (!ok) *s_err = 1;
+      // the warp's two chunks of 16 columns, read at once, so that the accumulator is handed back
+      // before the stores.  16-column chunks beyond the MMAs' columns lie in the part's zero padding,
+      // which no step writes (the iterate and operand arenas are zeroed when the workspace is
+      // bound); on a diagonal tile a chunk wholly left of the warp's first row holds only
+      // entries below the diagonal, which the mirror of the upper triangle writes
+      uint32_t v[16], v2[16];
+      bool has[2];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int cl = colq * 32 + h * 16;
+        has[h] = ok && cl < tc_tile_cols(p.s, t.tj) && !(dgt && cl + 16 <= quarter * 32);
+      }
+      {
+        const uint32_t tc = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(b * 128 + colq * 32);
+        if (has[0]) tmem_ld16(tc, v);
+        if (has[1]) tmem_ld16(tc + 16, v2);
+      }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(tempty(b));
       // sums back to the unscaled product: 2^-28 for FP16 operands of X 2^14 on both sides,
       // 2^(sig - 28) where the Xbar side is FP16 of Xbar 2^(14 - sig)
       const float ysc = XBAR16 ? pow2i(a.xb_sig[t.part] - 28) : Kind<KIND>::YSCALE;
       const float osc = XBAR16 ? pow2i(-a.xb_sig[a.nparts + t.part]) : 1.0f;  // Xbar_new's operand scale
       uint32_t amax = 0;  // FP16 adjoint: largest |Xbar_new| of the thread's entries (FP32 bits)
       double tY = 0.0, tN = 0.0;
-      if (ok) {
 #pragma unroll 1
-        for (int h = 0; h < 2; ++h) {
-          const int cl = colq * 32 + h * 16;
-          // 16-column chunks beyond the MMAs' columns lie in the part's zero padding, which
-          // no step writes (the iterate and operand arenas are zeroed when the workspace is
-          // bound); on a diagonal tile a chunk wholly left of the warp's first row holds only
-          // entries below the diagonal, which the mirror of the upper triangle writes
-          if (cl >= tc_tile_cols(p.s, t.tj) || (t.ti == t.tj && cl + 16 <= quarter * 32)) continue;
-          const int cbase = c0 + cl;
-          uint32_t v[16];
-          tmem_ld16(tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(b * 128 + cl), v);
+      for (int h = 0; h < 2; ++h) {
+        if (has[0]) {
+          const int cbase = c0 + colq * 32 + h * 16;
           float x[16];
 #pragma unroll
-          for (int j = 0; j < 16; ++j) x[j] = Xi[(int64_t)(cbase + j) * ld + r];
+          for (int j = 0; j < 16; ++j) x[j] = alf > 0 ? Xi[(int64_t)(cbase + j) * ld + r] : 0.0f;
           // the one diagonal entry of this half row, if any, picked out in FP32 and added in
           // FP64 once (an FP64 add in the unrolled loop would be issued for every element)
           float yd = 0.0f, zd = 0.0f;
@@ -721,45 +797,45 @@ __global__ void __launch_bounds__(TC_THREADS, 1) square_tc_persistent_kernel(TcS
             tN += (double)zd;
           }
           // diagonal tiles: keep the upper triangle (c >= r) and mirror it, so X stays exactly
-          // symmetric whatever order the tensor cores sum the split products in
+          // symmetric whatever order the tensor cores sum the split products in.  Eight columns
+          // per iteration, x turning in registers: straight-line code for 16 would be refetched for every tile
+          int64_t e = p.off + (int64_t)cbase * ld + r;
+#pragma unroll 1
+          for (int q2 = 0; q2 < 2; ++q2, e += 8 * ld) {
 #pragma unroll
-          for (int j = 0; j < 16; ++j) {
-            if (t.ti == t.tj && cbase + j < r) continue;
-            const int64_t e = (int64_t)(cbase + j) * ld + r;
-            Xo[e] = x[j];
-            store_operands<KIND, NPROD>(ohi, olo, p.off + e, XBAR16 ? x[j] * osc : x[j]);
-          }
-          if (t.ti == t.tj && cbase <= r) {
-            // the 16 x 16 blocks of a diagonal tile that straddle the diagonal: element stores
-            for (int j = 0; j < 16; ++j) {
-              if (cbase + j <= r) continue;
-              const int64_t e = (int64_t)r * ld + cbase + j;
-              Xo[e] = x[j];
-              store_operands<KIND, NPROD>(ohi, olo, p.off + e, XBAR16 ? x[j] * osc : x[j]);
+            for (int j = 0; j < 8; ++j)
+              store_element_if<KIND, NPROD>(!dgt || cbase + 8 * q2 + j >= r, Xo, ohi, olo, e + (int64_t)j * ld, x[j],
+                                            XBAR16 ? x[j] * osc : x[j]);
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+              const float y = x[j];
+              x[j] = x[8 + j];
+              x[8 + j] = y;
             }
-          } else if (!UPPER || t.ti == t.tj) {
-            // the mirrored row segment (all of it right of the diagonal): vector stores (the
-            // 16-bit kinds keep off-diagonal tiles upper only and mirror diagonal tiles only)
-            const int64_t e0 = (int64_t)r * ld + cbase;
-            float4* dst = reinterpret_cast<float4*>(Xo + e0);
+          }
+          if (!UPPER || dgt) {
+            // the mirrored entries (the 16-bit kinds keep off-diagonal tiles upper only), transposed
+            // among the lanes: lane l has column cbase + l % 16 of rows rb + j, which go to row
+            // cbase + l % 16 of columns rb + j
+            transpose16(x, lane);
+            int rb = r0 + quarter * 32 + (lane & 16);
+            const int c = cbase + (lane & 15);
+            int64_t em = p.off + (int64_t)rb * ld + c;
+#pragma unroll 1
+            for (int q2 = 0; q2 < 2; ++q2, rb += 8, em += 8 * ld) {
 #pragma unroll
-            for (int q = 0; q < 4; ++q) dst[q] = make_float4(x[4 * q], x[4 * q + 1], x[4 * q + 2], x[4 * q + 3]);
-            if (XBAR16) {
-              float xs[16];
+              for (int j = 0; j < 8; ++j)
+                store_element_if<KIND, NPROD>(!dgt || c > rb + j, Xo, ohi, olo, em + (int64_t)j * ld, x[j],
+                                              XBAR16 ? x[j] * osc : x[j]);
 #pragma unroll
-              for (int j = 0; j < 16; ++j) xs[j] = x[j] * osc;
-              store_operand_row<KIND, NPROD, 16>(ohi, olo, p.off + e0, xs);
-            } else {
-              store_operand_row<KIND, NPROD, 16>(ohi, olo, p.off + e0, x);
+              for (int j = 0; j < 8; ++j) x[j] = x[8 + j];
             }
           }
         }
-      } else {
-        *s_err = 1;
+        has[0] = has[1];
+#pragma unroll
+        for (int j = 0; j < 16; ++j) v[j] = v2[j];
       }
-      tc_fence_before();
-      __syncwarp();
-      if (lane == 0) mbar_arrive(tempty(b));
       if (XBAR16) {
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) amax = max(amax, __shfl_xor_sync(0xffffffffu, amax, o));
