@@ -57,7 +57,7 @@ struct WsLayout {
   size_t aop_maps;                // CUtensorMap[2 (S + 2)][nparts]
   size_t aop_maps_mn;             // the same, MN-major boxes
   size_t xb_sig, xb_max;          // int32[2][nparts] (scales read, written), uint32[nparts]
-  size_t mask;                    // uint8[nnz_p]: |P| > tau flags of gsp2_threshold_graph
+  size_t gdeg, growptr, gcol;     // gsp2_threshold_graph: int32[n], int64[n + 1], columns of a range of rows
   std::vector<size_t> tailf;      // low-precision adjoint: FP32 iterates of the FP64 tail, recomputed
   size_t slots, rslots, state, alpha, traces, idem, step_arena;
   size_t xchg;                 // ShardSlot of a shard plan's exchanges
@@ -259,6 +259,12 @@ extern "C" void gsp2_default_options(gsp2_options* o) {
 
 extern "C" const char* gsp2_last_error(gsp2_handle h) { return h ? h->err.c_str() : t_create_err.c_str(); }
 
+// Columns of the graph refresh that fit its buffer: the whole graph (at most two edges per
+// stored value of P and the diagonal) up to 64 MB, then ranges of rows (one row at least)
+static int64_t graph_cap(const gsp2_plan* h) {
+  return std::max<int64_t>(h->n, std::min<int64_t>(2 * h->pcolptr[(size_t)h->n] + h->n, int64_t(16) << 20));
+}
+
 static void build_layout(gsp2_plan* h) {
   WsLayout& L = h->L;
   h->use_oz = h->opt.precision == GSP2_PREC_FP64_EMU ||
@@ -308,7 +314,9 @@ static void build_layout(gsp2_plan* h) {
   L.idem = take(((size_t)h->opt.max_steps + HIST_EXTRA) * sizeof(double));
   L.step_arena = take(((size_t)h->total_steps + 1) * sizeof(double*));
   L.master_of_step = take(((size_t)h->opt.max_steps + 1 + MAX_TAIL) * sizeof(float*));
-  L.mask = take((size_t)h->pcolptr[(size_t)h->n]);
+  L.gdeg = take((size_t)h->n * sizeof(int32_t));
+  L.growptr = take(((size_t)h->n + 1) * sizeof(int64_t));
+  L.gcol = take((size_t)graph_cap(h) * sizeof(int32_t));
   const size_t ab = (size_t)h->arena_elems * sizeof(double);
   const int prec = h->opt.precision;
   if (!fp64_like(prec)) {
@@ -1593,55 +1601,42 @@ extern "C" gsp2_status gsp2_threshold_graph(gsp2_handle h, const double* d_pvals
   if (!d_pvals || !g_rowptr || !nnz || !(tau >= 0.0) || cap < 0) return fail(h, GSP2_E_ARG, "NULL argument or tau < 0");
   if (!h->ws) return fail(h, GSP2_E_STATE, "no workspace bound");
   cudaStream_t s = (cudaStream_t)stream;
-  const int64_t np = h->pcolptr[h->n];
-  std::vector<uint8_t> mask((size_t)np);
-  uint8_t* dmask = (uint8_t*)(h->ws + h->L.mask);
-  CU(h, launch_threshold(d_pvals, np, tau, dmask, s));
-  CU(h, cudaMemcpyAsync(mask.data(), dmask, (size_t)np, cudaMemcpyDeviceToHost, s));
-  CU(h, cudaStreamSynchronize(s));
+  const WsLayout& L = h->L;
+  char* w = h->ws;
   const int64_t n = h->n;
-  // edges (r, g) and (g, r) for every stored P_rg above tau, plus the diagonal
-  std::vector<int64_t> deg((size_t)n + 1, 0);
-  for (int64_t g = 0; g < n; ++g) {
-    ++deg[(size_t)g];
-    for (int64_t e = h->pcolptr[g]; e < h->pcolptr[g + 1]; ++e) {
-      const int32_t r = h->prowind[(size_t)e];
-      if (mask[(size_t)e] && r != g) {
-        ++deg[(size_t)r];
-        ++deg[(size_t)g];
-      }
-    }
-  }
-  std::vector<int64_t> rp((size_t)n + 1, 0);
-  for (int64_t i = 0; i < n; ++i) rp[(size_t)i + 1] = rp[(size_t)i] + deg[(size_t)i];
-  std::vector<int32_t> ci((size_t)rp[(size_t)n]);
-  std::vector<int64_t> fill(rp.begin(), rp.end() - 1);
-  for (int64_t g = 0; g < n; ++g) {
-    ci[(size_t)fill[(size_t)g]++] = (int32_t)g;
-    for (int64_t e = h->pcolptr[g]; e < h->pcolptr[g + 1]; ++e) {
-      const int32_t r = h->prowind[(size_t)e];
-      if (mask[(size_t)e] && r != g) {
-        ci[(size_t)fill[(size_t)r]++] = (int32_t)g;
-        ci[(size_t)fill[(size_t)g]++] = r;
-      }
-    }
-  }
-  // sort and deduplicate every row (an edge can come from both P_rg and P_gr), compacting
-  // the rows to the front of ci
-  int64_t out = 0;
-  g_rowptr[0] = 0;
-  for (int64_t i = 0; i < n; ++i) {
-    auto b = ci.begin() + rp[(size_t)i], e = ci.begin() + rp[(size_t)i + 1];
-    std::sort(b, e);
-    const int64_t m = std::unique(b, e) - b;
-    if (ci.begin() + out != b) std::copy(b, b + m, ci.begin() + out);  // out < rp[i]: moves left
-    out += m;
-    g_rowptr[i + 1] = out;
-  }
+  GraphArgs g{};
+  g.n = n;
+  g.p = d_pvals;
+  g.tau = tau;
+  g.parts = (const PartDesc*)(w + L.parts);
+  g.S = (const int32_t*)(w + L.S);
+  g.perm = (const int32_t*)(w + L.perm);
+  g.invperm = (const int32_t*)(w + L.invperm);
+  g.pcolptr = (const int64_t*)(w + L.pcolptr);
+  g.memptr = (const int64_t*)(w + L.memptr);
+  g.mempart = (const int32_t*)(w + L.mempart);
+  g.memloc = (const int32_t*)(w + L.memloc);
+  g.deg = (int32_t*)(w + L.gdeg);
+  g.rowptr = (int64_t*)(w + L.growptr);
+  CU(h, launch_graph_rowptr(g, h->num_sms, s));
+  CU(h, cudaMemcpyAsync(g_rowptr, g.rowptr, ((size_t)n + 1) * sizeof(int64_t), cudaMemcpyDeviceToHost, s));
+  CU(h, cudaStreamSynchronize(s));
+  const int64_t out = g_rowptr[n];
   *nnz = out;
   if (!g_colind) return GSP2_OK;
   if (cap < out) return fail(h, GSP2_E_ARG, "g_colind smaller than the graph (see *nnz)");
-  std::copy(ci.begin(), ci.begin() + out, g_colind);
+  int32_t* gcol = (int32_t*)(w + L.gcol);
+  const int64_t room = graph_cap(h);
+  for (int64_t r0 = 0; r0 < n;) {
+    // as many rows as the buffer holds
+    const int64_t* e = std::upper_bound(g_rowptr + r0, g_rowptr + n + 1, g_rowptr[r0] + room);
+    const int64_t r1 = (e - g_rowptr) - 1;
+    CU(h, launch_graph_rows(g, r0, r1 - r0, gcol, h->num_sms, s));
+    CU(h, cudaMemcpyAsync(g_colind + g_rowptr[r0], gcol, (size_t)(g_rowptr[r1] - g_rowptr[r0]) * sizeof(int32_t),
+                          cudaMemcpyDeviceToHost, s));
+    CU(h, cudaStreamSynchronize(s));
+    r0 = r1;
+  }
   return GSP2_OK;
 }
 

@@ -140,6 +140,19 @@ struct TcStepArgs {
 };
 constexpr int TC_SIG_MIN = -98, TC_SIG_MAX = 126;  // range of the FP16 adjoint's scale exponents
 
+// Arguments of the graph refresh (k_graph.cu).
+struct GraphArgs {
+  int64_t n;
+  const double* p;  // P in core columns
+  double tau;
+  const PartDesc* parts;
+  const int32_t *S, *perm, *invperm;
+  const int64_t *pcolptr, *memptr;
+  const int32_t *mempart, *memloc;
+  int32_t* deg;     // [n]
+  int64_t* rowptr;  // [n + 1]
+};
+
 // FP64 products rebuilt from FP16 digits (k_oz.cu)
 constexpr int OZ_SLICES = 5;  // digits per entry (11, 8, 11, 11 and 11 bits)
 constexpr int OZ_LOW = 2;     // digits the second pass of a tile multiplies

@@ -25,7 +25,9 @@ cudaError_t launch_square_fp64(const PartDesc* parts, const Tile* tiles, int nti
 cudaError_t launch_residual_fp64(const PartDesc* parts, const Tile* tiles, int ntiles, const double* x,
                                  const double* const* x_of_step, double* rslots, int64_t n, const StepCtl& ctl,
                                  cudaStream_t s);
-cudaError_t launch_threshold(const double* p, int64_t n, double tau, uint8_t* mask, cudaStream_t s);
+// graph refresh (k_graph.cu): the row pointers, then the columns of a range of rows into out
+cudaError_t launch_graph_rowptr(const GraphArgs& g, int nsm, cudaStream_t s);
+cudaError_t launch_graph_rows(const GraphArgs& g, int64_t row0, int64_t rows, int32_t* out, int nsm, cudaStream_t s);
 cudaError_t launch_square_fp32(const PartDesc* parts, const Tile* tiles, int ntiles, const float* xin, float* xout,
                                double2* slots, int nslots, const StepCtl& ctl, int step, cudaStream_t s);
 cudaError_t launch_scatter(const PartDesc* parts, const ColBlock* blocks, int nblocks, const int32_t* Sall,
