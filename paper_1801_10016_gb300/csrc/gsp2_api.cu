@@ -22,7 +22,7 @@ namespace {
 constexpr int BOUNDS_BLOCKS = 608;  // 152 SMs x 4
 
 struct WsLayout {
-  size_t parts, S, perm, invperm, tiles, tc_tiles, tc_wide, tc_wide_nb, gblocks, gblocks_ld, sblocks, pcolptr, rowptr,
+  size_t parts, S, perm, invperm, tiles, sq_tiles, tc_tiles, tc_wide, tc_wide_nb, gblocks, gblocks_ld, sblocks, pcolptr, rowptr,
       colind;
   size_t locptr, loc;  // the gathers' local indices of the stored entries of the rows S_k[j]
   size_t x0;           // Eq. 1 on the stored entries of H (FP64, per P-build)
@@ -94,7 +94,9 @@ struct gsp2_plan {
   std::vector<int64_t> locptr;           // per entry of S: its row's first slot in the local-index table
   int64_t nloc = 0;                      // slots of that table (stored entries of all rows S_k[j])
   std::vector<int32_t> mempart, memloc;  // part id, local index in S_part
-  std::vector<Tile> tiles;                 // 64x64 upper tiles (CUDA-core steps)
+  std::vector<Tile> tiles;                 // 64x64 upper tiles (FP32 steps)
+  std::vector<Tile> sq_tiles;              // 16x16 upper tiles (native FP64 steps, idempotency report)
+  int32_t nslots_sq = 0;
   std::vector<Tile> tc_tiles;              // 128x128 upper tiles (tensor-core steps)
   std::vector<Tile> tc_order;              // tc_tiles in the order of opt.tile_order (uploaded)
   std::vector<Tile> tc_wide;               // tile_shape 1: one or two column blocks per tile
@@ -284,6 +286,7 @@ static void build_layout(gsp2_plan* h) {
   L.mempart = take(h->mempart.size() * sizeof(int32_t));
   L.memloc = take(h->memloc.size() * sizeof(int32_t));
   L.tiles = take(h->tiles.size() * sizeof(Tile));
+  L.sq_tiles = take(h->sq_tiles.size() * sizeof(Tile));
   L.tc_tiles = take(h->tc_tiles.size() * sizeof(Tile));
   L.tc_wide = take(h->tc_wide.size() * sizeof(Tile));
   L.tc_wide_nb = take(h->tc_wide_nb.size());
@@ -302,10 +305,10 @@ static void build_layout(gsp2_plan* h) {
   L.locptr = take(h->locptr.size() * sizeof(int64_t));
   L.loc = take((size_t)h->nloc * sizeof(int32_t));
   L.x0 = take(h->colind.size() * sizeof(double));
-  const size_t nsl = std::max<size_t>({(size_t)h->nslots, (size_t)h->nslots_tc, h->gblocks.size(),
+  const size_t nsl = std::max<size_t>({(size_t)h->nslots, (size_t)h->nslots_sq, (size_t)h->nslots_tc, h->gblocks.size(),
                                         h->gblocks_ld.size(), (size_t)BOUNDS_BLOCKS, 1});
   L.slots = take(nsl * sizeof(double2));
-  L.rslots = take(std::max<size_t>(h->tiles.size(), 1) * sizeof(double));
+  L.rslots = take(std::max<size_t>({h->tiles.size(), h->sq_tiles.size(), 1}) * sizeof(double));
   L.state = take(sizeof(DevState));
   L.tile_ctr = take(sizeof(uint32_t));
   L.xchg = take(sizeof(ShardSlot));
@@ -648,6 +651,13 @@ static gsp2_status create_plan(int64_t n, const int64_t* rowptr, const int32_t* 
       for (int32_t j = 0; j < d.c; j += COLS_PER_BLOCK) h->sblocks.push_back(ColBlock{k, j});
     }
     h->nslots = slot;
+    for (int32_t k : order) {
+      const int32_t nt = (h->parts[k].s + SQ64_TILE - 1) / SQ64_TILE;
+      for (int32_t ti = 0; ti < nt; ++ti)
+        for (int32_t tj = ti; tj < nt; ++tj)
+          h->sq_tiles.push_back(Tile{k, ti, tj, ti == tj ? h->nslots_sq++ : -1});
+    }
+    if (h->sq_tiles.size() > (size_t)INT32_MAX) return bail(GSP2_E_ARG, "problem too large for one launch");
     if (h->tiles.size() > (size_t)INT32_MAX || h->gblocks.size() > (size_t)INT32_MAX)
       return bail(GSP2_E_ARG, "problem too large for one launch");
     build_layout(h);
@@ -882,6 +892,7 @@ extern "C" gsp2_status gsp2_bind_workspace(gsp2_handle h, void* d_ws, size_t byt
   for (size_t i = 0; i < tab.size(); ++i) tab[i] = (const double*)(h->ws + h->step_arena_off[i]);
   CU(h, up(L.step_arena, tab.data(), tab.size() * sizeof(double*)));
   CU(h, up(L.tiles, h->tiles.data(), h->tiles.size() * sizeof(Tile)));
+  CU(h, up(L.sq_tiles, h->sq_tiles.data(), h->sq_tiles.size() * sizeof(Tile)));
   order_tc_tiles(h, h->num_sms);
   CU(h, up(L.tc_tiles, h->tc_order.data(), h->tc_order.size() * sizeof(Tile)));
   CU(h, up(L.tc_wide, h->tcw_order.data(), h->tcw_order.size() * sizeof(Tile)));
@@ -1127,6 +1138,8 @@ static gsp2_status enqueue_forward(gsp2_plan* h, const double* hv, double* pv, i
   auto Sall = (const int32_t*)(w + L.S);
   auto perm = (const int32_t*)(w + L.perm);
   auto tiles = (const Tile*)(w + L.tiles);
+  auto sqt = (const Tile*)(w + L.sq_tiles);
+  const int nsq = (int)h->sq_tiles.size();
   auto gbl = (const ColBlock*)(w + L.gblocks_ld);  // every column up to ld, padding zeroed
   auto sbl = (const ColBlock*)(w + L.sblocks);
   auto pcol = (const int64_t*)(w + L.pcolptr);
@@ -1247,7 +1260,7 @@ static gsp2_status enqueue_forward(gsp2_plan* h, const double* hv, double* pv, i
         a.mode = tmode;
         CU(h, launch_oz_step(a, h->num_sms, s));
       } else
-        CU(h, launch_square_fp64(parts, tiles, (int)h->tiles.size(), d[t & 1], d[(t + 1) & 1], slots, h->nslots, ctl,
+        CU(h, launch_square_fp64(parts, sqt, nsq, d[t & 1], d[(t + 1) & 1], slots, h->nslots_sq, ctl,
                                  0, tmode, s));
     }
     if (!on()) return GSP2_OK;
@@ -1261,7 +1274,7 @@ static gsp2_status enqueue_forward(gsp2_plan* h, const double* hv, double* pv, i
         CU(h, launch_fixed_to_fp64(nullptr, d[T & 1], st, h->arena_elems, h->num_sms, s));
       if (ub) CU(h, launch_symmetrize(parts, (const Tile*)(w + L.tc_tiles), (int)h->tc_tiles.size(), nullptr, d[T & 1],
                                       st, s));
-      CU(h, launch_residual_fp64(parts, tiles, (int)h->tiles.size(), d[T & 1], nullptr, (double*)(w + L.rslots),
+      CU(h, launch_residual_fp64(parts, sqt, nsq, d[T & 1], nullptr, (double*)(w + L.rslots),
                                  h->n, ctl, s));
     }
     if (alpha_user)
@@ -1295,7 +1308,7 @@ static gsp2_status enqueue_forward(gsp2_plan* h, const double* hv, double* pv, i
       a.mode = SQ_FORWARD;
       CU(h, launch_oz_step(a, h->num_sms, s));
     } else
-      CU(h, launch_square_fp64(parts, tiles, (int)h->tiles.size(), xin, xout, slots, h->nslots, ctl, i, SQ_FORWARD,
+      CU(h, launch_square_fp64(parts, sqt, nsq, xin, xout, slots, h->nslots_sq, ctl, i, SQ_FORWARD,
                                s));
     if (!h->ev.empty()) CU(h, cudaEventRecordWithFlags(h->ev[2 * (i - 1) + 1], s, cudaEventRecordExternal));
   }
@@ -1311,7 +1324,7 @@ static gsp2_status enqueue_forward(gsp2_plan* h, const double* hv, double* pv, i
       CU(h, launch_symmetrize(parts, (const Tile*)(w + L.tc_tiles), (int)h->tc_tiles.size(),
                               (const double* const*)(w + L.step_arena), nullptr, st, s));
     }
-    CU(h, launch_residual_fp64(parts, tiles, (int)h->tiles.size(), nullptr, (const double* const*)(w + L.step_arena),
+    CU(h, launch_residual_fp64(parts, sqt, nsq, nullptr, (const double* const*)(w + L.step_arena),
                                (double*)(w + L.rslots), h->n, ctl, s));
   }
   if (mode == MODE_RECORD && alpha_user)
@@ -1853,14 +1866,14 @@ static gsp2_status enqueue_backward(gsp2_plan* h, const double* pbar, double* hb
   char* w = h->ws;
   auto parts = (const PartDesc*)(w + L.parts);
   auto Sall = (const int32_t*)(w + L.S);
-  auto tiles = (const Tile*)(w + L.tiles);
+  auto tiles = (const Tile*)(w + L.sq_tiles);
   auto gbl = (const ColBlock*)(w + L.gblocks);
   auto st = (DevState*)(w + L.state);
   auto alpha = (int8_t*)(w + L.alpha);
   double* xb0 = (double*)(w + L.xb0);
   double* xb1 = (double*)(w + L.xb1);
   const int k = h->opt.ckpt_every, M = backward_steps(h);
-  const int nt = (int)h->tiles.size();
+  const int nt = (int)h->sq_tiles.size();
   StepCtl ctl{st, alpha, (double*)(w + L.traces), (double*)(w + L.idem), h->nocc, h->opt.idem_tol,
               h->opt.trace_tol, MODE_REPLAY, M, 1, 0};
   CU(h, launch_adj_seed<double>(parts, gbl, (int)h->gblocks.size(), Sall, (const int32_t*)(w + L.invperm),

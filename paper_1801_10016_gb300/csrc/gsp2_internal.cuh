@@ -14,7 +14,8 @@
 namespace gsp2 {
 
 constexpr int LD_PAD = 128;      // ld_k multiple (tile edge of every square kernel)
-constexpr int SQ_TILE = 64;      // FP64 square tile edge
+constexpr int SQ_TILE = 64;      // FP32 square tile edge
+constexpr int SQ64_TILE = 16;    // FP64 square tile edge
 constexpr int TC_TILE = 128;     // tensor-core square tile edge
 constexpr int COLS_PER_BLOCK = 8;  // gather/scatter: one warp per column, 8 warps
 
@@ -24,7 +25,7 @@ struct PartDesc {
   int32_t s;     // core + halo size
   int32_t c;     // core count
   int32_t ld;    // padded leading dimension
-  int32_t nt;    // FP64 square tiles per edge: ceil(s / SQ_TILE)
+  int32_t nt;    // FP32 square tiles per edge: ceil(s / SQ_TILE)
 };
 
 struct Tile {  // one upper-triangular output tile of one part

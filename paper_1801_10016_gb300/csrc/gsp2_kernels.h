@@ -19,6 +19,7 @@ cudaError_t launch_x0_values(int64_t n, const int64_t* rowptr, const int32_t* co
 cudaError_t launch_locate(const PartDesc* parts, const ColBlock* blocks, int nblocks, const int32_t* Sall,
                           const int64_t* rowptr, const int32_t* colind, const int64_t* locptr, int32_t* loc,
                           cudaStream_t s);
+// FP64 steps and residual: SQ64_TILE tiles; FP32 steps: SQ_TILE tiles
 cudaError_t launch_square_fp64(const PartDesc* parts, const Tile* tiles, int ntiles, const double* xin,
                                double* xout, double2* slots, int nslots, const StepCtl& ctl, int step, int mode,
                                cudaStream_t s);

@@ -46,68 +46,71 @@ __global__ void __launch_bounds__(256) adj_seed_kernel(const PartDesc* __restric
   }
 }
 
-// One reverse step for every part.  Work item = one upper tile (ti <= tj);
+// One reverse step for every part.  Work item = one upper tile (ti <= tj) of edge
+// SQ64_TILE, as the forward steps (4,096 orbitals: 68.7 ms per backward with 64-tiles, 50.5 with 16);
 // Z_IJ = sum_k Xbar[I,k] X[k,J] + X[I,k] Xbar[k,J] with all four slices streamed from
 // columns k of the symmetric Xbar and X.  Result mirrored to (J, I).
 // The Xbar buffers alternate with (n - step) so that skipped steps keep the parity: input
 // xb[(n - step) & 1], output xb[(n - step + 1) & 1], n the steps applied by the forward;
 // steps above n are skipped.
-// Four consecutive elements (16-byte aligned for FP32, 32 for FP64) in vector stores.
-__device__ __forceinline__ void store4(double* p, double a, double b, double c, double d) {
-  reinterpret_cast<double2*>(p)[0] = make_double2(a, b);
-  reinterpret_cast<double2*>(p)[1] = make_double2(c, d);
-}
-__device__ __forceinline__ void store4(float* p, float a, float b, float c, float d) {
-  *reinterpret_cast<float4*>(p) = make_float4(a, b, c, d);
+// R consecutive elements (R elements aligned) in vector stores.
+template <int R>
+__device__ __forceinline__ void store_row(double* p, const double (&v)[R]) {
+  if constexpr (R == 1) {
+    *p = v[0];
+  } else {
+#pragma unroll
+    for (int i = 0; i < R; i += 2) *reinterpret_cast<double2*>(p + i) = make_double2(v[i], v[i + 1]);
+  }
 }
 
 template <typename T>
-struct AdjBK {
-  static constexpr int v = 64 / (int)sizeof(T);  // K slice: 8 (FP64) or 16 (FP32) = 16 B per thread
-};
-
-template <typename T>
-__global__ void __launch_bounds__(256, 2) adj_step_kernel(const PartDesc* __restrict__ parts,
+__global__ void __launch_bounds__(256, 4) adj_step_kernel(const PartDesc* __restrict__ parts,
                                                           const Tile* __restrict__ tiles, const T* __restrict__ Xall,
                                                           T* __restrict__ xb0, T* __restrict__ xb1,
                                                           const int8_t* __restrict__ alpha, const DevState* st,
                                                           int step) {
-  constexpr int ABK = AdjBK<T>::v;
+  static_assert(sizeof(T) == 8, "the native FP64 adjoint");
+  constexpr int EDGE = SQ64_TILE, ABK = 16;
+  constexpr int R = EDGE / 16;  // a thread's block is R x R
   const int n = *(volatile const int32_t*)&st->steps;
   if (step > n) return;
   const T* XBin = ((n - step) & 1) ? xb1 : xb0;
   T* XBout = ((n - step) & 1) ? xb0 : xb1;
-  __shared__ __align__(16) T S1[2][ABK][SQ_TILE];  // Xbar rows I
-  __shared__ __align__(16) T S2[2][ABK][SQ_TILE];  // X    rows J
-  __shared__ __align__(16) T S3[2][ABK][SQ_TILE];  // X    rows I
-  __shared__ __align__(16) T S4[2][ABK][SQ_TILE];  // Xbar rows J
+  __shared__ __align__(16) T S1[2][ABK][EDGE];  // Xbar rows I
+  __shared__ __align__(16) T S2[2][ABK][EDGE];  // X    rows J
+  __shared__ __align__(16) T S3[2][ABK][EDGE];  // X    rows I
+  __shared__ __align__(16) T S4[2][ABK][EDGE];  // Xbar rows J
   const Tile t = tiles[blockIdx.x];
   const PartDesc p = parts[t.part];
   const T* X = Xall + p.off;
   const T* B = XBin + p.off;
   const int64_t ld = p.ld;
-  const int r0 = t.ti * SQ_TILE, c0 = t.tj * SQ_TILE;
+  const int r0 = t.ti * EDGE, c0 = t.tj * EDGE;
   const int kend = (p.s + ABK - 1) / ABK * ABK;
   const int tid = threadIdx.x;
   const int tx = tid & 15, ty = tid >> 4;
 
   auto load_slice = [&](int buf, int k0) {
-    // ABK x 64 elements per operand = 256 16-byte chunks: one per thread per operand
+    // ABK x EDGE elements per operand: at most 256 16-byte chunks, one per thread per operand
     constexpr int EPC = 16 / (int)sizeof(T);
-    const int kr = tid / (SQ_TILE / EPC), c2 = (tid % (SQ_TILE / EPC)) * EPC;
-    const int64_t co = (int64_t)(k0 + kr) * ld;
-    cp_async16(&S1[buf][kr][c2], B + co + r0 + c2);
-    cp_async16(&S2[buf][kr][c2], X + co + c0 + c2);
-    cp_async16(&S3[buf][kr][c2], X + co + r0 + c2);
-    cp_async16(&S4[buf][kr][c2], B + co + c0 + c2);
+    static_assert(ABK * EDGE / EPC <= 256, "one chunk per thread");
+    const int kr = tid / (EDGE / EPC), c2 = (tid % (EDGE / EPC)) * EPC;
+    if (kr < ABK) {
+      const int64_t co = (int64_t)(k0 + kr) * ld;
+      cp_async16(&S1[buf][kr][c2], B + co + r0 + c2);
+      cp_async16(&S2[buf][kr][c2], X + co + c0 + c2);
+      cp_async16(&S3[buf][kr][c2], X + co + r0 + c2);
+      cp_async16(&S4[buf][kr][c2], B + co + c0 + c2);
+    }
     cp_async_commit();
   };
 
-  T acc[4][4];
+  T acc[R][R];
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int i = 0; i < R; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = T(0);
+    for (int j = 0; j < R; ++j) acc[i][j] = T(0);
 
   const int nk = kend / ABK;
   load_slice(0, 0);
@@ -122,40 +125,43 @@ __global__ void __launch_bounds__(256, 2) adj_step_kernel(const PartDesc* __rest
     __syncthreads();
 #pragma unroll
     for (int kk = 0; kk < ABK; ++kk) {
-      T a1[4], b1[4], a2[4], b2[4];
+      T a1[R], b1[R], a2[R], b2[R];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        a1[q] = S1[buf][kk][tx * 4 + q];
-        b1[q] = S2[buf][kk][ty * 4 + q];
-        a2[q] = S3[buf][kk][tx * 4 + q];
-        b2[q] = S4[buf][kk][ty * 4 + q];
+      for (int q = 0; q < R; ++q) {
+        a1[q] = S1[buf][kk][tx * R + q];
+        b1[q] = S2[buf][kk][ty * R + q];
+        a2[q] = S3[buf][kk][tx * R + q];
+        b2[q] = S4[buf][kk][ty * R + q];
       }
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
+      for (int i = 0; i < R; ++i)
 #pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fma(a2[i], b2[j], fma(a1[i], b1[j], acc[i][j]));
+        for (int j = 0; j < R; ++j) acc[i][j] = fma(a2[i], b2[j], fma(a1[i], b1[j], acc[i][j]));
     }
     __syncthreads();
   }
 
   const int8_t al = alpha[step];
   T* O = XBout + p.off;
-  const int rb = r0 + tx * 4, cb = c0 + ty * 4;
+  const int rb = r0 + tx * R, cb = c0 + ty * R;
 #pragma unroll
-  for (int j = 0; j < 4; ++j) {
+  for (int j = 0; j < R; ++j) {
     const int c = cb + j;
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
+    for (int i = 0; i < R; ++i) {
       const T z = acc[i][j];
       acc[i][j] = (al > 0) ? (T(2) * B[(int64_t)c * ld + rb + i] - z) : z;
     }
-    store4(O + (int64_t)c * ld + rb, acc[0][j], acc[1][j], acc[2][j], acc[3][j]);
+    T v[R];
+#pragma unroll
+    for (int i = 0; i < R; ++i) v[i] = acc[i][j];
+    store_row(O + (int64_t)c * ld + rb, v);
   }
   if (t.ti != t.tj) {
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
+    for (int i = 0; i < R; ++i) {
       const int r = rb + i;
-      store4(O + (int64_t)r * ld + cb, acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
+      store_row(O + (int64_t)r * ld + cb, acc[i]);
     }
   }
 }

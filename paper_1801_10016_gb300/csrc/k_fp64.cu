@@ -185,11 +185,16 @@ __global__ void __launch_bounds__(256) gather_kernel(const PartDesc* __restrict_
 // One purification step for every part (Eq. 2) on the CUDA cores, T = double (FP64
 // path and the FP64 tail of the low-precision paths) or float (FP32 path).
 //
-// Work item = one upper-triangular 64x64 output tile (ti <= tj) of one part.  X is
+// Work item = one upper-triangular EDGE x EDGE output tile (ti <= tj) of one part.  X is
 // symmetric, so both operands of Y = X X stream from columns of X: the A slice
 // X[I, k] is column k rows I, and the B slice X[k, J] = X[J, k] is column k rows J.
-// Each of the 256 threads owns a 4x4 block of the tile; 16-wide K slices are double
-// buffered in shared memory with cp.async.
+// Each of the 256 threads owns a (EDGE / 16)^2 block of the tile; 16-wide K slices are double
+// buffered in shared memory with cp.async.  The FP64 pipe of an SM issues 2 multiply-adds per
+// clock, so even one product per two shared-memory reads keeps it busy, and EDGE = 16 wastes the
+// least on padding and on SMs without a tile (a 64-tile of K = 200 holds its SM for 200 us):
+// 64 / 32 / 16 took 0.247 / 0.110 / 0.063 ms per step on 512 orbitals, 1.373 / 1.118 / 1.008 on
+// 4,096 and 23.96 / 22.14 / 21.33 on 8,000.  FP32 runs at 64 times the rate and keeps EDGE = 64.
+// Every element sums its products in the order of k whatever the tile.
 // Epilogue: X_new = Y (alpha = -1) or 2 X - Y (alpha = +1), written to (I, J) and
 // mirrored to (J, I); diagonal tiles add Tr_core[Y] and Tr_core[X_new] (FP64) to their
 // slot.  The last block sums the slots in a fixed order and runs the bookkeeping.
@@ -221,7 +226,7 @@ struct Vec2<float> {
 //               core columns j of its tile (and of the mirrored tile) to rslots, and the
 //               last block stores sqrt(sum / N) in the state.
 template <typename T>
-__global__ void __launch_bounds__(256, 2) square_simt_kernel(const PartDesc* __restrict__ parts,
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 2 : 4) square_simt_kernel(const PartDesc* __restrict__ parts,
                                                              const Tile* __restrict__ tiles,
                                                              const T* __restrict__ xin, T* __restrict__ xout,
                                                              double2* __restrict__ slots, int nslots, StepCtl ctl,
@@ -237,19 +242,21 @@ __global__ void __launch_bounds__(256, 2) square_simt_kernel(const PartDesc* __r
     if (stt == ST_NONFINITE || stt == ST_TIMEOUT) return;
     step = *(volatile int32_t*)&ctl.st->steps + 1;
   }
-  __shared__ __align__(16) T As[2][BK][SQ_TILE];
-  __shared__ __align__(16) T Bs[2][BK][SQ_TILE];
+  constexpr int EDGE = sizeof(T) == 4 ? SQ_TILE : SQ64_TILE;
+  constexpr int R = EDGE / 16;  // a thread's block is R x R
+  __shared__ __align__(16) T As[2][BK][EDGE];
+  __shared__ __align__(16) T Bs[2][BK][EDGE];
   const Tile t = tiles[blockIdx.x];
   const PartDesc p = parts[t.part];
   const T* xbase = (mode == SQ_RESIDUAL && xin_table) ? xin_table[step - 1] : xin;
   const T* X = xbase + p.off;
   const int64_t ld = p.ld;
-  const int r0 = t.ti * SQ_TILE, c0 = t.tj * SQ_TILE;
+  const int r0 = t.ti * EDGE, c0 = t.tj * EDGE;
   const int kend = (p.s + BK - 1) / BK * BK;
   const int tid = threadIdx.x;
   const int tx = tid & 15, ty = tid >> 4;
   constexpr int EPC = 16 / sizeof(T);             // elements per 16-byte chunk
-  constexpr int CPR = SQ_TILE / EPC;              // chunks per slice row
+  constexpr int CPR = EDGE / EPC;                 // chunks per slice row
   constexpr int CHUNKS = BK * CPR;                // chunks per operand slice
 
   auto load_slice = [&](int buf, int k0) {
@@ -263,11 +270,37 @@ __global__ void __launch_bounds__(256, 2) square_simt_kernel(const PartDesc* __r
     cp_async_commit();
   };
 
-  T acc[4][4];
+  T acc[R][R];
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+  for (int i = 0; i < R; ++i)
 #pragma unroll
-    for (int jj = 0; jj < 4; ++jj) acc[i][jj] = T(0);
+    for (int jj = 0; jj < R; ++jj) acc[i][jj] = T(0);
+  // R consecutive elements (vector accesses for R > 1)
+  auto get = [](const T* q, T (&v)[R]) {
+    if constexpr (R == 1) {
+      v[0] = *q;
+    } else {
+#pragma unroll
+      for (int i = 0; i < R; i += 2) {
+        const V2 x = *reinterpret_cast<const V2*>(q + i);
+        v[i] = x.x;
+        v[i + 1] = x.y;
+      }
+    }
+  };
+  auto put = [](T* q, const T (&v)[R]) {
+    if constexpr (R == 1) {
+      *q = v[0];
+    } else {
+#pragma unroll
+      for (int i = 0; i < R; i += 2) {
+        V2 x;
+        x.x = v[i];
+        x.y = v[i + 1];
+        *reinterpret_cast<V2*>(q + i) = x;
+      }
+    }
+  };
 
   const int nk = kend / BK;
   load_slice(0, 0);
@@ -282,28 +315,25 @@ __global__ void __launch_bounds__(256, 2) square_simt_kernel(const PartDesc* __r
     __syncthreads();
 #pragma unroll
     for (int kk = 0; kk < BK; ++kk) {
-      const V2 a01 = *reinterpret_cast<const V2*>(&As[buf][kk][tx * 4]);
-      const V2 a23 = *reinterpret_cast<const V2*>(&As[buf][kk][tx * 4 + 2]);
-      const V2 b01 = *reinterpret_cast<const V2*>(&Bs[buf][kk][ty * 4]);
-      const V2 b23 = *reinterpret_cast<const V2*>(&Bs[buf][kk][ty * 4 + 2]);
-      const T a[4] = {a01.x, a01.y, a23.x, a23.y};
-      const T b[4] = {b01.x, b01.y, b23.x, b23.y};
+      T a[R], b[R];
+      get(&As[buf][kk][tx * R], a);
+      get(&Bs[buf][kk][ty * R], b);
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
+      for (int i = 0; i < R; ++i)
 #pragma unroll
-        for (int jj = 0; jj < 4; ++jj) acc[i][jj] = fma(a[i], b[jj], acc[i][jj]);
+        for (int jj = 0; jj < R; ++jj) acc[i][jj] = fma(a[i], b[jj], acc[i][jj]);
     }
     __syncthreads();
   }
 
   if (mode == SQ_RESIDUAL) {
     double res = 0.0;
-    const int rb = r0 + tx * 4, cb = c0 + ty * 4;
+    const int rb = r0 + tx * R, cb = c0 + ty * R;
 #pragma unroll
-    for (int jj = 0; jj < 4; ++jj) {
+    for (int jj = 0; jj < R; ++jj) {
       const int c = cb + jj;
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
+      for (int i = 0; i < R; ++i) {
         const int r = rb + i;
         const double d = (double)acc[i][jj] - (double)X[(int64_t)c * ld + r];
         if (c < p.c) res += d * d;
@@ -333,32 +363,28 @@ __global__ void __launch_bounds__(256, 2) square_simt_kernel(const PartDesc* __r
 
   T* Y = xout + p.off;
   double tY = 0.0, tN = 0.0;
-  const int rb = r0 + tx * 4, cb = c0 + ty * 4;
-  // rb and cb are multiples of 4: a thread's block meets the diagonal only when rb == cb,
+  const int rb = r0 + tx * R, cb = c0 + ty * R;
+  // rb and cb are multiples of R: a thread's block meets the diagonal only when rb == cb,
   // at (i, i); its entries are added in FP64 outside the unrolled loop
-  T yd[4];
+  T yd[R];
 #pragma unroll
-  for (int i = 0; i < 4; ++i) yd[i] = acc[i][i];
+  for (int i = 0; i < R; ++i) yd[i] = acc[i][i];
 #pragma unroll
-  for (int jj = 0; jj < 4; ++jj) {
+  for (int jj = 0; jj < R; ++jj) {
     const int c = cb + jj;
-    const V2 x01 = *reinterpret_cast<const V2*>(X + (int64_t)c * ld + rb);
-    const V2 x23 = *reinterpret_cast<const V2*>(X + (int64_t)c * ld + rb + 2);
-    const T xv[4] = {x01.x, x01.y, x23.x, x23.y};
+    T xv[R], v[R];
+    get(X + (int64_t)c * ld + rb, xv);
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
+    for (int i = 0; i < R; ++i) {
       const T y = acc[i][jj];
       const T xn = (al > 0) ? (T(2) * xv[i] - y) : y;
       acc[i][jj] = xn;
+      v[i] = xn;
     }
-    V2 v;
-    v.x = acc[0][jj]; v.y = acc[1][jj];
-    *reinterpret_cast<V2*>(Y + (int64_t)c * ld + rb) = v;
-    v.x = acc[2][jj]; v.y = acc[3][jj];
-    *reinterpret_cast<V2*>(Y + (int64_t)c * ld + rb + 2) = v;
+    put(Y + (int64_t)c * ld + rb, v);
   }
   if (book && t.slot >= 0 && rb == cb) {
-    for (int i = 0; i < 4; ++i) {
+    for (int i = 0; i < R; ++i) {
       if (cb + i >= p.c) break;
       tY += (double)yd[i];
       tN += (double)acc[i][i];
@@ -366,14 +392,7 @@ __global__ void __launch_bounds__(256, 2) square_simt_kernel(const PartDesc* __r
   }
   if (t.ti != t.tj) {
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int r = rb + i;
-      V2 v;
-      v.x = acc[i][0]; v.y = acc[i][1];
-      *reinterpret_cast<V2*>(Y + (int64_t)r * ld + cb) = v;
-      v.x = acc[i][2]; v.y = acc[i][3];
-      *reinterpret_cast<V2*>(Y + (int64_t)r * ld + cb + 2) = v;
-    }
+    for (int i = 0; i < R; ++i) put(Y + (int64_t)(rb + i) * ld + cb, acc[i]);
   }
   if (!book) return;
   if (t.slot >= 0) {
