@@ -195,7 +195,7 @@ def run_reference(args):
     print(json.dumps(line), flush=True)
 
 
-OZ_DIGITS = 5  # digits of the fp64e step (11, 8, 11, 9 and 11 bits)
+OZ_DIGITS = 5  # digits of the fp64e step (11, 8, 11, 8 and 11 bits)
 OZ_PRODUCTS = OZ_DIGITS * (OZ_DIGITS + 1) // 2  # FP16 digit products per tile (15)
 
 

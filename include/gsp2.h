@@ -67,7 +67,7 @@ typedef enum {
   GSP2_PREC_BF16X3 = 4, /* split operands hi+lo in BF16, three products, FP32 accumulate */
   GSP2_PREC_TF32X3 = 5, /* split operands hi+lo in TF32, three products, FP32 accumulate */
   GSP2_PREC_FP64_EMU = 6, /* FP64 results; every product X X rebuilt from 5 digits of X (11, 8,
-                             11, 9 and 11 bits) held in FP16 (15 tensor-core products per tile, groups
+                             11, 8 and 11 bits) held in FP16 (15 tensor-core products per tile, groups
                              summed as 64-bit fixed point), master copy in that fixed point */
   GSP2_PREC_FP16X3 = 7  /* split operands hi+lo in FP16 of X 2^14 (22 bits like TF32X3, entries
                            down to 2^-28 in FP16's normal range), three products at the
@@ -126,15 +126,15 @@ typedef struct {
                               gsp2_autotune */
   int32_t split_k;         /* FP64_EMU steps: 1 = each upper tile's product as two work items, one
                               per half of its K (forward and rebuilt steps: the two halves of the
-                              K stages; adjoint reverse steps: Xbar X and X Xbar), their 64-bit
+                              K slices; adjoint reverse steps: Xbar X and X Xbar), their 64-bit
                               partial sums added by the second to finish (more, shorter items for
                               small problems); 0 = one item per tile; -1 (default) = 1 when the
-                              plan has at most 512 upper 128-tiles.  Needs every part above 128
-                              orbitals (else 0) and 2 x 128 KB of workspace per tile; gsp2_autotune
-                              may turn it off.  The 64-bit sums are exact and, in plans of at most
-                              512 upper tiles, items of either kind round their FP32 sums at the
-                              same K, so both give the same bits (larger plans agree to the last
-                              few) */
+                              plan has at most 38 upper 128-tiles.  Needs every part above 128
+                              orbitals (else 0) and 2 x 128 KB of workspace per tile (taken with -1 up
+                              to 512 tiles: gsp2_autotune may turn it on or off).  The 64-bit sums are
+                              exact; up to 512 tiles, plans with split_k set to 0 or 1 round their
+                              FP32 sums at the same K, so that both give the same bits (others
+                              agree to the last few) */
   int32_t tile_claim;      /* persistent 128 x 128 steps (tensor-core steps and reverse steps, FP64_EMU
                               forward and reverse steps): 1 (default) = each CTA takes its first
                               tile by its index and claims every next one from a counter in the

@@ -305,7 +305,7 @@ static void build_layout(gsp2_plan* h) {
   L.locptr = take(h->locptr.size() * sizeof(int64_t));
   L.loc = take((size_t)h->nloc * sizeof(int32_t));
   L.x0 = take(h->colind.size() * sizeof(double));
-  const size_t nsl = std::max<size_t>({(size_t)h->nslots, (size_t)h->nslots_sq, (size_t)h->nslots_tc, h->gblocks.size(),
+  const size_t nsl = std::max<size_t>({(size_t)h->nslots, (size_t)h->nslots_sq, 2 * (size_t)h->nslots_tc, h->gblocks.size(),
                                         h->gblocks_ld.size(), (size_t)BOUNDS_BLOCKS, 1});
   L.slots = take(nsl * sizeof(double2));
   L.rslots = take(std::max<size_t>({h->tiles.size(), h->sq_tiles.size(), 1}) * sizeof(double));
@@ -415,16 +415,18 @@ static void build_layout(gsp2_plan* h) {
   L.seg2.clear();
   L.oz_acc2 = 0;
   h->adj_overlap = h->opt.precision == GSP2_PREC_FP64_EMU && k > 1 && h->tc_tiles.size() <= 512;
-  // split-K work items: FP64_EMU plans whose parts all exceed 128 orbitals (so that both K
-  // halves of every pass hold at least one stage)
+  // split-K work items: FP64_EMU plans whose parts all exceed 128 orbitals (so that each K
+  // half holds at least one slice); by default they run where halves and column pieces together
+  // still leave an SM per item (24 tiles: 0.62 ms per forward against 0.68 without), while
+  // gsp2_autotune may turn them on for any plan with their buffers
   h->split_ok = h->opt.precision == GSP2_PREC_FP64_EMU && h->min_s > 128 &&
                 (h->opt.split_k == 1 || (h->opt.split_k < 0 && h->tc_tiles.size() <= 512));
-  h->split_on = h->split_ok;
-  h->halves = h->split_ok ||
-              (h->opt.precision == GSP2_PREC_FP64_EMU && h->min_s > 128 && h->tc_tiles.size() <= 512);
+  h->split_on = h->split_ok && (h->opt.split_k == 1 || h->tc_tiles.size() <= 152 / 4);
+  h->halves = h->split_on || (h->opt.precision == GSP2_PREC_FP64_EMU && h->min_s > 128 && h->opt.split_k == 0 &&
+                              h->tc_tiles.size() <= 512);
   if (h->split_ok) {
     L.split_acc = take(2 * h->tc_tiles.size() * 128 * 128 * sizeof(long long));
-    L.split_cnt = take(h->tc_tiles.size() * sizeof(uint32_t));
+    L.split_cnt = take(2 * h->tc_tiles.size() * sizeof(uint32_t));
     L.split_items = take(2 * h->tc_tiles.size() * sizeof(int32_t));
   }
   if (h->use_oz && k > 0) {
@@ -901,7 +903,7 @@ extern "C" gsp2_status gsp2_bind_workspace(gsp2_handle h, void* d_ws, size_t byt
     order_split_items(h, h->num_sms);
     CU(h, up(L.split_items, h->split_items.data(), h->split_items.size() * sizeof(int32_t)));
     // the per-tile counters of split items start at zero (every launch leaves them so)
-    CU(h, cudaMemsetAsync(h->ws + L.split_cnt, 0, h->tc_tiles.size() * sizeof(uint32_t), s));
+    CU(h, cudaMemsetAsync(h->ws + L.split_cnt, 0, 2 * h->tc_tiles.size() * sizeof(uint32_t), s));
   }
   CU(h, up(L.gblocks_ld, h->gblocks_ld.data(), h->gblocks_ld.size() * sizeof(ColBlock)));
   if (h->use_oz) {
@@ -1049,6 +1051,17 @@ extern "C" gsp2_status gsp2_bind_workspace(gsp2_handle h, void* d_ws, size_t byt
   return GSP2_OK;
 }
 
+// Column pieces per tile of the emulated steps: 2 (64 columns each) where that shortens the
+// longest row of items any SM takes.  A half-width item takes 0.62 of a whole one (its drains and
+// final pass are halved, its loads and MMAs are not).  Measured, ms per forward / backward with 1 and
+// 2 pieces: 24 tiles 0.80 -> 0.62 / 1.08 -> 0.79; 60 tiles 0.83 -> 0.65 / 1.32 -> 1.03; 152 tiles
+// 1.06 -> 1.12 / 1.98 -> 2.07; 193 tiles 1.50 -> 1.37 / 2.55 -> 2.51; 263 tiles 1.58 -> 1.67 / 2.95 ->
+// 3.29; 1,350 tiles 6.6 -> 8.4 / 18.8 -> 25.3.
+static int oz_pieces(int items, int sms) {
+  const int one = (items + sms - 1) / sms, two = (2 * items + sms - 1) / sms;
+  return 0.62 * two < (double)one ? 2 : 1;
+}
+
 // Arguments of the emulated FP64 step common to all its launches of a call.
 static OzStepArgs oz_args(gsp2_plan* h, const StepCtl& ctl) {
   const WsLayout& L = h->L;
@@ -1069,6 +1082,7 @@ static OzStepArgs oz_args(gsp2_plan* h, const StepCtl& ctl) {
   a.ctl = ctl;
   a.tile_ctr = h->opt.tile_claim ? (uint32_t*)(w + L.tile_ctr) : nullptr;
   a.halves = h->halves ? 1 : 0;
+  a.pieces = oz_pieces(a.ntiles * (h->split_on ? 2 : 1), h->num_sms);
   if (h->split_on) {
     a.split = 1;
     a.split_acc = (long long*)(w + L.split_acc);

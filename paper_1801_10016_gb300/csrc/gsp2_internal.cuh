@@ -155,7 +155,7 @@ struct GraphArgs {
 };
 
 // FP64 products rebuilt from FP16 digits (k_oz.cu)
-constexpr int OZ_SLICES = 5;  // digits per entry (11, 8, 11, 11 and 11 bits)
+constexpr int OZ_SLICES = 5;  // digits per entry (11, 8, 11, 8 and 11 bits)
 constexpr int OZ_LOW = 2;     // digits the second pass of a tile multiplies
 constexpr int OZ_MAX_GRID = 256;  // CTAs of the emulated step (one 128x128 int64 scratch each)
 constexpr int OZ_BK = 32;         // K per pipeline stage of the emulated step (64-byte rows)
@@ -198,6 +198,7 @@ struct OzStepArgs {
   // its 64-bit partial tile to split_acc[2 t + h] and the second of the two to finish
   // (split_cnt[t], left at zero) adds both and forms the tile (X_new, digits, traces)
   int split;
+  int pieces;            // column pieces of a tile, each an item of its own (1 or 2)
   int halves;            // the plan's items may be split: unsplit ones drain at the same boundary
   long long* split_acc;  // [2 ntiles][128 x 128], indexed by item code 2 t + h
   uint32_t* split_cnt;   // [ntiles]

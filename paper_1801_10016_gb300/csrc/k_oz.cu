@@ -4,28 +4,28 @@
 // FP16 products, in the spirit of the Ozaki splitting (Ozaki, Ogita, Oishi and Rump, 2012):
 //
 //   every entry of X (|x| <= 1: the spectrum of X stays in [0, 1]) is written with T = 5
-//   balanced digits of 11, 8, 11, 9 and 11 bits, x = sum_t S_t 2^{-e_t} + r with
-//   e = 11, 19, 30, 39, 50, |S_0| <= 2^11 |x| + 1, |S_t| at most half of digit t's range
-//   (t >= 1), |r| <= 2^-51 (+ 2^-57 from the fixed point); every S_t is an integer that FP16
+//   balanced digits of 11, 8, 11, 8 and 11 bits, x = sum_t S_t 2^{-e_t} + r with
+//   e = 11, 19, 30, 38, 49, |S_0| <= 2^11 |x| + 1, |S_t| at most half of digit t's range
+//   (t >= 1), |r| <= 2^-50 (+ 2^-57 from the fixed point); every S_t is an integer that FP16
 //   holds exactly (11 significant bits);
 //
 //   X X = sum_{a+b<T} 2^{-(e_a+e_b)} S_a S_b + (terms of order 2^-47): 15 products.
 //
-// The products are summed in FP32 in TMEM, in six accumulators.  Four of them hold integers
+// The products are summed in FP32 in TMEM, in six accumulators.  Five of them hold integers
 // (in units of their own scale) that stay below 2^24 and so are exact: (0,0), because
 // ||X||_2 <= 1 bounds sum_k |x_ik x_kj| by 1; (0,1) + (1,0) and (0,2) + (2,0), at most 2^19
 // and 2^22 times the row 1-norm sum_k |x_ik| (1 to 2 for the localised iterates of a gapped
 // system; for rows spread over all K columns the digits behave like independent values,
-// about 2^18 and 2^21); and (1,1), whose diagonal is a sum of squares, K 2^12.4 for digits
-// spread over their range.  The fifth, 2 [(1,2) + (2,1)] + (0,3) + (3,0) in units of 2^-50,
-// is exact too on localised iterates; on dense rows it is about sqrt(K) 2^17, and its
-// largest sums at K = 2048 round at 2^-49.  The width of digit 1 follows from (1,1) staying
-// below 2^24 up to K = 2048 (longer K is drained every 2048), that of digit 3 from the fifth
-// accumulator; digits 0 and 2 are as wide as FP16 allows, which leaves so little behind them
+// about 2^18 and 2^21); (1,1), whose diagonal is a sum of squares, K 2^12.4 for digits
+// spread over their range; and (1,2) + (2,1) + (0,3) + (3,0), about sqrt(K) 2^16 on dense rows.
+// The width of digit 1 follows from (1,1) staying below 2^24 up to K = 2048 (longer K is
+// drained every 2048), that of digit 3 from the fifth accumulator at the same K (with 9 bits its
+// largest sums passed 2^24 on dense rows, and the tensor core's truncation left 1.1e-13 at K = 2,049);
+// digits 0 and 2 are as wide as FP16 allows, which leaves so little behind them
 // that (1,3), (0,4), (2,2) and their mirrors, of order 2^-36 (2^-31 on the diagonal), share
 // the sixth accumulator, whose FP32 rounding lies below the dropped products.  Digits of 7
 // bits in BF16, whose 8-bit significand caps the width, took 7 digits and 28 products for an
-// error per entry of 1.3e-14 at K = 1,184 on dense rows; these give 0.8e-14.
+// error per entry of 1.25e-14 at K = 1,184 on dense rows; these give 1.0e-14.
 // The accumulators are added as integers into a 64-bit fixed point (resolution 2^-56; the
 // sixth rounded to it), and a final elementwise pass forms X_new = Y or 2X - Y on that
 // grid (the master copy of the iterate stays in this fixed point), the core traces in FP64,
@@ -49,20 +49,20 @@
 namespace gsp2 {
 
 // Digits of a value held in 64-bit fixed point v = x 2^56 (|x| < 2): rounded to
-// w = x 2^50, then written as balanced digits of 8, 11, 9 and 11 bits below S_0, so that
-// w = S_0 2^39 + S_1 2^31 + S_2 2^20 + S_3 2^11 + S_4 exactly.  The balanced digits of w are
+// w = x 2^49, then written as balanced digits of 8, 11, 8 and 11 bits below S_0, so that
+// w = S_0 2^38 + S_1 2^30 + S_2 2^19 + S_3 2^11 + S_4 exactly.  The balanced digits of w are
 // the plain bit fields of w + bias less half of each field's range, so each is one
-// shift-and-mask.  Digit t is stored as S_t 2^-rho_t with rho = -3, -4, -2, -2, 0: exact in
+// shift-and-mask.  Digit t is stored as S_t 2^-rho_t with rho = -3, -4, -2, -3, -1: exact in
 // FP16, and the products that share an accumulator land at one scale (rho_a + rho_b - e_a -
 // e_b is the same for (1,2) and (0,3), and for (1,3), (0,4) and (2,2)).  S_0 beyond 2^11
 // (|x| > 1, after low-precision steps) is kept even, which FP16 holds up to 2^12, and S_1
 // takes the rest.  Each value is a float whose significand
 // holds the field, less the same float of half its range: one AND/OR and one exact subtraction.
 __host__ __device__ constexpr int oz_e(int t) {  // x = sum_t S_t 2^-e_t
-  return t == 0 ? 11 : (t == 1 ? 19 : (t == 2 ? 30 : (t == 3 ? 39 : 50)));
+  return t == 0 ? 11 : (t == 1 ? 19 : (t == 2 ? 30 : (t == 3 ? 38 : 49)));
 }
 __host__ __device__ constexpr int oz_rho(int t) {  // stored: S_t 2^-rho_t
-  return t == 0 ? -3 : (t == 1 ? -4 : (t == 4 ? 0 : -2));
+  return t == 1 ? -4 : (t == 2 ? -2 : (t == 4 ? -1 : -3));
 }
 // Digit t, found biased by `half` at bit P of m (its field only): no shift is needed where the
 // field lies in the float's significand
@@ -73,14 +73,14 @@ __device__ __forceinline__ float digit_float(uint32_t m, uint32_t half) {
 }
 // Returns whether |S_0| > 2^11, where FP16 holds even integers only (digits_even).
 __device__ __forceinline__ bool digit_floats(long long v, float (&f)[OZ_SLICES]) {
-  // the rounding at 2^-50 and every field's bias in one addition; fields: S_4 bits 6-16, S_3
-  // 17-25, S_2 26-36, S_1 37-44, S_0 45-58
+  // the rounding at 2^-49 and every field's bias in one addition; fields: S_4 bits 7-17, S_3
+  // 18-25, S_2 26-36, S_1 37-44, S_0 45-58
   constexpr unsigned long long bias =
-      (1ull << 5) + (1024ull << 6) + (256ull << 17) + (1024ull << 26) + (128ull << 37) + (8192ull << 45);
+      (1ull << 6) + (1024ull << 7) + (128ull << 18) + (1024ull << 26) + (128ull << 37) + (8192ull << 45);
   const unsigned long long w = (unsigned long long)v + bias;
   const uint32_t lo = (uint32_t)w, hi = (uint32_t)(w >> 32);
-  f[4] = digit_float<4, 6>(lo & (2047u << 6), 1024u);
-  f[3] = digit_float<3, 14>((lo >> 3) & (511u << 14), 256u);
+  f[4] = digit_float<4, 7>(lo & (2047u << 7), 1024u);
+  f[3] = digit_float<3, 15>((lo >> 3) & (255u << 15), 128u);
   f[2] = digit_float<2, 0>(__funnelshift_r(lo, hi, 26) & 2047u, 1024u);
   f[1] = digit_float<1, 5>(hi & (255u << 5), 128u);
   f[0] = digit_float<0, 9>((hi >> 4) & (16383u << 9), 8192u);
@@ -373,6 +373,7 @@ struct alignas(16) OzItem {
   int64_t off, soff;
   int32_t code, ti, tj, slot;
   int32_t part, s, c, ld;
+  int32_t piece, pad[3];
 };
 constexpr int OZ_SMEM = OZ_UNITS * (int)OZ_UNIT_B + 1024 + 8 * (2 * OZ_UNITS + 4) + 16 + 16 * OZ_EPI_WARPS +
                         8 * 2 * OZ_RING + (int)sizeof(OzItem) * OZ_RING;
@@ -635,19 +636,26 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
   const CUtensorMap* maps_mn_b = reinterpret_cast<const CUtensorMap*>(a.maps_mn_b);
   // work items: the upper tiles, or (split K) each tile's two K halves
   const bool split = a.split != 0;
-  const int nitems = split ? 2 * a.ntiles : a.ntiles;
+  // column pieces of a tile, each an item of its own: 1 (128 columns) or 2 (64 columns)
+  const int pieces = a.pieces, pcols = 128 / pieces;
+  const int nitems = (split ? 2 * a.ntiles : a.ntiles) * pieces;
+  // columns of a piece that its MMAs cover
+  auto piece_cols = [&](int sz, int tj, int piece) {
+    return max(0, min(pcols, oz_tile_cols(sz, tj) - piece * pcols));
+  };
   // K slices [x, y) of an item of a part of size sz: all of them (the adjoint's first ns slices
   // multiply Xbar by X, the rest X by Xbar) or one half, up to or from slice z
   auto slices = [&](int sz, int half) {
     const int ns = (sz + OZ_BK - 1) / OZ_BK, all = ADJ ? 2 * ns : ns, mid = ADJ ? ns : (ns + 1) / 2;
     return make_int3(half == 1 ? mid : 0, half == 0 ? mid : all, mid);
   };
-  // end of the round of both passes that starts at slice c0: OZ_CHUNK slices, and (plans whose
-  // items may be split) never across the halves, so that a tile's sums are rounded alike
-  // whether one item forms it or two
+  // end of the round of both passes that starts at slice c0: rounds of equal length of at most
+  // OZ_CHUNK slices, and (plans whose items may be split) never across the halves, so that a
+  // tile's sums are rounded alike whether one item forms it or two
   auto round_end = [&](int c0, int3 kr) {
-    const int c1 = min(c0 + OZ_CHUNK, kr.y);
-    return a.halves && c0 < kr.z ? min(c1, kr.z) : c1;
+    const int left = (a.halves && c0 < kr.z ? min(kr.z, kr.y) : kr.y) - c0;
+    const int rounds = (left + OZ_CHUNK - 1) / OZ_CHUNK;
+    return c0 + (left + rounds - 1) / rounds;
   };
   // items claimed at run time (forward, tail and reverse steps; the list order) or dealt in turn
   // (the rebuilt iterates, which may run beside reverse steps and have no last block)
@@ -709,8 +717,9 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
           OzItem w;
           w.code = -1;
           if (it < nitems) {
-            w.code = split ? a.split_items[it] : it;
-            const Tile t = a.tiles[split ? w.code >> 1 : it];
+            w.piece = it % pieces;
+            w.code = split ? a.split_items[it / pieces] : it / pieces;
+            const Tile t = a.tiles[split ? w.code >> 1 : w.code];
             const PartDesc p = a.parts[t.part];
             w.ti = t.ti;
             w.tj = t.tj;
@@ -736,8 +745,10 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
       w.tj = __shfl_sync(0xffffffffu, s_items[q].tj, 0);
       w.part = __shfl_sync(0xffffffffu, s_items[q].part, 0);
       w.s = __shfl_sync(0xffffffffu, s_items[q].s, 0);
+      w.piece = __shfl_sync(0xffffffffu, s_items[q].piece, 0);
       if (op == 1 && lane == 0) mbar_arrive(item_empty(q));
       if (w.code < 0) break;
+      if (piece_cols(w.s, w.tj, w.piece) == 0) continue;
       const int half = split ? w.code & 1 : -1;
       const bool dg = !ADJ && w.ti == w.tj;  // X X on a diagonal tile: B is A
       const int blk = op == 0 ? w.ti : w.tj;
@@ -832,13 +843,18 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
       const int code = __shfl_sync(0xffffffffu, s_items[q].code, 0);
       const int ti = __shfl_sync(0xffffffffu, s_items[q].ti, 0), tj = __shfl_sync(0xffffffffu, s_items[q].tj, 0);
       const int sz = __shfl_sync(0xffffffffu, s_items[q].s, 0);
+      const int piece = __shfl_sync(0xffffffffu, s_items[q].piece, 0);
       if (lane == 0) mbar_arrive(item_empty(q));
       if (code < 0) break;
+      const int ncols = piece_cols(sz, tj, piece);
+      if (ncols == 0) continue;
       const int half = split ? code & 1 : -1;
       const bool dg = !ADJ && ti == tj;
       const int ns = (sz + OZ_BK - 1) / OZ_BK;
       const int3 kr = slices(sz, half);
-      const uint32_t idesc0 = IDESC | ((uint32_t)(oz_tile_cols(sz, tj) >> 3) << 17);
+      const uint32_t idesc0 = IDESC | ((uint32_t)(ncols >> 3) << 17);
+      // rows J of a piece start 64 rows into each digit tile: 64 B each K-major, one atom MN-major
+      const uint32_t poff = (uint32_t)piece * ((64u * OZ_BK * 2u) >> 4);
       // operands of slice ks, tile `off` of the units sa (rows I) and sb (rows J): those right of
       // the tile's own block came in MN-major (transpose bits 15 / 16); a K = 16 step advances
       // 32 B in a K-major row, 2 KB (16 K values) in an MN-major tile
@@ -851,7 +867,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
         o.alo = (uint32_t)(amn ? dm : dk) + ((unit(sa) + (uint32_t)off * OZ_DTILE) >> 4);
         o.adv_a = amn ? (2048u >> 4) : (32u >> 4);
         o.bhi = (uint32_t)((bmn ? dm : dk) >> 32);
-        o.blo = (uint32_t)(bmn ? dm : dk) + ((unit(sb) + (uint32_t)off * OZ_DTILE) >> 4);
+        o.blo = (uint32_t)(bmn ? dm : dk) + ((unit(sb) + (uint32_t)off * OZ_DTILE) >> 4) + poff;
         o.adv_b = bmn ? (2048u >> 4) : (32u >> 4);
         o.idesc = idesc0 | ((amn ? 1u : 0u) << 15) | ((bmn ? 1u : 0u) << 16);
         return o;
@@ -993,6 +1009,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
       t.ld = __shfl_sync(0xffffffffu, s_items[iq].ld, 0);
       t.off = __shfl_sync(0xffffffffu, s_items[iq].off, 0);
       t.soff = __shfl_sync(0xffffffffu, s_items[iq].soff, 0);
+      t.piece = __shfl_sync(0xffffffffu, s_items[iq].piece, 0);
       if (lane == 0) mbar_arrive(item_empty(iq));
       if (t.code < 0) break;
       const int code = t.code;
@@ -1007,22 +1024,26 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
       const int sg = ADJ ? a.sig[t.part] : 0;  // the adjoint's sums hold (Xbar X + X Xbar) / 2^sg
       // columns the MMAs covered; the 16-column chunks beyond them lie in the part's zero
       // padding, which no step writes (the arenas are zeroed when the workspace is bound)
-      const int ncols = oz_tile_cols(p.s, t.tj);
+      const int ncols = piece_cols(p.s, t.tj, t.piece);
+      if (ncols == 0) {  // a piece in the padding
+        if (!ADJ && !rec && diag && warp == 4 && lane == 0) a.slots[t.slot * pieces + t.piece] = make_double2(0.0, 0.0);
+        continue;
+      }
       // a diagonal tile keeps its upper triangle and mirrors it: a chunk wholly left of the
       // warp's first row (all its entries below the diagonal) is neither drained nor formed
       const int cskip = (t.ti == t.tj) ? quarter * 32 : 0;
       bool ok = true;
-      // the warp's chunks of 16 columns: the last one's sums stay in registers for the final
-      // pass, the other one's wait in the scratch tile (-1: no chunk)
-      const int clast = (colq * 32 + 16 < ncols && colq * 32 + 32 > cskip) ? 1
-                        : (colq * 32 < ncols && colq * 32 + 16 > cskip)   ? 0
-                                                                          : -1;
-      const int cfirst = clast == 1 && colq * 32 + 16 > cskip ? 0 : -1;
+      // the warp's chunks of 16 columns (pc0: its first column in the piece): the last one's sums stay
+      // in registers for the final pass, the other one's wait in the scratch tile (-1: no chunk)
+      const int nch = 2 / pieces, pc0 = colq * 16 * nch, tc0 = t.piece * pcols + pc0;
+      const bool on0 = pc0 < ncols && tc0 + 16 > cskip;
+      const bool on1 = nch == 2 && pc0 + 16 < ncols && tc0 + 32 > cskip;
+      const int clast = on1 ? 1 : (on0 ? 0 : -1), cfirst = on1 && on0 ? 0 : -1;
       // the previous iterate's lines of this warp (not written by this launch; read from HBM) come
       // to L2 while the MMAs run: lane l, column l of the warp's 32, two lines of 128 B
       if (alf > 0 && clast >= 0) {
-        const int c = t.tj * 128 + colq * 32 + lane;
-        if (c < p.s) {
+        const int c = t.tj * 128 + tc0 + lane;
+        if (lane < 16 * nch && c < p.s) {
           const double* x = xin + p.off + (int64_t)c * ld + t.ti * 128 + quarter * 32;
           asm volatile("prefetch.global.L2 [%0];\n prefetch.global.L2 [%0 + 128];\n" ::"l"(x));
         }
@@ -1042,8 +1063,8 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
 #pragma unroll 1
         for (int cc = 0; cc < 2 && ok; ++cc) {
           if (cc != clast && cc != cfirst) continue;
-          const int cl = colq * 32 + cc * 16;
-          const uint32_t tc = tmem + lane_off + (uint32_t)cl;
+          const int cl = tc0 + cc * 16;  // in the tile
+          const uint32_t tc = tmem + lane_off + (uint32_t)(pc0 + cc * 16);
           uint32_t w[16];
           if (pass == 0) {
             // the first pass's sum waits in the columns this warp has just drained (its own
@@ -1108,8 +1129,9 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
         __threadfence();
         asm volatile("bar.sync 1, %0;\n" ::"n"(32 * OZ_EPI_WARPS) : "memory");
         if (warp == 4 && lane == 0) {
-          const unsigned int before = atomicAdd(&a.split_cnt[ti], 1u);
-          if (before == 1u) a.split_cnt[ti] = 0u;  // both halves in: clear for the next launch
+          unsigned int* const cnt = &a.split_cnt[ti * pieces + t.piece];
+          const unsigned int before = atomicAdd(cnt, 1u);
+          if (before == 1u) *cnt = 0u;  // both halves in: clear for the next launch
           *s_half = (int)before;
         }
         asm volatile("bar.sync 1, %0;\n" ::"n"(32 * OZ_EPI_WARPS) : "memory");
@@ -1216,7 +1238,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
       for (int pc = 0; pc < 2 && ok; ++pc) {
         const int cc = pc == 0 ? clast : cfirst;
         if (cc < 0) continue;
-        const int cl = colq * 32 + cc * 16;
+        const int cl = tc0 + cc * 16;
         if (pc == 1) {
           const long long* zp = acc + (size_t)cl * 128 + m;
 #pragma unroll
@@ -1243,7 +1265,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
             sum.x += red[w].x;
             sum.y += red[w].y;
           }
-          a.slots[t.slot] = sum;
+          a.slots[t.slot * pieces + t.piece] = sum;
         }
         asm volatile("bar.sync 1, %0;\n" ::"n"(32 * OZ_EPI_WARPS) : "memory");
       }
@@ -1291,7 +1313,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
 
   if (last_block_ticket(&a.ctl.st->counter)) {
     double u = 0.0, w = 0.0;
-    for (int k = threadIdx.x; k < a.nslots; k += blockDim.x) {
+    for (int k = threadIdx.x; k < a.nslots * pieces; k += blockDim.x) {
       u += ld_cg(&a.slots[k].x);
       w += ld_cg(&a.slots[k].y);
     }
@@ -1326,7 +1348,7 @@ cudaError_t launch_oz_step(const OzStepArgs& a, int grid, cudaStream_t s, bool a
   auto kern = adjoint ? oz_step_kernel<true> : oz_step_kernel<false>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, OZ_SMEM);
   if (e != cudaSuccess) return e;
-  const int nitems = a.split ? 2 * a.ntiles : a.ntiles;
+  const int nitems = (a.split ? 2 * a.ntiles : a.ntiles) * a.pieces;
   int gr = grid < nitems ? grid : nitems;
   if (gr > OZ_MAX_GRID) gr = OZ_MAX_GRID;  // one scratch tile per CTA
   kern<<<gr, OZ_THREADS, OZ_SMEM, s>>>(a);
