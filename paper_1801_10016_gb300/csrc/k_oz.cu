@@ -589,23 +589,8 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
   // instruction descriptor without N (bits 17..22, N / 8): FP32 accumulate, FP16 A and B, M = 128
   constexpr uint32_t IDESC = (1u << 4) | ((128u >> 4) << 24);
 
-  int step = a.step;
   const bool rec = !ADJ && a.mode == SQ_RECOMPUTE;
-  int n = 0;
-  if (ADJ || rec) {
-    // reverse step `step` exists iff step <= n; a rebuilt X_step is read iff step < n
-    n = *(volatile int32_t*)&a.ctl.st->steps;
-    if (ADJ ? step > n : step >= n) return;
-  } else if (a.mode == SQ_FORWARD) {
-    if (*(volatile int32_t*)&a.ctl.st->stopped) return;
-  } else {
-    const int32_t stt = *(volatile int32_t*)&a.ctl.st->status;
-    if (stt == ST_NONFINITE || stt == ST_TIMEOUT) return;
-    step = *(volatile int32_t*)&a.ctl.st->steps + 1;
-  }
-  // digit buffers read / written (the adjoint's sets are passed explicitly)
-  const int dbi = (ADJ || rec) ? 0 : (step - 1) & 1, dbo = (ADJ || rec) ? 0 : step & 1;
-
+  pdl_release();
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
@@ -630,10 +615,6 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
   auto unit = [&](int s) { return base + (uint32_t)s * OZ_UNIT_B; };
   int32_t* abort_flag = &a.ctl.st->timeout;
   const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
-  const CUtensorMap* maps = reinterpret_cast<const CUtensorMap*>(a.maps) + (size_t)dbi * T * a.nparts;
-  const CUtensorMap* maps_mn = reinterpret_cast<const CUtensorMap*>(a.maps_mn) + (size_t)dbi * T * a.nparts;
-  const CUtensorMap* maps_b = reinterpret_cast<const CUtensorMap*>(a.maps_b);
-  const CUtensorMap* maps_mn_b = reinterpret_cast<const CUtensorMap*>(a.maps_mn_b);
   // work items: the upper tiles, or (split K) each tile's two K halves
   const bool split = a.split != 0;
   // column pieces of a tile, each an item of its own: 1 (128 columns) or 2 (64 columns)
@@ -685,6 +666,33 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
+
+  pdl_wait();  // everything below reads what the launch before wrote
+  int step = a.step;
+  bool run;
+  int n = 0;
+  if (ADJ || rec) {
+    // reverse step `step` exists iff step <= n; a rebuilt X_step is read iff step < n
+    n = *(volatile int32_t*)&a.ctl.st->steps;
+    run = ADJ ? step <= n : step < n;
+  } else if (a.mode == SQ_FORWARD) {
+    run = *(volatile int32_t*)&a.ctl.st->stopped == 0;
+  } else {
+    const int32_t stt = *(volatile int32_t*)&a.ctl.st->status;
+    run = stt != ST_NONFINITE && stt != ST_TIMEOUT;
+    step = *(volatile int32_t*)&a.ctl.st->steps + 1;
+  }
+  if (!run) {  // the loop has stopped: nothing to do
+    if (warp == 1) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;\n" ::"r"(tmem));
+    return;
+  }
+  // digit buffers read / written (the adjoint's sets are passed explicitly)
+  const int dbi = (ADJ || rec) ? 0 : (step - 1) & 1, dbo = (ADJ || rec) ? 0 : step & 1;
+
+  const CUtensorMap* maps = reinterpret_cast<const CUtensorMap*>(a.maps) + (size_t)dbi * T * a.nparts;
+  const CUtensorMap* maps_mn = reinterpret_cast<const CUtensorMap*>(a.maps_mn) + (size_t)dbi * T * a.nparts;
+  const CUtensorMap* maps_b = reinterpret_cast<const CUtensorMap*>(a.maps_b);
+  const CUtensorMap* maps_mn_b = reinterpret_cast<const CUtensorMap*>(a.maps_mn_b);
 
   // warp-collective bounded wait (the same outcome in every lane)
   auto wait = [&](uint32_t bar, uint32_t parity) {
@@ -1351,8 +1359,7 @@ cudaError_t launch_oz_step(const OzStepArgs& a, int grid, cudaStream_t s, bool a
   const int nitems = (a.split ? 2 * a.ntiles : a.ntiles) * a.pieces;
   int gr = grid < nitems ? grid : nitems;
   if (gr > OZ_MAX_GRID) gr = OZ_MAX_GRID;  // one scratch tile per CTA
-  kern<<<gr, OZ_THREADS, OZ_SMEM, s>>>(a);
-  return cudaGetLastError();
+  return launch_pdl(kern, gr, OZ_THREADS, OZ_SMEM, s, a);
 }
 
 cudaError_t launch_oz_gather(const PartDesc* parts, const ColBlock* blocks, int nblocks, const int32_t* Sall,

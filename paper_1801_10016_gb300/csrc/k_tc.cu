@@ -416,29 +416,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) square_tc_persistent_kernel(TcS
   // upper tile (two boxes of 64 rows, 8 KB apart, 128-byte swizzle, transpose bit)
   constexpr bool UPPER = KIND != 1;
 
-  int step = a.step;
-  int n = 0;
-  if (MODE != TC_STEP) {
-    // steps <= 0 count back from n (the tail steps); loop steps end at n - adj_tail, and
-    // the sweep never reads the loop's last iterate from a rebuild
-    n = *(volatile int32_t*)&a.ctl.st->steps;
-    if (step <= 0) {
-      step += n;
-      if (step < 1) return;
-    } else if (step > n - a.adj_tail || (MODE == TC_REBUILD && step == n - a.adj_tail)) {
-      return;
-    }
-  } else if (a.tail) {
-    const int32_t stt = *(volatile int32_t*)&a.ctl.st->status;
-    if (stt == ST_NONFINITE || stt == ST_TIMEOUT) return;
-    step = *(volatile int32_t*)&a.ctl.st->steps + 1;
-  } else if (*(volatile int32_t*)&a.ctl.st->stopped) {
-    return;
-  }
-  // iterate buffers read / written; the adjoint's Xbar: in (n - step) & 1, out the other
-  const int bi = MODE == TC_ADJOINT ? (n - step) & 1 : (step - 1) & 1;
-  const int bo = MODE == TC_ADJOINT ? bi ^ 1 : step & 1;
-
+  pdl_release();
   extern __shared__ uint8_t smem_raw[];
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
@@ -489,6 +467,36 @@ __global__ void __launch_bounds__(TC_THREADS, 1) square_tc_persistent_kernel(TcS
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
+
+  pdl_wait();  // everything below reads what the launch before wrote
+  int step = a.step;
+  bool run = true;
+  int n = 0;
+  if (MODE != TC_STEP) {
+    // steps <= 0 count back from n (the tail steps); loop steps end at n - adj_tail, and
+    // the sweep never reads the loop's last iterate from a rebuild
+    n = *(volatile int32_t*)&a.ctl.st->steps;
+    if (step <= 0) {
+      step += n;
+      run = step >= 1;
+    } else {
+      run = step <= n - a.adj_tail && !(MODE == TC_REBUILD && step == n - a.adj_tail);
+    }
+  } else if (a.tail) {
+    const int32_t stt = *(volatile int32_t*)&a.ctl.st->status;
+    run = stt != ST_NONFINITE && stt != ST_TIMEOUT;
+    step = *(volatile int32_t*)&a.ctl.st->steps + 1;
+  } else {
+    run = *(volatile int32_t*)&a.ctl.st->stopped == 0;
+  }
+  if (!run) {  // the loop has stopped, or the forward did not take this step
+    if (warp == 1) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 256;\n" ::"r"(tmem));
+    return;
+  }
+  // iterate buffers read / written; the adjoint's Xbar: in (n - step) & 1, out the other
+  const int bi = MODE == TC_ADJOINT ? (n - step) & 1 : (step - 1) & 1;
+  const int bo = MODE == TC_ADJOINT ? bi ^ 1 : step & 1;
+
 
   // warp-collective bounded wait (the same outcome in every lane)
   auto wait = [&](uint32_t bar, uint32_t parity) {
@@ -1217,8 +1225,7 @@ static cudaError_t launch_tc_persistent(const TcStepArgs& a, int grid, cudaStrea
   cudaError_t e = cudaFuncSetAttribute(square_tc_persistent_kernel<KIND, NPROD, MODE>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
-  square_tc_persistent_kernel<KIND, NPROD, MODE><<<grid, TC_THREADS, smem, s>>>(a);
-  return cudaGetLastError();
+  return launch_pdl(square_tc_persistent_kernel<KIND, NPROD, MODE>, grid, TC_THREADS, smem, s, a);
 }
 
 cudaError_t launch_tc_adjoint(const TcStepArgs& a, int grid, bool rebuild, cudaStream_t s) {
