@@ -282,6 +282,35 @@ __device__ __forceinline__ double2 block_sum2(double a, double b) {
   return r;
 }
 
+// The same ticket taken by one warp, after a block barrier that follows the block's partial
+// results: the other warps are done, and only this one reads all partials if true.
+__device__ __forceinline__ bool last_block_warp(unsigned int* counter) {
+  unsigned int t = 0;
+  if ((threadIdx.x & 31) == 0) {
+    __threadfence();
+    t = atomicAdd(counter, 1u);
+  }
+  const bool last = __shfl_sync(0xffffffffu, t, 0) == gridDim.x - 1;
+  if (last) __threadfence();
+  return last;
+}
+
+// Sum of n slots by one warp in a fixed order (every lane gets it).  A block of 640 threads that
+// sums them spends its time in FP64 adds of zeros: an FP64 instruction of a warp takes 16 cycles
+// of its SM's one FP64 pipe, 200 of them 1.7 us, and the barriers between them as much again
+// (from the last tile to the end of an emulated step, n = 512: 6.5 us so; a 22-step density 0.61
+// -> 0.54 ms with one warp here and for each diagonal tile's trace).
+__device__ __forceinline__ double2 warp_sum_slots(const double2* slots, int n) {
+  double a = 0.0, b = 0.0;
+#pragma unroll 4
+  for (int k = threadIdx.x & 31; k < n; k += 32) {
+    const double2 v = __ldcg(slots + k);
+    a += v.x;
+    b += v.y;
+  }
+  return make_double2(warp_sum(a), warp_sum(b));
+}
+
 // Bookkeeping of step `step` (0 = the initial guess X0), run by one thread of the
 // last block once the global sums are known:
 //   tN = Tr_core[X_step], tY = Tr_core[X_{step-1}^2] (unused for step 0).
@@ -300,30 +329,35 @@ __device__ __forceinline__ void finish_step(const StepCtl& c, int step, double t
     return;
   }
   DevState* st = c.st;
+  // everything this reads, in flight together: one thread runs this at the end of every step, and
+  // each load that waits for the one before costs the next step 0.4 us
+  const bool lagged = step >= 1 + c.stop_lag;
+  const double tprev = step > 0 ? c.traces[step - 1] : 0.0;
+  const double eprev = step > 0 && lagged ? c.idem[step - 1 - c.stop_lag] : 0.0;
+  const int nonfinite = st->nonfinite, status = st->status, tail_left = st->tail_left;
+  const int8_t al = c.alpha[step];
   c.traces[step] = tN;
   st->steps = step;
   bool stop = false, fire = false;
+  double e = 0.0;
   if (step > 0) {
-    const double e = c.traces[step - 1] - tY;
+    e = tprev - tY;
     c.idem[step - 1] = e;
-    if (c.mode == MODE_RECORD && step >= 1 + c.stop_lag && fabs(e) <= c.idem_tol &&
-        (e < 0.0 || e >= c.idem[step - 1 - c.stop_lag]))
-      fire = true;
-    if (!isfinite(e)) st->nonfinite = 1;
+    if (c.mode == MODE_RECORD && lagged && fabs(e) <= c.idem_tol && (e < 0.0 || e >= eprev)) fire = true;
   }
-  if (!isfinite(tN)) st->nonfinite = 1;
-  if (st->nonfinite) {
+  if (nonfinite || !isfinite(e) || !isfinite(tN)) {
+    st->nonfinite = 1;
     st->status = ST_NONFINITE;
     st->stopped = 1;
     return;
   }
-  if (c.mode == MODE_RECORD && st->tail_left > 0) {
+  if (c.mode == MODE_RECORD && tail_left > 0) {
     // this step was one of the alternating tail steps
-    st->tail_left -= 1;
-    if (st->tail_left == 0) {
+    st->tail_left = tail_left - 1;
+    if (tail_left == 1) {
       st->stopped = 1;
     } else {
-      c.alpha[step + 1] = (int8_t)(-c.alpha[step]);
+      c.alpha[step + 1] = (int8_t)(-al);
     }
     return;
   }
@@ -331,7 +365,7 @@ __device__ __forceinline__ void finish_step(const StepCtl& c, int step, double t
   if (fire) stop = true;
   if (!stop && cap) {
     stop = true;
-    if (c.mode == MODE_RECORD && step > 0 && !(fabs(c.idem[step - 1]) <= c.idem_tol)) st->status = ST_NOT_CONVERGED;
+    if (c.mode == MODE_RECORD && step > 0 && !(fabs(e) <= c.idem_tol)) st->status = ST_NOT_CONVERGED;
   }
   if (stop && c.mode == MODE_RECORD && c.tail_steps > 0) {
     // start the tail: first branch from the trace rule, then alternating
@@ -341,7 +375,7 @@ __device__ __forceinline__ void finish_step(const StepCtl& c, int step, double t
   }
   if (stop) {
     st->stopped = 1;
-    if (c.mode == MODE_REPLAY && st->status == ST_OK) {
+    if (c.mode == MODE_REPLAY && status == ST_OK) {
       const double d = tN - (double)c.nocc;
       if (!(fabs(d) <= c.trace_tol)) st->status = ST_TRACE;
     }

@@ -395,17 +395,18 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 2 : 4) square_simt_kerne
     for (int i = 0; i < R; ++i) put(Y + (int64_t)(rb + i) * ld + cb, acc[i]);
   }
   if (!book) return;
+  // the 16 threads tx == ty hold the diagonal's entries: one warp adds them
+  __shared__ double2 red[16];
+  if (t.slot >= 0 && tx == ty) red[tx] = make_double2(tY, tN);
+  __syncthreads();
+  if (tid >= 32) return;
   if (t.slot >= 0) {
-    const double2 s = block_sum2(tY, tN);
+    const double2 v = tid < 16 ? red[tid] : make_double2(0.0, 0.0);
+    const double2 s = make_double2(warp_sum(v.x), warp_sum(v.y));
     if (tid == 0) slots[t.slot] = s;
   }
-  if (last_block_ticket(&ctl.st->counter)) {
-    double a = 0.0, b = 0.0;
-    for (int k = tid; k < nslots; k += blockDim.x) {
-      a += ld_cg(&slots[k].x);
-      b += ld_cg(&slots[k].y);
-    }
-    const double2 s = block_sum2(a, b);
+  if (last_block_warp(&ctl.st->counter)) {
+    const double2 s = warp_sum_slots(slots, nslots);
     if (tid == 0) {
       if (mode == SQ_FORWARD) {
         finish_step(ctl, step, s.y, s.x);

@@ -375,7 +375,7 @@ struct alignas(16) OzItem {
   int32_t part, s, c, ld;
   int32_t piece, pad[3];
 };
-constexpr int OZ_SMEM = OZ_UNITS * (int)OZ_UNIT_B + 1024 + 8 * (2 * OZ_UNITS + 4) + 16 + 16 * OZ_EPI_WARPS +
+constexpr int OZ_SMEM = OZ_UNITS * (int)OZ_UNIT_B + 1024 + 8 * (2 * OZ_UNITS + 4) + 16 + 16 * 128 +
                         8 * 2 * OZ_RING + (int)sizeof(OzItem) * OZ_RING;
 static_assert(OZ_LOW_SUB * OZ_LOW <= OZ_SLICES, "a unit holds the second pass's slices");
 static_assert((2 * OZ_UNITS + 4) % 2 == 0, "alignment of the reduction slots and items");
@@ -599,12 +599,12 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(sb + OZ_UNITS * OZ_UNIT_B + 8 * (2 * OZ_UNITS + 4));
   int* s_err = reinterpret_cast<int*>(tmem_slot + 1);
   int* s_half = reinterpret_cast<int*>(tmem_slot + 2);  // split K: halves of the tile done before
-  double2* red = reinterpret_cast<double2*>(sb + OZ_UNITS * OZ_UNIT_B + 8 * (2 * OZ_UNITS + 4) + 16);
+  longlong2* red = reinterpret_cast<longlong2*>(sb + OZ_UNITS * OZ_UNIT_B + 8 * (2 * OZ_UNITS + 4) + 16);
   // warp 0's producer takes each next tile (claimed from a counter in global memory, or dealt)
   // and passes it on with its part through a ring (full: taken; empty: read by the other
   // producer, the MMA thread and every epilogue warp)
-  const uint32_t ring_bars = smem_u32(red + OZ_EPI_WARPS);
-  OzItem* s_items = reinterpret_cast<OzItem*>(reinterpret_cast<uint8_t*>(red + OZ_EPI_WARPS) + 8 * 2 * OZ_RING);
+  const uint32_t ring_bars = smem_u32(red + 128);
+  OzItem* s_items = reinterpret_cast<OzItem*>(reinterpret_cast<uint8_t*>(red + 128) + 8 * 2 * OZ_RING);
   auto item_full = [&](int q) { return ring_bars + 8u * q; };
   auto item_empty = [&](int q) { return ring_bars + 8u * (OZ_RING + q); };
   auto full = [&](int s) { return bars + 8u * s; };
@@ -1261,19 +1261,21 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
       }
       if (ADJ && ok && r < p.s && rown != 0.0f) atomicAdd(&a.normf[p.soff + r], rown);
       if (!ADJ && !rec && diag) {
-        // one conversion and FP64 sum per thread (zero where another warp has the entry)
-        const bool core = ok && r < p.c;
-        const double tY = warp_sum(core ? from_fixed(sgn < 0 ? -yd : yd) : 0.0);
-        const double tN = warp_sum(core ? from_fixed(xd) : 0.0);
-        if (lane == 0) red[warp - 4] = make_double2(tY, tN);
+        // the thread that has a diagonal entry leaves it (sgn Y, X_new) in shared memory; one warp
+        // converts and adds them.  A reduction in every warp would be 160 FP64 instructions, 16
+        // cycles each.
+        if (m >= tc0 && m < tc0 + 16 * nch) red[m] = make_longlong2(yd, xd);
         asm volatile("bar.sync 1, %0;\n" ::"n"(32 * OZ_EPI_WARPS) : "memory");
-        if (warp == 4 && lane == 0) {
+        if (warp == 4) {
           double2 sum = make_double2(0.0, 0.0);
-          for (int w = 0; w < OZ_EPI_WARPS; ++w) {
-            sum.x += red[w].x;
-            sum.y += red[w].y;
+          for (int q = t.piece * pcols + lane; q < min(p.c - t.ti * 128, (t.piece + 1) * pcols); q += 32) {
+            const longlong2 e = red[q];
+            sum.x += from_fixed(sgn < 0 ? -e.x : e.x);
+            sum.y += from_fixed(e.y);
           }
-          a.slots[t.slot * pieces + t.piece] = sum;
+          sum.x = warp_sum(sum.x);
+          sum.y = warp_sum(sum.y);
+          if (lane == 0) a.slots[t.slot * pieces + t.piece] = sum;
         }
         asm volatile("bar.sync 1, %0;\n" ::"n"(32 * OZ_EPI_WARPS) : "memory");
       }
@@ -1295,10 +1297,16 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
       for (int k = warp; k < a.nparts; k += OZ_THREADS / 32) {
         const PartDesc p = a.parts[k];
         float mx = 0.0f;
-        for (int rr = lane; rr < p.s; rr += 32) {
-          float* q = a.normf + p.soff + rr;
-          mx = fmaxf(mx, __ldcg(q));
-          *q = 0.0f;
+        // loads in flight together, eight per lane
+        for (int r0 = lane; r0 < p.s; r0 += 32 * 8) {
+          float v[8];
+#pragma unroll
+          for (int q = 0; q < 8; ++q) v[q] = r0 + 32 * q < p.s ? __ldcg(a.normf + p.soff + r0 + 32 * q) : 0.0f;
+#pragma unroll
+          for (int q = 0; q < 8; ++q) {
+            mx = fmaxf(mx, v[q]);
+            if (r0 + 32 * q < p.s) a.normf[p.soff + r0 + 32 * q] = 0.0f;
+          }
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
@@ -1319,13 +1327,8 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
     return;
   }
 
-  if (last_block_ticket(&a.ctl.st->counter)) {
-    double u = 0.0, w = 0.0;
-    for (int k = threadIdx.x; k < a.nslots * pieces; k += blockDim.x) {
-      u += ld_cg(&a.slots[k].x);
-      w += ld_cg(&a.slots[k].y);
-    }
-    const double2 sum = block_sum2(u, w);
+  if (warp == 0 && last_block_warp(&a.ctl.st->counter)) {
+    const double2 sum = warp_sum_slots(a.slots, a.nslots * pieces);
     if (threadIdx.x == 0) {
       if (a.ctl.st->timeout) {
         a.ctl.st->status = ST_TIMEOUT;

@@ -276,13 +276,8 @@ __global__ void __launch_bounds__(256, 2) square_tc_kernel(TcStepArgs a) {
     const double2 sum = block_sum2(tY, tN);
     if (threadIdx.x == 0) a.slots[t.slot] = sum;
   }
-  if (last_block_ticket(&a.ctl.st->counter)) {
-    double u = 0.0, w = 0.0;
-    for (int k = threadIdx.x; k < a.nslots; k += blockDim.x) {
-      u += ld_cg(&a.slots[k].x);
-      w += ld_cg(&a.slots[k].y);
-    }
-    const double2 sum = block_sum2(u, w);
+  if (warp == 0 && last_block_warp(&a.ctl.st->counter)) {
+    const double2 sum = warp_sum_slots(a.slots, a.nslots);
     if (threadIdx.x == 0) {
       if (a.ctl.st->timeout) {
         a.ctl.st->status = ST_TIMEOUT;
@@ -424,7 +419,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) square_tc_persistent_kernel(TcS
   const uint32_t bars = base + STAGES * STAGE_B;  // full[S], empty[S], tfull[2], tempty[2]
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(sb + STAGES * STAGE_B + 8 * (2 * STAGES + 4));
   int* s_err = reinterpret_cast<int*>(tmem_slot + 1);
-  double2* red = reinterpret_cast<double2*>(sb + STAGES * STAGE_B + 8 * (2 * STAGES + 4) + 16);
+  float2* red = reinterpret_cast<float2*>(sb + STAGES * STAGE_B + 8 * (2 * STAGES + 4) + 16);
   auto full = [&](int s) { return bars + 8u * s; };
   auto empty = [&](int s) { return bars + 8u * (STAGES + s); };
   auto tfull = [&](int b) { return bars + 8u * (2 * STAGES + b); };
@@ -438,8 +433,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1) square_tc_persistent_kernel(TcS
   // producer, the MMA warp and the epilogue warps through a ring in shared memory (full:
   // taken; empty: read by all of them)
   const bool dyn = a.tile_ctr != nullptr && MODE != TC_REBUILD;
-  const uint32_t ring_bars = smem_u32(red + TC_EPI_WARPS);
-  TcItem* s_items = reinterpret_cast<TcItem*>(reinterpret_cast<uint8_t*>(red + TC_EPI_WARPS) + 8 * 2 * TC_RING);
+  const uint32_t ring_bars = smem_u32(red + 128);
+  TcItem* s_items = reinterpret_cast<TcItem*>(reinterpret_cast<uint8_t*>(red + 128) + 8 * 2 * TC_RING);
   auto item_full = [&](int q) { return ring_bars + 8u * q; };
   auto item_empty = [&](int q) { return ring_bars + 8u * (TC_RING + q); };
 
@@ -780,7 +775,6 @@ __global__ void __launch_bounds__(TC_THREADS, 1) square_tc_persistent_kernel(TcS
       const float ysc = XBAR16 ? pow2i(a.xb_sig[t.part] - 28) : Kind<KIND>::YSCALE;
       const float osc = XBAR16 ? pow2i(-a.xb_sig[a.nparts + t.part]) : 1.0f;  // Xbar_new's operand scale
       uint32_t amax = 0;  // FP16 adjoint: largest |Xbar_new| of the thread's entries (FP32 bits)
-      double tY = 0.0, tN = 0.0;
 #pragma unroll 1
       for (int h = 0; h < 2; ++h) {
         if (has[0]) {
@@ -788,8 +782,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1) square_tc_persistent_kernel(TcS
           float x[16];
 #pragma unroll
           for (int j = 0; j < 16; ++j) x[j] = alf > 0 ? Xi[(int64_t)(cbase + j) * ld + r] : 0.0f;
-          // the one diagonal entry of this half row, if any, picked out in FP32 and added in
-          // FP64 once (an FP64 add in the unrolled loop would be issued for every element)
+          // the one diagonal entry of this half row, if any, goes to shared memory; one warp adds
+          // the tile's in FP64
           float yd = 0.0f, zd = 0.0f;
 #pragma unroll
           for (int j = 0; j < 16; ++j) {
@@ -800,10 +794,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) square_tc_persistent_kernel(TcS
             x[j] = z;
             if (XBAR16) amax = max(amax, __float_as_uint(z) & 0x7FFFFFFFu);  // NaN bits exceed Inf
           }
-          if (MODE == TC_STEP && diag && r >= cbase && r < cbase + 16 && r < p.c) {
-            tY += (double)yd;
-            tN += (double)zd;
-          }
+          if (MODE == TC_STEP && diag && r >= cbase && r < cbase + 16) red[m] = make_float2(yd, zd);
           // diagonal tiles: keep the upper triangle (c >= r) and mirror it, so X stays exactly
           // symmetric whatever order the tensor cores sum the split products in.  Eight columns
           // per iteration, x turning in registers: straight-line code for 16 would be refetched for every tile
@@ -850,18 +841,19 @@ __global__ void __launch_bounds__(TC_THREADS, 1) square_tc_persistent_kernel(TcS
         if (lane == 0 && amax != 0) atomicMax(&a.xb_max[t.part], amax);
       }
       if (MODE == TC_STEP && diag) {
-        // fixed-order reduction over the epilogue warps (named barrier 1)
-        tY = warp_sum(tY);
-        tN = warp_sum(tN);
-        if (lane == 0) red[warp - 4] = make_double2(tY, tN);
+        // fixed-order sum of the diagonal's core entries by one warp (named barrier 1); a reduction
+        // in every warp would be 160 FP64 instructions, 16 cycles each
         asm volatile("bar.sync 1, %0;\n" ::"n"(32 * TC_EPI_WARPS) : "memory");
-        if (warp == 4 && lane == 0) {
+        if (warp == 4) {
           double2 acc = make_double2(0.0, 0.0);
-          for (int w = 0; w < TC_EPI_WARPS; ++w) {
-            acc.x += red[w].x;
-            acc.y += red[w].y;
+          for (int q = lane; q < min(p.c - r0, 128); q += 32) {
+            const float2 e = red[q];
+            acc.x += (double)e.x;
+            acc.y += (double)e.y;
           }
-          a.slots[t.slot] = acc;
+          acc.x = warp_sum(acc.x);
+          acc.y = warp_sum(acc.y);
+          if (lane == 0) a.slots[t.slot] = acc;
         }
         asm volatile("bar.sync 1, %0;\n" ::"n"(32 * TC_EPI_WARPS) : "memory");
       }
@@ -895,13 +887,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1) square_tc_persistent_kernel(TcS
   }
   if (MODE != TC_STEP) return;
 
-  if (last_block_ticket(&a.ctl.st->counter)) {
-    double u = 0.0, w = 0.0;
-    for (int k = threadIdx.x; k < a.nslots; k += blockDim.x) {
-      u += ld_cg(&a.slots[k].x);
-      w += ld_cg(&a.slots[k].y);
-    }
-    const double2 sum = block_sum2(u, w);
+  if (warp == 0 && last_block_warp(&a.ctl.st->counter)) {
+    const double2 sum = warp_sum_slots(a.slots, a.nslots);
     if (threadIdx.x == 0) {
       if (a.ctl.st->timeout) {
         a.ctl.st->status = ST_TIMEOUT;
@@ -1180,13 +1167,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1) square_tc_wide_kernel(TcStepArg
   if (warp == 1) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;\n" ::"r"(tmem));
   if (threadIdx.x == 0 && *s_err) a.ctl.st->timeout = 1;
 
-  if (last_block_ticket(&a.ctl.st->counter)) {
-    double u = 0.0, w = 0.0;
-    for (int k = threadIdx.x; k < a.nslots; k += blockDim.x) {
-      u += ld_cg(&a.slots[k].x);
-      w += ld_cg(&a.slots[k].y);
-    }
-    const double2 sum = block_sum2(u, w);
+  if (warp == 0 && last_block_warp(&a.ctl.st->counter)) {
+    const double2 sum = warp_sum_slots(a.slots, a.nslots);
     if (threadIdx.x == 0) {
       if (a.ctl.st->timeout) {
         a.ctl.st->status = ST_TIMEOUT;
@@ -1221,7 +1203,7 @@ static cudaError_t launch_tc_persistent(const TcStepArgs& a, int grid, cudaStrea
   constexpr int NOPS = NPROD == 3 ? 4 : 2;
   constexpr int STAGES = NPROD == 3 ? 3 : 4;
   const int smem =
-      STAGES * NOPS * (int)kTileBytes + 1024 + 8 * (2 * STAGES + 4) + 16 + 16 * TC_EPI_WARPS + 8 * 2 * TC_RING + (int)sizeof(TcItem) * TC_RING;
+      STAGES * NOPS * (int)kTileBytes + 1024 + 8 * (2 * STAGES + 4) + 16 + 8 * 128 + 8 * 2 * TC_RING + (int)sizeof(TcItem) * TC_RING;
   cudaError_t e = cudaFuncSetAttribute(square_tc_persistent_kernel<KIND, NPROD, MODE>,
                                        cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
