@@ -49,7 +49,7 @@ struct DevState {
   int32_t fp64_steps;
   int32_t timeout;     // a bounded device wait gave up
   int32_t tail_left;   // FP64 path: alternating tail steps still to run (0: none)
-  int32_t pad[4];
+  double inv_hi, inv_lo;  // 1 / (eps_max - eps_min) = inv_hi + inv_lo; inv_hi = 0: to be divided by
 };
 
 enum : int32_t { ST_OK = 0, ST_NOT_CONVERGED = 5, ST_TRACE = 6, ST_NONFINITE = 7, ST_TIMEOUT = 9 };
@@ -215,6 +215,26 @@ constexpr int32_t OZ_SIG_NONFINITE = 0x7FFF;  // scale of a part whose Xbar hold
 
 __device__ __forceinline__ double ld_cg(const double* p) { return __ldcg(p); }
 
+// Programmatic dependent launch: the next launch of the stream may become resident (its blocks
+// set up barriers and TMEM while this one drains), and this one waits here until the launch
+// before it has completed and its writes are visible.
+__device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
+template <typename... Params, typename... Args>
+cudaError_t launch_pdl(void (*kern)(Params...), int grid, int threads, size_t smem, cudaStream_t s, const Args&... a) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, static_cast<Params>(a)...);
+}
+
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -309,6 +329,64 @@ __device__ __forceinline__ double2 warp_sum_slots(const double2* slots, int n) {
     b += v.y;
   }
   return make_double2(warp_sum(a), warp_sum(b));
+}
+
+// One column of the initial guess, assembled by a warp in shared memory and written once.
+// Rows [0, rend) (a multiple of 128) come in chunks: zeros, then the entries t < nq of the row's
+// list whose local index lj[t] falls there, put(index, xq[t]) each, then out(first row, the
+// chunk's rows).  Zeros written to the arena, entries scattered over them there and the column
+// read back for its digits cost a pass over memory more, the arena being larger than L2 in every
+// large plan: n = 30000, 256 parts, 0.66 -> 0.49 ms for fixed point and digits (2 GB, 0.29 ms at the
+// copy rate; the rest is the chain row -> list -> value, hidden by the warps in flight) and 0.54 ->
+// 0.38 ms for FP32 and two FP16 operands.
+constexpr int GATHER_BATCH = 4;   // entries per lane in flight (8: 7 % slower for the warps its registers cost)
+constexpr int GATHER_ROWS = 512;  // 4 KB of 8-byte words a warp: 6 blocks of 8 warps an SM
+template <typename T, typename Put, typename Out>
+__device__ __forceinline__ void gather_column(T* buf, int rend, int nq, const int32_t* __restrict__ lj,
+                                              const double* __restrict__ xq, int lane, Put put, Out out) {
+  for (int r0 = 0; r0 < rend; r0 += GATHER_ROWS) {
+    const int m = min(GATHER_ROWS, rend - r0);
+    for (int i = lane; i < (int)(m * sizeof(T) / 16); i += 32) reinterpret_cast<uint4*>(buf)[i] = make_uint4(0, 0, 0, 0);
+    __syncwarp();
+    for (int t0 = lane; t0 < nq; t0 += 32 * GATHER_BATCH) {
+      int a[GATHER_BATCH];
+      double x[GATHER_BATCH];
+#pragma unroll
+      for (int u = 0; u < GATHER_BATCH; ++u) a[u] = t0 + 32 * u < nq ? lj[t0 + 32 * u] - r0 : -1;
+#pragma unroll
+      for (int u = 0; u < GATHER_BATCH; ++u)  // -1 (not in the part) and the other chunks' rows fall outside
+        x[u] = a[u] >= 0 && a[u] < m ? xq[t0 + 32 * u] : 0.0;
+#pragma unroll
+      for (int u = 0; u < GATHER_BATCH; ++u)
+        if (a[u] >= 0 && a[u] < m) buf[a[u]] = put(a[u] + r0, x[u]);
+    }
+    __syncwarp();
+    for (int r = 0; r < m; r += 128) out(r0 + r, buf + r);
+    __syncwarp();
+  }
+}
+
+// Sum of one value per warp (zero where a warp has none) in warp order, to slots[blockIdx.x]; then
+// the last block forms T_0 from all blocks' slots.  `v` lies in shared memory, one per warp.
+__device__ __forceinline__ bool gather_traces(const double* v, double* slots, unsigned int* counter, double& sum) {
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double a = 0.0;
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) a += v[w];
+    slots[blockIdx.x] = a;
+  }
+  if (!last_block_ticket(counter)) return false;
+  double a = 0.0;
+#pragma unroll 8
+  for (unsigned int k = threadIdx.x; k < gridDim.x; k += blockDim.x) a += ld_cg(&slots[k]);
+  a = warp_sum(a);
+  __shared__ double red[32];
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = a;
+  __syncthreads();
+  sum = 0.0;
+  if (threadIdx.x == 0)
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) sum += red[w];
+  return threadIdx.x == 0;
 }
 
 // Bookkeeping of step `step` (0 = the initial guess X0), run by one thread of the

@@ -9,8 +9,28 @@ namespace gsp2 {
 // ------------------------------------------------------------------------------------
 // Gershgorin bounds (Section 2.1): eps_min = min_i (H_ii - R_i), eps_max = max_i (H_ii
 // + R_i), R_i = sum_{j != i} |H_ij|.  One warp per row; block min/max into a slot; the
-// last block reduces the slots and resets the per-call state.
+// last block reduces the slots.  What bounds it is FP64 instructions (one warp's takes the SM's FP64
+// pipe about 30 cycles) and the latency of a row's list: only the sum of |H_ij| uses them, the diagonal
+// goes by shuffle, a row's two bounds wait until a lane has one of 32 rows, and minima and maxima are
+// taken on integers.  One thread reducing 608 slots took 70 us of every call: n = 512 84 -> 11 us,
+// n = 30000 (9.2 M entries) 157 -> 76 us.
 // ------------------------------------------------------------------------------------
+// Doubles (not NaN) as integers of the same order.
+__device__ __forceinline__ unsigned long long ordered_bits(double v) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(v);
+  return b ^ (b >> 63 ? ~0ull : 1ull << 63);
+}
+__device__ __forceinline__ double from_ordered_bits(unsigned long long k) {
+  return __longlong_as_double((long long)(k ^ (k >> 63 ? 1ull << 63 : ~0ull)));
+}
+__device__ __forceinline__ void warp_minmax(unsigned long long& lo, unsigned long long& hi) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    lo = min(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+    hi = max(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+  }
+}
+constexpr int BOUNDS_UNROLL = 4;  // entries per lane in flight
 __global__ void __launch_bounds__(256) bounds_kernel(int64_t n, const int64_t* __restrict__ rowptr,
                                                      const int32_t* __restrict__ colind,
                                                      const double* __restrict__ vals,
@@ -18,41 +38,90 @@ __global__ void __launch_bounds__(256) bounds_kernel(int64_t n, const int64_t* _
   const int lane = threadIdx.x & 31;
   const int64_t warp = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int64_t nwarps = (int64_t)gridDim.x * (blockDim.x >> 5);
+  pdl_release();
+  pdl_wait();
   double lo = INFINITY, hi = -INFINITY;
-  int bad = 0;
+  int bad = 0, rows = 0;
+  double d = 0.0, rad = 0.0;  // lane l: diagonal and radius of the warp's row l of the last 32
   for (int64_t i = warp; i < n; i += nwarps) {
-    double rad = 0.0, dia = 0.0;
-    for (int64_t p = rowptr[i] + lane; p < rowptr[i + 1]; p += 32) {
-      const double v = vals[p];
-      if (!isfinite(v)) bad = 1;
-      if (colind[p] == i) dia = v; else rad += fabs(v);
-    }
-    rad = warp_sum(rad);
-    dia = warp_sum(dia);  // exactly one lane holds the diagonal
-    lo = fmin(lo, dia - rad);
-    hi = fmax(hi, dia + rad);
-  }
-  __shared__ double s_lo[8], s_hi[8];
-  __shared__ int s_bad;
-  if (threadIdx.x == 0) s_bad = 0;
-  __syncthreads();
-  if (bad) s_bad = 1;
-  if (lane == 0) { s_lo[threadIdx.x >> 5] = lo; s_hi[threadIdx.x >> 5] = hi; }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    for (int w = 1; w < (int)(blockDim.x >> 5); ++w) { lo = fmin(lo, s_lo[w]); hi = fmax(hi, s_hi[w]); }
-    slots[blockIdx.x] = make_double2(lo, hi);
-    if (s_bad) st->nonfinite = 1;
-  }
-  if (last_block_ticket(&st->counter)) {
-    if (threadIdx.x == 0) {
-      double a = INFINITY, b = -INFINITY;
-      for (unsigned int k = 0; k < gridDim.x; ++k) {
-        a = fmin(a, ld_cg(&slots[k].x));
-        b = fmax(b, ld_cg(&slots[k].y));
+    const int64_t p1 = rowptr[i + 1];
+    double sum = 0.0, dia = 0.0;
+    bool own = false;
+    for (int64_t p0 = rowptr[i] + lane; p0 < p1; p0 += 32 * BOUNDS_UNROLL) {
+      double v[BOUNDS_UNROLL];
+      int32_t c[BOUNDS_UNROLL];
+#pragma unroll
+      for (int u = 0; u < BOUNDS_UNROLL; ++u) {
+        const bool in = p0 + 32 * u < p1;
+        v[u] = in ? vals[p0 + 32 * u] : 0.0;
+        c[u] = in ? colind[p0 + 32 * u] : -1;
       }
+#pragma unroll
+      for (int u = 0; u < BOUNDS_UNROLL; ++u) {
+        if (((unsigned long long)__double_as_longlong(v[u]) >> 52 & 0x7FF) == 0x7FF) bad = 1;
+        if (c[u] == i) {
+          dia = v[u];
+          own = true;
+        } else if (p0 + 32 * u < p1) {
+          sum += fabs(v[u]);
+        }
+      }
+    }
+    sum = warp_sum(sum);
+    const unsigned int who = __ballot_sync(0xffffffffu, own);  // at most one lane has the diagonal
+    dia = __shfl_sync(0xffffffffu, dia, who ? __ffs(who) - 1 : 0);
+    if (lane == (rows & 31)) {
+      d = dia;
+      rad = sum;
+    }
+    if ((++rows & 31) == 0 || i + nwarps >= n) {
+      if (lane <= ((rows - 1) & 31)) {
+        lo = fmin(lo, d - rad);
+        hi = fmax(hi, d + rad);
+      }
+    }
+  }
+  // the rest compares the doubles as integers (no NaN among them)
+  unsigned long long klo = ordered_bits(lo), khi = ordered_bits(hi);
+  __shared__ unsigned long long s_lo[8], s_hi[8];
+  auto block_minmax = [&]() {  // thread 0 ends with the block's
+    warp_minmax(klo, khi);
+    __syncthreads();
+    if (lane == 0) {
+      s_lo[threadIdx.x >> 5] = klo;
+      s_hi[threadIdx.x >> 5] = khi;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0)
+      for (int w = 1; w < (int)(blockDim.x >> 5); ++w) {
+        klo = min(klo, s_lo[w]);
+        khi = max(khi, s_hi[w]);
+      }
+  };
+  if (bad) st->nonfinite = 1;
+  block_minmax();
+  if (threadIdx.x == 0) slots[blockIdx.x] = make_double2(from_ordered_bits(klo), from_ordered_bits(khi));
+  if (last_block_ticket(&st->counter)) {
+    klo = ~0ull;
+    khi = 0ull;
+#pragma unroll 4
+    for (unsigned int k = threadIdx.x; k < gridDim.x; k += blockDim.x) {
+      const double2 v = __ldcg(&slots[k]);
+      klo = min(klo, ordered_bits(v.x));
+      khi = max(khi, ordered_bits(v.y));
+    }
+    block_minmax();
+    if (threadIdx.x == 0) {
+      const double a = from_ordered_bits(klo), b = from_ordered_bits(khi);
       st->eps_min = a;
       st->eps_max = b;
+      // x0_values_kernel divides by b - a as a product with 1 / (b - a) held in two doubles
+      // (multiplication by a constant: Brisebarre and Muller, IEEE Trans. Comput. 57, 2008): two FP64
+      // instructions instead of a division, within (1/2 + 2^-50) ulp; not where the reciprocal or
+      // its error would leave the normal range
+      const double den = b - a, h = 1.0 / den;
+      st->inv_hi = den >= 0x1p-900 && den <= 0x1p900 ? h : 0.0;
+      st->inv_lo = fma(-den, h, 1.0) / den;
       if (!isfinite(a) || !isfinite(b) || !(b > a)) st->nonfinite = 1;
       st->counter = 0;
     }
@@ -80,20 +149,31 @@ __global__ void reset_kernel(DevState* st, int8_t* alpha, const int8_t* alpha_in
 // Eq. 1 on the stored entries of H, once per P-build: x0[q] = (eps_max [col = row] - H_q) /
 // (eps_max - eps_min).  Every entry lies in several parts (each of which gathers it), so
 // dividing once here keeps the divisions, which run on GB300's slow FP64 pipe, out of the
-// gathers.  One warp per row.
+// gathers.  One warp per row.  Two FP64 instructions an entry bound it: 9.2 M entries 208 -> 117 us
+// (a division took about ten).
 // ------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) x0_values_kernel(int64_t n, const int64_t* __restrict__ rowptr,
                                                         const int32_t* __restrict__ colind,
                                                         const double* __restrict__ vals, const DevState* st,
                                                         double* __restrict__ x0) {
-  const double emax = st->eps_max, emin = st->eps_min;
-  const double den = emax - emin;
+  pdl_release();
+  pdl_wait();
+  const double emax = st->eps_max, h = st->inv_hi, l = st->inv_lo;
   const int lane = threadIdx.x & 31;
   const int64_t w0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nw = ((int64_t)gridDim.x * blockDim.x) >> 5;
-  for (int64_t g = w0; g < n; g += nw)
-    for (int64_t q = rowptr[g] + lane; q < rowptr[g + 1]; q += 32)
-      x0[q] = (colind[q] == g) ? (emax - vals[q]) / den : (0.0 - vals[q]) / den;
+  for (int64_t g = w0; g < n; g += nw) {
+    const int64_t q1 = rowptr[g + 1];
+#pragma unroll 4
+    for (int64_t q = rowptr[g] + lane; q < q1; q += 32) {
+      const double v = vals[q];
+      // 0 - v without an FP64 instruction (0 for either zero)
+      const long long w = __double_as_longlong(v);
+      double a = __longlong_as_double(w << 1 == 0 ? 0ll : (long long)((unsigned long long)w ^ 1ull << 63));
+      if (colind[q] == g) a = emax - v;
+      x0[q] = h != 0.0 ? fma(a, h, a * l) : a / (emax - st->eps_min);
+    }
+  }
 }
 
 // ------------------------------------------------------------------------------------
@@ -131,7 +211,7 @@ __global__ void __launch_bounds__(256) locate_kernel(const PartDesc* __restrict_
 // Blocks store the core-diagonal sum of their columns; the last block forms T_0 and
 // chooses the first branch.
 // ------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) gather_kernel(const PartDesc* __restrict__ parts,
+__global__ void __launch_bounds__(256, 6) gather_kernel(const PartDesc* __restrict__ parts,
                                                      const ColBlock* __restrict__ blocks,
                                                      const int32_t* __restrict__ Sall,
                                                      const int64_t* __restrict__ rowptr,
@@ -139,45 +219,47 @@ __global__ void __launch_bounds__(256) gather_kernel(const PartDesc* __restrict_
                                                      const int64_t* __restrict__ locptr,
                                                      const double* __restrict__ x0, double* __restrict__ arena,
                                                      double* __restrict__ slots, StepCtl ctl) {
+  __shared__ __align__(16) double cols[COLS_PER_BLOCK][GATHER_ROWS];
+  __shared__ double s_tr[COLS_PER_BLOCK];
+  pdl_release();
+  pdl_wait();
   const ColBlock b = blocks[blockIdx.x];
   const PartDesc p = parts[b.part];
-  const int lane = threadIdx.x & 31;
-  const int j = b.j0 + (threadIdx.x >> 5);
-  const int32_t* S = Sall + p.soff;
-  double tr = 0.0;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int j = b.j0 + w;
+  if (lane == 0) s_tr[w] = 0.0;
+  __syncwarp();
   // columns [s, ld) are zero padding: the squares read it up to the tile edge, and the
   // emulated steps up to ld (their K slices are packed within 128-blocks)
   if (j < p.ld) {
-    double* col = arena + p.off + (int64_t)j * p.ld;
-    for (int r = lane; r < p.ld; r += 32) col[r] = 0.0;
-    __syncwarp();
+    double* const col = arena + p.off + (int64_t)j * p.ld;
+    int64_t q0 = 0;
+    int nq = 0;
+    const int32_t* lj = loc;
     if (j < p.s) {
-      const int32_t g = S[j];
-      const int64_t q0 = rowptr[g], nq = rowptr[g + 1] - q0;
-      const int32_t* lj = loc + locptr[p.soff + j];
-      for (int64_t t = lane; t < nq; t += 32) {
-        const int a = lj[t];
-        const int64_t q = q0 + t;
-        if (a >= 0) {
-          const double x = x0[q];
-          col[a] = x;
-          if (a == j && j < p.c) tr = x;
-        }
-      }
+      const int32_t g = Sall[p.soff + j];
+      q0 = rowptr[g];
+      nq = (int)(rowptr[g + 1] - q0);
+      lj = loc + locptr[p.soff + j];
     }
+    gather_column(
+        cols[w], p.ld, nq, lj, x0 + q0, lane,
+        [&](int a, double x) {
+          if (a == j && j < p.c) s_tr[w] = x;
+          return x;
+        },
+        [&](int r, const double* v) {
+          const double2* v2 = reinterpret_cast<const double2*>(v);
+          double2* c2 = reinterpret_cast<double2*>(col + r);
+          c2[lane] = v2[lane];
+          c2[32 + lane] = v2[32 + lane];
+        });
   }
-  const double2 t = block_sum2(tr, 0.0);
-  if (threadIdx.x == 0) slots[blockIdx.x] = t.x;
-  if (last_block_ticket(&ctl.st->counter)) {
-    double2 acc = make_double2(0.0, 0.0);
-    double a = 0.0;
-    for (unsigned int k = threadIdx.x; k < gridDim.x; k += blockDim.x) a += ld_cg(&slots[k]);
-    acc = block_sum2(a, 0.0);
-    if (threadIdx.x == 0) {
-      if (ctl.st->nonfinite) ctl.st->status = ST_NONFINITE;
-      finish_step(ctl, 0, acc.x, 0.0);
-      ctl.st->counter = 0;
-    }
+  double sum;
+  if (gather_traces(s_tr, slots, &ctl.st->counter, sum)) {
+    if (ctl.st->nonfinite) ctl.st->status = ST_NONFINITE;
+    finish_step(ctl, 0, sum, 0.0);
+    ctl.st->counter = 0;
   }
 }
 
@@ -498,22 +580,21 @@ cudaError_t launch_reset(DevState* st, int8_t* alpha, const int8_t* alpha_in, in
 
 cudaError_t launch_bounds(int64_t n, const int64_t* rowptr, const int32_t* colind, const double* vals,
                           double2* slots, int nblocks, DevState* st, cudaStream_t s) {
-  bounds_kernel<<<nblocks, 256, 0, s>>>(n, rowptr, colind, vals, slots, st);
-  return cudaGetLastError();
+  const int64_t rows = (n + 7) / 8;  // a warp for each row, at most nblocks blocks
+  return launch_pdl(bounds_kernel, (int)(rows < nblocks ? rows : nblocks), 256, 0, s, n, rowptr, colind, vals, slots, st);
 }
 
 cudaError_t launch_gather(const PartDesc* parts, const ColBlock* blocks, int nblocks, const int32_t* Sall,
                           const int64_t* rowptr, const int32_t* loc, const int64_t* locptr, const double* x0,
                           double* arena, double* slots, const StepCtl& ctl, cudaStream_t s) {
-  gather_kernel<<<nblocks, 32 * COLS_PER_BLOCK, 0, s>>>(parts, blocks, Sall, rowptr, loc, locptr, x0, arena,
-                                                       slots, ctl);
-  return cudaGetLastError();
+  return launch_pdl(gather_kernel, nblocks, 32 * COLS_PER_BLOCK, 0, s, parts, blocks, Sall, rowptr, loc, locptr, x0,
+                    arena, slots, ctl);
 }
 
 cudaError_t launch_x0_values(int64_t n, const int64_t* rowptr, const int32_t* colind, const double* vals,
                              const DevState* st, double* x0, int nsm, cudaStream_t s) {
-  x0_values_kernel<<<8 * nsm, 256, 0, s>>>(n, rowptr, colind, vals, st, x0);
-  return cudaGetLastError();
+  const int64_t rows = (n + 7) / 8;
+  return launch_pdl(x0_values_kernel, (int)(rows < 8 * nsm ? rows : 8 * nsm), 256, 0, s, n, rowptr, colind, vals, st, x0);
 }
 
 cudaError_t launch_locate(const PartDesc* parts, const ColBlock* blocks, int nblocks, const int32_t* Sall,

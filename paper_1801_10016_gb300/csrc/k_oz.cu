@@ -158,63 +158,59 @@ __global__ void __launch_bounds__(256) oz_convert_slice_kernel(const PartDesc* _
 
 // Gather of the emulated path: Eq. 1 and the digits of X0 in one pass.  One warp per column
 // j < ld assembles the rows of column j of X0 on or above its diagonal block, the only ones
-// the emulated steps read (zeros, then the stored entries of row S_j of H that fall there,
+// the emulated steps read: zeros and the stored entries of row S_j of H that fall there,
 // at the local indices of the plan's table (locate_kernel), with the values of Eq. 1 from
-// x0_values_kernel, each stored in the 64-bit
-// fixed point x 2^56 of the emulated steps' master), then reads them back from L1/L2 and
-// writes their digits, coalesced (rows outside the part are zero).  Blocks store
-// the core-diagonal sum of their columns; the last block forms T_0 and takes the first
-// branch.
-__global__ void __launch_bounds__(32 * COLS_PER_BLOCK) oz_gather_kernel(
+// x0_values_kernel, each stored in the 64-bit fixed point x 2^56 of the emulated steps' master
+// and as digits.  Blocks store the core-diagonal sum of their columns; the last block forms T_0
+// and takes the first branch.
+__global__ void __launch_bounds__(32 * COLS_PER_BLOCK, 6) oz_gather_kernel(
     const PartDesc* __restrict__ parts, const ColBlock* __restrict__ blocks, const int32_t* __restrict__ Sall,
     const int64_t* __restrict__ rowptr, const int32_t* __restrict__ loc, const int64_t* __restrict__ locptr,
     const double* __restrict__ x0, double* __restrict__ arena, OzSlices dig, double* __restrict__ slots,
     StepCtl ctl) {
+  __shared__ __align__(16) long long cols[COLS_PER_BLOCK][GATHER_ROWS];
+  __shared__ double s_tr[COLS_PER_BLOCK];
+  pdl_release();
+  pdl_wait();
   const ColBlock b = blocks[blockIdx.x];
   const PartDesc p = parts[b.part];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int j = b.j0 + w;
-  const int32_t* S = Sall + p.soff;
-  long long* col = reinterpret_cast<long long*>(arena) + p.off + (int64_t)j * p.ld;
-  double tr = 0.0;
+  if (lane == 0) s_tr[w] = 0.0;
+  __syncwarp();
   if (j < p.ld) {
     const int rend = min(p.ld, (j / 128 + 1) * 128);
-    for (int r = lane; r < rend; r += 32) col[r] = 0ll;
-    __syncwarp();
+    const int64_t cbase = p.off + (int64_t)j * p.ld;  // a multiple of 128, as rend
+    long long* const col = reinterpret_cast<long long*>(arena) + cbase;
+    int64_t q0 = 0;
+    int nq = 0;
+    const int32_t* lj = loc;
     if (j < p.s) {
-      const int32_t g = S[j];
-      const int64_t q0 = rowptr[g], nq = rowptr[g + 1] - q0;
-      const int32_t* lj = loc + locptr[p.soff + j];
-      for (int64_t t = lane; t < nq; t += 32) {
-        const int a = lj[t];
-        const int64_t q = q0 + t;
-        if (a >= 0 && a < rend) {
-          const double x = x0[q];
-          col[a] = to_fixed(x);
-          if (a == j && j < p.c) tr = x;
-        }
-      }
+      const int32_t g = Sall[p.soff + j];
+      q0 = rowptr[g];
+      nq = (int)(rowptr[g + 1] - q0);
+      lj = loc + locptr[p.soff + j];
     }
-    __syncwarp();  // the lanes' stores to the column are visible to the whole warp
-    const int64_t cbase = p.off + (int64_t)j * p.ld;
-    for (int r = 4 * lane; r < rend; r += 128) {  // rend and cbase are multiples of 128
-      long long v[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) v[i] = col[r + i];
-      store_digits4(dig.s, cbase + r, v);
-    }
+    gather_column(
+        cols[w], rend, nq, lj, x0 + q0, lane,
+        [&](int a, double x) {
+          if (a == j && j < p.c) s_tr[w] = x;
+          return to_fixed(x);
+        },
+        [&](int r, const long long* v) {
+          const longlong2* v2 = reinterpret_cast<const longlong2*>(v);
+          longlong2* c2 = reinterpret_cast<longlong2*>(col + r);
+          c2[lane] = v2[lane];
+          c2[32 + lane] = v2[32 + lane];
+          const longlong2 a = v2[2 * lane], c = v2[2 * lane + 1];
+          store_digits4(dig.s, cbase + r + 4 * lane, {a.x, a.y, c.x, c.y});
+        });
   }
-  const double2 t = block_sum2(tr, 0.0);
-  if (threadIdx.x == 0) slots[blockIdx.x] = t.x;
-  if (last_block_ticket(&ctl.st->counter)) {
-    double a = 0.0;
-    for (unsigned int k = threadIdx.x; k < gridDim.x; k += blockDim.x) a += ld_cg(&slots[k]);
-    const double2 acc = block_sum2(a, 0.0);
-    if (threadIdx.x == 0) {
-      if (ctl.st->nonfinite) ctl.st->status = ST_NONFINITE;
-      finish_step(ctl, 0, acc.x, 0.0);
-      ctl.st->counter = 0;
-    }
+  double sum;
+  if (gather_traces(s_tr, slots, &ctl.st->counter, sum)) {
+    if (ctl.st->nonfinite) ctl.st->status = ST_NONFINITE;
+    finish_step(ctl, 0, sum, 0.0);
+    ctl.st->counter = 0;
   }
 }
 
@@ -1368,9 +1364,8 @@ cudaError_t launch_oz_step(const OzStepArgs& a, int grid, cudaStream_t s, bool a
 cudaError_t launch_oz_gather(const PartDesc* parts, const ColBlock* blocks, int nblocks, const int32_t* Sall,
                              const int64_t* rowptr, const int32_t* loc, const int64_t* locptr, const double* x0,
                              double* arena, const OzSlices& dig, double* slots, const StepCtl& ctl, cudaStream_t s) {
-  oz_gather_kernel<<<nblocks, 32 * COLS_PER_BLOCK, 0, s>>>(parts, blocks, Sall, rowptr, loc, locptr, x0, arena, dig,
-                                                            slots, ctl);
-  return cudaGetLastError();
+  return launch_pdl(oz_gather_kernel, nblocks, 32 * COLS_PER_BLOCK, 0, s, parts, blocks, Sall, rowptr, loc, locptr, x0,
+                    arena, dig, slots, ctl);
 }
 
 cudaError_t launch_oz_adj_scale(const PartDesc* parts, int nparts, const Tile* tiles, int ntiles, const double* xb0,

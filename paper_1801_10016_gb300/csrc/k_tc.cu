@@ -38,6 +38,27 @@ __device__ __forceinline__ void store_operands(void* hi, void* lo, int64_t e, fl
   }
 }
 
+// Store the operand(s) of four consecutive elements starting at element e (a multiple of 4).
+template <int KIND, int NPROD>
+__device__ __forceinline__ void store_operand_quad(void* hi, void* lo, int64_t e, const float (&x)[4]) {
+  uint32_t h[4], l[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const auto v = Operand<KIND>::bits(x[i]);
+    h[i] = v;
+    if (NPROD == 3) l[i] = Operand<KIND>::bits(x[i] - Operand<KIND>::value(v));
+  }
+  if (KIND != 1) {
+    *reinterpret_cast<uint2*>(reinterpret_cast<uint16_t*>(hi) + e) = make_uint2(h[0] | h[1] << 16, h[2] | h[3] << 16);
+    if (NPROD == 3)
+      *reinterpret_cast<uint2*>(reinterpret_cast<uint16_t*>(lo) + e) = make_uint2(l[0] | l[1] << 16, l[2] | l[3] << 16);
+  } else {
+    *reinterpret_cast<uint4*>(reinterpret_cast<uint32_t*>(hi) + e) = make_uint4(h[0], h[1], h[2], h[3]);
+    if (NPROD == 3)
+      *reinterpret_cast<uint4*>(reinterpret_cast<uint32_t*>(lo) + e) = make_uint4(l[0], l[1], l[2], l[3]);
+  }
+}
+
 // Store the operand(s) of N consecutive elements x[0..N-1] (N a multiple of 8) starting at
 // element e (16-byte aligned) with vector stores.
 template <int KIND, int NPROD, int N>
@@ -1328,7 +1349,7 @@ cudaError_t launch_square_tc(int kind, int nprod, const TcStepArgs& a, int ntile
 // 16-bit steps read no others).  T_0 is summed in FP64 from the stored FP32 values.
 // KIND = -1: FP32 master only (CUDA-core FP32 path).
 template <int KIND, int NPROD>
-__global__ void __launch_bounds__(256) gather_lp_kernel(const PartDesc* __restrict__ parts,
+__global__ void __launch_bounds__(256, 8) gather_lp_kernel(const PartDesc* __restrict__ parts,
                                                         const ColBlock* __restrict__ blocks,
                                                         const int32_t* __restrict__ Sall,
                                                         const int64_t* __restrict__ rowptr,
@@ -1337,50 +1358,47 @@ __global__ void __launch_bounds__(256) gather_lp_kernel(const PartDesc* __restri
                                                         const double* __restrict__ x0, float* __restrict__ master,
                                                         void* op_hi, void* op_lo, double* __restrict__ slots,
                                                         StepCtl ctl, int upper_rows) {
+  __shared__ __align__(16) float cols[COLS_PER_BLOCK][GATHER_ROWS];
+  __shared__ double s_tr[COLS_PER_BLOCK];
+  pdl_release();
+  pdl_wait();
   const ColBlock b = blocks[blockIdx.x];
   const PartDesc p = parts[b.part];
-  const int lane = threadIdx.x & 31;
-  const int j = b.j0 + (threadIdx.x >> 5);
-  const int32_t* S = Sall + p.soff;
-  double tr = 0.0;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int j = b.j0 + w;
+  if (lane == 0) s_tr[w] = 0.0;
+  __syncwarp();
   if (j < p.ld) {
     const int64_t cbase = p.off + (int64_t)j * p.ld;
     const int rend = upper_rows ? min(p.ld, (j / 128 + 1) * 128) : p.ld;
-    float* col = master + cbase;
-    for (int r = lane; r < rend; r += 32) col[r] = 0.0f;
-    __syncwarp();
+    int64_t q0 = 0;
+    int nq = 0;
+    const int32_t* lj = loc;
     if (j < p.s) {
-      const int32_t g = S[j];
-      const int64_t q0 = rowptr[g], nq = rowptr[g + 1] - q0;
-      const int32_t* lj = loc + locptr[p.soff + j];
-      for (int64_t t = lane; t < nq; t += 32) {
-        const int a = lj[t];
-        const int64_t q = q0 + t;
-        if (a >= 0 && a < rend) {
-          const double x = x0[q];
+      const int32_t g = Sall[p.soff + j];
+      q0 = rowptr[g];
+      nq = (int)(rowptr[g + 1] - q0);
+      lj = loc + locptr[p.soff + j];
+    }
+    gather_column(
+        cols[w], rend, nq, lj, x0 + q0, lane,
+        [&](int a, double x) {
           const float xf = (float)x;
-          col[a] = xf;
-          if (a == j && j < p.c) tr = (double)xf;
-        }
-      }
-    }
-    if (KIND >= 0) {
-      __syncwarp();  // the lanes' stores to the column are visible to the whole warp
-      for (int r = lane; r < rend; r += 32)
-        store_operands<(KIND < 0 ? 0 : KIND), NPROD>(op_hi, op_lo, cbase + r, col[r]);
-    }
+          if (a == j && j < p.c) s_tr[w] = (double)xf;
+          return xf;
+        },
+        [&](int r, const float* v) {
+          const float4 x = reinterpret_cast<const float4*>(v)[lane];
+          const int64_t e = cbase + r + 4 * lane;
+          *reinterpret_cast<float4*>(master + e) = x;
+          if (KIND >= 0) store_operand_quad<(KIND < 0 ? 0 : KIND), NPROD>(op_hi, op_lo, e, {x.x, x.y, x.z, x.w});
+        });
   }
-  const double2 t = block_sum2(tr, 0.0);
-  if (threadIdx.x == 0) slots[blockIdx.x] = t.x;
-  if (last_block_ticket(&ctl.st->counter)) {
-    double acc = 0.0;
-    for (unsigned int k = threadIdx.x; k < gridDim.x; k += blockDim.x) acc += ld_cg(&slots[k]);
-    const double2 sum = block_sum2(acc, 0.0);
-    if (threadIdx.x == 0) {
-      if (ctl.st->nonfinite) ctl.st->status = ST_NONFINITE;
-      finish_step(ctl, 0, sum.x, 0.0);
-      ctl.st->counter = 0;
-    }
+  double sum;
+  if (gather_traces(s_tr, slots, &ctl.st->counter, sum)) {
+    if (ctl.st->nonfinite) ctl.st->status = ST_NONFINITE;
+    finish_step(ctl, 0, sum, 0.0);
+    ctl.st->counter = 0;
   }
 }
 
@@ -1388,25 +1406,22 @@ cudaError_t launch_gather_lp(int kind, int nprod, const PartDesc* parts, const C
                              const int32_t* Sall, const int64_t* rowptr, const int32_t* loc, const int64_t* locptr,
                              const double* x0, float* master, void* op_hi, void* op_lo, double* slots,
                              const StepCtl& ctl, cudaStream_t s, int upper_rows) {
-  const dim3 g(nblocks), b(32 * COLS_PER_BLOCK);
+  auto go = [&](auto kern) {
+    return launch_pdl(kern, nblocks, 32 * COLS_PER_BLOCK, 0, s, parts, blocks, Sall, rowptr, loc, locptr, x0, master,
+                      op_hi, op_lo, slots, ctl, upper_rows);
+  };
   if (kind < 0)
-    gather_lp_kernel<-1, 1><<<g, b, 0, s>>>(parts, blocks, Sall, rowptr, loc, locptr, x0, master, op_hi, op_lo,
-                                            slots, ctl, upper_rows);
+    return go(gather_lp_kernel<-1, 1>);
   else if (kind == 0 && nprod == 1)
-    gather_lp_kernel<0, 1><<<g, b, 0, s>>>(parts, blocks, Sall, rowptr, loc, locptr, x0, master, op_hi, op_lo,
-                                           slots, ctl, upper_rows);
+    return go(gather_lp_kernel<0, 1>);
   else if (kind == 0 && nprod == 3)
-    gather_lp_kernel<0, 3><<<g, b, 0, s>>>(parts, blocks, Sall, rowptr, loc, locptr, x0, master, op_hi, op_lo,
-                                           slots, ctl, upper_rows);
+    return go(gather_lp_kernel<0, 3>);
   else if (kind == 1 && nprod == 1)
-    gather_lp_kernel<1, 1><<<g, b, 0, s>>>(parts, blocks, Sall, rowptr, loc, locptr, x0, master, op_hi, op_lo,
-                                           slots, ctl, upper_rows);
+    return go(gather_lp_kernel<1, 1>);
   else if (kind == 1 && nprod == 3)
-    gather_lp_kernel<1, 3><<<g, b, 0, s>>>(parts, blocks, Sall, rowptr, loc, locptr, x0, master, op_hi, op_lo,
-                                           slots, ctl, upper_rows);
+    return go(gather_lp_kernel<1, 3>);
   else if (kind == 2 && nprod == 3)
-    gather_lp_kernel<2, 3><<<g, b, 0, s>>>(parts, blocks, Sall, rowptr, loc, locptr, x0, master, op_hi, op_lo,
-                                           slots, ctl, upper_rows);
+    return go(gather_lp_kernel<2, 3>);
   else
     return cudaErrorInvalidValue;
   return cudaGetLastError();

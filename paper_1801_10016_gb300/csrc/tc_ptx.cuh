@@ -177,26 +177,6 @@ __device__ __forceinline__ void mma_col(int op, uint32_t tmem, uint64_t a, uint6
   }
 }
 #undef GSP2_MMA_COL
-// Programmatic dependent launch: the next launch of the stream may become resident (its blocks
-// set up barriers and TMEM while this one drains), and this one waits here until the launch
-// before it has completed and its writes are visible.
-__device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
-template <typename Args>
-cudaError_t launch_pdl(void (*kern)(Args), int grid, int threads, size_t smem, cudaStream_t s, const Args& a) {
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3((unsigned)grid);
-  cfg.blockDim = dim3((unsigned)threads);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = s;
-  cudaLaunchAttribute at{};
-  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at.val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = &at;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kern, a);
-}
-
 // True in one lane of a converged warp.
 __device__ __forceinline__ bool elect_one() {
   uint32_t p;
