@@ -913,18 +913,18 @@ extern "C" gsp2_status gsp2_bind_workspace(gsp2_handle h, void* d_ws, size_t byt
     if (!enc || q != cudaDriverEntryPointSuccess)
       return fail(h, GSP2_E_CUDA, "cuTensorMapEncodeTiled not available from the driver");
     const size_t np = h->parts.size();
-    // per digit set, K-major and MN-major maps whose boxes take all OZ_SLICES digits (the
-    // high pass) or the first OZ_LOW (the low pass) of a tile slice in one request; a set's
-    // digit arenas lie one arena apart (consecutive equal allocations)
+    // per digit set, K-major and MN-major maps whose boxes take one digit of a wide tile slice, or
+    // all OZ_SLICES digits (the high pass) or the first OZ_LOW (the low pass) of a narrow one in one
+    // request; a set's digit arenas lie one arena apart (consecutive equal allocations)
     const size_t dstride = (size_t)h->arena_elems * 2;
     auto encode_set = [&](unsigned char* mk, unsigned char* mm, const size_t* dig) -> int {
       for (int t = 1; t < OZ_SLICES; ++t)
         if (dig[t] != dig[0] + (size_t)t * dstride) return -1;
-      int r = encode_part_maps_digits(enc, mk, mm, h->parts.data(), (int)np, h->ws + dig[0], dstride, OZ_SLICES,
-                                      OZ_SLICES, OZ_BK);
-      if (r == 0)
-        r = encode_part_maps_digits(enc, mk + np * 128, mm + np * 128, h->parts.data(), (int)np, h->ws + dig[0],
-                                    dstride, OZ_SLICES, OZ_LOW, OZ_BK);
+      const int digits[3] = {1, OZ_SLICES, OZ_LOW}, bk[3] = {OZ_BK_WIDE, OZ_BK, OZ_BK};
+      int r = 0;
+      for (int m = 0; m < 3 && r == 0; ++m)
+        r = encode_part_maps_digits(enc, mk + m * np * 128, mm + m * np * 128, h->parts.data(), (int)np,
+                                    h->ws + dig[0], dstride, OZ_SLICES, digits[m], bk[m]);
       return r;
     };
     std::vector<unsigned char> maps((size_t)2 * OZ_SLICES * np * 128, 0), maps_mn(maps.size(), 0);
@@ -1062,6 +1062,19 @@ static int oz_pieces(int items, int sms) {
   return 0.62 * two < (double)one ? 2 : 1;
 }
 
+// Wide K slices (one digit tile per request, 128-byte rows) where whole tiles fill the chip and their
+// K is long: the loads take 0.77 of the narrow form's time and an item's sums stay in registers, but the
+// tensor pipe waits longer for an item's first slice and at each change of passes.  Measured
+// (narrow / wide, forward and backward; K the tiles' mean part size): 748 tiles of K 344 0.97, 0.95; 1,841
+// of 368 0.96, 0.95; 306 of 622 1.00, 0.97; 498 of 650 1.02, 1.03; 977 of 500 1.01, 1.02; 2,288 of 554 1.02,
+// 1.02; 3,198 of 772 1.05, 1.05; 528 of 4,000 1.10, 1.13.
+static bool oz_wide(const gsp2_plan* h) {
+  const int64_t tiles = (int64_t)h->tc_tiles.size();
+  int64_t k = 0;
+  for (const Tile& t : h->tc_tiles) k += h->parts[t.part].s;
+  return tiles > 3 * (int64_t)h->num_sms && k >= 512 * tiles;
+}
+
 // Arguments of the emulated FP64 step common to all its launches of a call.
 static OzStepArgs oz_args(gsp2_plan* h, const StepCtl& ctl) {
   const WsLayout& L = h->L;
@@ -1082,7 +1095,8 @@ static OzStepArgs oz_args(gsp2_plan* h, const StepCtl& ctl) {
   a.ctl = ctl;
   a.tile_ctr = h->opt.tile_claim ? (uint32_t*)(w + L.tile_ctr) : nullptr;
   a.halves = h->halves ? 1 : 0;
-  a.pieces = oz_pieces(a.ntiles * (h->split_on ? 2 : 1), h->num_sms);
+  a.wide = oz_wide(h) ? 1 : 0;
+  a.pieces = a.wide ? 1 : oz_pieces(a.ntiles * (h->split_on ? 2 : 1), h->num_sms);
   if (h->split_on) {
     a.split = 1;
     a.split_acc = (long long*)(w + L.split_acc);

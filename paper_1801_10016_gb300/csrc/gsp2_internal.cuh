@@ -158,7 +158,8 @@ struct GraphArgs {
 constexpr int OZ_SLICES = 5;  // digits per entry (11, 8, 11, 8 and 11 bits)
 constexpr int OZ_LOW = 2;     // digits the second pass of a tile multiplies
 constexpr int OZ_MAX_GRID = 256;  // CTAs of the emulated step (one 128x128 int64 scratch each)
-constexpr int OZ_BK = 32;         // K per pipeline stage of the emulated step (64-byte rows)
+constexpr int OZ_BK = 32;         // K per slice of the emulated step, narrow form (64-byte rows)
+constexpr int OZ_BK_WIDE = 64;    // the same, wide form (128-byte rows)
 
 struct OzSlices {
   uint16_t* s[OZ_SLICES];  // FP16 digit arenas (same element indexing as the arenas)
@@ -174,11 +175,11 @@ struct OzStepArgs {
   const PartDesc* parts;
   const Tile* tiles;   // 128x128 upper tiles
   int ntiles;
-  const void* maps;    // per digit buffer (OZ_SLICES x nparts maps apart): CUtensorMap[2][nparts], K-major
-                       // boxes of all OZ_SLICES digits ([0]) or the first OZ_LOW ([1]) of a tile slice
-  const void* maps_mn; // the same with MN-major boxes (each tile 128 rows x OZ_BK columns as two 64-row atoms,
-                       // 128-byte swizzle)
-  const void* maps_b;    // adjoint: the same two K-major map arrays over the digits of Xbar / 2^sig
+  const void* maps;    // per digit buffer (OZ_SLICES x nparts maps apart): CUtensorMap[3][nparts], K-major
+                       // boxes of one digit of a wide tile slice ([0]), of all OZ_SLICES ([1]) or the
+                       // first OZ_LOW ([2]) digits of a narrow one
+  const void* maps_mn; // the same with MN-major boxes (each tile 128 rows x K columns as two 64-row atoms)
+  const void* maps_b;    // adjoint: the same K-major maps over the digits of Xbar / 2^sig
   const void* maps_mn_b; // the same, MN-major
   int32_t* sig;          // adjoint: per-part scale exponent of Xbar's digits (OZ_SIG_NONFINITE: NaN),
                          // replaced by the new Xbar's scale by the last block of the step
@@ -198,7 +199,8 @@ struct OzStepArgs {
   // its 64-bit partial tile to split_acc[2 t + h] and the second of the two to finish
   // (split_cnt[t], left at zero) adds both and forms the tile (X_new, digits, traces)
   int split;
-  int pieces;            // column pieces of a tile, each an item of its own (1 or 2)
+  int pieces;            // column pieces of a tile, each an item of its own (1 or 2; wide: 1)
+  int wide;              // K slices of OZ_BK_WIDE in a ring of single digit tiles, not of OZ_BK in units of five
   int halves;            // the plan's items may be split: unsplit ones drain at the same boundary
   long long* split_acc;  // [2 ntiles][128 x 128], indexed by item code 2 t + h
   uint32_t* split_cnt;   // [ntiles]

@@ -42,6 +42,8 @@
 // order 2^-47 2^sig.
 #include <cuda.h>
 
+#include <type_traits>
+
 #include "gsp2_internal.cuh"
 #include "gsp2_kernels.h"
 #include "tc_ptx.cuh"
@@ -336,31 +338,42 @@ __global__ void __launch_bounds__(256) oz_digits_kernel(const PartDesc* __restri
 // The 15 digit products of a tile need six FP32 accumulators of 128 TMEM columns, more than
 // the 512 columns of an SM, so a tile takes two passes over K: first the 12 products other
 // than (0,0), (0,1) and (1,0) (all five digits, columns 0-511), then those three (digits 0
-// and 1, columns 0-255).  A unit of the TMA ring holds one operand (rows I or rows J) of the
-// pass: one K = OZ_BK slice of all five digits, or in the second pass two slices of two
-// digits; diagonal tiles load rows I only.  Each distinct digit tile is loaded once per slice
-// and feeds all its products (one K = 16 FP16 MMA each).  Five units of 40 KB keep two and a
-// half slices in flight.  The epilogue warps turn the first pass's sums into 64-bit fixed
-// point (2^-56) and park them in TMEM columns 256-511, which the second pass leaves alone;
-// after it they add its sums, hand all 512 columns back and keep the tile's sums in a
-// per-CTA scratch tile (L2-resident) for the final pass, which forms X_new = Y or 2X - Y,
+// and 1, columns 0-255).  Each distinct digit tile is loaded once per K slice and pass and feeds all its
+// products (one K = 16 FP16 MMA each); diagonal tiles load rows I only.  The K slices come in one of
+// two forms, chosen by the plan (oz_wide in gsp2_api.cu):
+//   narrow, K = 32: a unit of the TMA ring holds one operand (rows I or rows J) of the pass, one slice
+//   of all five digits in one request, or in the second pass two slices of two digits.  Five units of
+//   40 KB keep two and a half slices in flight.
+//   wide, K = 64: the ring holds 13 single digit tiles of 16 KB.  A K-major tile then has 128-byte
+//   rows, which L2 serves in 0.77 of the time of 64-byte ones (the loads of a step alone, n = 30000: 1.17
+//   and 0.90 ms), a tile is given back as soon as its last product is issued, and the MMA warp waits
+//   for the tiles in two groups (a wait per tile left the tensor pipe idle: 2.16 ms a step instead of
+//   1.59).  Padding of K beyond the next multiple of 16 is not multiplied.
+// The epilogue warps turn the passes' sums into 64-bit fixed point (2^-56): narrow, those of the first
+// pass are parked in TMEM columns 256-511, which the second pass leaves alone, and the tile's in a
+// per-CTA scratch tile (L2-resident); wide, all stay in registers, so that a pass's columns are
+// handed back after nothing but their own reads.  The final pass forms X_new = Y or 2X - Y,
 // writes the master copy (64-bit fixed point) and the digits of X_new (into the other
 // digit buffer) at (I, J) and mirrored at (J, I) (diagonal tiles from their upper
 // triangle), and adds the core traces, while the MMAs of the next tile's first pass run.  The new
 // iterate is written with evict-first stores: the next step reads it after this launch,
 // and keeping it out of L2 leaves room for the digit panels the running tiles share.  The last block
-// runs the step bookkeeping.  K beyond OZ_CHUNK slices is taken in rounds of both passes, the
-// later ones adding to the scratch tile, so that the sums stay exact (see the top).
+// runs the step bookkeeping.  K beyond 2048 is taken in rounds of both passes, so that the sums stay
+// exact (see the top).  n = 30000 (256 parts), per step: narrow 1.69, wide 1.59 ms; the MMAs at the
+// measured 16-bit peak take 1.15, without loads or epilogue 1.29, with loads 1.32, with drains 1.43.
 //
-// 20 warps: warps 0 and 2 lane 0 TMA (rows I and rows J: one thread's work per unit would hold
+// 20 warps: warps 0 and 2 TMA (rows I and rows J: one warp's work per tile would hold
 // the ring back), warp 1 TMEM owner and MMA issuer, warps 4..19 epilogue
 // (warp w: TMEM lanes 32 (w % 4) .. + 31, columns 32 ((w - 4) / 4) .. + 31 of each group,
 // in two chunks of 16), sized so that four epilogue warps per scheduler hide latency.
-constexpr int OZ_UNITS = 5;                                      // operand units of the TMA ring
-constexpr uint32_t OZ_DTILE = 128u * OZ_BK * 2u;                 // one digit tile: 128 rows x 64 B
-constexpr uint32_t OZ_UNIT_B = OZ_SLICES * OZ_DTILE;             // one operand's digit tiles
+constexpr int OZ_UNITS = 5;                                      // narrow: operand units of the TMA ring
+constexpr uint32_t OZ_UNIT_B = OZ_SLICES * 128u * OZ_BK * 2u;    // one operand's digit tiles
 constexpr int OZ_LOW_SUB = 2;                                    // K slices per unit of the second pass
-constexpr int OZ_CHUNK = 2048 / OZ_BK;                           // K slices per round of both passes
+constexpr int OZ_TILES = 13;                                     // wide: digit tiles in the TMA ring
+constexpr int OZ_GROUPS = 8;  // wide: barriers of tile groups per operand, more than the ring holds (2 tiles or more)
+constexpr int OZ_HEAD = 3;    // wide: steps of the first pass whose tiles come as its first group
+constexpr uint32_t OZ_RING_B = OZ_TILES * 128u * OZ_BK_WIDE * 2u;
+constexpr int OZ_BARS = 2 * OZ_GROUPS + OZ_TILES + 4 + 1;        // mbarriers of the ring (padded to 16 bytes)
 constexpr int OZ_EPI_WARPS = 16;                                 // 4 per TMEM lane quarter
 constexpr int OZ_THREADS = 32 * (4 + OZ_EPI_WARPS);
 constexpr int OZ_RING = 4;  // dynamic schedule: tiles claimed ahead of the MMA and epilogue warps
@@ -371,10 +384,11 @@ struct alignas(16) OzItem {
   int32_t part, s, c, ld;
   int32_t piece, pad[3];
 };
-constexpr int OZ_SMEM = OZ_UNITS * (int)OZ_UNIT_B + 1024 + 8 * (2 * OZ_UNITS + 4) + 16 + 16 * 128 +
+constexpr int OZ_SMEM = (int)OZ_RING_B + 1024 + 8 * OZ_BARS + 16 + 16 * 128 +
                         8 * 2 * OZ_RING + (int)sizeof(OzItem) * OZ_RING;
+static_assert(OZ_UNITS * OZ_UNIT_B <= OZ_RING_B && OZ_UNITS <= OZ_GROUPS, "the narrow ring within the wide one's space");
 static_assert(OZ_LOW_SUB * OZ_LOW <= OZ_SLICES, "a unit holds the second pass's slices");
-static_assert((2 * OZ_UNITS + 4) % 2 == 0, "alignment of the reduction slots and items");
+static_assert(OZ_BARS % 2 == 0, "alignment of the reduction slots and items");
 static_assert(OZ_SMEM <= 232448, "shared memory of the emulated step");
 
 // Columns of tile column block tj that an MMA must cover: those inside the part, rounded up
@@ -386,21 +400,21 @@ __host__ __device__ constexpr int oz_tile_cols(int s, int tj) {
 // Accumulators (first TMEM column): of the first pass, (1,3), (0,4) and (2,2) in columns
 // 0-127, (1,2) and (0,3) in 128-255, (0,2) in 256-383 and (1,1) in 384-511; of the second,
 // (0,0) in 0-127 and (0,1) in 128-255.  The second pass can start once the columns 0-255 are
-// read, and columns 256-511 then hold the first pass's 64-bit sums (low and high words).
+// read, and columns 256-511 then hold the first pass's 64-bit sums (narrow: low and high words).
 constexpr uint32_t OZ_PARK_LO = 256, OZ_PARK_HI = 384;
 __host__ __device__ constexpr bool oz_low_pass(int a, int b) { return a + b <= 1; }
 __host__ __device__ constexpr uint32_t oz_col(int a, int b) {
   return a + b == 0 || a + b == 4 ? 0u : (a + b == 2 ? (a == 1 ? 384u : 256u) : 128u);
 }
-// products of A digit q in a pass: (q, b) for lo <= b < hi
+// Narrow slices: products of A digit q in a pass: (q, b) for lo <= b < hi
 template <bool LOW>
-__host__ __device__ constexpr int oz_b_lo(int q) { return LOW ? 0 : (q < 2 ? 2 - q : 0); }
+__host__ __device__ constexpr int oz_q_lo(int q) { return LOW ? 0 : (q < 2 ? 2 - q : 0); }
 template <bool LOW>
-__host__ __device__ constexpr int oz_b_hi(int q) { return (LOW ? OZ_LOW : OZ_SLICES) - q; }
+__host__ __device__ constexpr int oz_q_hi(int q) { return (LOW ? OZ_LOW : OZ_SLICES) - q; }
 
 // Descriptors of one K slice: lower words at the slice's first digit tile, upper words,
 // advance of a K = 16 step (16-byte units) and instruction descriptor.
-struct OzOperands {
+struct OzNarrow {
   uint32_t alo, ahi, blo, bhi, adv_a, adv_b, idesc;
 };
 
@@ -412,12 +426,12 @@ struct OzOperands {
 // instead of once per product (the MMAs' shared-memory reads, A and B, set the pace of the
 // tensor pipe otherwise).
 template <bool LOW, int KK>
-__device__ __forceinline__ void oz_issue(uint32_t tmem, const OzOperands& o, bool first_k) {
-  constexpr uint32_t step = OZ_DTILE >> 4;
+__device__ __forceinline__ void oz_issue_narrow(uint32_t tmem, const OzNarrow& o, bool first_k) {
+  constexpr uint32_t step = (128u * OZ_BK * 2u) >> 4;
   const uint32_t alo = o.alo + (KK ? KK * o.adv_a : 0u), blo = o.blo + (KK ? KK * o.adv_b : 0u);
 #pragma unroll
   for (int q = 0; q < (LOW ? OZ_LOW : OZ_SLICES); ++q) {
-    const int b0 = oz_b_lo<LOW>(q), b1 = oz_b_hi<LOW>(q);
+    const int b0 = oz_q_lo<LOW>(q), b1 = oz_q_hi<LOW>(q);
 #pragma unroll
     for (int b = b0; b < b1; ++b) {
       const int op = (b1 - b0 == 1) ? 0 : (b == b0 ? 1 : (b == b1 - 1 ? 3 : 2));
@@ -425,6 +439,54 @@ __device__ __forceinline__ void oz_issue(uint32_t tmem, const OzOperands& o, boo
       const bool opens = q == 0 || (q == 1 && b == 1);
       mma_f16_lo(op, tmem + oz_col(q, b), alo + (uint32_t)q * step, o.ahi, blo + (uint32_t)b * step, o.bhi, o.idesc,
                  (KK == 0 && opens && first_k) ? 0u : 1u);
+    }
+  }
+}
+
+// Wide slices: the digit tiles of a K slice come and are used in this order: in step i of a pass over T digits
+// digit T - 1 - i of rows I, then digit i of rows J, and the products (T - 1 - i, b), lo <= b <= i, of
+// the pass follow.  A tile of rows I is then done, and tiles of rows J not long after they came, so
+// that a ring of single tiles refills while the slice is still being multiplied.
+template <bool LOW>
+__host__ __device__ constexpr int oz_digits() { return LOW ? OZ_LOW : OZ_SLICES; }
+template <bool LOW>
+__host__ __device__ constexpr int oz_b_lo(int i) {
+  const int q = oz_digits<LOW>() - 1 - i;
+  return LOW ? 0 : (q < 2 ? 2 - q : 0);
+}
+// the step after which digit b of rows J is done
+template <bool LOW>
+__host__ __device__ constexpr int oz_b_last(int b) {
+  int last = 0;
+  for (int i = 0; i < oz_digits<LOW>(); ++i)
+    if (oz_b_lo<LOW>(i) <= b && b <= i) last = i;
+  return last;
+}
+
+// Descriptors of one K slice: lower words of the digit tiles' descriptors, upper words, advance of a
+// K = 16 step (16-byte units), instruction descriptor and K = 16 steps.
+struct OzWide {
+  uint32_t a[OZ_SLICES], b[OZ_SLICES], ahi, bhi, adv_a, adv_b, idesc;
+  int steps;
+};
+
+// The MMAs of step I of one slice of a pass, K = 16 steps [K0, K1), fully unrolled.  The products of an
+// A digit follow one another and share their A operand through the collector buffer, so each A digit
+// tile is read from shared memory once per K = 16 step instead of once per product (the MMAs'
+// shared-memory reads, A and B, set the pace of the tensor pipe otherwise).
+template <bool LOW, int I, int K0, int K1>
+__device__ __forceinline__ void oz_issue_wide(uint32_t tmem, const OzWide& o, bool first) {
+  constexpr int q = oz_digits<LOW>() - 1 - I, b0 = oz_b_lo<LOW>(I);
+#pragma unroll
+  for (int kk = K0; kk < K1; ++kk) {
+    if (kk >= o.steps) break;
+#pragma unroll
+    for (int b = b0; b <= I; ++b) {
+      const int op = I == b0 ? 0 : (b == b0 ? 1 : (b == I ? 3 : 2));
+      // the first product into each accumulator: (1,0), (0,0); (4,0), (3,0), (2,0), (1,1)
+      const bool opens = b == 0 || (!LOW && q == 1 && b == 1);
+      mma_f16_lo(op, tmem + oz_col(q, b), o.a[q] + (uint32_t)kk * o.adv_a, o.ahi, o.b[b] + (uint32_t)kk * o.adv_b, o.bhi,
+                 o.idesc, (kk == 0 && opens && first) ? 0u : 1u);
     }
   }
 }
@@ -579,9 +641,12 @@ __device__ __forceinline__ void store_digits_if(bool on, uint16_t* d, size_t dst
       : "memory");
 }
 
-template <bool ADJ>
+template <bool ADJ, bool WIDE>
 __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
   constexpr int T = OZ_SLICES;
+  constexpr int BK = WIDE ? OZ_BK_WIDE : OZ_BK;  // K per slice
+  constexpr int CHUNK = 2048 / BK;               // K slices per round of both passes
+  constexpr uint32_t DTILE = 128u * BK * 2u;     // one digit tile: 128 rows x 64 or 128 B
   // instruction descriptor without N (bits 17..22, N / 8): FP32 accumulate, FP16 A and B, M = 128
   constexpr uint32_t IDESC = (1u << 4) | ((128u >> 4) << 24);
 
@@ -591,11 +656,11 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t base = (raw + 1023u) & ~1023u;
   uint8_t* sb = smem_raw + (base - raw);
-  const uint32_t bars = base + OZ_UNITS * OZ_UNIT_B;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(sb + OZ_UNITS * OZ_UNIT_B + 8 * (2 * OZ_UNITS + 4));
+  const uint32_t bars = base + OZ_RING_B;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(sb + OZ_RING_B + 8 * OZ_BARS);
   int* s_err = reinterpret_cast<int*>(tmem_slot + 1);
   int* s_half = reinterpret_cast<int*>(tmem_slot + 2);  // split K: halves of the tile done before
-  longlong2* red = reinterpret_cast<longlong2*>(sb + OZ_UNITS * OZ_UNIT_B + 8 * (2 * OZ_UNITS + 4) + 16);
+  longlong2* red = reinterpret_cast<longlong2*>(sb + OZ_RING_B + 8 * OZ_BARS + 16);
   // warp 0's producer takes each next tile (claimed from a counter in global memory, or dealt)
   // and passes it on with its part through a ring (full: taken; empty: read by the other
   // producer, the MMA thread and every epilogue warp)
@@ -603,12 +668,13 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
   OzItem* s_items = reinterpret_cast<OzItem*>(reinterpret_cast<uint8_t*>(red + 128) + 8 * 2 * OZ_RING);
   auto item_full = [&](int q) { return ring_bars + 8u * q; };
   auto item_empty = [&](int q) { return ring_bars + 8u * (OZ_RING + q); };
-  auto full = [&](int s) { return bars + 8u * s; };
-  auto empty = [&](int s) { return bars + 8u * (OZ_UNITS + s); };
+  auto full = [&](int op, uint32_t g) { return bars + 8u * (op * OZ_GROUPS + g % OZ_GROUPS); };  // rows I 0, rows J 1
+  auto empty = [&](int s) { return bars + 8u * (2 * OZ_GROUPS + s); };
   // accumulator barriers: [0] first pass, [1] second
-  auto afull = [&](int pass) { return bars + 8u * (2 * OZ_UNITS + pass); };
-  auto aempty = [&](int pass) { return bars + 8u * (2 * OZ_UNITS + 2 + pass); };
-  auto unit = [&](int s) { return base + (uint32_t)s * OZ_UNIT_B; };
+  auto afull = [&](int pass) { return bars + 8u * (2 * OZ_GROUPS + OZ_TILES + pass); };
+  auto aempty = [&](int pass) { return bars + 8u * (2 * OZ_GROUPS + OZ_TILES + 2 + pass); };
+  auto tile_addr = [&](uint32_t s) { return base + s * DTILE; };                       // wide
+  auto unit = [&](int s) { return base + (uint32_t)s * OZ_UNIT_B; };                   // narrow
   int32_t* abort_flag = &a.ctl.st->timeout;
   const int warp = __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0), lane = threadIdx.x & 31;
   // work items: the upper tiles, or (split K) each tile's two K halves
@@ -623,35 +689,32 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
   // K slices [x, y) of an item of a part of size sz: all of them (the adjoint's first ns slices
   // multiply Xbar by X, the rest X by Xbar) or one half, up to or from slice z
   auto slices = [&](int sz, int half) {
-    const int ns = (sz + OZ_BK - 1) / OZ_BK, all = ADJ ? 2 * ns : ns, mid = ADJ ? ns : (ns + 1) / 2;
+    const int ns = (sz + BK - 1) / BK, all = ADJ ? 2 * ns : ns, mid = ADJ ? ns : (ns + 1) / 2;
     return make_int3(half == 1 ? mid : 0, half == 0 ? mid : all, mid);
   };
   // end of the round of both passes that starts at slice c0: rounds of equal length of at most
-  // OZ_CHUNK slices, and (plans whose items may be split) never across the halves, so that a
+  // CHUNK slices, and (plans whose items may be split) never across the halves, so that a
   // tile's sums are rounded alike whether one item forms it or two
   auto round_end = [&](int c0, int3 kr) {
     const int left = (a.halves && c0 < kr.z ? min(kr.z, kr.y) : kr.y) - c0;
-    const int rounds = (left + OZ_CHUNK - 1) / OZ_CHUNK;
+    const int rounds = (left + CHUNK - 1) / CHUNK;
     return c0 + (left + rounds - 1) / rounds;
   };
   // items claimed at run time (forward, tail and reverse steps; the list order) or dealt in turn
   // (the rebuilt iterates, which may run beside reverse steps and have no last block)
   const bool dyn = a.tile_ctr != nullptr && !rec;
 
-  if (threadIdx.x == 0) {
-    for (int s = 0; s < OZ_UNITS; ++s) {
-      mbar_init(full(s), 1);
-      mbar_init(empty(s), 1);
+  if (warp == 0) {
+    for (int q = lane; q < 2 * OZ_GROUPS + OZ_TILES; q += 32) mbar_init(bars + 8u * q, 1);
+    if (lane < 2) {
+      mbar_init(afull(lane), 1);
+      mbar_init(aempty(lane), OZ_EPI_WARPS);
     }
-    for (int q = 0; q < 2; ++q) {
-      mbar_init(afull(q), 1);
-      mbar_init(aempty(q), OZ_EPI_WARPS);
+    if (lane < OZ_RING) {
+      mbar_init(item_full(lane), 1);
+      mbar_init(item_empty(lane), 2 + OZ_EPI_WARPS);
     }
-    for (int q = 0; q < OZ_RING; ++q) {
-      mbar_init(item_full(q), 1);
-      mbar_init(item_empty(q), 2 + OZ_EPI_WARPS);
-    }
-    *s_err = 0;
+    if (lane == 0) *s_err = 0;
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
   }
   if (warp == 1) {
@@ -663,6 +726,29 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
   tc_fence_after();
   const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
 
+  // the first item's tables, which no launch writes, before the launch before this one is done
+  OzItem first;
+  auto read_item = [&](int it) {
+    OzItem w;
+    w.piece = it % pieces;
+    w.code = split ? a.split_items[it / pieces] : it / pieces;
+    const Tile t = a.tiles[split ? w.code >> 1 : w.code];
+    const PartDesc p = a.parts[t.part];
+    w.ti = t.ti;
+    w.tj = t.tj;
+    w.slot = t.slot;
+    w.part = t.part;
+    w.off = p.off;
+    w.soff = p.soff;
+    w.s = p.s;
+    w.c = p.c;
+    w.ld = p.ld;
+    return w;
+  };
+  if (threadIdx.x == 0) {
+    first.code = -1;
+    if ((int)blockIdx.x < nitems) first = read_item(blockIdx.x);
+  }
   pdl_wait();  // everything below reads what the launch before wrote
   int step = a.step;
   bool run;
@@ -698,8 +784,9 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
     // Like the issuing warp below, the whole warp walks the units with warp-uniform values and
     // one elected lane issues the loads.
     const int op = warp >> 1;      // 0: rows I, 1: rows J
-    uint32_t su = 0, ph = 0;       // next unit of the ring and its phase
-    uint32_t used = 0, phase = 0;  // units this warp has filled, and the phases of the last fills
+    uint32_t su = 0, ph = 0;       // next tile or unit of the ring and its phase
+    uint32_t grp = 0;              // wide: groups of tiles this warp has begun
+    uint32_t used = 0, phase = 0;  // narrow: units this warp has filled, and the phases of the last fills
     bool bad = false;
     // dynamic: the first item is blockIdx.x, the next ones gridDim.x + the counter's count,
     // each claimed one item ahead so that the atomic's latency hides behind an item's loads
@@ -718,22 +805,10 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
             it = nxt;
             if (it < nitems) nxt = (int)gridDim.x + (int)atomicAdd(a.tile_ctr, 1u);
           }
-          OzItem w;
-          w.code = -1;
-          if (it < nitems) {
-            w.piece = it % pieces;
-            w.code = split ? a.split_items[it / pieces] : it / pieces;
-            const Tile t = a.tiles[split ? w.code >> 1 : w.code];
-            const PartDesc p = a.parts[t.part];
-            w.ti = t.ti;
-            w.tj = t.tj;
-            w.slot = t.slot;
-            w.part = t.part;
-            w.off = p.off;
-            w.soff = p.soff;
-            w.s = p.s;
-            w.c = p.c;
-            w.ld = p.ld;
+          OzItem w = first;
+          if (v > 0) {
+            w.code = -1;
+            if (it < nitems) w = read_item(it);
           }
           s_items[q] = w;
           mbar_arrive(item_full(q));
@@ -756,85 +831,150 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
       const int half = split ? w.code & 1 : -1;
       const bool dg = !ADJ && w.ti == w.tj;  // X X on a diagonal tile: B is A
       const int blk = op == 0 ? w.ti : w.tj;
-      const int ns = (w.s + OZ_BK - 1) / OZ_BK;
+      const int ns = (w.s + BK - 1) / BK;
       const int3 kr = slices(w.s, half);
-      // the next unit of this thread; false if the wait gave up
-      auto acquire = [&](uint32_t bytes, uint32_t& u) {
-        if (op == 1 && ++su == OZ_UNITS) {
-          su = 0;
-          ph ^= 1;
+      if constexpr (WIDE) {
+        // ring places of this pass over: `by` tiles on
+        auto advance = [&](uint32_t by) {
+          su += by;
+          if (su >= OZ_TILES) {
+            su -= OZ_TILES;
+            ph ^= 1;
+          }
+        };
+        // The tiles of one slice of a pass over T digits: rows I from the last digit down, rows J from
+        // the first up, in turn; on a diagonal tile rows I alone.  The MMA warp waits for them in groups
+        // (one barrier each): three and two of the five digits, both of the second pass's, or all of a
+        // diagonal tile.  K-major from columns `blk` of the tiles on or above the diagonal (slice
+        // block <= blk), else MN-major from rows `blk` of the tile (blk, slice).  The adjoint's first
+        // ns slices take Xbar for rows I and X for rows J, the rest X for rows I and Xbar for rows J
+        auto slice = [&](int ks, int T) {
+          const bool h2 = ADJ && ks >= ns;
+          const bool xb = ADJ && (op == 0) != h2;
+          const int k0 = (h2 ? ks - ns : ks) * BK;
+          const bool kmajor = k0 / 128 <= blk;
+          const CUtensorMap* const map =
+              (kmajor ? (xb ? maps_b : maps) : (xb ? maps_mn_b : maps_mn)) + w.part;
+          // which of the slice's places are free already (a lane each)
+          uint32_t at = su + (uint32_t)(dg ? lane : 2 * lane + op), fr = ph;
+          if (at >= OZ_TILES) {
+            at -= OZ_TILES;
+            fr ^= 1u;
+          }
+          const uint32_t ready = __ballot_sync(0xffffffffu, lane < T && mbar_test(empty(at), fr ^ 1u));
+          for (int i = 0; i < T; ++i) {
+            if (op == 1) advance(1);
+            if (!(ready >> i & 1u) && !wait(empty(su), ph ^ 1u)) {
+              bad = true;
+              return;
+            }
+            const bool head = i == 0 || (i == OZ_HEAD && !dg);
+            grp += head;
+            const uint32_t bar = full(op, grp - 1u);
+            const int dig = op == 0 ? T - 1 - i : i;
+            if (elect_one()) {
+              if (head) mbar_expect_tx(bar, DTILE * (uint32_t)(T == OZ_LOW || dg ? T : (i == 0 ? OZ_HEAD : T - OZ_HEAD)));
+              if (kmajor) tma_load_3d(tile_addr(su), map, k0, blk * 128, dig, bar);
+              else tma_load_4d(tile_addr(su), map, 0, k0, 2 * blk, dig, bar);
+            }
+            advance(op == 0 && !dg ? 2 : 1);
+          }
+        };
+        if (op == 1 && dg) {  // rows I only: this warp's place in the ring moves past them
+          const uint32_t by = su + (uint32_t)((kr.y - kr.x) * (OZ_SLICES + OZ_LOW));
+          ph ^= (by / OZ_TILES) & 1u;
+          su = by % OZ_TILES;
+          continue;
         }
-        u = su;
-        if (!wait(empty(u), ph ^ 1u)) return false;
-        if (elect_one()) mbar_expect_tx(full(u), bytes);
-        used |= 1u << u;
-        phase = (phase & ~(1u << u)) | (ph << u);
-        if (++su == OZ_UNITS) {
-          su = 0;
-          ph ^= 1;
-        }
-        if (op == 0 && !dg && ++su == OZ_UNITS) {
-          su = 0;
-          ph ^= 1;
-        }
-        return true;
-      };
-      // one request brings a slice's digit tiles: K-major from columns `blk` of the tiles on or
-      // above the diagonal (slice block <= blk), else MN-major from rows `blk` of the tile (blk,
-      // slice).  The adjoint's first ns slices take Xbar for rows I and X for rows J, the rest
-      // X for rows I and Xbar for rows J
-      auto load = [&](uint32_t dst, uint32_t bar, int ks, size_t at) {
-        const bool h2 = ADJ && ks >= ns;
-        const bool xb = ADJ && (op == 0) != h2;
-        const int k0 = (h2 ? ks - ns : ks) * OZ_BK;
-        if (elect_one()) {
-          if (k0 / 128 <= blk) tma_load_3d(dst, (xb ? maps_b : maps) + at, k0, blk * 128, 0, bar);
-          else tma_load_4d(dst, (xb ? maps_mn_b : maps_mn) + at, 0, k0, 2 * blk, 0, bar);  // 64-row atoms x digits
-        }
-      };
-      if (op == 1 && dg) {  // rows I only: this thread's place in the ring moves past them
-        for (int c0 = kr.x, c1; c0 < kr.y; c0 = c1) {
+        for (int c0 = kr.x, c1; c0 < kr.y && !bad; c0 = c1) {
           c1 = round_end(c0, kr);
-          su += (uint32_t)(c1 - c0 + (c1 - c0 + OZ_LOW_SUB - 1) / OZ_LOW_SUB);
+          for (int kb = c0; kb < c1 && !bad; ++kb) slice(kb, OZ_SLICES);
+          for (int kb = c0; kb < c1 && !bad; ++kb) slice(kb, OZ_LOW);
         }
-        ph ^= (su / OZ_UNITS) & 1u;
-        su %= OZ_UNITS;
-        continue;
-      }
-      for (int c0 = kr.x, c1; c0 < kr.y && !bad; c0 = c1) {
-        c1 = round_end(c0, kr);
-        uint32_t u;
-        for (int kb = c0; kb < c1; ++kb) {
-          if (!acquire(T * OZ_DTILE, u)) {
-            bad = true;
-            break;
+      } else {
+        // the next unit of this thread; false if the wait gave up
+        auto acquire = [&](uint32_t bytes, uint32_t& u) {
+          if (op == 1 && ++su == OZ_UNITS) {
+            su = 0;
+            ph ^= 1;
           }
-          load(unit(u), full(u), kb, (size_t)w.part);
+          u = su;
+          if (!wait(empty(u), ph ^ 1u)) return false;
+          if (elect_one()) mbar_expect_tx(full(0, u), bytes);
+          used |= 1u << u;
+          phase = (phase & ~(1u << u)) | (ph << u);
+          if (++su == OZ_UNITS) {
+            su = 0;
+            ph ^= 1;
+          }
+          if (op == 0 && !dg && ++su == OZ_UNITS) {
+            su = 0;
+            ph ^= 1;
+          }
+          return true;
+        };
+        // one request brings a slice's digit tiles: K-major from columns `blk` of the tiles on or
+        // above the diagonal (slice block <= blk), else MN-major from rows `blk` of the tile (blk,
+        // slice).  The adjoint's first ns slices take Xbar for rows I and X for rows J, the rest
+        // X for rows I and Xbar for rows J
+        auto load = [&](uint32_t dst, uint32_t bar, int ks, size_t at) {
+          const bool h2 = ADJ && ks >= ns;
+          const bool xb = ADJ && (op == 0) != h2;
+          const int k0 = (h2 ? ks - ns : ks) * BK;
+          if (elect_one()) {
+            if (k0 / 128 <= blk) tma_load_3d(dst, (xb ? maps_b : maps) + at, k0, blk * 128, 0, bar);
+            else tma_load_4d(dst, (xb ? maps_mn_b : maps_mn) + at, 0, k0, 2 * blk, 0, bar);  // 64-row atoms x digits
+          }
+        };
+        if (op == 1 && dg) {  // rows I only: this thread's place in the ring moves past them
+          for (int c0 = kr.x, c1; c0 < kr.y; c0 = c1) {
+            c1 = round_end(c0, kr);
+            su += (uint32_t)(c1 - c0 + (c1 - c0 + OZ_LOW_SUB - 1) / OZ_LOW_SUB);
+          }
+          ph ^= (su / OZ_UNITS) & 1u;
+          su %= OZ_UNITS;
+          continue;
         }
-        for (int kb = c0; kb < c1 && !bad; kb += OZ_LOW_SUB) {
-          const int m = min(OZ_LOW_SUB, c1 - kb);
-          if (!acquire((uint32_t)(m * OZ_LOW) * OZ_DTILE, u)) {
-            bad = true;
-            break;
+        for (int c0 = kr.x, c1; c0 < kr.y && !bad; c0 = c1) {
+          c1 = round_end(c0, kr);
+          uint32_t u;
+          for (int kb = c0; kb < c1; ++kb) {
+            if (!acquire(T * DTILE, u)) {
+              bad = true;
+              break;
+            }
+            load(unit(u), full(0, u), kb, (size_t)a.nparts + w.part);
           }
-          for (int x = 0; x < m; ++x)
-            load(unit(u) + (uint32_t)(x * OZ_LOW) * OZ_DTILE, full(u), kb + x, (size_t)a.nparts + w.part);
+          for (int kb = c0; kb < c1 && !bad; kb += OZ_LOW_SUB) {
+            const int m = min(OZ_LOW_SUB, c1 - kb);
+            if (!acquire((uint32_t)(m * OZ_LOW) * DTILE, u)) {
+              bad = true;
+              break;
+            }
+            for (int x = 0; x < m; ++x)
+              load(unit(u) + (uint32_t)(x * OZ_LOW) * DTILE, full(0, u), kb + x, (size_t)2 * a.nparts + w.part);
+          }
         }
       }
     }
     if (bad) {
       *s_err = 1;
-      for (uint32_t u = 0; u < (uint32_t)OZ_UNITS; ++u)
-        if (used >> u & 1u) (void)mbar_wait_own(full(u), phase >> u & 1u);
+      // loads in flight still write shared memory: wait for them on this warp's own limit
+      if (WIDE) {
+        for (uint32_t g = grp > OZ_GROUPS - 1 ? grp - (OZ_GROUPS - 1) : 0; g < grp; ++g)
+          (void)mbar_wait_own(full(op, g), (g / OZ_GROUPS) & 1);
+      } else {
+        for (uint32_t u = 0; u < (uint32_t)OZ_UNITS; ++u)
+          if (used >> u & 1u) (void)mbar_wait_own(full(0, u), phase >> u & 1u);
+      }
     }
   } else if (warp == 1) {
     // The whole warp walks the slices with warp-uniform values (the item's fields through a
     // shuffle), so that descriptors are formed in uniform registers, and one elected lane
-    // issues.  The issuing warp's own work between two slices (barrier tests, descriptors, commits) would
-    // leave the tensor pipe idle: the descriptors of the next unit are formed between the two K = 16
-    // steps of a slice, while the first step's MMAs run.
-    uint32_t su = 0, ph = 0;  // next unit of the ring and its phase
-    int last = -1;            // last unit released by a commit
+    // issues.  A step's MMAs (4 to 12) keep the tensor pipe busy while the next step's tiles are waited for.
+    uint32_t su = 0, ph = 0;  // next tile or unit of the ring and its phase
+    uint32_t ga = 0, gb = 0;  // wide: groups of tiles of rows I and rows J taken
+    int last = -1;            // last tile or unit released by a commit
     uint32_t lastph = 0;
     int v = 0, r = 0;  // items taken, rounds of both passes done by this CTA
     bool bad = false;
@@ -854,116 +994,235 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
       if (ncols == 0) continue;
       const int half = split ? code & 1 : -1;
       const bool dg = !ADJ && ti == tj;
-      const int ns = (sz + OZ_BK - 1) / OZ_BK;
+      const int ns = (sz + BK - 1) / BK;
       const int3 kr = slices(sz, half);
       const uint32_t idesc0 = IDESC | ((uint32_t)(ncols >> 3) << 17);
-      // rows J of a piece start 64 rows into each digit tile: 64 B each K-major, one atom MN-major
-      const uint32_t poff = (uint32_t)piece * ((64u * OZ_BK * 2u) >> 4);
-      // operands of slice ks, tile `off` of the units sa (rows I) and sb (rows J): those right of
-      // the tile's own block came in MN-major (transpose bits 15 / 16); a K = 16 step advances
-      // 32 B in a K-major row, 2 KB (16 K values) in an MN-major tile
-      const uint64_t dk = smem_desc_sw<2 * OZ_BK>(0), dm = smem_desc_mn128(0, OZ_DTILE / 2);
-      auto operands = [&](int ks, uint32_t sa, uint32_t sb, int off) {
-        const int kt = (ADJ && ks >= ns ? ks - ns : ks) / (128 / OZ_BK);
-        const bool amn = kt > ti, bmn = kt > tj;
-        OzOperands o;
-        o.ahi = (uint32_t)((amn ? dm : dk) >> 32);
-        o.alo = (uint32_t)(amn ? dm : dk) + ((unit(sa) + (uint32_t)off * OZ_DTILE) >> 4);
-        o.adv_a = amn ? (2048u >> 4) : (32u >> 4);
-        o.bhi = (uint32_t)((bmn ? dm : dk) >> 32);
-        o.blo = (uint32_t)(bmn ? dm : dk) + ((unit(sb) + (uint32_t)off * OZ_DTILE) >> 4) + poff;
-        o.adv_b = bmn ? (2048u >> 4) : (32u >> 4);
-        o.idesc = idesc0 | ((amn ? 1u : 0u) << 15) | ((bmn ? 1u : 0u) << 16);
-        return o;
-      };
-      // the units of the next K step of the ring: rows I, rows J (the same on a diagonal tile)
-      uint32_t sa, pa, sb, pb;
-      auto take = [&]() {
-        sa = su;
-        pa = ph;
-        if (++su == OZ_UNITS) {
-          su = 0;
-          ph ^= 1;
+      if constexpr (WIDE) {
+        const uint64_t dk = smem_desc_sw<2 * BK>(0), dm = smem_desc_mn128(0, DTILE / 2);
+        // the ring's tile `off` places past s0 (phase p0)
+        auto place = [&](uint32_t s0, uint32_t off) { return s0 + off >= OZ_TILES ? s0 + off - OZ_TILES : s0 + off; };
+        auto parity = [&](uint32_t s0, uint32_t p0, uint32_t off) { return s0 + off >= OZ_TILES ? p0 ^ 1u : p0; };
+        // the next group of tiles of each operand has come (a diagonal tile's serves both)
+        auto loaded = [&]() {
+          bool in = mbar_wait(full(0, ga), (ga / OZ_GROUPS) & 1, abort_flag);
+          ++ga;
+          if (!dg) {
+            in = in && mbar_wait(full(1, gb), (gb / OZ_GROUPS) & 1, abort_flag);
+            ++gb;
+          }
+          return __all_sync(0xffffffffu, in) != 0;
+        };
+        // The tiles of a slice lie in the ring in the order the producers fill it (rows I and rows J in
+        // turn; on a diagonal tile rows I alone, the tile of a digit serving both).  Descriptors of
+        // slice ks, whose first tile is the next of the ring.  Blocks right of the tile's own came in
+        // MN-major (transpose bits 15 / 16); a K = 16 step advances 32 B in a K-major row, 2 KB (16 K
+        // values) in an MN-major tile
+        OzWide o;
+        auto prepare = [&](auto low, int ks) {
+          constexpr int N = oz_digits<decltype(low)::value>();
+          const int kp = ADJ && ks >= ns ? ks - ns : ks, kt = kp / (128 / BK);
+          const bool amn = kt > ti, bmn = kt > tj;
+          const uint32_t alo = (uint32_t)(amn ? dm : dk) + (base >> 4), blo = (uint32_t)(bmn ? dm : dk) + (base >> 4);
+          o.ahi = (uint32_t)((amn ? dm : dk) >> 32);
+          o.bhi = (uint32_t)((bmn ? dm : dk) >> 32);
+          o.adv_a = amn ? (2048u >> 4) : (32u >> 4);
+          o.adv_b = bmn ? (2048u >> 4) : (32u >> 4);
+          o.idesc = idesc0 | ((amn ? 1u : 0u) << 15) | ((bmn ? 1u : 0u) << 16);
+          o.steps = min(BK / 16, (sz - kp * BK + 15) / 16);
+  #pragma unroll
+          for (int q = 0; q < N; ++q) {
+            o.a[q] = alo + place(su, dg ? N - 1 - q : 2 * (N - 1 - q)) * (DTILE >> 4);
+            o.b[q] = blo + place(su, dg ? N - 1 - q : 2 * q + 1) * (DTILE >> 4);
+          }
+        };
+        // The MMAs of the prepared slice.  Before the last K = 16 step of a group of tiles
+        // the next group is waited for, and before that of the slice the next one's descriptors are formed
+        // (next()): the tensor pipe has the products issued so far to work on meanwhile.  Every MMA issued is committed, also where a wait gives up.
+        auto slice = [&](auto low, bool first, auto next) {
+          constexpr bool LOW = decltype(low)::value;
+          constexpr int N = oz_digits<LOW>();
+          const uint32_t s0 = su, p0 = ph;
+          const OzWide c = o;
+          su += (uint32_t)(dg ? N : 2 * N);
+          if (su >= OZ_TILES) {
+            su -= OZ_TILES;
+            ph ^= 1;
+          }
+          bool good = true;
+          auto step = [&](auto idx) {
+            constexpr int I = decltype(idx)::value;
+            constexpr bool ends = I == N - 1 || I == OZ_HEAD - 1;  // of a group
+            if (!good) return;
+            if (elect_one()) oz_issue_wide<LOW, I, 0, BK / 16 - 1>(tmem, c, first);
+            bool more = true;
+            if constexpr (I == N - 1) more = next();
+            if (ends && more && (I == N - 1 || !dg)) good = loaded();
+            if (elect_one()) {
+              oz_issue_wide<LOW, I, BK / 16 - 1, BK / 16>(tmem, c, first);
+              if (!dg) {
+                mma_commit(empty(place(s0, 2 * I)));
+  #pragma unroll
+                for (int b = 0; b <= I; ++b)
+                  if (oz_b_last<LOW>(b) == I) mma_commit(empty(place(s0, 2 * b + 1)));
+              } else if (I == N - 1) {
+  #pragma unroll
+                for (int q = 0; q < N; ++q) mma_commit(empty(place(s0, q)));
+              }
+            }
+            last = (int)place(s0, dg ? 0 : 2 * I);
+            lastph = parity(s0, p0, dg ? 0 : 2 * I);
+          };
+          step(std::integral_constant<int, 0>());
+          step(std::integral_constant<int, 1>());
+          if constexpr (!LOW) {
+            step(std::integral_constant<int, 2>());
+            step(std::integral_constant<int, 3>());
+            step(std::integral_constant<int, 4>());
+          }
+          return good;
+        };
+        prepare(std::false_type(), kr.x);
+        bad = !loaded();
+        for (int c0 = kr.x, c1; c0 < kr.y && !bad; c0 = c1, ++r) {
+          c1 = round_end(c0, kr);
+          // first pass: it reuses the columns of the previous round's second
+          if (r > 0 && !wait(aempty(1), (r - 1) & 1)) {
+            bad = true;
+            break;
+          }
+          tc_fence_after();
+          for (int kb = c0; kb < c1 && !bad; ++kb)
+            bad = !slice(std::false_type(), kb == c0, [&]() {
+              if (kb + 1 < c1) prepare(std::false_type(), kb + 1);
+              else prepare(std::true_type(), c0);
+              return true;
+            });
+          if (bad) break;
+          if (elect_one()) mma_commit(afull(0));
+          // second pass: it reuses columns of this round's first
+          if (!wait(aempty(0), r & 1)) {
+            bad = true;
+            break;
+          }
+          tc_fence_after();
+          for (int kb = c0; kb < c1 && !bad; ++kb)
+            bad = !slice(std::true_type(), kb == c0, [&]() {
+              if (kb + 1 < c1) prepare(std::true_type(), kb + 1);
+              else if (c1 < kr.y) prepare(std::false_type(), c1);
+              else return false;
+              return true;
+            });
+          if (!bad && elect_one()) mma_commit(afull(1));
         }
-        sb = sa;
-        pb = pa;
-        if (!dg) {
-          sb = su;
-          pb = ph;
+      } else {
+        // rows J of a piece start 64 rows into each digit tile: 64 B each K-major, one atom MN-major
+        const uint32_t poff = (uint32_t)piece * ((64u * BK * 2u) >> 4);
+        // operands of slice ks, tile `off` of the units sa (rows I) and sb (rows J): those right of
+        // the tile's own block came in MN-major (transpose bits 15 / 16); a K = 16 step advances
+        // 32 B in a K-major row, 2 KB (16 K values) in an MN-major tile
+        const uint64_t dk = smem_desc_sw<2 * BK>(0), dm = smem_desc_mn128(0, DTILE / 2);
+        auto operands = [&](int ks, uint32_t sa, uint32_t sb, int off) {
+          const int kt = (ADJ && ks >= ns ? ks - ns : ks) / (128 / BK);
+          const bool amn = kt > ti, bmn = kt > tj;
+          OzNarrow o;
+          o.ahi = (uint32_t)((amn ? dm : dk) >> 32);
+          o.alo = (uint32_t)(amn ? dm : dk) + ((unit(sa) + (uint32_t)off * DTILE) >> 4);
+          o.adv_a = amn ? (2048u >> 4) : (32u >> 4);
+          o.bhi = (uint32_t)((bmn ? dm : dk) >> 32);
+          o.blo = (uint32_t)(bmn ? dm : dk) + ((unit(sb) + (uint32_t)off * DTILE) >> 4) + poff;
+          o.adv_b = bmn ? (2048u >> 4) : (32u >> 4);
+          o.idesc = idesc0 | ((amn ? 1u : 0u) << 15) | ((bmn ? 1u : 0u) << 16);
+          return o;
+        };
+        // the units of the next K step of the ring: rows I, rows J (the same on a diagonal tile)
+        uint32_t sa, pa, sb, pb;
+        auto take = [&]() {
+          sa = su;
+          pa = ph;
           if (++su == OZ_UNITS) {
             su = 0;
             ph ^= 1;
           }
-        }
-      };
-      auto loaded = [&]() {
-        if (!wait(full(sa), pa) || (!dg && !wait(full(sb), pb))) return false;
-        tc_fence_after();
-        return true;
-      };
-      auto release = [&](uint32_t ua, uint32_t ub, uint32_t pub) {
-        if (elect_one()) {
-          mma_commit(empty(ua));
-          if (!dg) mma_commit(empty(ub));
-        }
-        last = (int)ub;
-        lastph = pub;
-      };
-      for (int c0 = kr.x, c1; c0 < kr.y && !bad; c0 = c1, ++r) {
-        c1 = round_end(c0, kr);
-        // first pass: it reuses the columns of the previous round's second
-        take();
-        OzOperands o = operands(c0, sa, sb, 0);
-        if (r > 0 && !wait(aempty(1), (r - 1) & 1)) {
-          bad = true;
-          break;
-        }
-        tc_fence_after();
-        for (int kb = c0; kb < c1; ++kb) {
-          if (!loaded()) {
-            bad = true;
-            break;
+          sb = sa;
+          pb = pa;
+          if (!dg) {
+            sb = su;
+            pb = ph;
+            if (++su == OZ_UNITS) {
+              su = 0;
+              ph ^= 1;
+            }
           }
-          if (elect_one()) oz_issue<false, 0>(tmem, o, kb == c0);
-          const OzOperands cur = o;
-          const uint32_t ua = sa, ub = sb, pub = pb;
-          take();  // after the last slice: the first unit of the second pass
-          if (kb + 1 < c1) o = operands(kb + 1, sa, sb, 0);
-          if (elect_one()) oz_issue<false, 1>(tmem, cur, false);
-          release(ua, ub, pub);
-        }
-        if (bad) break;
-        if (elect_one()) mma_commit(afull(0));
-        // second pass: it reuses columns of this round's first
-        o = operands(c0, sa, sb, 0);
-        if (!wait(aempty(0), r & 1)) {
-          bad = true;
-          break;
-        }
-        tc_fence_after();
-        for (int kb = c0; kb < c1; kb += OZ_LOW_SUB) {
-          const bool two = kb + 1 < c1;
-          if (!loaded()) {
-            bad = true;
-            break;
-          }
+        };
+        auto loaded = [&]() {
+          if (!wait(full(0, sa), pa) || (!dg && !wait(full(0, sb), pb))) return false;
+          tc_fence_after();
+          return true;
+        };
+        auto release = [&](uint32_t ua, uint32_t ub, uint32_t pub) {
           if (elect_one()) {
-            oz_issue<true, 0>(tmem, o, kb == c0);
-            oz_issue<true, 1>(tmem, o, false);
+            mma_commit(empty(ua));
+            if (!dg) mma_commit(empty(ub));
           }
-          const uint32_t ua = sa, ub = sb, pub = pb;
-          if (two) o = operands(kb + 1, sa, sb, OZ_LOW);
-          const bool more = kb + OZ_LOW_SUB < c1;
-          if (two && elect_one()) oz_issue<true, 0>(tmem, o, false);
-          const OzOperands cur = o;
-          if (more) {
-            take();
-            o = operands(kb + OZ_LOW_SUB, sa, sb, 0);
+          last = (int)ub;
+          lastph = pub;
+        };
+        for (int c0 = kr.x, c1; c0 < kr.y && !bad; c0 = c1, ++r) {
+          c1 = round_end(c0, kr);
+          // first pass: it reuses the columns of the previous round's second
+          take();
+          OzNarrow o = operands(c0, sa, sb, 0);
+          if (r > 0 && !wait(aempty(1), (r - 1) & 1)) {
+            bad = true;
+            break;
           }
-          if (two && elect_one()) oz_issue<true, 1>(tmem, cur, false);
-          release(ua, ub, pub);
+          tc_fence_after();
+          for (int kb = c0; kb < c1; ++kb) {
+            if (!loaded()) {
+              bad = true;
+              break;
+            }
+            if (elect_one()) oz_issue_narrow<false, 0>(tmem, o, kb == c0);
+            const OzNarrow cur = o;
+            const uint32_t ua = sa, ub = sb, pub = pb;
+            take();  // after the last slice: the first unit of the second pass
+            if (kb + 1 < c1) o = operands(kb + 1, sa, sb, 0);
+            if (elect_one()) oz_issue_narrow<false, 1>(tmem, cur, false);
+            release(ua, ub, pub);
+          }
+          if (bad) break;
+          if (elect_one()) mma_commit(afull(0));
+          // second pass: it reuses columns of this round's first
+          o = operands(c0, sa, sb, 0);
+          if (!wait(aempty(0), r & 1)) {
+            bad = true;
+            break;
+          }
+          tc_fence_after();
+          for (int kb = c0; kb < c1; kb += OZ_LOW_SUB) {
+            const bool two = kb + 1 < c1;
+            if (!loaded()) {
+              bad = true;
+              break;
+            }
+            if (elect_one()) {
+              oz_issue_narrow<true, 0>(tmem, o, kb == c0);
+              oz_issue_narrow<true, 1>(tmem, o, false);
+            }
+            const uint32_t ua = sa, ub = sb, pub = pb;
+            if (two) o = operands(kb + 1, sa, sb, OZ_LOW);
+            const bool more = kb + OZ_LOW_SUB < c1;
+            if (two && elect_one()) oz_issue_narrow<true, 0>(tmem, o, false);
+            const OzNarrow cur = o;
+            if (more) {
+              take();
+              o = operands(kb + OZ_LOW_SUB, sa, sb, 0);
+            }
+            if (two && elect_one()) oz_issue_narrow<true, 1>(tmem, cur, false);
+            release(ua, ub, pub);
+          }
+          if (!bad && elect_one()) mma_commit(afull(1));
         }
-        if (!bad && elect_one()) mma_commit(afull(1));
       }
     }
     if (bad) {
@@ -983,13 +1242,9 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
     else if (a.mode == SQ_TAIL_NEXT) alf = (int8_t)(-a.ctl.alpha[step - 1]);
     else alf = a.ctl.alpha[step];
     // the adjoint's Xbar ping-pong: in = buffer (n - step) & 1, out = the other
-    const double* xin = a.xin;
-    double* xout = a.xout;
-    if (ADJ && ((n - step) & 1)) {
-      xin = a.xout;
-      xout = const_cast<double*>(a.xin);
-    }
-    long long* const xq = reinterpret_cast<long long*>(xout);
+    const bool flip = ADJ && ((n - step) & 1);
+    auto xin = [&]() { return flip ? (const double*)a.xout : a.xin; };
+    auto xq = [&]() { return reinterpret_cast<long long*>(flip ? const_cast<double*>(a.xin) : a.xout); };
     // the sums are formed with the sign the step needs: X_new = 2X + z, z = -Y, or z = Y alone
     const int sgn = alf > 0 ? -1 : 1;
     // the digit arenas of a set lie one arena apart
@@ -1002,19 +1257,28 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
         *s_err = 1;
         break;
       }
-      OzItem t;  // warp-uniform
+      // the item's fields (warp-uniform); wide: read again after the drains, which need the registers
+      OzItem t;
+      auto fields = [&]() {
+        const volatile OzItem& w = s_items[iq];
+        t.ti = __shfl_sync(0xffffffffu, w.ti, 0);
+        t.tj = __shfl_sync(0xffffffffu, w.tj, 0);
+        t.slot = __shfl_sync(0xffffffffu, w.slot, 0);
+        t.part = __shfl_sync(0xffffffffu, w.part, 0);
+        t.s = __shfl_sync(0xffffffffu, w.s, 0);
+        t.c = __shfl_sync(0xffffffffu, w.c, 0);
+        t.ld = __shfl_sync(0xffffffffu, w.ld, 0);
+        t.off = __shfl_sync(0xffffffffu, w.off, 0);
+        t.soff = __shfl_sync(0xffffffffu, w.soff, 0);
+        t.piece = __shfl_sync(0xffffffffu, w.piece, 0);
+      };
+      auto done = [&]() {  // with the item
+        __syncwarp();
+        if (lane == 0) mbar_arrive(item_empty(iq));
+      };
       t.code = __shfl_sync(0xffffffffu, s_items[iq].code, 0);
-      t.ti = __shfl_sync(0xffffffffu, s_items[iq].ti, 0);
-      t.tj = __shfl_sync(0xffffffffu, s_items[iq].tj, 0);
-      t.slot = __shfl_sync(0xffffffffu, s_items[iq].slot, 0);
-      t.part = __shfl_sync(0xffffffffu, s_items[iq].part, 0);
-      t.s = __shfl_sync(0xffffffffu, s_items[iq].s, 0);
-      t.c = __shfl_sync(0xffffffffu, s_items[iq].c, 0);
-      t.ld = __shfl_sync(0xffffffffu, s_items[iq].ld, 0);
-      t.off = __shfl_sync(0xffffffffu, s_items[iq].off, 0);
-      t.soff = __shfl_sync(0xffffffffu, s_items[iq].soff, 0);
-      t.piece = __shfl_sync(0xffffffffu, s_items[iq].piece, 0);
-      if (lane == 0) mbar_arrive(item_empty(iq));
+      fields();
+      if (!WIDE) done();
       if (t.code < 0) break;
       const int code = t.code;
       const int ti = split ? code >> 1 : code, half = split ? code & 1 : -1;
@@ -1022,107 +1286,154 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
       // finishes the tile reads; otherwise the sums wait in this CTA's scratch tile
       long long* const acc = split ? a.split_acc + (size_t)code * (128 * 128) : cta_acc;
       const OzItem& p = t;
-      const int64_t ld = p.ld;
-      const int r = t.ti * 128 + m;
-      const bool diag = t.slot >= 0;
-      const int sg = ADJ ? a.sig[t.part] : 0;  // the adjoint's sums hold (Xbar X + X Xbar) / 2^sg
       // columns the MMAs covered; the 16-column chunks beyond them lie in the part's zero
       // padding, which no step writes (the arenas are zeroed when the workspace is bound)
       const int ncols = piece_cols(p.s, t.tj, t.piece);
       if (ncols == 0) {  // a piece in the padding
-        if (!ADJ && !rec && diag && warp == 4 && lane == 0) a.slots[t.slot * pieces + t.piece] = make_double2(0.0, 0.0);
+        if (!ADJ && !rec && t.slot >= 0 && warp == 4 && lane == 0)
+          a.slots[t.slot * pieces + t.piece] = make_double2(0.0, 0.0);
+        if (WIDE) done();
         continue;
       }
       // a diagonal tile keeps its upper triangle and mirrors it: a chunk wholly left of the
       // warp's first row (all its entries below the diagonal) is neither drained nor formed
       const int cskip = (t.ti == t.tj) ? quarter * 32 : 0;
       bool ok = true;
-      // the warp's chunks of 16 columns (pc0: its first column in the piece): the last one's sums stay
-      // in registers for the final pass, the other one's wait in the scratch tile (-1: no chunk)
+      // the warp's chunks of 16 columns (pc0: its first column in the piece)
       const int nch = 2 / pieces, pc0 = colq * 16 * nch, tc0 = t.piece * pcols + pc0;
       const bool on0 = pc0 < ncols && tc0 + 16 > cskip;
       const bool on1 = nch == 2 && pc0 + 16 < ncols && tc0 + 32 > cskip;
-      const int clast = on1 ? 1 : (on0 ? 0 : -1), cfirst = on1 && on0 ? 0 : -1;
       // the previous iterate's lines of this warp (not written by this launch; read from HBM) come
       // to L2 while the MMAs run: lane l, column l of the warp's 32, two lines of 128 B
-      if (alf > 0 && clast >= 0) {
+      if (alf > 0 && (on0 || on1)) {
         const int c = t.tj * 128 + tc0 + lane;
         if (lane < 16 * nch && c < p.s) {
-          const double* x = xin + p.off + (int64_t)c * ld + t.ti * 128 + quarter * 32;
+          const double* x = xin() + p.off + (int64_t)c * p.ld + t.ti * 128 + quarter * 32;
           asm volatile("prefetch.global.L2 [%0];\n prefetch.global.L2 [%0 + 128];\n" ::"l"(x));
         }
       }
-      long long z[16];
       // the two passes of every round: read the accumulators' sums (integers at their scales,
-      // held exactly in FP32, but for the sixth) and add them as 64-bit integers, parked in
-      // TMEM between the passes and then in the scratch tile (thread-private entries: column
-      // cl, row m) or in registers; each pass hands its columns back
+      // held exactly in FP32, but for the sixth) and add them as 64-bit integers; each pass hands its
+      // columns back
+      long long z[16];
       const int3 kr = slices(p.s, half);
-      for (int c0 = kr.x, pass = 0; c0 < kr.y; pass ^= 1) {
-        ok = __all_sync(0xffffffffu, mbar_wait(afull(pass), rd & 1, abort_flag)) && ok;
-        tc_fence_after();
-        // the first pass hands its columns back as soon as the warp's last chunk has read
-        // columns 0-255, which the second reuses
-        bool released = false;
-#pragma unroll 1
-        for (int cc = 0; cc < 2 && ok; ++cc) {
-          if (cc != clast && cc != cfirst) continue;
-          const int cl = tc0 + cc * 16;  // in the tile
-          const uint32_t tc = tmem + lane_off + (uint32_t)(pc0 + cc * 16);
-          uint32_t w[16];
-          if (pass == 0) {
-            // the first pass's sum waits in the columns this warp has just drained (its own
-            // columns among 256-511), which the second pass leaves alone
-#pragma unroll
-            for (int j = 0; j < 16; ++j) z[j] = (long long)(sgn < 0 ? kOzOffset : 0ull - kOzOffset);
-            oz_drain_high_a(tc, sgn, z);
-            if (cc == clast) {
-              tc_fence_before();
-              __syncwarp();
-              if (lane == 0) mbar_arrive(aempty(0));
-              released = true;
-            }
-            oz_drain_high_b(tc, sgn, z);
-#pragma unroll
-            for (int j = 0; j < 16; ++j) w[j] = (uint32_t)(unsigned long long)z[j];
-            tmem_st16(tc + OZ_PARK_LO, w);
-#pragma unroll
-            for (int j = 0; j < 16; ++j) w[j] = (uint32_t)((unsigned long long)z[j] >> 32);
-            tmem_st16(tc + OZ_PARK_HI, w);
-          } else {
-            tmem_ld16(tc + OZ_PARK_LO, w);
-#pragma unroll
-            for (int j = 0; j < 16; ++j) z[j] = (long long)(unsigned long long)w[j];
-            tmem_ld16(tc + OZ_PARK_HI, w);
-#pragma unroll
-            for (int j = 0; j < 16; ++j) z[j] += (long long)((unsigned long long)w[j] << 32);
-            oz_drain_low(tc, sgn, z);
-            if (cc == clast) {
-              tc_fence_before();
-              __syncwarp();
-              if (lane == 0) mbar_arrive(aempty(1));
-              released = true;
-            }
-            long long* zp = acc + (size_t)cl * 128 + m;
-            if (c0 > kr.x) {  // the rounds before
-#pragma unroll
-              for (int j = 0; j < 16; ++j) z[j] += zp[(size_t)j * 128];
-            }
-            if (split || cc != clast || round_end(c0, kr) < kr.y) {
-#pragma unroll
-              for (int j = 0; j < 16; ++j) zp[(size_t)j * 128] = z[j];
-            }
-          }
-        }
-        if (pass == 0) tmem_wait_st();
-        if (!released) {
+      if constexpr (WIDE) {
+        // Both chunks' sums stay in registers.  The tensor pipe stands still from a pass's last product
+        // until the columns the next pass starts in have been read by every warp, so nothing but that
+        // comes first: of the first pass columns 0-255 of both chunks, then the rest while the second
+        // pass runs.
+        long long z1[16];
+        const uint32_t tc = tmem + lane_off + (uint32_t)pc0;
+        auto hand_back = [&](int pass) {
           tc_fence_before();
           __syncwarp();
           if (lane == 0) mbar_arrive(aempty(pass));
+        };
+#pragma unroll
+        for (int j = 0; j < 16; ++j) z[j] = z1[j] = 0ll;
+        for (int c0 = kr.x; c0 < kr.y; c0 = round_end(c0, kr), ++rd) {
+          const long long less = (long long)(sgn < 0 ? kOzOffset : 0ull - kOzOffset);
+#pragma unroll
+          for (int j = 0; j < 16; ++j) {
+            z[j] += less;
+            z1[j] += less;
+          }
+          ok = __all_sync(0xffffffffu, mbar_wait(afull(0), rd & 1, abort_flag)) && ok;
+          tc_fence_after();
+          if (ok && on0) oz_drain_high_a(tc, sgn, z);
+          if (ok && on1) oz_drain_high_a(tc + 16, sgn, z1);
+          hand_back(0);
+          if (ok && on0) oz_drain_high_b(tc, sgn, z);
+          if (ok && on1) oz_drain_high_b(tc + 16, sgn, z1);
+          ok = __all_sync(0xffffffffu, mbar_wait(afull(1), rd & 1, abort_flag)) && ok;
+          tc_fence_after();
+          if (ok && on0) oz_drain_low(tc, sgn, z);
+          if (ok && on1) oz_drain_low(tc + 16, sgn, z1);
+          hand_back(1);
         }
-        if (pass == 1) {
-          c0 = round_end(c0, kr);
-          ++rd;
+        // the sums leave the registers for a scratch tile (thread-private entries: column cl, row m):
+        // both chunks' of a split item, else the one the final pass takes second
+        auto put = [&](int cl, const long long (&v)[16]) {
+          long long* zp = acc + (size_t)cl * 128 + m;
+#pragma unroll
+          for (int j = 0; j < 16; ++j) zp[(size_t)j * 128] = v[j];
+        };
+        if (on0 && (split || on1)) put(tc0, z);
+        if (on1) {
+          if (split) put(tc0 + 16, z1);
+#pragma unroll
+          for (int j = 0; j < 16; ++j) z[j] = z1[j];
+        }
+      } else {
+        const int clast = on1 ? 1 : (on0 ? 0 : -1), cfirst = on1 && on0 ? 0 : -1;
+        // one chunk's sums at a time, parked in TMEM between the passes and then in the scratch tile
+        // (thread-private entries: column cl, row m) or, the last one's, in registers
+        for (int c0 = kr.x, pass = 0; c0 < kr.y; pass ^= 1) {
+          ok = __all_sync(0xffffffffu, mbar_wait(afull(pass), rd & 1, abort_flag)) && ok;
+          tc_fence_after();
+          // the first pass hands its columns back as soon as the warp's last chunk has read
+          // columns 0-255, which the second reuses
+          bool released = false;
+#pragma unroll 1
+          for (int cc = 0; cc < 2 && ok; ++cc) {
+            if (cc != clast && cc != cfirst) continue;
+            const int cl = tc0 + cc * 16;  // in the tile
+            const uint32_t tc = tmem + lane_off + (uint32_t)(pc0 + cc * 16);
+            uint32_t w[16];
+            if (pass == 0) {
+              // the first pass's sum waits in the columns this warp has just drained (its own
+              // columns among 256-511), which the second pass leaves alone
+#pragma unroll
+              for (int j = 0; j < 16; ++j) z[j] = (long long)(sgn < 0 ? kOzOffset : 0ull - kOzOffset);
+              oz_drain_high_a(tc, sgn, z);
+              if (cc == clast) {
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(aempty(0));
+                released = true;
+              }
+              oz_drain_high_b(tc, sgn, z);
+#pragma unroll
+              for (int j = 0; j < 16; ++j) w[j] = (uint32_t)(unsigned long long)z[j];
+              tmem_st16(tc + OZ_PARK_LO, w);
+#pragma unroll
+              for (int j = 0; j < 16; ++j) w[j] = (uint32_t)((unsigned long long)z[j] >> 32);
+              tmem_st16(tc + OZ_PARK_HI, w);
+            } else {
+              tmem_ld16(tc + OZ_PARK_LO, w);
+#pragma unroll
+              for (int j = 0; j < 16; ++j) z[j] = (long long)(unsigned long long)w[j];
+              tmem_ld16(tc + OZ_PARK_HI, w);
+#pragma unroll
+              for (int j = 0; j < 16; ++j) z[j] += (long long)((unsigned long long)w[j] << 32);
+              oz_drain_low(tc, sgn, z);
+              if (cc == clast) {
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(aempty(1));
+                released = true;
+              }
+              long long* zp = acc + (size_t)cl * 128 + m;
+              if (c0 > kr.x) {  // the rounds before
+#pragma unroll
+                for (int j = 0; j < 16; ++j) z[j] += zp[(size_t)j * 128];
+              }
+              if (split || cc != clast || round_end(c0, kr) < kr.y) {
+#pragma unroll
+                for (int j = 0; j < 16; ++j) zp[(size_t)j * 128] = z[j];
+              }
+            }
+          }
+          if (pass == 0) tmem_wait_st();
+          if (!released) {
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(aempty(pass));
+          }
+          if (pass == 1) {
+            c0 = round_end(c0, kr);
+            ++rd;
+          }
         }
       }
       if (!ok) *s_err = 1;
@@ -1139,7 +1450,10 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
           *s_half = (int)before;
         }
         asm volatile("bar.sync 1, %0;\n" ::"n"(32 * OZ_EPI_WARPS) : "memory");
-        if (*s_half == 0) continue;
+        if (*s_half == 0) {
+          if (WIDE) done();
+          continue;
+        }
         __threadfence();
         other = a.split_acc + (size_t)(code ^ 1) * (128 * 128);
       }
@@ -1148,112 +1462,216 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
       // tiles on or above the diagonal are kept (the next step reads the rest MN-major from
       // them); a diagonal tile mirrors its upper triangle, transposed among the lanes so that the
       // mirrored columns are written 128 B (master) and 32 B (each digit) at a time
+      if (WIDE) {
+        fields();
+        done();
+      }
+      const int64_t ld = p.ld;
+      const int r = t.ti * 128 + m;
+      const bool diag = t.slot >= 0;
+      const int sg = ADJ ? a.sig[t.part] : 0;  // the adjoint's sums hold (Xbar X + X Xbar) / 2^sg
       long long yd = 0ll, xd = 0ll;  // diagonal entry (r, r) of sgn Y and X_new
       float rown = 0.0f;             // adjoint: squared norm of row r over this thread's upper entries
-      auto stored = [&](long long xf) {  // the word stored: fixed point (forward) or FP64 bits (adjoint)
-        if (!ADJ) return xf;
+      auto stored = [&](long long xf) {  // adjoint: the FP64 word stored
         return sg == OZ_SIG_NONFINITE ? 0x7FF8000000000000ll : __double_as_longlong(from_fixed(xf, sg));
       };
       const bool dgt = t.ti == t.tj;
-      // A tile is formed once, so straight-line code for all 16 columns of a chunk would be fetched
-      // from L2 as often as it runs (a diagonal tile took 42,000 cycles, most of them waiting
-      // for instructions): the columns are taken eight at a time in loops, z turning in registers.
-      auto chunk = [&](int cl) {
-        const int cbase = t.tj * 128 + cl;
-        // element (first row of the warp, column cbase), uniform; the lane's row is added to it
-        int64_t e = p.off + (int64_t)cbase * ld + (t.ti * 128 + quarter * 32);
-        float coln[16];  // adjoint: squares of the entries (r, c) for the norms of rows c
-#pragma unroll 1
-        for (int b = 0; b < 2; ++b, e += 8 * ld) {
-          const int cb = cbase + 8 * b;
-          long long xn[8];  // the forward iterates are kept in the fixed point itself; the adjoint's Xbar in FP64
+      if constexpr (WIDE) {
+        // A tile is formed once, so straight-line code for all 16 columns of a chunk would be fetched
+        // from L2 as often as it runs (a diagonal tile took 42,000 cycles, most of them waiting
+        // for instructions): the columns are stored four at a time in a loop, z turning in registers, and
+        // a diagonal tile's mirrored entries go through the same loop a second time.
+        auto chunk = [&](int cl) {
+          const int cbase = t.tj * 128 + cl;
+          // element (row r, column cbase)
+          int64_t e = p.off + (int64_t)cbase * ld + r;
+          constexpr int B = ADJ ? 8 : 16;  // columns read together
 #pragma unroll
-          for (int j = 0; j < 8; ++j)
-            xn[j] = alf > 0 ? __ldg(reinterpret_cast<const long long*>(xin) + (e + (int64_t)j * ld) + lane) : 0ll;
+          for (int h = 0; h < 16; h += B) {
+            long long xn[B];  // the forward iterates are kept in the fixed point itself; the adjoint's Xbar in FP64
 #pragma unroll
-          for (int j = 0; j < 8; ++j) {
-            const int c = cb + j;
-            const bool upper = !dgt || c >= r;
-            const long long xf = 2 * (ADJ ? to_fixed(__longlong_as_double(xn[j]), sg) : xn[j]) + z[j];
-            if (!ADJ && dgt && c == r) {  // the thread's one diagonal entry, if it has it
-              yd = z[j];
-              xd = xf;
-            }
-            if (ADJ) {
-              float f = 0.0f;
-              if (upper && r < p.s && c < p.s) f = fixed_to_f32_abs(xf);
-              // every stored entry (r, c) adds to the norm of row r, and of row c unless c = r
-              rown = fmaf(f, f, rown);
-              coln[j] = coln[8 + j];
-              coln[8 + j] = c != r ? f * f : 0.0f;
-            }
-            xn[j] = stored(xf);
-            store_word_if(upper, xq + (e + (int64_t)j * ld) + lane, xn[j]);
-          }
-          if (!ADJ) {
+            for (int j = 0; j < B; ++j)
+              xn[j] = alf > 0 ? __ldg(reinterpret_cast<const long long*>(xin()) + e + (int64_t)(h + j) * ld) : 0ll;
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-              uint32_t dw[OZ_SLICES][2];  // four columns' digits, two packed per word
-              digits4({xn[4 * h], xn[4 * h + 1], xn[4 * h + 2], xn[4 * h + 3]}, dw);
-#pragma unroll
-              for (int w = 0; w < 4; ++w) {
-                uint16_t* d = a.digits[dbo].s[0] + (e + (int64_t)(4 * h + w) * ld) + lane;
-                store_digits_if(!dgt || cb + 4 * h + w >= r, d, dstr, dw, w);
+            for (int j = 0; j < B; ++j) {
+              const long long xf = 2 * (ADJ ? to_fixed(__longlong_as_double(xn[j]), sg) : xn[j]) + z[h + j];
+              if (!ADJ && dgt && cbase + h + j == r) {  // the thread's one diagonal entry, if it has it
+                yd = z[h + j];
+                xd = xf;
               }
+              z[h + j] = xf;
             }
           }
+          if constexpr (ADJ) {
+            // every stored entry (r, c) adds to the norm of row r, and of row c unless c = r
+            float coln[16];
 #pragma unroll
-          for (int j = 0; j < 8; ++j) {
-            z[j] = z[8 + j];
-            z[8 + j] = xn[j];
+            for (int j = 0; j < 16; ++j) {
+              const int c = cbase + j;
+              const float f = (!dgt || c >= r) && r < p.s && c < p.s ? fixed_to_f32_abs(z[j]) : 0.0f;
+              rown = fmaf(f, f, rown);
+              coln[j] = c != r ? f * f : 0.0f;
+            }
+            int col;
+            const float cs = warp_colsum16(coln, lane, col);
+            if (!(lane & 1) && cbase + col < p.s && cs != 0.0f) atomicAdd(&a.normf[p.soff + cbase + col], cs);
+#pragma unroll
+            for (int j = 0; j < 16; ++j) z[j] = stored(z[j]);
           }
-        }
-        if (dgt) {
-          // the mirrored entries: lane l has column cbase + l % 16 of rows rb + j, which go to row
-          // cbase + l % 16 of columns rb + j
-          transpose16(z, lane);
-          int rb = t.ti * 128 + quarter * 32 + (lane & 16);
-          const int c = cbase + (lane & 15);
-          int64_t em = p.off + (int64_t)rb * ld + c;
+          // first the thread's own entries: row r, columns cbase + j, those on or above the diagonal.  Then,
+          // of a diagonal tile, z transposed: lane l has column c = cbase + l % 16 of rows rb + j, which
+          // go to row c of columns rb + j, those below it.  Entry j is stored if at + dir j >= 0.
+          int at = dgt ? cbase - r : 128, dir = 1;
 #pragma unroll 1
-          for (int b = 0; b < 4; ++b, rb += 4, em += 4 * ld) {
+          for (int b = 0;; ++b, e += 4 * ld, at += 4 * dir) {
+            if (b == 4) {
+              if (!dgt) break;
+              transpose16(z, lane);
+              const int rb = t.ti * 128 + quarter * 32 + (lane & 16), c = cbase + (lane & 15);
+              e = p.off + (int64_t)rb * ld + c;
+              at = c - rb - 1;
+              dir = -1;
+            }
+            if (b == 8) break;
 #pragma unroll
-            for (int j = 0; j < 4; ++j)
-              store_word_if(c > rb + j, xq + em + (int64_t)j * ld, z[j]);
+            for (int j = 0; j < 4; ++j) store_word_if(at + dir * j >= 0, xq() + e + (int64_t)j * ld, z[j]);
             if (!ADJ) {
-              uint32_t dw[OZ_SLICES][2];
+              uint32_t dw[OZ_SLICES][2];  // four entries' digits, two packed per word
               digits4({z[0], z[1], z[2], z[3]}, dw);
 #pragma unroll
-              for (int w = 0; w < 4; ++w) {
-                store_digits_if(c > rb + w, a.digits[dbo].s[0] + em + (int64_t)w * ld, dstr, dw, w);
+              for (int j = 0; j < 4; ++j)
+                store_digits_if(at + dir * j >= 0, a.digits[dbo].s[0] + e + (int64_t)j * ld, dstr, dw, j);
+            }
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+              const long long w = z[j];
+              z[j] = z[4 + j];
+              z[4 + j] = z[8 + j];
+              z[8 + j] = z[12 + j];
+              z[12 + j] = w;
+            }
+          }
+        };
+#pragma unroll 1
+        for (int cc = 1; cc >= 0 && ok; --cc) {
+          if (!(cc ? on1 : on0)) continue;
+          const int cl = tc0 + cc * 16;
+          if (cc == 0 && on1) {
+            const long long* zp = acc + (size_t)cl * 128 + m;
+#pragma unroll
+            for (int j = 0; j < 16; ++j) z[j] = zp[(size_t)j * 128];
+          }
+          if (other) {
+            const long long* zo = other + (size_t)cl * 128 + m;
+#pragma unroll
+            for (int j = 0; j < 16; ++j) z[j] += __ldcg(zo + (size_t)j * 128);
+          }
+          chunk(cl);
+        }
+      } else {
+        // the columns are taken eight at a time in loops, the mirrored entries in one of their own: where
+        // a CTA has one or two items, the wide form's loop takes longer (n = 512 density 0.46 against
+        // 0.45 ms), its columns being read before any are stored
+        const double* const xi = xin();
+        long long* const xo = xq();
+        const int clast = on1 ? 1 : (on0 ? 0 : -1), cfirst = on1 && on0 ? 0 : -1;
+        auto chunk = [&](int cl) {
+          const int cbase = t.tj * 128 + cl;
+          // element (first row of the warp, column cbase), uniform; the lane's row is added to it
+          int64_t e = p.off + (int64_t)cbase * ld + (t.ti * 128 + quarter * 32);
+          float coln[16];  // adjoint: squares of the entries (r, c) for the norms of rows c
+#pragma unroll 1
+          for (int b = 0; b < 2; ++b, e += 8 * ld) {
+            const int cb = cbase + 8 * b;
+            long long xn[8];  // the forward iterates are kept in the fixed point itself; the adjoint's Xbar in FP64
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+              xn[j] = alf > 0 ? __ldg(reinterpret_cast<const long long*>(xi) + (e + (int64_t)j * ld) + lane) : 0ll;
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+              const int c = cb + j;
+              const bool upper = !dgt || c >= r;
+              const long long xf = 2 * (ADJ ? to_fixed(__longlong_as_double(xn[j]), sg) : xn[j]) + z[j];
+              if (!ADJ && dgt && c == r) {  // the thread's one diagonal entry, if it has it
+                yd = z[j];
+                xd = xf;
+              }
+              if (ADJ) {
+                float f = 0.0f;
+                if (upper && r < p.s && c < p.s) f = fixed_to_f32_abs(xf);
+                // every stored entry (r, c) adds to the norm of row r, and of row c unless c = r
+                rown = fmaf(f, f, rown);
+                coln[j] = coln[8 + j];
+                coln[8 + j] = c != r ? f * f : 0.0f;
+              }
+              xn[j] = ADJ ? stored(xf) : xf;
+              store_word_if(upper, xo + (e + (int64_t)j * ld) + lane, xn[j]);
+            }
+            if (!ADJ) {
+#pragma unroll
+              for (int h = 0; h < 2; ++h) {
+                uint32_t dw[OZ_SLICES][2];  // four columns' digits, two packed per word
+                digits4({xn[4 * h], xn[4 * h + 1], xn[4 * h + 2], xn[4 * h + 3]}, dw);
+#pragma unroll
+                for (int w = 0; w < 4; ++w) {
+                  uint16_t* d = a.digits[dbo].s[0] + (e + (int64_t)(4 * h + w) * ld) + lane;
+                  store_digits_if(!dgt || cb + 4 * h + w >= r, d, dstr, dw, w);
+                }
               }
             }
 #pragma unroll
-            for (int j = 0; j < 12; ++j) z[j] = z[j + 4];
+            for (int j = 0; j < 8; ++j) {
+              z[j] = z[8 + j];
+              z[8 + j] = xn[j];
+            }
           }
-        }
-        if constexpr (ADJ) {
-          int col;
-          const float cs = warp_colsum16(coln, lane, col);
-          if (!(lane & 1) && cbase + col < p.s && cs != 0.0f) atomicAdd(&a.normf[p.soff + cbase + col], cs);
-        }
-      };
+          if (dgt) {
+            // the mirrored entries: lane l has column cbase + l % 16 of rows rb + j, which go to row
+            // cbase + l % 16 of columns rb + j
+            transpose16(z, lane);
+            int rb = t.ti * 128 + quarter * 32 + (lane & 16);
+            const int c = cbase + (lane & 15);
+            int64_t em = p.off + (int64_t)rb * ld + c;
 #pragma unroll 1
-      for (int pc = 0; pc < 2 && ok; ++pc) {
-        const int cc = pc == 0 ? clast : cfirst;
-        if (cc < 0) continue;
-        const int cl = tc0 + cc * 16;
-        if (pc == 1) {
-          const long long* zp = acc + (size_t)cl * 128 + m;
+            for (int b = 0; b < 4; ++b, rb += 4, em += 4 * ld) {
 #pragma unroll
-          for (int j = 0; j < 16; ++j) z[j] = zp[(size_t)j * 128];
-        }
-        if (other) {
-          const long long* zo = other + (size_t)cl * 128 + m;
+              for (int j = 0; j < 4; ++j)
+                store_word_if(c > rb + j, xo + em + (int64_t)j * ld, z[j]);
+              if (!ADJ) {
+                uint32_t dw[OZ_SLICES][2];
+                digits4({z[0], z[1], z[2], z[3]}, dw);
 #pragma unroll
-          for (int j = 0; j < 16; ++j) z[j] += __ldcg(zo + (size_t)j * 128);
+                for (int w = 0; w < 4; ++w) {
+                  store_digits_if(c > rb + w, a.digits[dbo].s[0] + em + (int64_t)w * ld, dstr, dw, w);
+                }
+              }
+#pragma unroll
+              for (int j = 0; j < 12; ++j) z[j] = z[j + 4];
+            }
+          }
+          if constexpr (ADJ) {
+            int col;
+            const float cs = warp_colsum16(coln, lane, col);
+            if (!(lane & 1) && cbase + col < p.s && cs != 0.0f) atomicAdd(&a.normf[p.soff + cbase + col], cs);
+          }
+        };
+#pragma unroll 1
+        for (int pc = 0; pc < 2 && ok; ++pc) {
+          const int cc = pc == 0 ? clast : cfirst;
+          if (cc < 0) continue;
+          const int cl = tc0 + cc * 16;
+          if (pc == 1) {
+            const long long* zp = acc + (size_t)cl * 128 + m;
+#pragma unroll
+            for (int j = 0; j < 16; ++j) z[j] = zp[(size_t)j * 128];
+          }
+          if (other) {
+            const long long* zo = other + (size_t)cl * 128 + m;
+#pragma unroll
+            for (int j = 0; j < 16; ++j) z[j] += __ldcg(zo + (size_t)j * 128);
+          }
+          chunk(cl);
         }
-        chunk(cl);
       }
       if (ADJ && ok && r < p.s && rown != 0.0f) atomicAdd(&a.normf[p.soff + r], rown);
       if (!ADJ && !rec && diag) {
@@ -1352,7 +1770,8 @@ cudaError_t launch_oz_convert_slice(const PartDesc* parts, const ColBlock* block
 }
 
 cudaError_t launch_oz_step(const OzStepArgs& a, int grid, cudaStream_t s, bool adjoint) {
-  auto kern = adjoint ? oz_step_kernel<true> : oz_step_kernel<false>;
+  auto kern = a.wide ? (adjoint ? oz_step_kernel<true, true> : oz_step_kernel<false, true>)
+                     : (adjoint ? oz_step_kernel<true, false> : oz_step_kernel<false, false>);
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, OZ_SMEM);
   if (e != cudaSuccess) return e;
   const int nitems = (a.split ? 2 * a.ntiles : a.ntiles) * a.pieces;

@@ -34,6 +34,17 @@ __device__ __forceinline__ uint64_t global_ns() {
   return t;
 }
 
+// Whether the phase of this parity is done, without waiting.
+__device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
+  uint32_t done;
+  asm volatile(
+      "{\n .reg .pred p;\n mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
+      : "=r"(done)
+      : "r"(bar), "r"(parity)
+      : "memory");
+  return done != 0;
+}
+
 // Bounded wait: gives up after kWaitNs nanoseconds, or at once when another block
 // has already given up (the shared abort flag), and then raises the flag itself.
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, int32_t* abort_flag) {
@@ -104,13 +115,13 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t addr) {
 // width: 8-row groups 8 ROW bytes apart.
 template <int ROW>
 __device__ __forceinline__ uint64_t smem_desc_sw(uint32_t addr) {
-  static_assert(ROW == 32 || ROW == 64, "32- or 64-byte rows");
+  static_assert(ROW == 32 || ROW == 64 || ROW == 128, "32-, 64- or 128-byte rows");
   uint64_t d = 0;
   d |= (uint64_t)((addr >> 4) & 0x3FFF);
   d |= (uint64_t)(16 >> 4) << 16;         // leading byte offset (unused for swizzled K-major)
   d |= (uint64_t)((8 * ROW) >> 4) << 32;  // stride byte offset: next 8-row group
   d |= (uint64_t)1 << 46;                 // descriptor version
-  d |= (uint64_t)(ROW == 32 ? 6 : 4) << 61;  // 32- or 64-byte swizzle
+  d |= (uint64_t)(ROW == 32 ? 6 : (ROW == 64 ? 4 : 2)) << 61;  // 32-, 64- or 128-byte swizzle
   return d;
 }
 
