@@ -351,6 +351,24 @@ struct alignas(16) TcItem {
 };
 enum : int { TC_STEP = 0, TC_REBUILD = 1, TC_ADJOINT = 2 };
 
+// The 16-bit operand(s) of two elements e, e + 1 (e even), scaled as bits() scales one.
+template <int KIND, int NPROD>
+__device__ __forceinline__ void store_operand_pair(void* hi, void* lo, int64_t e, float x0, float x1) {
+  static_assert(KIND != 1, "16-bit kinds");
+  auto pack = [](float a, float b) {
+    uint32_t w;
+    if (KIND == 0) asm("cvt.rn.bf16x2.f32 %0, %1, %2;\n" : "=r"(w) : "f"(b), "f"(a));
+    else asm("cvt.rn.f16x2.f32 %0, %1, %2;\n" : "=r"(w) : "f"(b * 16384.0f), "f"(a * 16384.0f));
+    return w;
+  };
+  const uint32_t h = pack(x0, x1);
+  *reinterpret_cast<uint32_t*>(reinterpret_cast<uint16_t*>(hi) + e) = h;
+  if (NPROD == 3) {
+    const float h0 = Operand<KIND>::value((uint16_t)h), h1 = Operand<KIND>::value((uint16_t)(h >> 16));
+    *reinterpret_cast<uint32_t*>(reinterpret_cast<uint16_t*>(lo) + e) = pack(x0 - h0, x1 - h1);
+  }
+}
+
 // Predicated stores of one element (master and operands): the columns of a diagonal tile differ
 // in the lanes that store, and a branch per column costs more than the stores.
 template <int KIND, int NPROD>
@@ -731,6 +749,11 @@ __global__ void __launch_bounds__(TC_THREADS, 1) square_tc_persistent_kernel(TcS
     // in two halves of 16
     const int quarter = warp & 3, colq = (warp - 4) >> 2;
     const int m = quarter * 32 + lane;
+    int8_t alf;
+    if (MODE != TC_STEP) alf = a.ctl.alpha[step];  // the recorded branch
+    else if (a.tail == 1) alf = (a.ctl.traces[step - 1] <= (double)a.ctl.nocc) ? (int8_t)1 : (int8_t)-1;
+    else if (a.tail == 2) alf = (int8_t)(-a.ctl.alpha[step - 1]);
+    else alf = a.ctl.alpha[step];
     for (int i = 0;; ++i) {
       const int q = i % TC_RING;
       const bool got = __all_sync(0xffffffffu, mbar_wait(item_full(q), (i / TC_RING) & 1, abort_flag));
@@ -751,11 +774,6 @@ __global__ void __launch_bounds__(TC_THREADS, 1) square_tc_persistent_kernel(TcS
       if (t.part < 0) break;
       const TcItem& p = t;
       const int b = i & 1, u = i >> 1;
-      int8_t alf;
-      if (MODE != TC_STEP) alf = a.ctl.alpha[step];  // the recorded branch
-      else if (a.tail == 1) alf = (a.ctl.traces[step - 1] <= (double)a.ctl.nocc) ? (int8_t)1 : (int8_t)-1;
-      else if (a.tail == 2) alf = (int8_t)(-a.ctl.alpha[step - 1]);
-      else alf = a.ctl.alpha[step];
       const float* Xi = (MODE == TC_REBUILD ? a.xin : a.master[bi]) + p.off;
       float* Xo = MODE == TC_REBUILD ? a.xout : a.master[bo];
       void* ohi = MODE == TC_REBUILD ? a.xo_hi : a.op_hi[bo];
@@ -800,55 +818,85 @@ __global__ void __launch_bounds__(TC_THREADS, 1) square_tc_persistent_kernel(TcS
       for (int h = 0; h < 2; ++h) {
         if (has[0]) {
           const int cbase = c0 + colq * 32 + h * 16;
-          float x[16];
+          if (UPPER && !dgt) {
+            // Lanes l, l + 1 (l even) have rows r, r + 1 of 16 columns: they trade every second column, so
+            // that each has both rows of eight columns (those of its own parity).  The previous iterate, the
+            // new one and its operands then move two rows at a time, in half as many loads and stores.
+            // n = 30000, FP16x3: 0.405 / 0.421 -> 0.401 / 0.415 ms a step (Y / 2X - Y), n = 8000 0.100 -> 0.098:
+            // the epilogue's instructions are not what is left above the MMAs' 0.30 ms, its traffic beside the
+            // operand loads is.
+            const bool odd = lane & 1;
+            float2 y[8], x[8];
 #pragma unroll
-          for (int j = 0; j < 16; ++j) x[j] = alf > 0 ? Xi[(int64_t)(cbase + j) * ld + r] : 0.0f;
-          // the one diagonal entry of this half row, if any, goes to shared memory; one warp adds
-          // the tile's in FP64
-          float yd = 0.0f, zd = 0.0f;
-#pragma unroll
-          for (int j = 0; j < 16; ++j) {
-            const float y = __uint_as_float(v[j]) * ysc;
-            const float z = (alf > 0) ? (2.0f * x[j] - y) : y;
-            yd = (cbase + j == r) ? y : yd;
-            zd = (cbase + j == r) ? z : zd;
-            x[j] = z;
-            if (XBAR16) amax = max(amax, __float_as_uint(z) & 0x7FFFFFFFu);  // NaN bits exceed Inf
-          }
-          if (MODE == TC_STEP && diag && r >= cbase && r < cbase + 16) red[m] = make_float2(yd, zd);
-          // diagonal tiles: keep the upper triangle (c >= r) and mirror it, so X stays exactly
-          // symmetric whatever order the tensor cores sum the split products in.  Eight columns
-          // per iteration, x turning in registers: straight-line code for 16 would be refetched for every tile
-          int64_t e = p.off + (int64_t)cbase * ld + r;
-#pragma unroll 1
-          for (int q2 = 0; q2 < 2; ++q2, e += 8 * ld) {
-#pragma unroll
-            for (int j = 0; j < 8; ++j)
-              store_element_if<KIND, NPROD>(!dgt || cbase + 8 * q2 + j >= r, Xo, ohi, olo, e + (int64_t)j * ld, x[j],
-                                            XBAR16 ? x[j] * osc : x[j]);
-#pragma unroll
-            for (int j = 0; j < 8; ++j) {
-              const float y = x[j];
-              x[j] = x[8 + j];
-              x[8 + j] = y;
+            for (int k = 0; k < 8; ++k) {
+              const uint32_t got = __shfl_xor_sync(0xffffffffu, odd ? v[2 * k] : v[2 * k + 1], 1);
+              y[k].x = __uint_as_float(odd ? got : v[2 * k]);
+              y[k].y = __uint_as_float(odd ? v[2 * k + 1] : got);
             }
-          }
-          if (!UPPER || dgt) {
-            // the mirrored entries (the 16-bit kinds keep off-diagonal tiles upper only), transposed
-            // among the lanes: lane l has column cbase + l % 16 of rows rb + j, which go to row
-            // cbase + l % 16 of columns rb + j
-            transpose16(x, lane);
-            int rb = r0 + quarter * 32 + (lane & 16);
-            const int c = cbase + (lane & 15);
-            int64_t em = p.off + (int64_t)rb * ld + c;
+            const int64_t e = (int64_t)(cbase + odd) * ld + (r & ~1);
+#pragma unroll
+            for (int k = 0; k < 8; ++k)
+              x[k] = alf > 0 ? *reinterpret_cast<const float2*>(Xi + e + (int64_t)(2 * k) * ld) : make_float2(0.0f, 0.0f);
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+              const float y0 = y[k].x * ysc, y1 = y[k].y * ysc;
+              const float z0 = (alf > 0) ? (2.0f * x[k].x - y0) : y0, z1 = (alf > 0) ? (2.0f * x[k].y - y1) : y1;
+              if (XBAR16) amax = max(amax, max(__float_as_uint(z0) & 0x7FFFFFFFu, __float_as_uint(z1) & 0x7FFFFFFFu));
+              const int64_t o = p.off + e + (int64_t)(2 * k) * ld;
+              *reinterpret_cast<float2*>(Xo + o) = make_float2(z0, z1);
+              store_operand_pair<UPPER ? KIND : 0, NPROD>(ohi, olo, o, XBAR16 ? z0 * osc : z0, XBAR16 ? z1 * osc : z1);
+            }
+          } else {
+            float x[16];
+#pragma unroll
+            for (int j = 0; j < 16; ++j) x[j] = alf > 0 ? Xi[(int64_t)(cbase + j) * ld + r] : 0.0f;
+            // the one diagonal entry of this half row, if any, goes to shared memory; one warp adds
+            // the tile's in FP64
+            float yd = 0.0f, zd = 0.0f;
+#pragma unroll
+            for (int j = 0; j < 16; ++j) {
+              const float y = __uint_as_float(v[j]) * ysc;
+              const float z = (alf > 0) ? (2.0f * x[j] - y) : y;
+              yd = (cbase + j == r) ? y : yd;
+              zd = (cbase + j == r) ? z : zd;
+              x[j] = z;
+              if (XBAR16) amax = max(amax, __float_as_uint(z) & 0x7FFFFFFFu);  // NaN bits exceed Inf
+            }
+            if (MODE == TC_STEP && diag && r >= cbase && r < cbase + 16) red[m] = make_float2(yd, zd);
+            // diagonal tiles: keep the upper triangle (c >= r) and mirror it, so X stays exactly
+            // symmetric whatever order the tensor cores sum the split products in.  Eight columns
+            // per iteration, x turning in registers: straight-line code for 16 would be refetched for every tile
+            int64_t e = p.off + (int64_t)cbase * ld + r;
 #pragma unroll 1
-            for (int q2 = 0; q2 < 2; ++q2, rb += 8, em += 8 * ld) {
+            for (int q2 = 0; q2 < 2; ++q2, e += 8 * ld) {
 #pragma unroll
               for (int j = 0; j < 8; ++j)
-                store_element_if<KIND, NPROD>(!dgt || c > rb + j, Xo, ohi, olo, em + (int64_t)j * ld, x[j],
+                store_element_if<KIND, NPROD>(!dgt || cbase + 8 * q2 + j >= r, Xo, ohi, olo, e + (int64_t)j * ld, x[j],
                                               XBAR16 ? x[j] * osc : x[j]);
 #pragma unroll
-              for (int j = 0; j < 8; ++j) x[j] = x[8 + j];
+              for (int j = 0; j < 8; ++j) {
+                const float y = x[j];
+                x[j] = x[8 + j];
+                x[8 + j] = y;
+              }
+            }
+            if (!UPPER || dgt) {
+              // the mirrored entries (the 16-bit kinds keep off-diagonal tiles upper only), transposed
+              // among the lanes: lane l has column cbase + l % 16 of rows rb + j, which go to row
+              // cbase + l % 16 of columns rb + j
+              transpose16(x, lane);
+              int rb = r0 + quarter * 32 + (lane & 16);
+              const int c = cbase + (lane & 15);
+              int64_t em = p.off + (int64_t)rb * ld + c;
+#pragma unroll 1
+              for (int q2 = 0; q2 < 2; ++q2, rb += 8, em += 8 * ld) {
+#pragma unroll
+                for (int j = 0; j < 8; ++j)
+                  store_element_if<KIND, NPROD>(!dgt || c > rb + j, Xo, ohi, olo, em + (int64_t)j * ld, x[j],
+                                                XBAR16 ? x[j] * osc : x[j]);
+#pragma unroll
+                for (int j = 0; j < 8; ++j) x[j] = x[8 + j];
+              }
             }
           }
         }
