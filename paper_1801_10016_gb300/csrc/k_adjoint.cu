@@ -168,9 +168,11 @@ __global__ void __launch_bounds__(256, 4) adj_step_kernel(const PartDesc* __rest
 
 // dL/dH on the CSR pattern: for every stored (r, col), the sum over the parts k that
 // hold r (membership list of r) and col of -Xbar0_k[col, r] / (eps_max - eps_min), in
-// the fixed membership order (ascending part id).  One warp per row, lanes over the row's entries.  With
-// upper_block > 0 only the tiles of that edge on or above the diagonal hold Xbar0 (the
-// emulated adjoint); the symmetric entry is read from there.
+// the fixed membership order (ascending part id).  HBAR_WARPS warps per row, lanes over the row's
+// entries: the chain entry -> its column's parts -> Xbar0 is all latency (one warp per row: 71 us on
+// 4,096 orbitals and 217 us on 8,000, four 35 and 148).  With upper_block > 0 only the tiles of that
+// edge on or above the diagonal hold Xbar0 (the emulated adjoint); the symmetric entry is read from there.
+constexpr int HBAR_WARPS = 4;
 template <typename T>
 __global__ void __launch_bounds__(256) adj_hbar_kernel(int64_t n, const int64_t* __restrict__ rowptr,
                                                        const int32_t* __restrict__ colind,
@@ -184,13 +186,15 @@ __global__ void __launch_bounds__(256) adj_hbar_kernel(int64_t n, const int64_t*
                                                        int upper_block) {
   const int nsteps = st->steps;
   const T* XB = (nsteps & 1) ? xb1 : xb0;
-  const double scale = -1.0 / (st->eps_max - st->eps_min);
+  // the bounds kernel's 1 / (eps_max - eps_min), correctly rounded; a division in every thread took 7 us
+  const double scale = -(st->inv_hi != 0.0 ? st->inv_hi : 1.0 / (st->eps_max - st->eps_min));
   const int lane = threadIdx.x & 31;
   const int64_t warp = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   const int64_t nwarps = (int64_t)gridDim.x * (blockDim.x >> 5);
-  for (int64_t r = warp; r < n; r += nwarps) {
+  for (int64_t w = warp; w < n * HBAR_WARPS; w += nwarps) {
+    const int64_t r = w / HBAR_WARPS;
     const int64_t m0 = memptr[r], m1 = memptr[r + 1];
-    for (int64_t q = rowptr[r] + lane; q < rowptr[r + 1]; q += 32) {
+    for (int64_t q = rowptr[r] + 32 * (w % HBAR_WARPS) + lane; q < rowptr[r + 1]; q += 32 * HBAR_WARPS) {
       const int32_t col = colind[q];
       // the parts holding both r and col: the intersection of their membership lists, both
       // in ascending part order, walked as a merge (the same parts in the same order as a
@@ -232,7 +236,8 @@ cudaError_t launch_adj_hbar(int64_t n, const int64_t* rowptr, const int32_t* col
                             const int32_t* mempart, const int32_t* memloc, const PartDesc* parts,
                             const int32_t* Sall, const T* xb0, const T* xb1, double* hbar, const DevState* st,
                             cudaStream_t s, int upper_block) {
-  adj_hbar_kernel<T><<<608, 256, 0, s>>>(n, rowptr, colind, memptr, mempart, memloc, parts, Sall, xb0, xb1, hbar, st,
+  const int64_t blocks = (n * HBAR_WARPS + 7) / 8;
+  adj_hbar_kernel<T><<<(int)(blocks < 1216 ? blocks : 1216), 256, 0, s>>>(n, rowptr, colind, memptr, mempart, memloc, parts, Sall, xb0, xb1, hbar, st,
                                          upper_block);
   return cudaGetLastError();
 }

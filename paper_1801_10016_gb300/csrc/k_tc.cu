@@ -1284,7 +1284,9 @@ cudaError_t launch_tc_adjoint(const TcStepArgs& a, int grid, bool rebuild, cudaS
   return rebuild ? launch_tc_persistent<2, 3, TC_REBUILD>(a, g, s) : launch_tc_persistent<2, 3, TC_ADJOINT>(a, g, s);
 }
 
-// FP16 hi + lo operands of an FP32 arena, one warp per column up to ld: of x 2^-sig[part]
+// FP16 hi + lo operands of an FP32 arena, one warp per column up to ld, the rows on or above its
+// diagonal block (all that the reverse steps read), four a lane (4,096 orbitals: 18 -> 9 us a launch, of whole
+// columns an entry a lane): of x 2^-sig[part]
 // (the FP16 adjoint's seed Xbar; sig NULL: of x, an iterate).  Skipped where need > n - tail
 // (a checkpoint the reverse sweep does not reach).
 __global__ void __launch_bounds__(256) split_f16_kernel(const PartDesc* __restrict__ parts,
@@ -1299,7 +1301,11 @@ __global__ void __launch_bounds__(256) split_f16_kernel(const PartDesc* __restri
   if (j >= p.ld) return;
   const float f = sig ? pow2i(-sig[b.part]) : 1.0f;
   const int64_t cbase = p.off + (int64_t)j * p.ld;
-  for (int r = lane; r < p.ld; r += 32) store_operands<2, 3>(hi, lo, cbase + r, x[cbase + r] * f);
+  const int rend = min(p.ld, (j / 128 + 1) * 128);
+  for (int r = 4 * lane; r < rend; r += 128) {  // rend and cbase are multiples of 128
+    const float4 v = *reinterpret_cast<const float4*>(x + cbase + r);
+    store_operand_quad<2, 3>(hi, lo, cbase + r, {v.x * f, v.y * f, v.z * f, v.w * f});
+  }
 }
 
 // Scales of the seed Xbar's FP16 operands: each part's largest |x| into xb_max (one warp
