@@ -31,12 +31,12 @@ PEAKS_FILE = os.path.join(ROOT, "MEASURED_PEAKS.json")
 # nominal dense rates (TFLOP/s) used to derive a dtype's peak from the measured bf16 one
 NOMINAL = {"bf16": 2250.0, "tf32": 1100.0, "fp64": 1.25}
 # DRAM bytes (read + write) per launch of the step kernel, from one ncu capture of the kernel
-# as it is now (the summaries are under profiles/): each step on tb8k (tb30k's part sizes)
+# as it is now (the summaries are under profiles/), the mean of a Y and a 2X - Y step: each on tb8k (tb30k's part sizes)
 # scaled to tb30k by arena elements; an entry is dropped when its kernel changes, and the
 # line then reports null
 TB8K_TO_TB30K = 191545344 / 38469632
-TRAFFIC = {("tb30k", "fp64"): 0.5270e9 * TB8K_TO_TB30K, ("tb30k", "fp64e"): 1.0497e9 * TB8K_TO_TB30K,
-           ("tb30k", "fp16x3"): 0.2712e9 * TB8K_TO_TB30K, ("tb30k", "tf32x3"): 0.7313e9 * TB8K_TO_TB30K}
+TRAFFIC = {("tb30k", "fp64"): 0.4998e9 * TB8K_TO_TB30K, ("tb30k", "fp64e"): 0.6776e9 * TB8K_TO_TB30K,
+           ("tb30k", "fp16x3"): 0.2392e9 * TB8K_TO_TB30K, ("tb30k", "tf32x3"): 0.7147e9 * TB8K_TO_TB30K}
 
 
 def dist_env():
@@ -230,7 +230,7 @@ def fp64_roofline(precision, sizes, avg_launch_ms, peaks, src, workload):
     import numpy as np
     if precision == "fp64e":
         flops = alg_flops(sizes, OZ_PRODUCTS)
-        exe = tc_exec_flops(sizes, 32, OZ_PRODUCTS, trim=True)
+        exe = tc_exec_flops(sizes, 16, OZ_PRODUCTS, trim=True)  # wide slices: K rounded to an MMA's 16
         t = avg_launch_ms / 1e3
         achieved = flops / t / 1e12
         peak = peaks["bf16_tflops"]
