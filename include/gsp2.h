@@ -68,7 +68,11 @@ typedef enum {
   GSP2_PREC_TF32X3 = 5, /* split operands hi+lo in TF32, three products, FP32 accumulate */
   GSP2_PREC_FP64_EMU = 6, /* FP64 results; every product X X rebuilt from 5 digits of X (11, 8,
                              11, 8 and 11 bits) held in FP16 (15 tensor-core products per tile, groups
-                             summed as 64-bit fixed point), master copy in that fixed point */
+                             summed as 64-bit fixed point), master copy in that fixed point.  An
+                             entry of X X is off by about 1e-14 (rms 0.3e-15 sqrt(K), K = core + halo
+                             size); by at most K 2^-49 where entries of one magnitude make the
+                             products left out add up.  Such parts also take 2 to 4 times as long: their
+                             digit sums are added up in shorter rounds, which keeps them exact */
   GSP2_PREC_FP16X3 = 7  /* split operands hi+lo in FP16 of X 2^14 (22 bits like TF32X3, entries
                            down to 2^-28 in FP16's normal range), three products at the
                            16-bit tensor rate, FP32 accumulate, sums scaled back by 2^-28 */

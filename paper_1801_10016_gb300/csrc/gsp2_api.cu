@@ -39,6 +39,7 @@ struct WsLayout {
   size_t oz_slice[2][OZ_SLICES];  // FP16 digit arenas, two buffers (read / written by a step)
   size_t oz_maps;                 // CUtensorMap[2][OZ_SLICES][nparts], K-major boxes
   size_t oz_maps_mn;              // the same, MN-major boxes
+  size_t oz_coh;                  // coherent parts (OzStepArgs), forward and adjoint: int32[2][nparts] and OzAgain each
   size_t oz_acc;                  // int64[OZ_MAX_GRID][128 * 128] partial sums of the emulated step
   // emulated FP64 adjoint: digit sets 0..k-1 hold X_{c0+j} of a checkpoint segment, set k
   // holds Xbar / 2^sig; their tensor maps; row norms and per-part scales of Xbar
@@ -261,6 +262,9 @@ extern "C" void gsp2_default_options(gsp2_options* o) {
 
 extern "C" const char* gsp2_last_error(gsp2_handle h) { return h ? h->err.c_str() : t_create_err.c_str(); }
 
+// Words of the list of coherent parts (OzStepArgs) of one direction.
+static size_t oz_coh_words(size_t nparts) { return 2 * nparts + sizeof(OzAgain) / sizeof(int32_t); }
+
 // Columns of the graph refresh that fit its buffer: the whole graph (at most two edges per
 // stored value of P and the diagonal) up to 64 MB, then ranges of rows (one row at least)
 static int64_t graph_cap(const gsp2_plan* h) {
@@ -383,6 +387,7 @@ static void build_layout(gsp2_plan* h) {
       L.oz_maps = take((size_t)2 * OZ_SLICES * h->parts.size() * 128);
       L.oz_maps_mn = take((size_t)2 * OZ_SLICES * h->parts.size() * 128);
       L.oz_acc = take((size_t)OZ_MAX_GRID * 128 * 128 * 8);
+      L.oz_coh = take(2 * oz_coh_words(h->parts.size()) * sizeof(int32_t));
     }
     L.arena0 = L.d[0];
     L.arena1 = L.d[1];
@@ -408,6 +413,7 @@ static void build_layout(gsp2_plan* h) {
     L.oz_maps = take((size_t)2 * OZ_SLICES * h->parts.size() * 128);
     L.oz_maps_mn = take((size_t)2 * OZ_SLICES * h->parts.size() * 128);
     L.oz_acc = take((size_t)OZ_MAX_GRID * 128 * 128 * 8);
+    L.oz_coh = take(2 * oz_coh_words(h->parts.size()) * sizeof(int32_t));
   }
   L.adj_dig.clear();
   L.adj_maps = L.adj_maps_mn = L.adj_norm = L.adj_sig = L.adj_normf = 0;
@@ -1093,6 +1099,9 @@ static OzStepArgs oz_args(gsp2_plan* h, const StepCtl& ctl) {
   a.nslots = h->nslots_tc;
   a.acc = (long long*)(w + L.oz_acc);
   a.ctl = ctl;
+  a.coh = (int32_t*)(w + L.oz_coh);
+  a.coh_new = a.coh + a.nparts;
+  a.again = (OzAgain*)(a.coh + 2 * a.nparts);
   a.tile_ctr = h->opt.tile_claim ? (uint32_t*)(w + L.tile_ctr) : nullptr;
   a.halves = h->halves ? 1 : 0;
   a.wide = oz_wide(h) ? 1 : 0;
@@ -1185,7 +1194,7 @@ static gsp2_status enqueue_forward(gsp2_plan* h, const double* hv, double* pv, i
   auto on = [&]() { return seg >= seg_lo && seg <= seg_hi; };
   if (on()) {
     CU(h, launch_reset(st, alpha, mode == MODE_REPLAY ? alpha_user : nullptr, nsteps, h->opt.max_steps + HIST_EXTRA,
-                       s));
+                       h->use_oz ? (int32_t*)(w + L.oz_coh) : nullptr, (int)h->parts.size(), s));
     CU(h, launch_bounds(h->n, rp, ci, hv, slots, BOUNDS_BLOCKS, st, s));
     CU(h, launch_x0_values(h->n, rp, ci, hv, st, x0, h->num_sms, s));
   }
@@ -1786,6 +1795,7 @@ static gsp2_status enqueue_backward_emu(gsp2_plan* h, const double* pbar, double
   int32_t* sig = (int32_t*)(w + L.adj_sig);
   const int k = h->opt.ckpt_every, M = backward_steps(h);
   const int np = (int)h->parts.size();
+  int32_t* coh = (int32_t*)(w + L.oz_coh) + oz_coh_words(np);  // the reverse steps' own
   StepCtl ctl{st, alpha, (double*)(w + L.traces), (double*)(w + L.idem), h->nocc, h->opt.idem_tol,
               h->opt.trace_tol, MODE_REPLAY, M, 1, 0};
   // digit set j of buffer b (the iterates X_{c0+j} of a checkpoint segment), and Xbar's set
@@ -1833,6 +1843,9 @@ static gsp2_status enqueue_backward_emu(gsp2_plan* h, const double* pbar, double
       a.maps_mn_b = smaps(L.adj_maps_mn, xset);
       a.sig = sig;
       a.normf = normf;
+      a.coh = coh;
+      a.coh_new = coh + np;
+      a.again = (OzAgain*)(coh + 2 * np);
       a.xin = xb0;
       a.xout = xb1;
       a.step = i;
@@ -1846,7 +1859,7 @@ static gsp2_status enqueue_backward_emu(gsp2_plan* h, const double* pbar, double
     CU(h, cudaMemsetAsync(normf, 0, h->S.size() * sizeof(float), s));
     CU(h, launch_adj_seed<double>(parts, gbl, (int)h->gblocks.size(), Sall, (const int32_t*)(w + L.invperm),
                                   (const int64_t*)(w + L.pcolptr), pbar, xb0, s));
-    CU(h, launch_oz_adj_scale(parts, np, tct, ntc, xb0, xb1, 0, norm, sig, st, s));
+    CU(h, launch_oz_adj_scale(parts, np, tct, ntc, xb0, xb1, 0, norm, sig, coh, st, s));
     CU(h, launch_oz_digits(parts, gbl_ld, ngb, xb0, xb1, 0, 0, dset(xset), sig, st, s));
     return GSP2_OK;
   };

@@ -8,6 +8,7 @@
 //     ascending), the scatter permutation, the work lists and the per-step state.
 #pragma once
 
+#include <cstddef>
 #include <cstdint>
 #include <cuda_runtime.h>
 
@@ -42,15 +43,19 @@ struct DevState {
   double eps_min, eps_max;
   double idem_fro;     // idempotency report of the final P (core columns), -1 if not run
   unsigned int counter;
-  int32_t stopped;     // 1: no further purification steps this call
+  int32_t tail_left;   // FP64 path: alternating tail steps still to run (0: none)
+  int32_t stopped;     // 1: no further purification steps this call (read with the next word)
+  int32_t coherent;    // emulated steps: some part was found coherent (OzStepArgs)
   int32_t steps;       // purification steps applied so far
   int32_t status;      // gsp2_status detected on the device
   int32_t nonfinite;   // set by any block that meets NaN/Inf
   int32_t fp64_steps;
   int32_t timeout;     // a bounded device wait gave up
-  int32_t tail_left;   // FP64 path: alternating tail steps still to run (0: none)
+  int32_t pad;
   double inv_hi, inv_lo;  // 1 / (eps_max - eps_min) = inv_hi + inv_lo; inv_hi = 0: to be divided by
 };
+
+static_assert(offsetof(DevState, stopped) % 8 == 0, "stopped and coherent are read together");
 
 enum : int32_t { ST_OK = 0, ST_NOT_CONVERGED = 5, ST_TRACE = 6, ST_NONFINITE = 7, ST_TIMEOUT = 9 };
 enum : int32_t { MODE_RECORD = 0, MODE_REPLAY = 1 };
@@ -165,6 +170,14 @@ struct OzSlices {
   uint16_t* s[OZ_SLICES];  // FP16 digit arenas (same element indexing as the arenas)
 };
 
+// Where the blocks of a launch meet to form coherent parts again.
+struct OzAgain {
+  int32_t go;    // the launch's place (oz_step_kernel): its items are done, its coherent parts' can be taken again
+  int32_t ctr;   // items taken (of all items, those of other parts being passed over)
+  int32_t done;  // items done
+  int32_t pad;
+};
+
 // One emulated step: digits of X_{step-1} are read from buffer (step-1)&1 and the digits
 // of X_step written to buffer step&1 (SQ_FORWARD and the tail modes).  SQ_RECOMPUTE (the
 // adjoint's rebuilt iterates) reads the digit set `maps` points at and writes digits[0],
@@ -202,6 +215,11 @@ struct OzStepArgs {
   int pieces;            // column pieces of a tile, each an item of its own (1 or 2; wide: 1)
   int wide;              // K slices of OZ_BK_WIDE in a ring of single digit tiles, not of OZ_BK in units of five
   int halves;            // the plan's items may be split: unsplit ones drain at the same boundary
+  // Parts whose digits are coherent (some sum of digit products reached 2^24): coh[part] is the step that
+  // found it (adjoint: counted back from the last step), OZ_INCOHERENT if none; coh_new[part] is set by
+  // the items of a launch, and cleared by its last block once the part has been formed again in brief rounds
+  int32_t *coh, *coh_new;
+  OzAgain* again;
   long long* split_acc;  // [2 ntiles][128 x 128], indexed by item code 2 t + h
   uint32_t* split_cnt;   // [ntiles]
   const int32_t* split_items;  // [2 ntiles]: item codes in the order the CTAs take them
@@ -211,11 +229,18 @@ struct OzStepArgs {
   // b + gridDim.x, ...
   uint32_t* tile_ctr;
 };
+constexpr int32_t OZ_INCOHERENT = 0x7FFFFFFF;
 constexpr int32_t OZ_SIG_NONFINITE = 0x7FFF;  // scale of a part whose Xbar holds NaN or Inf
 
 // ------------------------------------------------------------------ device helpers
 
 __device__ __forceinline__ double ld_cg(const double* p) { return __ldcg(p); }
+// Two consecutive words (8-byte aligned) in one volatile load.
+__device__ __forceinline__ uint2 ld_volatile2(const void* p) {
+  uint2 v;
+  asm volatile("ld.volatile.global.v2.u32 {%0, %1}, [%2];\n" : "=r"(v.x), "=r"(v.y) : "l"(p) : "memory");
+  return v;
+}
 
 // Programmatic dependent launch: the next launch of the stream may become resident (its blocks
 // set up barriers and TMEM while this one drains), and this one waits here until the launch

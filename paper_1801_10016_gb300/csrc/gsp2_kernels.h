@@ -5,8 +5,8 @@
 
 namespace gsp2 {
 
-cudaError_t launch_reset(DevState* st, int8_t* alpha, const int8_t* alpha_in, int n_in, int n_alpha,
-                         cudaStream_t s);
+cudaError_t launch_reset(DevState* st, int8_t* alpha, const int8_t* alpha_in, int n_in, int n_alpha, int32_t* coh,
+                         int nparts, cudaStream_t s);
 cudaError_t launch_bounds(int64_t n, const int64_t* rowptr, const int32_t* colind, const double* vals,
                           double2* slots, int nblocks, DevState* st, cudaStream_t s);
 cudaError_t launch_gather(const PartDesc* parts, const ColBlock* blocks, int nblocks, const int32_t* Sall,
@@ -71,8 +71,8 @@ cudaError_t launch_oz_gather(const PartDesc* parts, const ColBlock* blocks, int 
                              double* arena, const OzSlices& dig, double* slots, const StepCtl& ctl, cudaStream_t s);
 // the emulated adjoint's Xbar digits: row norms and per-part scales, then the digits
 cudaError_t launch_oz_adj_scale(const PartDesc* parts, int nparts, const Tile* tiles, int ntiles, const double* xb0,
-                                const double* xb1, int after, double* norm, int32_t* sig, const DevState* st,
-                                cudaStream_t s);
+                                const double* xb1, int after, double* norm, int32_t* sig, int32_t* coh,
+                                const DevState* st, cudaStream_t s);
 cudaError_t launch_oz_digits(const PartDesc* parts, const ColBlock* blocks, int nblocks, const double* x0,
                              const double* x1, int after, int need, const OzSlices& out, const int32_t* sig,
                              const DevState* st, cudaStream_t s);

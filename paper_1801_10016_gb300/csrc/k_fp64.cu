@@ -128,8 +128,10 @@ __global__ void __launch_bounds__(256) bounds_kernel(int64_t n, const int64_t* _
   }
 }
 
-// Resets the per-call state; must run before bounds_kernel on the same stream.
-__global__ void reset_kernel(DevState* st, int8_t* alpha, const int8_t* alpha_in, int n_in, int n_alpha) {
+// Resets the per-call state, and (emulated steps) the list of coherent parts coh[2][nparts], again; must run
+// before bounds_kernel on the same stream.
+__global__ void reset_kernel(DevState* st, int8_t* alpha, const int8_t* alpha_in, int n_in, int n_alpha, int32_t* coh,
+                             int nparts) {
   if (threadIdx.x == 0 && blockIdx.x == 0) {
     st->stopped = 0;
     st->steps = 0;
@@ -138,11 +140,15 @@ __global__ void reset_kernel(DevState* st, int8_t* alpha, const int8_t* alpha_in
     st->fp64_steps = 0;
     st->timeout = 0;
     st->tail_left = 0;
+    st->coherent = 0;
     st->idem_fro = -1.0;
     st->counter = 0;
   }
   for (int i = threadIdx.x; i < n_alpha; i += blockDim.x)
     alpha[i] = (alpha_in != nullptr && i >= 1 && i <= n_in) ? alpha_in[i - 1] : (int8_t)0;
+  if (coh)
+    for (int i = threadIdx.x; i < 2 * nparts + (int)(sizeof(OzAgain) / 4); i += blockDim.x)
+      coh[i] = i < nparts ? OZ_INCOHERENT : 0;
 }
 
 // ------------------------------------------------------------------------------------
@@ -572,9 +578,9 @@ __global__ void __launch_bounds__(256) symmetrize_kernel(const PartDesc* __restr
 // ------------------------------------------------------------------------------------
 // launch wrappers
 // ------------------------------------------------------------------------------------
-cudaError_t launch_reset(DevState* st, int8_t* alpha, const int8_t* alpha_in, int n_in, int n_alpha,
-                         cudaStream_t s) {
-  reset_kernel<<<1, 256, 0, s>>>(st, alpha, alpha_in, n_in, n_alpha);
+cudaError_t launch_reset(DevState* st, int8_t* alpha, const int8_t* alpha_in, int n_in, int n_alpha, int32_t* coh,
+                         int nparts, cudaStream_t s) {
+  reset_kernel<<<1, 256, 0, s>>>(st, alpha, alpha_in, n_in, n_alpha, coh, nparts);
   return cudaGetLastError();
 }
 

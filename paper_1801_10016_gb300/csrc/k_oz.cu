@@ -12,12 +12,12 @@
 //   X X = sum_{a+b<T} 2^{-(e_a+e_b)} S_a S_b + (terms of order 2^-47): 15 products.
 //
 // The products are summed in FP32 in TMEM, in six accumulators.  Five of them hold integers
-// (in units of their own scale) that stay below 2^24 and so are exact: (0,0), because
+// (in units of their own scale), which FP32 keeps exactly while they stay below 2^24: (0,0), because
 // ||X||_2 <= 1 bounds sum_k |x_ik x_kj| by 1; (0,1) + (1,0) and (0,2) + (2,0), at most 2^19
 // and 2^22 times the row 1-norm sum_k |x_ik| (1 to 2 for the localised iterates of a gapped
-// system; for rows spread over all K columns the digits behave like independent values,
+// system; for rows spread over all K columns whose digits behave like independent values,
 // about 2^18 and 2^21); (1,1), whose diagonal is a sum of squares, K 2^12.4 for digits
-// spread over their range; and (1,2) + (2,1) + (0,3) + (3,0), about sqrt(K) 2^16 on dense rows.
+// spread over their range; and (1,2) + (2,1) + (0,3) + (3,0), about sqrt(K) 2^16 on such rows.
 // The width of digit 1 follows from (1,1) staying below 2^24 up to K = 2048 (longer K is
 // drained every 2048), that of digit 3 from the fifth accumulator at the same K (with 9 bits its
 // largest sums passed 2^24 on dense rows, and the tensor core's truncation left 1.1e-13 at K = 2,049);
@@ -26,6 +26,18 @@
 // the sixth accumulator, whose FP32 rounding lies below the dropped products.  Digits of 7
 // bits in BF16, whose 8-bit significand caps the width, took 7 digits and 28 products for an
 // error per entry of 1.25e-14 at K = 1,184 on dense rows; these give 1.0e-14.
+//
+// That is how digits behave on most inputs, not a bound.  On coherent rows (entries of one magnitude,
+// or slowly varying: the projectors of a Hadamard matrix, of a metallic ring, of rank 1) sums reach
+// 2^26 in (0,2) and 2^28 in (1,2) + (0,3), and truncation there left up to 2.4e-11 a step.  So the drains
+// look at every sum, and a part of which one has reached 2^24 is formed again, by the last block of the same launch,
+// in brief rounds: the accumulators are drained every 32 columns, within which the digits' ranges
+// bound every sum by 2^23.8 (rows of 0 <= X <= 1 have off-diagonal 2-norm <= 1/2, and 32 such entries add up to at
+// most (1 + sqrt(33)) / 2; the adjoint's operands likewise).  From the next step on the part takes brief rounds at once.
+// What a coherent row then loses is the products left out, whose bound is K 2^-49 (4.8e-12 met at K =
+// 4,096; the seven digits of 7 bits left out 1.5 times that).  A partial sum that passes 2^24 and comes back in
+// every tile of its part would not be seen; (1,1) cannot do so (Cauchy-Schwarz against the diagonal),
+// and on the inputs above the largest partial sum lies within 2^0.3 of the largest sum.
 // The accumulators are added as integers into a 64-bit fixed point (resolution 2^-56; the
 // sixth rounded to it), and a final elementwise pass forms X_new = Y or 2X - Y on that
 // grid (the master copy of the iterate stays in this fixed point), the core traces in FP64,
@@ -269,13 +281,19 @@ __global__ void __launch_bounds__(256) oz_norm_kernel(const PartDesc* __restrict
 
 // Scale of each part's Xbar digits: the smallest sig with 2^sig >= 2 max_r ||xbar_r||_2
 // (with a relative margin of 2^-20 over the rounding of the FP64 sums), 0 for a zero Xbar,
-// OZ_SIG_NONFINITE where a row norm is NaN or Inf.  Clears the norms for the next step.
-// One CTA per part.
+// OZ_SIG_NONFINITE where a row norm is NaN or Inf.  Clears the norms for the next step, and at the
+// seed the list of coherent parts coh[2][nparts], again.  One CTA per part.
 __global__ void __launch_bounds__(256) oz_scale_kernel(const PartDesc* __restrict__ parts, int after,
                                                        double* __restrict__ norm, int32_t* __restrict__ sig,
-                                                       const DevState* st) {
+                                                       int32_t* __restrict__ coh, const DevState* st) {
   const int n = *(volatile const int32_t*)&st->steps;
   if (after > n) return;
+  if (after == 0 && threadIdx.x == 0) {
+    coh[blockIdx.x] = OZ_INCOHERENT;
+    coh[gridDim.x + blockIdx.x] = 0;
+    if (blockIdx.x == 0)
+      for (int i = 0; i < (int)(sizeof(OzAgain) / 4); ++i) coh[2 * gridDim.x + i] = 0;
+  }
   const PartDesc p = parts[blockIdx.x];
   __shared__ double smax[8];
   double m = 0.0;
@@ -358,8 +376,8 @@ __global__ void __launch_bounds__(256) oz_digits_kernel(const PartDesc* __restri
 // triangle), and adds the core traces, while the MMAs of the next tile's first pass run.  The new
 // iterate is written with evict-first stores: the next step reads it after this launch,
 // and keeping it out of L2 leaves room for the digit panels the running tiles share.  The last block
-// runs the step bookkeeping.  K beyond 2048 is taken in rounds of both passes, so that the sums stay
-// exact (see the top).  n = 30000 (256 parts), per step: narrow 1.69, wide 1.59 ms; the MMAs at the
+// runs the step bookkeeping, after it has formed again the parts whose sums were found too large (brief
+// items, see the top).  K beyond 2048 is taken in rounds of both passes.  n = 30000 (256 parts), per step: narrow 1.69, wide 1.59 ms; the MMAs at the
 // measured 16-bit peak take 1.15, without loads or epilogue 1.29, with loads 1.32, with drains 1.43.
 //
 // 20 warps: warps 0 and 2 TMA (rows I and rows J: one warp's work per tile would hold
@@ -377,13 +395,16 @@ constexpr int OZ_BARS = 2 * OZ_GROUPS + OZ_TILES + 4 + 1;        // mbarriers of
 constexpr int OZ_EPI_WARPS = 16;                                 // 4 per TMEM lane quarter
 constexpr int OZ_THREADS = 32 * (4 + OZ_EPI_WARPS);
 constexpr int OZ_RING = 4;  // dynamic schedule: tiles claimed ahead of the MMA and epilogue warps
-// a claimed item as the producer passes it on: code < 0 ends the walk
+// a claimed item as the producer passes it on (code < 0: none)
 struct alignas(16) OzItem {
   int64_t off, soff;
   int32_t code, ti, tj, slot;
   int32_t part, s, c, ld;
-  int32_t piece, pad[3];
+  int32_t piece, brief;  // brief: rounds of one K = 32 slice
+  int32_t rounds, pad;   // rounds of both passes
 };
+constexpr int OZ_END = -1, OZ_PAUSE = -2;  // codes of no item: the walk ends; it waits for the last block's decision
+
 constexpr int OZ_SMEM = (int)OZ_RING_B + 1024 + 8 * OZ_BARS + 16 + 16 * 128 +
                         8 * 2 * OZ_RING + (int)sizeof(OzItem) * OZ_RING;
 static_assert(OZ_UNITS * OZ_UNIT_B <= OZ_RING_B && OZ_UNITS <= OZ_GROUPS, "the narrow ring within the wide one's space");
@@ -498,12 +519,14 @@ __host__ __device__ constexpr uint32_t oz_magic(int M) { return ((uint32_t)(150 
 // z[j] += sgn (u[j] + oz_magic(M)) 2^SHIFT for one accumulator of one 16-column chunk, where
 // u = v 2^M is the integer its FP32 sums v hold at the scale 2^-M (the sixth accumulator: v 2^M
 // rounded); the constants oz_magic(M) 2^SHIFT of all accumulators are taken off once, where z
-// starts (oz_offset; 64-bit arithmetic modulo 2^64).  A chunk whose integers all lie below
+// starts (kOzOffset; 64-bit arithmetic modulo 2^64).  A chunk whose integers all lie below
 // 2^22 in magnitude is converted without the conversion unit, through the float bits, and a 32 x 32 ->
 // 64-bit multiply-add (by the power of two, or on the upper word for shifts of 32 and more)
 // accumulates it; any other chunk goes through the exact rounding conversion of v 2^M (|u| < 2^31).
-template <int M, int SHIFT>
-__device__ __forceinline__ void oz_drain_slot(uint32_t taddr, int sgn, long long (&z)[16]) {
+// EXACT: mark(largest |u| 2^-24) where FP32 need not have held an integer: from 2^24 on, which only the second
+// branch can meet (EVERY: always).
+template <int M, int SHIFT, bool EXACT, bool EVERY, typename Mark>
+__device__ __forceinline__ void oz_drain_slot(uint32_t taddr, int sgn, const Mark& mark, long long (&z)[16]) {
   uint32_t v[16];
   tmem_ld16(taddr, v);
   const float magic = __uint_as_float(oz_magic(M));
@@ -511,6 +534,8 @@ __device__ __forceinline__ void oz_drain_slot(uint32_t taddr, int sgn, long long
   float mx = 0.0f;
 #pragma unroll
   for (int j = 0; j < 16; ++j) mx = fmaxf(mx, fabsf(__uint_as_float(v[j])));
+  const float to1 = __uint_as_float((uint32_t)(103 + M) << 23);  // 2^(M - 24)
+  if (EXACT && EVERY) mark(mx * to1);
   if (__all_sync(0xffffffffu, mx < lim)) {
     const int32_t mult = sgn * (1 << (SHIFT & 31));
 #pragma unroll
@@ -523,6 +548,7 @@ __device__ __forceinline__ void oz_drain_slot(uint32_t taddr, int sgn, long long
       }
     }
   } else {
+    if (EXACT && !EVERY && mx * to1 >= 1.0f) mark(mx * to1);
     const float scale = __uint_as_float((uint32_t)(127 + M) << 23);  // 2^M
 #pragma unroll
     for (int j = 0; j < 16; ++j) {
@@ -540,27 +566,31 @@ struct OzSlot {
   static constexpr int M = oz_rho(A) + oz_rho(B) - (oz_e(A) + oz_e(B) - GRID);
   static constexpr int SHIFT = 56 - GRID;
   static constexpr unsigned long long offset = (unsigned long long)oz_magic(M) << SHIFT;
-  static __device__ __forceinline__ void drain(uint32_t taddr, int sgn, long long (&z)[16]) {
-    oz_drain_slot<M, SHIFT>(taddr + oz_col(A, B), sgn, z);
+  template <bool EVERY, typename Mark>
+  static __device__ __forceinline__ void drain(uint32_t taddr, int sgn, const Mark& mark, long long (&z)[16]) {
+    oz_drain_slot<M, SHIFT, GRID == oz_e(A) + oz_e(B), EVERY>(taddr + oz_col(A, B), sgn, mark, z);
   }
 };
 using OzSixth = OzSlot<0, 4, 56>;
 
 // The first pass of one chunk, in two halves: the columns the second pass reuses, then the
 // columns that hold the sums from then on, into z (negated for sgn < 0).
-__device__ __forceinline__ void oz_drain_high_a(uint32_t taddr, int sgn, long long (&z)[16]) {
-  OzSixth::drain(taddr, sgn, z);
-  OzSlot<0, 3>::drain(taddr, sgn, z);
+template <bool EVERY, typename Mark>
+__device__ __forceinline__ void oz_drain_high_a(uint32_t taddr, int sgn, const Mark& mark, long long (&z)[16]) {
+  OzSixth::template drain<EVERY>(taddr, sgn, mark, z);
+  OzSlot<0, 3>::template drain<EVERY>(taddr, sgn, mark, z);
 }
-__device__ __forceinline__ void oz_drain_high_b(uint32_t taddr, int sgn, long long (&z)[16]) {
-  OzSlot<0, 2>::drain(taddr, sgn, z);
-  OzSlot<1, 1>::drain(taddr, sgn, z);
+template <bool EVERY, typename Mark>
+__device__ __forceinline__ void oz_drain_high_b(uint32_t taddr, int sgn, const Mark& mark, long long (&z)[16]) {
+  OzSlot<0, 2>::template drain<EVERY>(taddr, sgn, mark, z);
+  OzSlot<1, 1>::template drain<EVERY>(taddr, sgn, mark, z);
 }
 
 // The second pass of one chunk into z.
-__device__ __forceinline__ void oz_drain_low(uint32_t taddr, int sgn, long long (&z)[16]) {
-  OzSlot<0, 0>::drain(taddr, sgn, z);
-  OzSlot<0, 1>::drain(taddr, sgn, z);
+template <bool EVERY, typename Mark>
+__device__ __forceinline__ void oz_drain_low(uint32_t taddr, int sgn, const Mark& mark, long long (&z)[16]) {
+  OzSlot<0, 0>::template drain<EVERY>(taddr, sgn, mark, z);
+  OzSlot<0, 1>::template drain<EVERY>(taddr, sgn, mark, z);
 }
 
 // Where z starts: less the constants that the six drains of a round add.
@@ -641,11 +671,77 @@ __device__ __forceinline__ void store_digits_if(bool on, uint16_t* d, size_t dst
       : "memory");
 }
 
+// K slices of a part of size sz; brief items count slices of 32 in either form (wide: halves of the
+// loaded ones).
+template <bool WIDE>
+__device__ __forceinline__ int oz_nslices(int sz, bool brief) {
+  constexpr int BK = WIDE ? OZ_BK_WIDE : OZ_BK;
+  return brief ? (sz + OZ_BK - 1) / OZ_BK : (sz + BK - 1) / BK;
+}
+// K slices [x, y) of an item: all of them (the adjoint's first ns slices multiply Xbar by X, the rest X
+// by Xbar) or one half (0, 1; -1 none), up to or from slice z.
 template <bool ADJ, bool WIDE>
-__global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
+__device__ __forceinline__ int3 oz_slices(int sz, int half, bool brief) {
+  const int ns = oz_nslices<WIDE>(sz, brief), all = ADJ ? 2 * ns : ns, mid = ADJ ? ns : (ns + 1) / 2;
+  return make_int3(half == 1 ? mid : 0, half == 0 ? mid : all, mid);
+}
+// End of the round of both passes that starts at slice c0: rounds of equal length of at most 2048 columns,
+// and (halves: plans whose items may be split) never across the halves, so that a tile's sums are
+// rounded alike whether one item forms it or two; one slice of a brief item.
+template <bool WIDE>
+__device__ __forceinline__ int oz_round_end(int c0, int3 kr, bool halves, bool brief) {
+  constexpr int CHUNK = 2048 / (WIDE ? OZ_BK_WIDE : OZ_BK);
+  if (brief) return c0 + 1;
+  const int left = (halves && c0 < kr.z ? min(kr.z, kr.y) : kr.y) - c0;
+  if (left <= CHUNK) return c0 + left;
+  const int rounds = (left + CHUNK - 1) / CHUNK;
+  return c0 + (left + rounds - 1) / rounds;
+}
+// How many rounds an item takes.
+template <bool WIDE>
+__device__ __forceinline__ int oz_rounds(int3 kr, bool halves, bool brief) {
+  constexpr int CHUNK = 2048 / (WIDE ? OZ_BK_WIDE : OZ_BK);
+  if (brief) return kr.y - kr.x;
+  if (halves && kr.x < kr.z && kr.z < kr.y) return (kr.z - kr.x + CHUNK - 1) / CHUNK + (kr.y - kr.z + CHUNK - 1) / CHUNK;
+  return (kr.y - kr.x + CHUNK - 1) / CHUNK;
+}
+
+// Opens (by a warp) the taking again of coherent parts' items.
+__device__ __noinline__ void oz_open_again(OzAgain* again, int place) {
+  if ((threadIdx.x & 31) == 0) again->ctr = again->done = 0;
+  __threadfence();
+  __syncwarp();
+  if ((threadIdx.x & 31) == 0) *(volatile int32_t*)&again->go = place;
+}
+// Item `it` of the launch, with its part's tables; brief where its part was found coherent up to step `brief_to`
+// (negative: no part was, or it may not be read yet).
+template <bool ADJ, bool WIDE>
+__device__ __forceinline__ void oz_read_item(const OzStepArgs& a, int it, int brief_to, OzItem* w) {
+  const int code = a.split ? a.split_items[it / a.pieces] : it / a.pieces;
+  const Tile t = a.tiles[a.split ? code >> 1 : code];
+  // in flight beside the part's tables: the loads of an item wait for this chain
+  int32_t coh = OZ_INCOHERENT;
+  if (brief_to >= 0) coh = *(volatile int32_t*)&a.coh[t.part];
+  const PartDesc p = a.parts[t.part];
+  const bool brief = coh <= brief_to;
+  w->code = code;
+  w->piece = it % a.pieces;
+  w->ti = t.ti;
+  w->tj = t.tj;
+  w->slot = t.slot;
+  w->part = t.part;
+  w->off = p.off;
+  w->soff = p.soff;
+  w->s = p.s;
+  w->c = p.c;
+  w->ld = p.ld;
+  w->brief = brief;
+  w->rounds = oz_rounds<WIDE>(oz_slices<ADJ, WIDE>(p.s, a.split ? code & 1 : -1, brief), a.halves, brief);
+}
+template <bool ADJ, bool WIDE>
+__global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(const __grid_constant__ OzStepArgs a) {
   constexpr int T = OZ_SLICES;
   constexpr int BK = WIDE ? OZ_BK_WIDE : OZ_BK;  // K per slice
-  constexpr int CHUNK = 2048 / BK;               // K slices per round of both passes
   constexpr uint32_t DTILE = 128u * BK * 2u;     // one digit tile: 128 rows x 64 or 128 B
   // instruction descriptor without N (bits 17..22, N / 8): FP32 accumulate, FP16 A and B, M = 128
   constexpr uint32_t IDESC = (1u << 4) | ((128u >> 4) << 24);
@@ -660,6 +756,10 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(sb + OZ_RING_B + 8 * OZ_BARS);
   int* s_err = reinterpret_cast<int*>(tmem_slot + 1);
   int* s_half = reinterpret_cast<int*>(tmem_slot + 2);  // split K: halves of the tile done before
+  // 1: a sum has reached 2^24.  From the decision at the pause on: 8, and 2 where this block ends the launch, 4 where it
+  // forms coherent parts again, 16 while warp 3 waits for that
+  __shared__ int s_walk;
+  __shared__ int s_taken;  // items taken again
   longlong2* red = reinterpret_cast<longlong2*>(sb + OZ_RING_B + 8 * OZ_BARS + 16);
   // warp 0's producer takes each next tile (claimed from a counter in global memory, or dealt)
   // and passes it on with its part through a ring (full: taken; empty: read by the other
@@ -686,20 +786,6 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
   auto piece_cols = [&](int sz, int tj, int piece) {
     return max(0, min(pcols, oz_tile_cols(sz, tj) - piece * pcols));
   };
-  // K slices [x, y) of an item of a part of size sz: all of them (the adjoint's first ns slices
-  // multiply Xbar by X, the rest X by Xbar) or one half, up to or from slice z
-  auto slices = [&](int sz, int half) {
-    const int ns = (sz + BK - 1) / BK, all = ADJ ? 2 * ns : ns, mid = ADJ ? ns : (ns + 1) / 2;
-    return make_int3(half == 1 ? mid : 0, half == 0 ? mid : all, mid);
-  };
-  // end of the round of both passes that starts at slice c0: rounds of equal length of at most
-  // CHUNK slices, and (plans whose items may be split) never across the halves, so that a
-  // tile's sums are rounded alike whether one item forms it or two
-  auto round_end = [&](int c0, int3 kr) {
-    const int left = (a.halves && c0 < kr.z ? min(kr.z, kr.y) : kr.y) - c0;
-    const int rounds = (left + CHUNK - 1) / CHUNK;
-    return c0 + (left + rounds - 1) / rounds;
-  };
   // items claimed at run time (forward, tail and reverse steps; the list order) or dealt in turn
   // (the rebuilt iterates, which may run beside reverse steps and have no last block)
   const bool dyn = a.tile_ctr != nullptr && !rec;
@@ -714,7 +800,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
       mbar_init(item_full(lane), 1);
       mbar_init(item_empty(lane), 2 + OZ_EPI_WARPS);
     }
-    if (lane == 0) *s_err = 0;
+    if (lane == 0) *s_err = s_walk = s_taken = 0;
     asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
   }
   if (warp == 1) {
@@ -727,38 +813,22 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
   const uint32_t tmem = __shfl_sync(0xffffffffu, *tmem_slot, 0);
 
   // the first item's tables, which no launch writes, before the launch before this one is done
-  OzItem first;
-  auto read_item = [&](int it) {
-    OzItem w;
-    w.piece = it % pieces;
-    w.code = split ? a.split_items[it / pieces] : it / pieces;
-    const Tile t = a.tiles[split ? w.code >> 1 : w.code];
-    const PartDesc p = a.parts[t.part];
-    w.ti = t.ti;
-    w.tj = t.tj;
-    w.slot = t.slot;
-    w.part = t.part;
-    w.off = p.off;
-    w.soff = p.soff;
-    w.s = p.s;
-    w.c = p.c;
-    w.ld = p.ld;
-    return w;
-  };
   if (threadIdx.x == 0) {
-    first.code = -1;
-    if ((int)blockIdx.x < nitems) first = read_item(blockIdx.x);
+    if ((int)blockIdx.x < nitems) oz_read_item<ADJ, WIDE>(a, blockIdx.x, -1, s_items);
+    else s_items->code = rec ? OZ_END : OZ_PAUSE;
   }
   pdl_wait();  // everything below reads what the launch before wrote
   int step = a.step;
-  bool run;
+  bool run, coherent = true;  // whether some part may have been found coherent
   int n = 0;
   if (ADJ || rec) {
     // reverse step `step` exists iff step <= n; a rebuilt X_step is read iff step < n
     n = *(volatile int32_t*)&a.ctl.st->steps;
     run = ADJ ? step <= n : step < n;
   } else if (a.mode == SQ_FORWARD) {
-    run = *(volatile int32_t*)&a.ctl.st->stopped == 0;
+    const uint2 v = ld_volatile2(&a.ctl.st->stopped);
+    run = v.x == 0;
+    coherent = v.y != 0;
   } else {
     const int32_t stt = *(volatile int32_t*)&a.ctl.st->status;
     run = stt != ST_NONFINITE && stt != ST_TIMEOUT;
@@ -767,6 +837,12 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
   if (!run) {  // the loop has stopped: nothing to do
     if (warp == 1) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;\n" ::"r"(tmem));
     return;
+  }
+  // a part's items take brief rounds after the step that found it coherent (a rebuilt step: from that one on)
+  const int place = ADJ ? n - step + 1 : step, brief_to = !coherent ? -1 : (rec ? place : place - 1);
+  if (threadIdx.x == 0 && brief_to >= 0 && s_items->code >= 0 && a.coh[s_items->part] <= brief_to) {
+    s_items->brief = 1;
+    s_items->rounds = oz_rounds<WIDE>(oz_slices<ADJ, WIDE>(s_items->s, split ? s_items->code & 1 : -1, true), false, true);
   }
   // digit buffers read / written (the adjoint's sets are passed explicitly)
   const int dbi = (ADJ || rec) ? 0 : (step - 1) & 1, dbo = (ADJ || rec) ? 0 : step & 1;
@@ -780,6 +856,19 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
   auto wait = [&](uint32_t bar, uint32_t parity) {
     return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag)) != 0;
   };
+  // The pause of the walk, passed once by every warp, after its part of this CTA's items: when the last block of
+  // the launch has come here, parts found coherent are formed again.
+  auto pause = [&]() {
+    tc_fence_before();
+    asm volatile("bar.sync 2, %0;\n" ::"n"(OZ_THREADS) : "memory");
+  };
+  auto decision = [&]() {  // (every warp but warp 0, which takes it)
+    pause();
+    asm volatile("bar.sync 2, %0;\n" ::"n"(OZ_THREADS) : "memory");
+    tc_fence_after();
+    return (*(volatile int*)&s_walk & 4) != 0;
+  };
+  auto paused = [&]() { return rec || (*(volatile int*)&s_walk & 8) != 0; };  // (rebuilt steps have no pause)
   if (warp == 0 || warp == 2) {
     // Like the issuing warp below, the whole warp walks the units with warp-uniform values and
     // one elected lane issues the loads.
@@ -793,6 +882,46 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
     int nxt = nitems;
     if (op == 0 && lane == 0 && dyn && (int)blockIdx.x < nitems)
       nxt = (int)gridDim.x + (int)atomicAdd(a.tile_ctr, 1u);
+    int redo = -1;  // warp 0, after the pause: items taken again
+    // Warp 0 takes this CTA's ticket, with a mark in its upper half if a sum has reached 2^24; the last
+    // block of the launch to take one knows so whether any has, and all items are done then.  Blocks whose ticket
+    // shows such a sum wait a while for that (warp 3: the wait in this loop, even as a call, made every
+    // step 1.5 % slower) and help; no block depends on a helper, and none waits in a launch without such a sum.
+    // One part of 1,500: 7.3 ms a density with helpers, 29 without; of 4,096 85 and 426.
+    auto decide = [&]() {
+      if (op != 0) return decision();
+      pause();
+      redo = 0;
+      const unsigned int found = *(volatile int*)&s_walk & 1 ? 0x10000u : 0u;
+      unsigned int t = 0;
+      if (lane == 0) {
+        if (*(volatile int*)s_err) a.ctl.st->timeout = 1;
+        __threadfence();
+        t = found + atomicAdd(&a.ctl.st->counter, found + 1u);
+      }
+      t = __shfl_sync(0xffffffffu, t, 0);
+      int walk = 8;
+      if ((t & 0xFFFFu) == gridDim.x - 1) {
+        __threadfence();
+        walk = 10;
+        if (t >> 16 && *(volatile int32_t*)&a.ctl.st->timeout == 0) {
+          walk = 12;
+          if constexpr (ADJ) {  // the norms of the rows formed again are summed again too
+            for (int k = 0; k < a.nparts; ++k)
+              if (__ldcg(a.coh_new + k) && a.coh[k] > brief_to)
+                for (int r = lane; r < a.parts[k].s; r += 32) a.normf[a.parts[k].soff + r] = 0.0f;
+          }
+          oz_open_again(a.again, place);
+        }
+      } else if (t >> 16) {
+        walk = 24;
+      }
+      if (lane == 0) *(volatile int*)&s_walk = walk;
+      __syncwarp();
+      asm volatile("bar.arrive 3, 64;\n" ::: "memory");
+      asm volatile("bar.sync 2, %0;\n" ::"n"(OZ_THREADS) : "memory");
+      return (*(volatile int*)&s_walk & 4) != 0;
+    };
     for (int v = 0, it = blockIdx.x; !bad; ++v, it += gridDim.x) {
       const int q = v % OZ_RING;
       if (op == 0) {
@@ -805,12 +934,18 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
             it = nxt;
             if (it < nitems) nxt = (int)gridDim.x + (int)atomicAdd(a.tile_ctr, 1u);
           }
-          OzItem w = first;
           if (v > 0) {
-            w.code = -1;
-            if (it < nitems) w = read_item(it);
+            do {  // after the pause: those of parts found coherent by this launch
+              if (redo >= 0) it = atomicAdd(&a.again->ctr, 1);
+              if (it >= nitems) {
+                s_taken = redo;
+                s_items[q].code = redo >= 0 || rec ? OZ_END : OZ_PAUSE;
+                break;
+              }
+              if (redo >= 0) ++redo;
+              oz_read_item<ADJ, WIDE>(a, it, redo >= 0 ? OZ_INCOHERENT : brief_to, s_items + q);
+            } while (redo >= 0 && !(__ldcg(a.coh_new + s_items[q].part) && a.coh[s_items[q].part] > brief_to));
           }
-          s_items[q] = w;
           mbar_arrive(item_full(q));
         }
         __syncwarp();
@@ -825,15 +960,18 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
       w.part = __shfl_sync(0xffffffffu, s_items[q].part, 0);
       w.s = __shfl_sync(0xffffffffu, s_items[q].s, 0);
       w.piece = __shfl_sync(0xffffffffu, s_items[q].piece, 0);
+      const bool brief = __shfl_sync(0xffffffffu, s_items[q].brief, 0) != 0;
       if (op == 1 && lane == 0) mbar_arrive(item_empty(q));
+      if (w.code == OZ_PAUSE && decide()) continue;
       if (w.code < 0) break;
       if (piece_cols(w.s, w.tj, w.piece) == 0) continue;
       const int half = split ? w.code & 1 : -1;
       const bool dg = !ADJ && w.ti == w.tj;  // X X on a diagonal tile: B is A
       const int blk = op == 0 ? w.ti : w.tj;
-      const int ns = (w.s + BK - 1) / BK;
-      const int3 kr = slices(w.s, half);
+      const int ns = oz_nslices<WIDE>(w.s, brief);
+      const int3 kr = oz_slices<ADJ, WIDE>(w.s, half, brief);
       if constexpr (WIDE) {
+        const int unit = brief ? OZ_BK : BK;  // brief: a slice's tiles hold its 32 columns and 32 that are not multiplied
         // ring places of this pass over: `by` tiles on
         auto advance = [&](uint32_t by) {
           su += by;
@@ -851,7 +989,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
         auto slice = [&](int ks, int T) {
           const bool h2 = ADJ && ks >= ns;
           const bool xb = ADJ && (op == 0) != h2;
-          const int k0 = (h2 ? ks - ns : ks) * BK;
+          const int k0 = (h2 ? ks - ns : ks) * unit;
           const bool kmajor = k0 / 128 <= blk;
           const CUtensorMap* const map =
               (kmajor ? (xb ? maps_b : maps) : (xb ? maps_mn_b : maps_mn)) + w.part;
@@ -887,7 +1025,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
           continue;
         }
         for (int c0 = kr.x, c1; c0 < kr.y && !bad; c0 = c1) {
-          c1 = round_end(c0, kr);
+          c1 = oz_round_end<WIDE>(c0, kr, a.halves, brief);
           for (int kb = c0; kb < c1 && !bad; ++kb) slice(kb, OZ_SLICES);
           for (int kb = c0; kb < c1 && !bad; ++kb) slice(kb, OZ_LOW);
         }
@@ -928,7 +1066,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
         };
         if (op == 1 && dg) {  // rows I only: this thread's place in the ring moves past them
           for (int c0 = kr.x, c1; c0 < kr.y; c0 = c1) {
-            c1 = round_end(c0, kr);
+            c1 = oz_round_end<WIDE>(c0, kr, a.halves, brief);
             su += (uint32_t)(c1 - c0 + (c1 - c0 + OZ_LOW_SUB - 1) / OZ_LOW_SUB);
           }
           ph ^= (su / OZ_UNITS) & 1u;
@@ -936,7 +1074,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
           continue;
         }
         for (int c0 = kr.x, c1; c0 < kr.y && !bad; c0 = c1) {
-          c1 = round_end(c0, kr);
+          c1 = oz_round_end<WIDE>(c0, kr, a.halves, brief);
           uint32_t u;
           for (int kb = c0; kb < c1; ++kb) {
             if (!acquire(T * DTILE, u)) {
@@ -967,6 +1105,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
         for (uint32_t u = 0; u < (uint32_t)OZ_UNITS; ++u)
           if (used >> u & 1u) (void)mbar_wait_own(full(0, u), phase >> u & 1u);
       }
+      if (!paused()) (void)decide();
     }
   } else if (warp == 1) {
     // The whole warp walks the slices with warp-uniform values (the item's fields through a
@@ -988,19 +1127,22 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
       const int ti = __shfl_sync(0xffffffffu, s_items[q].ti, 0), tj = __shfl_sync(0xffffffffu, s_items[q].tj, 0);
       const int sz = __shfl_sync(0xffffffffu, s_items[q].s, 0);
       const int piece = __shfl_sync(0xffffffffu, s_items[q].piece, 0);
+      const bool brief = __shfl_sync(0xffffffffu, s_items[q].brief, 0) != 0;
       if (lane == 0) mbar_arrive(item_empty(q));
+      if (code == OZ_PAUSE && decision()) continue;
       if (code < 0) break;
       const int ncols = piece_cols(sz, tj, piece);
       if (ncols == 0) continue;
       const int half = split ? code & 1 : -1;
       const bool dg = !ADJ && ti == tj;
-      const int ns = (sz + BK - 1) / BK;
-      const int3 kr = slices(sz, half);
+      const int ns = oz_nslices<WIDE>(sz, brief);
+      const int3 kr = oz_slices<ADJ, WIDE>(sz, half, brief);
       const uint32_t idesc0 = IDESC | ((uint32_t)(ncols >> 3) << 17);
       if constexpr (WIDE) {
+        const int unit = brief ? OZ_BK : BK;
         const uint64_t dk = smem_desc_sw<2 * BK>(0), dm = smem_desc_mn128(0, DTILE / 2);
         // the ring's tile `off` places past s0 (phase p0)
-        auto place = [&](uint32_t s0, uint32_t off) { return s0 + off >= OZ_TILES ? s0 + off - OZ_TILES : s0 + off; };
+        auto at = [&](uint32_t s0, uint32_t off) { return s0 + off >= OZ_TILES ? s0 + off - OZ_TILES : s0 + off; };
         auto parity = [&](uint32_t s0, uint32_t p0, uint32_t off) { return s0 + off >= OZ_TILES ? p0 ^ 1u : p0; };
         // the next group of tiles of each operand has come (a diagonal tile's serves both)
         auto loaded = [&]() {
@@ -1020,7 +1162,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
         OzWide o;
         auto prepare = [&](auto low, int ks) {
           constexpr int N = oz_digits<decltype(low)::value>();
-          const int kp = ADJ && ks >= ns ? ks - ns : ks, kt = kp / (128 / BK);
+          const int k0 = (ADJ && ks >= ns ? ks - ns : ks) * unit, kt = k0 / 128;
           const bool amn = kt > ti, bmn = kt > tj;
           const uint32_t alo = (uint32_t)(amn ? dm : dk) + (base >> 4), blo = (uint32_t)(bmn ? dm : dk) + (base >> 4);
           o.ahi = (uint32_t)((amn ? dm : dk) >> 32);
@@ -1028,11 +1170,11 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
           o.adv_a = amn ? (2048u >> 4) : (32u >> 4);
           o.adv_b = bmn ? (2048u >> 4) : (32u >> 4);
           o.idesc = idesc0 | ((amn ? 1u : 0u) << 15) | ((bmn ? 1u : 0u) << 16);
-          o.steps = min(BK / 16, (sz - kp * BK + 15) / 16);
+          o.steps = min(unit / 16, (sz - k0 + 15) / 16);
   #pragma unroll
           for (int q = 0; q < N; ++q) {
-            o.a[q] = alo + place(su, dg ? N - 1 - q : 2 * (N - 1 - q)) * (DTILE >> 4);
-            o.b[q] = blo + place(su, dg ? N - 1 - q : 2 * q + 1) * (DTILE >> 4);
+            o.a[q] = alo + at(su, dg ? N - 1 - q : 2 * (N - 1 - q)) * (DTILE >> 4);
+            o.b[q] = blo + at(su, dg ? N - 1 - q : 2 * q + 1) * (DTILE >> 4);
           }
         };
         // The MMAs of the prepared slice.  Before the last K = 16 step of a group of tiles
@@ -1060,16 +1202,16 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
             if (elect_one()) {
               oz_issue_wide<LOW, I, BK / 16 - 1, BK / 16>(tmem, c, first);
               if (!dg) {
-                mma_commit(empty(place(s0, 2 * I)));
+                mma_commit(empty(at(s0, 2 * I)));
   #pragma unroll
                 for (int b = 0; b <= I; ++b)
-                  if (oz_b_last<LOW>(b) == I) mma_commit(empty(place(s0, 2 * b + 1)));
+                  if (oz_b_last<LOW>(b) == I) mma_commit(empty(at(s0, 2 * b + 1)));
               } else if (I == N - 1) {
   #pragma unroll
-                for (int q = 0; q < N; ++q) mma_commit(empty(place(s0, q)));
+                for (int q = 0; q < N; ++q) mma_commit(empty(at(s0, q)));
               }
             }
-            last = (int)place(s0, dg ? 0 : 2 * I);
+            last = (int)at(s0, dg ? 0 : 2 * I);
             lastph = parity(s0, p0, dg ? 0 : 2 * I);
           };
           step(std::integral_constant<int, 0>());
@@ -1084,7 +1226,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
         prepare(std::false_type(), kr.x);
         bad = !loaded();
         for (int c0 = kr.x, c1; c0 < kr.y && !bad; c0 = c1, ++r) {
-          c1 = round_end(c0, kr);
+          c1 = oz_round_end<WIDE>(c0, kr, a.halves, brief);
           // first pass: it reuses the columns of the previous round's second
           if (r > 0 && !wait(aempty(1), (r - 1) & 1)) {
             bad = true;
@@ -1168,7 +1310,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
           lastph = pub;
         };
         for (int c0 = kr.x, c1; c0 < kr.y && !bad; c0 = c1, ++r) {
-          c1 = round_end(c0, kr);
+          c1 = oz_round_end<WIDE>(c0, kr, a.halves, brief);
           // first pass: it reuses the columns of the previous round's second
           take();
           OzNarrow o = operands(c0, sa, sb, 0);
@@ -1277,11 +1419,14 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
         if (lane == 0) mbar_arrive(item_empty(iq));
       };
       t.code = __shfl_sync(0xffffffffu, s_items[iq].code, 0);
+      const bool brief = __shfl_sync(0xffffffffu, s_items[iq].brief, 0) != 0;
+      int rounds = __shfl_sync(0xffffffffu, s_items[iq].rounds, 0);
       fields();
-      if (!WIDE) done();
+      if (!WIDE || t.code < 0) done();
+      if (t.code == OZ_PAUSE && decision()) continue;
       if (t.code < 0) break;
       const int code = t.code;
-      const int ti = split ? code >> 1 : code, half = split ? code & 1 : -1;
+      const int ti = split ? code >> 1 : code;
       // a split item's 64-bit partial goes to its own tile of split_acc, which the item that
       // finishes the tile reads; otherwise the sums wait in this CTA's scratch tile
       long long* const acc = split ? a.split_acc + (size_t)code * (128 * 128) : cta_acc;
@@ -1299,6 +1444,18 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
       // warp's first row (all its entries below the diagonal) is neither drained nor formed
       const int cskip = (t.ti == t.tj) ? quarter * 32 : 0;
       bool ok = true;
+      // A sum has reached 2^24: the last block of the launch is to form the part again.  (Kept to the end of an item in
+      // the wide form, whose registers that suits: marked as in the narrow one it spills 370 bytes and takes 3 %
+      // longer; the narrow one, marking at the end, takes 0.7 % longer at n = 512.)
+      float top = 0.0f;
+      auto mark_part = [&](int part) {  // (of a brief item, which can reach 2^24 only if X has left [0, 1], it does nothing)
+        a.coh_new[part] = 1;
+        atomicOr(&s_walk, 1);  // (brief items come after the decision)
+      };
+      auto mark = [&](float m) {
+        if (WIDE) top = fmaxf(top, m);
+        else mark_part(t.part);
+      };
       // the warp's chunks of 16 columns (pc0: its first column in the piece)
       const int nch = 2 / pieces, pc0 = colq * 16 * nch, tc0 = t.piece * pcols + pc0;
       const bool on0 = pc0 < ncols && tc0 + 16 > cskip;
@@ -1316,7 +1473,6 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
       // held exactly in FP32, but for the sixth) and add them as 64-bit integers; each pass hands its
       // columns back
       long long z[16];
-      const int3 kr = slices(p.s, half);
       if constexpr (WIDE) {
         // Both chunks' sums stay in registers.  The tensor pipe stands still from a pass's last product
         // until the columns the next pass starts in have been read by every warp, so nothing but that
@@ -1331,7 +1487,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
         };
 #pragma unroll
         for (int j = 0; j < 16; ++j) z[j] = z1[j] = 0ll;
-        for (int c0 = kr.x; c0 < kr.y; c0 = round_end(c0, kr), ++rd) {
+        for (; rounds > 0; --rounds, ++rd) {
           const long long less = (long long)(sgn < 0 ? kOzOffset : 0ull - kOzOffset);
 #pragma unroll
           for (int j = 0; j < 16; ++j) {
@@ -1340,15 +1496,15 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
           }
           ok = __all_sync(0xffffffffu, mbar_wait(afull(0), rd & 1, abort_flag)) && ok;
           tc_fence_after();
-          if (ok && on0) oz_drain_high_a(tc, sgn, z);
-          if (ok && on1) oz_drain_high_a(tc + 16, sgn, z1);
+          if (ok && on0) oz_drain_high_a<WIDE>(tc, sgn, mark, z);
+          if (ok && on1) oz_drain_high_a<WIDE>(tc + 16, sgn, mark, z1);
           hand_back(0);
-          if (ok && on0) oz_drain_high_b(tc, sgn, z);
-          if (ok && on1) oz_drain_high_b(tc + 16, sgn, z1);
+          if (ok && on0) oz_drain_high_b<WIDE>(tc, sgn, mark, z);
+          if (ok && on1) oz_drain_high_b<WIDE>(tc + 16, sgn, mark, z1);
           ok = __all_sync(0xffffffffu, mbar_wait(afull(1), rd & 1, abort_flag)) && ok;
           tc_fence_after();
-          if (ok && on0) oz_drain_low(tc, sgn, z);
-          if (ok && on1) oz_drain_low(tc + 16, sgn, z1);
+          if (ok && on0) oz_drain_low<WIDE>(tc, sgn, mark, z);
+          if (ok && on1) oz_drain_low<WIDE>(tc + 16, sgn, mark, z1);
           hand_back(1);
         }
         // the sums leave the registers for a scratch tile (thread-private entries: column cl, row m):
@@ -1368,7 +1524,8 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
         const int clast = on1 ? 1 : (on0 ? 0 : -1), cfirst = on1 && on0 ? 0 : -1;
         // one chunk's sums at a time, parked in TMEM between the passes and then in the scratch tile
         // (thread-private entries: column cl, row m) or, the last one's, in registers
-        for (int c0 = kr.x, pass = 0; c0 < kr.y; pass ^= 1) {
+        const int all = rounds;
+        for (int pass = 0; rounds > 0; pass ^= 1) {
           ok = __all_sync(0xffffffffu, mbar_wait(afull(pass), rd & 1, abort_flag)) && ok;
           tc_fence_after();
           // the first pass hands its columns back as soon as the warp's last chunk has read
@@ -1385,14 +1542,14 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
               // columns among 256-511), which the second pass leaves alone
 #pragma unroll
               for (int j = 0; j < 16; ++j) z[j] = (long long)(sgn < 0 ? kOzOffset : 0ull - kOzOffset);
-              oz_drain_high_a(tc, sgn, z);
+              oz_drain_high_a<WIDE>(tc, sgn, mark, z);
               if (cc == clast) {
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) mbar_arrive(aempty(0));
                 released = true;
               }
-              oz_drain_high_b(tc, sgn, z);
+              oz_drain_high_b<WIDE>(tc, sgn, mark, z);
 #pragma unroll
               for (int j = 0; j < 16; ++j) w[j] = (uint32_t)(unsigned long long)z[j];
               tmem_st16(tc + OZ_PARK_LO, w);
@@ -1406,7 +1563,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
               tmem_ld16(tc + OZ_PARK_HI, w);
 #pragma unroll
               for (int j = 0; j < 16; ++j) z[j] += (long long)((unsigned long long)w[j] << 32);
-              oz_drain_low(tc, sgn, z);
+              oz_drain_low<WIDE>(tc, sgn, mark, z);
               if (cc == clast) {
                 tc_fence_before();
                 __syncwarp();
@@ -1414,11 +1571,11 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
                 released = true;
               }
               long long* zp = acc + (size_t)cl * 128 + m;
-              if (c0 > kr.x) {  // the rounds before
+              if (rounds < all) {  // the rounds before
 #pragma unroll
                 for (int j = 0; j < 16; ++j) z[j] += zp[(size_t)j * 128];
               }
-              if (split || cc != clast || round_end(c0, kr) < kr.y) {
+              if (split || cc != clast || rounds > 1) {
 #pragma unroll
                 for (int j = 0; j < 16; ++j) zp[(size_t)j * 128] = z[j];
               }
@@ -1431,12 +1588,15 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
             if (lane == 0) mbar_arrive(aempty(pass));
           }
           if (pass == 1) {
-            c0 = round_end(c0, kr);
+            --rounds;
             ++rd;
           }
         }
       }
       if (!ok) *s_err = 1;
+      if constexpr (WIDE)
+        if (__any_sync(0xffffffffu, top >= 1.0f) && lane == 0 && !rec && *(volatile int*)&s_items[iq].brief == 0)
+          mark_part(*(volatile int*)&s_items[iq].part);
       // split K: the first half to finish leaves its partial; the second adds the first's
       // (64-bit integers: exact, so which one finishes first does not matter) and forms the tile
       const long long* other = nullptr;
@@ -1695,19 +1855,68 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
       }
     }
   }
-  tc_fence_before();
-  __syncthreads();
+  if (warp == 3) {
+    if (!rec) {
+      pause();
+      asm volatile("bar.sync 3, 64;\n" ::: "memory");  // warp 0's word
+      if (*(volatile int*)&s_walk & 16) {
+        if (lane == 0) {
+          const uint64_t until = global_ns() + 2000000ull;  // no longer than two items take
+          bool ready;
+          while (!(ready = *(volatile int32_t*)&a.again->go == place) && *(volatile int32_t*)abort_flag == 0 &&
+                 global_ns() < until)
+            __nanosleep(500);
+          __threadfence();
+          *(volatile int*)&s_walk = ready ? 12 : 8;
+        }
+        __syncwarp();
+      }
+      asm volatile("bar.arrive 2, %0;\n" ::"n"(OZ_THREADS) : "memory");
+    }
+  } else if (!paused()) {
+    (void)decision();
+  }
+  int walk = *(volatile int*)&s_walk;
+  if (rec || walk & 4) {  // else the pause was the end
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    if (walk & 4) {  // the block whose items are the last to be done ends the launch
+      if (threadIdx.x == 0) {
+        __threadfence();
+        const int taken = s_taken;
+        s_walk = taken > 0 && atomicAdd(&a.again->done, taken) + taken == nitems ? 14 : 12;
+        __threadfence();
+      }
+      __syncthreads();
+      walk = s_walk;
+    }
+  }
   if (warp == 1) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;\n" ::"r"(tmem));
   if (threadIdx.x == 0 && *s_err) {
     a.ctl.st->timeout = 1;
-    if (ADJ || rec) a.ctl.st->status = ST_TIMEOUT;  // no step bookkeeping follows
+    if (ADJ || rec || walk & 4) a.ctl.st->status = ST_TIMEOUT;  // no step bookkeeping follows
+    if (walk & 4) {
+      a.ctl.st->stopped = 1;
+      a.ctl.st->counter = 0;
+      if (dyn) *a.tile_ctr = 0u;
+    }
   }
-  if (rec) return;
+  if (rec || !(walk & 2)) return;
+  if (walk & 4 && warp == 3) {
+    for (int k = lane; k < a.nparts; k += 32)
+      if (a.coh_new[k]) {
+        a.coh[k] = min(a.coh[k], place);
+        a.coh_new[k] = 0;
+      }
+    if (!ADJ && lane == 0) a.ctl.st->coherent = 1;
+  }
   if (ADJ) {
+    __threadfence();
     // the last block: each part's new scale from the largest squared row norm m (on the grid
     // of the old scale sg): the smallest e with 2^e >= 2 sqrt(m) (1 + 2^-10), the margin
     // covering the truncated squares and the FP32 sums; the norms are cleared for the next step
-    if (last_block_ticket(&a.ctl.st->counter)) {
+    {
       for (int k = warp; k < a.nparts; k += OZ_THREADS / 32) {
         const PartDesc p = a.parts[k];
         float mx = 0.0f;
@@ -1741,7 +1950,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(OzStepArgs a) {
     return;
   }
 
-  if (warp == 0 && last_block_warp(&a.ctl.st->counter)) {
+  if (warp == 0) {
     const double2 sum = warp_sum_slots(a.slots, a.nslots * pieces);
     if (threadIdx.x == 0) {
       if (a.ctl.st->timeout) {
@@ -1788,12 +1997,12 @@ cudaError_t launch_oz_gather(const PartDesc* parts, const ColBlock* blocks, int 
 }
 
 cudaError_t launch_oz_adj_scale(const PartDesc* parts, int nparts, const Tile* tiles, int ntiles, const double* xb0,
-                                const double* xb1, int after, double* norm, int32_t* sig, const DevState* st,
-                                cudaStream_t s) {
+                                const double* xb1, int after, double* norm, int32_t* sig, int32_t* coh,
+                                const DevState* st, cudaStream_t s) {
   if (ntiles > 0) oz_norm_kernel<<<ntiles, 256, 0, s>>>(parts, tiles, xb0, xb1, after, norm, st);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  oz_scale_kernel<<<nparts, 256, 0, s>>>(parts, after, norm, sig, st);
+  oz_scale_kernel<<<nparts, 256, 0, s>>>(parts, after, norm, sig, coh, st);
   return cudaGetLastError();
 }
 
