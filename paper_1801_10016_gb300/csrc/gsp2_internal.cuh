@@ -244,7 +244,9 @@ __device__ __forceinline__ uint2 ld_volatile2(const void* p) {
 
 // Programmatic dependent launch: the next launch of the stream may become resident (its blocks
 // set up barriers and TMEM while this one drains), and this one waits here until the launch
-// before it has completed and its writes are visible.
+// before it has completed and its writes are visible.  What that launch writes is read by plain loads: the
+// read-only path (__ldg, const __restrict__) is for data that does not change while a kernel runs, and
+// these kernels run while it still does.
 __device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
 template <typename... Params, typename... Args>
@@ -370,7 +372,7 @@ constexpr int GATHER_BATCH = 4;   // entries per lane in flight (8: 7 % slower f
 constexpr int GATHER_ROWS = 512;  // 4 KB of 8-byte words a warp: 6 blocks of 8 warps an SM
 template <typename T, typename Put, typename Out>
 __device__ __forceinline__ void gather_column(T* buf, int rend, int nq, const int32_t* __restrict__ lj,
-                                              const double* __restrict__ xq, int lane, Put put, Out out) {
+                                              const double* xq, int lane, Put put, Out out) {
   for (int r0 = 0; r0 < rend; r0 += GATHER_ROWS) {
     const int m = min(GATHER_ROWS, rend - r0);
     for (int i = lane; i < (int)(m * sizeof(T) / 16); i += 32) reinterpret_cast<uint4*>(buf)[i] = make_uint4(0, 0, 0, 0);

@@ -223,7 +223,7 @@ __global__ void __launch_bounds__(256, 6) gather_kernel(const PartDesc* __restri
                                                      const int64_t* __restrict__ rowptr,
                                                      const int32_t* __restrict__ loc,
                                                      const int64_t* __restrict__ locptr,
-                                                     const double* __restrict__ x0, double* __restrict__ arena,
+                                                     const double* x0, double* __restrict__ arena,
                                                      double* __restrict__ slots, StepCtl ctl) {
   __shared__ __align__(16) double cols[COLS_PER_BLOCK][GATHER_ROWS];
   __shared__ double s_tr[COLS_PER_BLOCK];

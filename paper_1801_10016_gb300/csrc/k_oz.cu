@@ -180,7 +180,7 @@ __global__ void __launch_bounds__(256) oz_convert_slice_kernel(const PartDesc* _
 __global__ void __launch_bounds__(32 * COLS_PER_BLOCK, 6) oz_gather_kernel(
     const PartDesc* __restrict__ parts, const ColBlock* __restrict__ blocks, const int32_t* __restrict__ Sall,
     const int64_t* __restrict__ rowptr, const int32_t* __restrict__ loc, const int64_t* __restrict__ locptr,
-    const double* __restrict__ x0, double* __restrict__ arena, OzSlices dig, double* __restrict__ slots,
+    const double* x0, double* __restrict__ arena, OzSlices dig, double* __restrict__ slots,
     StepCtl ctl) {
   __shared__ __align__(16) long long cols[COLS_PER_BLOCK][GATHER_ROWS];
   __shared__ double s_tr[COLS_PER_BLOCK];
@@ -1651,7 +1651,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(const __grid_con
             long long xn[B];  // the forward iterates are kept in the fixed point itself; the adjoint's Xbar in FP64
 #pragma unroll
             for (int j = 0; j < B; ++j)
-              xn[j] = alf > 0 ? __ldg(reinterpret_cast<const long long*>(xin()) + e + (int64_t)(h + j) * ld) : 0ll;
+              xn[j] = alf > 0 ? reinterpret_cast<const long long*>(xin())[e + (int64_t)(h + j) * ld] : 0ll;
 #pragma unroll
             for (int j = 0; j < B; ++j) {
               const long long xf = 2 * (ADJ ? to_fixed(__longlong_as_double(xn[j]), sg) : xn[j]) + z[h + j];
@@ -1746,7 +1746,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(const __grid_con
             long long xn[8];  // the forward iterates are kept in the fixed point itself; the adjoint's Xbar in FP64
 #pragma unroll
             for (int j = 0; j < 8; ++j)
-              xn[j] = alf > 0 ? __ldg(reinterpret_cast<const long long*>(xi) + (e + (int64_t)j * ld) + lane) : 0ll;
+              xn[j] = alf > 0 ? reinterpret_cast<const long long*>(xi)[(e + (int64_t)j * ld) + lane] : 0ll;
 #pragma unroll
             for (int j = 0; j < 8; ++j) {
               const int c = cb + j;

@@ -1409,7 +1409,7 @@ __global__ void __launch_bounds__(256, 8) gather_lp_kernel(const PartDesc* __res
                                                         const int64_t* __restrict__ rowptr,
                                                         const int32_t* __restrict__ loc,
                                                         const int64_t* __restrict__ locptr,
-                                                        const double* __restrict__ x0, float* __restrict__ master,
+                                                        const double* x0, float* __restrict__ master,
                                                         void* op_hi, void* op_lo, double* __restrict__ slots,
                                                         StepCtl ctl, int upper_rows) {
   __shared__ __align__(16) float cols[COLS_PER_BLOCK][GATHER_ROWS];
