@@ -985,7 +985,12 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(const __grid_con
         // (one barrier each): three and two of the five digits, both of the second pass's, or all of a
         // diagonal tile.  K-major from columns `blk` of the tiles on or above the diagonal (slice
         // block <= blk), else MN-major from rows `blk` of the tile (blk, slice).  The adjoint's first
-        // ns slices take Xbar for rows I and X for rows J, the rest X for rows I and Xbar for rows J
+        // ns slices take Xbar for rows I and X for rows J, the rest X for rows I and Xbar for rows J.
+        // A place is waited for when its turn comes, never looked at ahead: 13 being odd, it changes its
+        // producer every lap, and this warp knows that the phase before the one it waits for is over only from its
+        // last own fill (it lies 11 places before the tile whose release that was).  With a look at all five places
+        // at a slice's start, rows J's last could be taken as free one phase early, the release of rows J's third
+        // tile becoming visible after that of rows I's last, and a live digit tile was overwritten.
         auto slice = [&](int ks, int T) {
           const bool h2 = ADJ && ks >= ns;
           const bool xb = ADJ && (op == 0) != h2;
@@ -993,16 +998,9 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(const __grid_con
           const bool kmajor = k0 / 128 <= blk;
           const CUtensorMap* const map =
               (kmajor ? (xb ? maps_b : maps) : (xb ? maps_mn_b : maps_mn)) + w.part;
-          // which of the slice's places are free already (a lane each)
-          uint32_t at = su + (uint32_t)(dg ? lane : 2 * lane + op), fr = ph;
-          if (at >= OZ_TILES) {
-            at -= OZ_TILES;
-            fr ^= 1u;
-          }
-          const uint32_t ready = __ballot_sync(0xffffffffu, lane < T && mbar_test(empty(at), fr ^ 1u));
           for (int i = 0; i < T; ++i) {
             if (op == 1) advance(1);
-            if (!(ready >> i & 1u) && !wait(empty(su), ph ^ 1u)) {
+            if (!wait(empty(su), ph ^ 1u)) {
               bad = true;
               return;
             }

@@ -34,17 +34,6 @@ __device__ __forceinline__ uint64_t global_ns() {
   return t;
 }
 
-// Whether the phase of this parity is done, without waiting.
-__device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
-  uint32_t done;
-  asm volatile(
-      "{\n .reg .pred p;\n mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
-      : "=r"(done)
-      : "r"(bar), "r"(parity)
-      : "memory");
-  return done != 0;
-}
-
 // Bounded wait: gives up after kWaitNs nanoseconds, or at once when another block
 // has already given up (the shared abort flag), and then raises the flag itself.
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, int32_t* abort_flag) {
