@@ -133,12 +133,12 @@ typedef struct {
                               K slices; adjoint reverse steps: Xbar X and X Xbar), their 64-bit
                               partial sums added by the second to finish (more, shorter items for
                               small problems); 0 = one item per tile; -1 (default) = 1 when the
-                              plan has at most 38 upper 128-tiles.  Needs every part above 128
-                              orbitals (else 0) and 2 x 128 KB of workspace per tile (taken with -1 up
-                              to 512 tiles: gsp2_autotune may turn it on or off).  The 64-bit sums are
-                              exact; up to 512 tiles, plans with split_k set to 0 or 1 round their
-                              FP32 sums at the same K, so that both give the same bits (others
-                              agree to the last few) */
+                              plan has at most a quarter as many upper 128-tiles as the device has SMs
+                              (38 on GB300).  Needs every part above 128 orbitals (else 0) and
+                              2 x 128 KB of workspace per tile.  The 64-bit sums are exact; up to 512
+                              tiles, plans with split_k set to 0 or 1, and those that split by default,
+                              round their FP32 sums at the same K whether split or not, so that both
+                              give the same bits (others agree to the last few) */
   int32_t tile_claim;      /* persistent 128 x 128 steps (tensor-core steps and reverse steps, FP64_EMU
                               forward and reverse steps): 1 (default) = each CTA takes its first
                               tile by its index and claims every next one from a counter in the
@@ -308,11 +308,11 @@ typedef struct {
  * that applies to the plan's precision -- tensor-core steps: persistent 128 x 128 tiles in
  * tile orders 0 and 1, each with claimed tiles and with the static deal, 128 x 256 tiles in
  * either order, and one CTA per tile; FP64_EMU steps: the three tile orders with claimed
- * tiles, tile order 2 with the static deal, and for small plans split-K work items;
+ * tiles, tile order 2 with the static deal, and for small plans the other orders with the static
+ * deal, or split-K work items (plans whose split and whole items round at the same K);
  * FP64 and FP32: the only schedule -- and keeps the fastest in the plan (gsp2_plan_query
- * reports it).  Every candidate without split-K work items computes bitwise the same P (a
- * tile's arithmetic does not depend on the CTA that runs it); split-K agrees to the last
- * bits.
+ * reports it).  Every candidate computes bitwise the same P (a tile's arithmetic does not depend on
+ * the CTA that runs it).
  *  d_hvals, d_pvals  as for gsp2_density; d_pvals is overwritten
  *  rep               optional output
  * Synchronises `stream`.  Errors: GSP2_E_ARG, GSP2_E_STATE (no workspace), GSP2_E_CUDA, or

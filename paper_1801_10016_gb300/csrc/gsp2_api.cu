@@ -113,6 +113,7 @@ struct gsp2_plan {
   bool use_oz = false;      // FP64 products from FP16 digits (fp64e steps or emulated tail steps)
   bool split_ok = false;    // emulated steps: buffers for split-K work items are in the workspace
   bool split_on = false;    // emulated steps split each tile's K into two work items
+  bool split_tuned = false; // gsp2_autotune has chosen
   bool halves = false;      // unsplit items drain at the halves too: bitwise the sums of split ones
   std::vector<int64_t> pcolptr;
   std::vector<int32_t> prowind;
@@ -123,7 +124,7 @@ struct gsp2_plan {
   char* ws = nullptr;
   size_t ws_size = 0;
   int device = -1;
-  int num_sms = 0;
+  int num_sms = 152;  // of GB300; of the device once a workspace is bound
   cudaStream_t cap_stream = nullptr;
   // emulated adjoint of small plans: the iterates of the next checkpoint segment are rebuilt
   // on a side stream while the reverse steps of the current one run (two digit-set buffers)
@@ -269,6 +270,16 @@ static size_t oz_coh_words(size_t nparts) { return 2 * nparts + sizeof(OzAgain) 
 // stored value of P and the diagonal) up to 64 MB, then ranges of rows (one row at least)
 static int64_t graph_cap(const gsp2_plan* h) {
   return std::max<int64_t>(h->n, std::min<int64_t>(2 * h->pcolptr[(size_t)h->n] + h->n, int64_t(16) << 20));
+}
+
+// Split-K work items unless the options or gsp2_autotune say otherwise: where halves and column pieces together
+// still leave an SM per item (24 tiles on 152 SMs: 0.62 ms per forward against 0.68 without).  A plan that splits, or
+// might have, drains unsplit items at the halves too: both give the same bits.
+static void default_split(gsp2_plan* h) {
+  if (h->split_tuned) return;
+  h->split_on = h->split_ok && (h->opt.split_k == 1 || h->tc_tiles.size() <= (size_t)h->num_sms / 4);
+  h->halves = h->split_on || (h->opt.precision == GSP2_PREC_FP64_EMU && h->min_s > 128 && h->opt.split_k == 0 &&
+                              h->tc_tiles.size() <= 512);
 }
 
 static void build_layout(gsp2_plan* h) {
@@ -422,14 +433,11 @@ static void build_layout(gsp2_plan* h) {
   L.oz_acc2 = 0;
   h->adj_overlap = h->opt.precision == GSP2_PREC_FP64_EMU && k > 1 && h->tc_tiles.size() <= 512;
   // split-K work items: FP64_EMU plans whose parts all exceed 128 orbitals (so that each K
-  // half holds at least one slice); by default they run where halves and column pieces together
-  // still leave an SM per item (24 tiles: 0.62 ms per forward against 0.68 without), while
-  // gsp2_autotune may turn them on for any plan with their buffers
+  // half holds at least one slice); whether they are used by default is decided when a device is bound
+  // (default_split), so the buffers are there for as many tiles as any device would split
   h->split_ok = h->opt.precision == GSP2_PREC_FP64_EMU && h->min_s > 128 &&
-                (h->opt.split_k == 1 || (h->opt.split_k < 0 && h->tc_tiles.size() <= 512));
-  h->split_on = h->split_ok && (h->opt.split_k == 1 || h->tc_tiles.size() <= 152 / 4);
-  h->halves = h->split_on || (h->opt.precision == GSP2_PREC_FP64_EMU && h->min_s > 128 && h->opt.split_k == 0 &&
-                              h->tc_tiles.size() <= 512);
+                (h->opt.split_k == 1 || (h->opt.split_k < 0 && h->tc_tiles.size() <= OZ_MAX_GRID / 4));
+  default_split(h);
   if (h->split_ok) {
     L.split_acc = take(2 * h->tc_tiles.size() * 128 * 128 * sizeof(long long));
     L.split_cnt = take(2 * h->tc_tiles.size() * sizeof(uint32_t));
@@ -868,6 +876,7 @@ extern "C" gsp2_status gsp2_bind_workspace(gsp2_handle h, void* d_ws, size_t byt
   int dev = 0;
   CU(h, cudaGetDevice(&dev));
   CU(h, cudaDeviceGetAttribute(&h->num_sms, cudaDevAttrMultiProcessorCount, dev));
+  default_split(h);
   cudaStream_t s = (cudaStream_t)stream;
   drop_graph(h);
   h->ws = (char*)d_ws;
@@ -1534,8 +1543,11 @@ extern "C" gsp2_status gsp2_autotune(gsp2_handle h, const double* d_hvals, doubl
   if (!fp64_like(prec) && prec_kind(prec) >= 0)
     cand = {{0, 0, 0, 0, 1}, {0, 1, 0, 0, 1}, {0, 0, 0, 0, 0}, {0, 1, 0, 0, 0},
             {0, 0, 1, 0, 0}, {0, 1, 1, 0, 0}, {1, 0, 0, 0, 0}};
-  else if (prec == GSP2_PREC_FP64_EMU && h->split_ok)
+  else if (prec == GSP2_PREC_FP64_EMU && h->split_ok && h->halves)
     cand = {{0, 0, 0, 0, 1}, {0, 1, 0, 0, 1}, {0, 2, 0, 0, 1}, {0, 0, 0, 1, 1}, {0, 1, 0, 1, 1}, {0, 2, 0, 0, 0}};
+  else if (prec == GSP2_PREC_FP64_EMU && h->tc_tiles.size() <= 512 && h->min_s > 128 && h->opt.split_k < 0)
+    // split items would round at other K than this plan's whole ones: the choice must not change the results
+    cand = {{0, 0, 0, 0, 1}, {0, 1, 0, 0, 1}, {0, 2, 0, 0, 1}, {0, 0, 0, 0, 0}, {0, 1, 0, 0, 0}, {0, 2, 0, 0, 0}};
   else if (prec == GSP2_PREC_FP64_EMU) cand = {{0, 0, 0, 0, 1}, {0, 1, 0, 0, 1}, {0, 2, 0, 0, 1}, {0, 2, 0, 0, 0}};
   else cand = {{h->opt.tc_schedule, h->opt.tile_order, h->opt.tile_shape, sp, h->opt.tile_claim}};
   cudaEvent_t e0 = nullptr, e1 = nullptr;
@@ -1552,6 +1564,7 @@ extern "C" gsp2_status gsp2_autotune(gsp2_handle h, const double* d_hvals, doubl
     h->opt.tile_order = c.order;
     h->opt.tile_shape = c.shape;
     h->split_on = c.split != 0 && h->split_ok;
+    h->split_tuned = true;
     order_tc_tiles(h, h->num_sms);
     if (h->tc_order.empty()) return cudaSuccess;
     cudaError_t e = cudaMemcpyAsync(h->ws + h->L.tc_tiles, h->tc_order.data(), h->tc_order.size() * sizeof(Tile),
