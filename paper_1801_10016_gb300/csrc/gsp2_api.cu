@@ -1008,7 +1008,7 @@ extern "C" gsp2_status gsp2_bind_workspace(gsp2_handle h, void* d_ws, size_t byt
     {
       // every iterate and operand arena starts zeroed, so that the padding no step writes
       // stays zero for the steps and conversions that read whole 128-column blocks: the
-      // CUDA-core steps work in 64-column tiles up to roundup(s, 64), the tensor-core steps
+      // CUDA-core steps work in tiles of 16 (FP64) or 64 (FP32) columns, the tensor-core steps
       // skip the 16-column chunks beyond roundup(s, 16)
       const size_t af = (size_t)h->arena_elems * sizeof(float);
       const size_t ab = (size_t)h->arena_elems * sizeof(double);
@@ -1768,16 +1768,6 @@ extern "C" gsp2_status gsp2_step_times(gsp2_handle h, float* ms, int32_t cap) {
   return GSP2_OK;
 }
 
-// Queue the adjoint on `s`: seed, then per checkpoint segment (last first) the
-// recomputed iterates and the reverse steps, then the scatter-add onto H.  The
-// schedule covers max_steps; kernels for steps beyond the applied count return at once.
-// Adjoint of an emulated-FP64 plan on the BF16 tensor cores.  For each checkpoint segment
-// the iterates X_{c0} .. X_{c0+k-1} are rebuilt as digit sets (digits of the checkpoint,
-// then emulated steps with the recorded branches); every reverse step multiplies the
-// digits of X_{i-1} with those of Xbar / 2^sig and leaves the new Xbar's per-part scales
-// (from its row norms, summed in the step's epilogue), and the new digits follow.  The
-// seed's scales come from a separate norm pass.  Xbar is kept in its upper 128-tiles like
-// the forward iterates.
 // Steps the adjoint schedules (launches for steps the forward did not apply return at once):
 // max_steps (FP64 plans: plus their tail steps), or the applied count once gsp2_sync_status
 // has read it (the loop's steps for the low-precision plans, whose FP64 tail steps are
@@ -1789,6 +1779,13 @@ static int backward_steps(gsp2_plan* h) {
   return h->known_steps >= T ? std::min(h->known_steps - T, h->opt.max_steps) : h->opt.max_steps;
 }
 
+// Adjoint of an emulated-FP64 plan on the FP16 tensor cores.  For each checkpoint segment
+// the iterates X_{c0} .. X_{c0+k-1} are rebuilt as digit sets (digits of the checkpoint,
+// then emulated steps with the recorded branches); every reverse step multiplies the
+// digits of X_{i-1} with those of Xbar / 2^sig and leaves the new Xbar's per-part scales
+// (from its row norms, summed in the step's epilogue), and the new digits follow.  The
+// seed's scales come from a separate norm pass.  Xbar is kept in its upper 128-tiles like
+// the forward iterates.
 static gsp2_status enqueue_backward_emu(gsp2_plan* h, const double* pbar, double* hbar, cudaStream_t s) {
   const WsLayout& L = h->L;
   char* w = h->ws;
@@ -1914,6 +1911,9 @@ static gsp2_status enqueue_backward_emu(gsp2_plan* h, const double* pbar, double
   return GSP2_OK;
 }
 
+// Queue the adjoint on `s`: seed, then per checkpoint segment (last first) the
+// recomputed iterates and the reverse steps, then the scatter-add onto H.  The
+// schedule covers max_steps; kernels for steps beyond the applied count return at once.
 static gsp2_status enqueue_backward(gsp2_plan* h, const double* pbar, double* hbar, cudaStream_t s) {
   if (h->opt.precision == GSP2_PREC_FP64_EMU) return enqueue_backward_emu(h, pbar, hbar, s);
   const WsLayout& L = h->L;

@@ -53,17 +53,6 @@ __global__ void __launch_bounds__(256) adj_seed_kernel(const PartDesc* __restric
 // The Xbar buffers alternate with (n - step) so that skipped steps keep the parity: input
 // xb[(n - step) & 1], output xb[(n - step + 1) & 1], n the steps applied by the forward;
 // steps above n are skipped.
-// R consecutive elements (R elements aligned) in vector stores.
-template <int R>
-__device__ __forceinline__ void store_row(double* p, const double (&v)[R]) {
-  if constexpr (R == 1) {
-    *p = v[0];
-  } else {
-#pragma unroll
-    for (int i = 0; i < R; i += 2) *reinterpret_cast<double2*>(p + i) = make_double2(v[i], v[i + 1]);
-  }
-}
-
 template <typename T>
 __global__ void __launch_bounds__(256, 4) adj_step_kernel(const PartDesc* __restrict__ parts,
                                                           const Tile* __restrict__ tiles, const T* __restrict__ Xall,
@@ -72,7 +61,7 @@ __global__ void __launch_bounds__(256, 4) adj_step_kernel(const PartDesc* __rest
                                                           int step) {
   static_assert(sizeof(T) == 8, "the native FP64 adjoint");
   constexpr int EDGE = SQ64_TILE, ABK = 16;
-  constexpr int R = EDGE / 16;  // a thread's block is R x R
+  static_assert(EDGE == 16, "one entry of the tile a thread");
   const int n = *(volatile const int32_t*)&st->steps;
   if (step > n) return;
   const T* XBin = ((n - step) & 1) ? xb1 : xb0;
@@ -106,12 +95,7 @@ __global__ void __launch_bounds__(256, 4) adj_step_kernel(const PartDesc* __rest
     cp_async_commit();
   };
 
-  T acc[R][R];
-#pragma unroll
-  for (int i = 0; i < R; ++i)
-#pragma unroll
-    for (int j = 0; j < R; ++j) acc[i][j] = T(0);
-
+  T acc = T(0);
   const int nk = kend / ABK;
   load_slice(0, 0);
   for (int it = 0; it < nk; ++it) {
@@ -124,46 +108,17 @@ __global__ void __launch_bounds__(256, 4) adj_step_kernel(const PartDesc* __rest
     }
     __syncthreads();
 #pragma unroll
-    for (int kk = 0; kk < ABK; ++kk) {
-      T a1[R], b1[R], a2[R], b2[R];
-#pragma unroll
-      for (int q = 0; q < R; ++q) {
-        a1[q] = S1[buf][kk][tx * R + q];
-        b1[q] = S2[buf][kk][ty * R + q];
-        a2[q] = S3[buf][kk][tx * R + q];
-        b2[q] = S4[buf][kk][ty * R + q];
-      }
-#pragma unroll
-      for (int i = 0; i < R; ++i)
-#pragma unroll
-        for (int j = 0; j < R; ++j) acc[i][j] = fma(a2[i], b2[j], fma(a1[i], b1[j], acc[i][j]));
-    }
+    for (int kk = 0; kk < ABK; ++kk)
+      acc = fma(S3[buf][kk][tx], S4[buf][kk][ty], fma(S1[buf][kk][tx], S2[buf][kk][ty], acc));
     __syncthreads();
   }
 
   const int8_t al = alpha[step];
   T* O = XBout + p.off;
-  const int rb = r0 + tx * R, cb = c0 + ty * R;
-#pragma unroll
-  for (int j = 0; j < R; ++j) {
-    const int c = cb + j;
-#pragma unroll
-    for (int i = 0; i < R; ++i) {
-      const T z = acc[i][j];
-      acc[i][j] = (al > 0) ? (T(2) * B[(int64_t)c * ld + rb + i] - z) : z;
-    }
-    T v[R];
-#pragma unroll
-    for (int i = 0; i < R; ++i) v[i] = acc[i][j];
-    store_row(O + (int64_t)c * ld + rb, v);
-  }
-  if (t.ti != t.tj) {
-#pragma unroll
-    for (int i = 0; i < R; ++i) {
-      const int r = rb + i;
-      store_row(O + (int64_t)r * ld + cb, acc[i]);
-    }
-  }
+  const int64_t r = r0 + tx, c = c0 + ty;
+  const T z = al > 0 ? T(2) * B[c * ld + r] - acc : acc;
+  O[c * ld + r] = z;
+  if (t.ti != t.tj) O[r * ld + c] = z;
 }
 
 // dL/dH on the CSR pattern: for every stored (r, col), the sum over the parts k that

@@ -597,22 +597,6 @@ __device__ __forceinline__ void oz_drain_low(uint32_t taddr, int sgn, const Mark
 constexpr unsigned long long kOzOffset = OzSixth::offset + OzSlot<0, 3>::offset + OzSlot<0, 2>::offset +
                                          OzSlot<1, 1>::offset + OzSlot<0, 0>::offset + OzSlot<0, 1>::offset;
 
-// z of a warp's 32 rows x 16 columns (lane l, z[j]: row l, column j) transposed within each half
-// warp: lane l, z[j] becomes row 16 (l / 16) + j, column l % 16.
-__device__ __forceinline__ void transpose16(long long (&z)[16], int lane) {
-#pragma unroll
-  for (int d = 8; d > 0; d >>= 1) {
-    const bool up = lane & d;
-#pragma unroll
-    for (int j = 0; j < 16; ++j) {
-      if (j & d) continue;
-      const long long got = __shfl_xor_sync(0xffffffffu, up ? z[j] : z[j + d], d);
-      if (up) z[j] = got;
-      else z[j + d] = got;
-    }
-  }
-}
-
 // |v| 2^-56 as FP32 (integer instructions, truncated: at most 2^-23 below), for the row
 // norms of the adjoint's new Xbar on its fixed-point grid.
 __device__ __forceinline__ float fixed_to_f32_abs(long long v) {
@@ -644,10 +628,6 @@ __device__ __forceinline__ float warp_colsum16(const float (&v)[16], int lane, i
   return a1;
 }
 
-// ADJ: the adjoint step (see the top of the file): K runs over [Xbar | X] x [X ; Xbar],
-// diagonal tiles load both operands, the epilogue forms Xbar_new in FP64 without digits
-// or traces and adds its squared row norms (FP32, on the grid of the input scale); the last
-// block turns them into each part's new scale.
 // Predicated evict-first stores: the columns of a diagonal tile differ in the lanes that store,
 // and a branch per column costs more than the stores.
 __device__ __forceinline__ void store_word_if(bool on, long long* q, long long v) {
@@ -738,6 +718,10 @@ __device__ __forceinline__ void oz_read_item(const OzStepArgs& a, int it, int br
   w->brief = brief;
   w->rounds = oz_rounds<WIDE>(oz_slices<ADJ, WIDE>(p.s, a.split ? code & 1 : -1, brief), a.halves, brief);
 }
+// ADJ: the adjoint step (see the top of the file): K runs over [Xbar | X] x [X ; Xbar],
+// diagonal tiles load both operands, the epilogue forms Xbar_new in FP64 without digits
+// or traces and adds its squared row norms (FP32, on the grid of the input scale); the block that ends the
+// launch turns them into each part's new scale.
 template <bool ADJ, bool WIDE>
 __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(const __grid_constant__ OzStepArgs a) {
   constexpr int T = OZ_SLICES;

@@ -412,22 +412,6 @@ __device__ __forceinline__ void store_element_if(bool on, float* master, void* h
   }
 }
 
-// x of a warp's 32 rows x 16 columns (lane l, x[j]: row l, column j) transposed within each half
-// warp: lane l, x[j] becomes row 16 (l / 16) + j, column l % 16.
-__device__ __forceinline__ void transpose16(float (&x)[16], int lane) {
-#pragma unroll
-  for (int d = 8; d > 0; d >>= 1) {
-    const bool up = lane & d;
-#pragma unroll
-    for (int j = 0; j < 16; ++j) {
-      if (j & d) continue;
-      const float got = __shfl_xor_sync(0xffffffffu, up ? x[j] : x[j + d], d);
-      if (up) x[j] = got;
-      else x[j + d] = got;
-    }
-  }
-}
-
 template <int KIND, int NPROD, int MODE = TC_STEP>
 __global__ void __launch_bounds__(TC_THREADS, 1) square_tc_persistent_kernel(TcStepArgs a) {
   constexpr int NOPS = NPROD == 3 ? 4 : 2;
@@ -1476,9 +1460,7 @@ cudaError_t launch_gather_lp(int kind, int nprod, const PartDesc* parts, const C
     return go(gather_lp_kernel<1, 3>);
   else if (kind == 2 && nprod == 3)
     return go(gather_lp_kernel<2, 3>);
-  else
-    return cudaErrorInvalidValue;
-  return cudaGetLastError();
+  return cudaErrorInvalidValue;
 }
 
 // FP32 master of the last low-precision iterate -> FP64 arena for the tail steps.

@@ -34,6 +34,23 @@ __device__ __forceinline__ uint64_t global_ns() {
   return t;
 }
 
+// x of a warp's 32 rows x 16 columns (lane l, x[j]: row l, column j) transposed within each half
+// warp: lane l, x[j] becomes row 16 (l / 16) + j, column l % 16.
+template <typename T>
+__device__ __forceinline__ void transpose16(T (&x)[16], int lane) {
+#pragma unroll
+  for (int d = 8; d > 0; d >>= 1) {
+    const bool up = lane & d;
+#pragma unroll
+    for (int j = 0; j < 16; ++j) {
+      if (j & d) continue;
+      const T got = __shfl_xor_sync(0xffffffffu, up ? x[j] : x[j + d], d);
+      if (up) x[j] = got;
+      else x[j + d] = got;
+    }
+  }
+}
+
 // Bounded wait: gives up after kWaitNs nanoseconds, or at once when another block
 // has already given up (the shared abort flag), and then raises the flag itself.
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, int32_t* abort_flag) {
