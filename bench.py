@@ -35,7 +35,7 @@ NOMINAL = {"bf16": 2250.0, "tf32": 1100.0, "fp64": 1.25}
 # scaled to tb30k by arena elements; an entry is dropped when its kernel changes, and the
 # line then reports null
 TB8K_TO_TB30K = 191545344 / 38469632
-TRAFFIC = {("tb30k", "fp64"): 0.4998e9 * TB8K_TO_TB30K, ("tb30k", "fp64e"): 0.6776e9 * TB8K_TO_TB30K,
+TRAFFIC = {("tb30k", "fp64"): 0.4998e9 * TB8K_TO_TB30K, ("tb30k", "fp64e"): 0.6774e9 * TB8K_TO_TB30K,
            ("tb30k", "fp16x3"): 0.2392e9 * TB8K_TO_TB30K, ("tb30k", "tf32x3"): 0.7147e9 * TB8K_TO_TB30K}
 
 

@@ -377,8 +377,9 @@ __global__ void __launch_bounds__(256) oz_digits_kernel(const PartDesc* __restri
 // iterate is written with evict-first stores: the next step reads it after this launch,
 // and keeping it out of L2 leaves room for the digit panels the running tiles share.  The last block
 // runs the step bookkeeping, after it has formed again the parts whose sums were found too large (brief
-// items, see the top).  K beyond 2048 is taken in rounds of both passes.  n = 30000 (256 parts), per step: narrow 1.69, wide 1.59 ms; the MMAs at the
-// measured 16-bit peak take 1.15, without loads or epilogue 1.29, with loads 1.32, with drains 1.43.
+// items, see the top).  K beyond 2048 is taken in rounds of both passes.  n = 30000 (256 parts), per step:
+// narrow 1.69, wide 1.59 ms before the drains looked at every sum, 1.62 since; the MMAs at the measured 16-bit
+// peak take 1.15, without loads or epilogue 1.29, with loads 1.32, with drains 1.43.
 //
 // 20 warps: warps 0 and 2 TMA (rows I and rows J: one warp's work per tile would hold
 // the ring back), warp 1 TMEM owner and MMA issuer, warps 4..19 epilogue
@@ -826,7 +827,8 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(const __grid_con
   const int place = ADJ ? n - step + 1 : step, brief_to = !coherent ? -1 : (rec ? place : place - 1);
   if (threadIdx.x == 0 && brief_to >= 0 && s_items->code >= 0 && a.coh[s_items->part] <= brief_to) {
     s_items->brief = 1;
-    s_items->rounds = oz_rounds<WIDE>(oz_slices<ADJ, WIDE>(s_items->s, split ? s_items->code & 1 : -1, true), false, true);
+    s_items->rounds =
+        oz_rounds<WIDE>(oz_slices<ADJ, WIDE>(s_items->s, split ? s_items->code & 1 : -1, true), false, true);
   }
   // digit buffers read / written (the adjoint's sets are passed explicitly)
   const int dbi = (ADJ || rec) ? 0 : (step - 1) & 1, dbo = (ADJ || rec) ? 0 : step & 1;
@@ -1430,7 +1432,7 @@ __global__ void __launch_bounds__(OZ_THREADS, 1) oz_step_kernel(const __grid_con
       // the wide form, whose registers that suits: marked as in the narrow one it spills 370 bytes and takes 3 %
       // longer; the narrow one, marking at the end, takes 0.7 % longer at n = 512.)
       float top = 0.0f;
-      auto mark_part = [&](int part) {  // (of a brief item, which can reach 2^24 only if X has left [0, 1], it does nothing)
+      auto mark_part = [&](int part) {  // (a brief item reaches 2^24 only if X has left [0, 1]; it is not formed again)
         a.coh_new[part] = 1;
         atomicOr(&s_walk, 1);  // (brief items come after the decision)
       };
