@@ -167,3 +167,56 @@ def test_reverse_step_on_a_seed_of_one_value(n):
     print(f"n={n}: sums 2^{np.log2(t0 + t1):.1f}, left out {(l0 + l1):.1e}, max|dHbar| {err:.2e} of {tol:.2e}")
     assert t0 + t1 >= 2.0 ** 24
     assert err <= tol
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("split", [-1, 1])
+def test_one_coherent_part_among_others(split):
+    """A ring of 1,500 in one part beside six gapped blocks of 160 in parts of their own: P and Hbar against the
+    native FP64 path on the same branches (the parts formed again and rebuilt among the others), and the same bits
+    for claimed and dealt items, either order, and launches without a graph."""
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import __graft_entry__
+    __graft_entry__.build()
+    from paper_1801_10016_gb300 import gsp2
+    rng = np.random.default_rng(12)
+    sizes = [160, 160, 160, 1500, 160, 160, 160]
+    blocks = []
+    for m in sizes:
+        if m == 1500:
+            blocks.append(ring(m))
+        else:
+            b = rng.standard_normal((m, m)) * 0.02
+            blocks.append(np.diag(np.where(np.arange(m) % 2, 1.2, -1.2)) + 0.5 * (b + b.T))
+    n = sum(sizes)
+    starts = np.concatenate([[0], np.cumsum(sizes)])
+    part = np.repeat(np.arange(len(sizes), dtype=np.int32), sizes)
+    rowptr = np.concatenate([[0], np.cumsum(np.repeat(sizes, sizes))]).astype(np.int64)
+    colind = np.concatenate([np.arange(starts[k], starts[k + 1]) for k, m in enumerate(sizes) for _ in range(m)]).astype(np.int32)
+    h = torch.from_numpy(np.concatenate([b.ravel() for b in blocks])).to("cuda:0")
+
+    def make(precision, **kw):
+        return gsp2.GSP2(n, rowptr, colind, n // 2, part, len(sizes), np.zeros(n + 1, np.int64), np.zeros(0, np.int32),
+                         device="cuda:0", precision=precision, max_steps=36, fp64_tail_steps=0, ckpt_every=5, **kw)
+
+    plan = make("fp64e", split_k=split)
+    p = plan.density(h)
+    alphas = plan.history()["alphas"]
+    torch.manual_seed(5)
+    pb = torch.randn(plan.nnz_p, dtype=torch.float64, device="cuda:0")
+    hb = plan.backward(pb)
+    alpha = torch.zeros(plan.alpha_len, dtype=torch.int8, device="cuda:0")
+    alpha[:len(alphas)] = torch.tensor(alphas, dtype=torch.int8)
+    ref = make("fp64")
+    want = ref.density(h, alpha=alpha, mode="replay", nsteps=len(alphas))
+    want_h = ref.backward(pb)
+    err, err_h = float((p - want).abs().max()), float((hb - want_h).abs().max())
+    scale = max(1.0, float(want_h.abs().max()))
+    print(f"split {split}: {len(alphas)} steps, max|dP| {err:.1e}, max|dHbar| {err_h:.1e} of {scale:.1e}")
+    assert err <= 1e-10 and err_h <= 1e-9 * scale
+    for kw in (dict(tile_claim=0), dict(tile_order=0), dict(use_graph=0)):
+        other = make("fp64e", split_k=split, **kw)
+        assert torch.equal(other.density(h), p), kw
+        assert torch.equal(other.backward(pb), hb), kw
